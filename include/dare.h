@@ -249,7 +249,7 @@ dare_status_t dare_rmsnorm(const void* x, const float* gain, void* y, int64_t ro
                            void* cuda_stream);
 /* *tau_out (device) = the k-th smallest of n_tokens float32 scores (k clamped to [0, n_tokens]; k = 0: -inf,
  * k = n_tokens or beyond the scores that are numbers: +inf), the threshold that reuses the k least-drifted tokens under
- * Eq. 2 (Sec. 3.1).  One CTA, exact; 1 <= n_tokens <= 2^24. */
+ * Eq. 2 (Sec. 3.1).  Exact; 1 <= n_tokens <= 2^24. */
 dare_status_t dare_score_kth(const float* scores, int64_t n_tokens, int64_t k, float* tau_out, void* cuda_stream);
 size_t dare_select_compact_scratch_bytes(int64_t n_tokens);
 dare_status_t dare_select_compact(const float* scores, int64_t n_tokens, float threshold, int32_t* idx, int32_t* count,

@@ -93,15 +93,19 @@ dare_status_t check_handle(const dare_layer_t* L) {
 }  // namespace
 namespace dare {
 // A step that was asked to reuse its k least-drifted tokens works its threshold out from the scores the Q projection
-// just left (one more kernel ahead of the selection); returns where the selection finds it, or nullptr when the
-// caller's threshold applies (also on a first step and in dense mode, which refresh everything anyway).
-const float* step_threshold_on_device(dare_layer* L, const StepGeom& g, int mode, cudaStream_t st, int* launches) {
-  L->last_tau_on_device = false;
-  if (L->reuse_count < 0 || !L->has_prev || mode == DARE_MODE_DENSE) return nullptr;
-  launch_kth_score(L->buf.scores, g.tokens(), L->reuse_count, L->buf.tau_dev, st);
+// just left: inside the selection kernel, or with very many tokens one launch ahead of it.  Without such a request, on a
+// first step and in dense mode (which refresh everything anyway) the caller's threshold applies.
+void select_step(dare_layer* L, const StepGeom& g, int mode, float tau, bool beside_predecessor, cudaStream_t st,
+                 int* launches) {
+  const Buffers& B = L->buf;
+  const bool all = !L->has_prev || mode == DARE_MODE_DENSE;
+  const bool own = L->reuse_count >= 0 && !all, inside = own && kth_score_in_select(g.tokens());
+  L->last_tau_on_device = own;
+  if (own && !inside) { launch_kth_score(B.scores, g.tokens(), L->reuse_count, B.tau_dev, st); ++*launches; }
+  launch_select(B.scores, tau, all, g, B.idx, B.count, B.batch_off, B.delta, st, beside_predecessor,
+                own ? B.tau_dev : nullptr, inside ? L->reuse_count : -1);
   ++*launches;
-  L->last_tau_on_device = true;
-  return L->buf.tau_dev;
+  if (L->inject) inject_selection_error(L, g, st);
 }
 // Diagnostics (dare_layer_debug_inject): overwrites one value of the selection just made, once.
 void inject_selection_error(dare_layer* L, const StepGeom& g, cudaStream_t st) {
@@ -132,10 +136,7 @@ dare_status_t step_simt(dare_layer_t* L, const T* x, const StepGeom& g, int mode
   launch_q_post_simt<T>(B.tmp, d, B.rope_cs, B.q_prev, B.scores, has_prev, (T*)B.q, g, st); ++launches;
   // lines 4-5: refresh set as a compacted index list; Sec. 4 staleness
   prof_mark(L, SLOT_SELECT, st);
-  const float* tau_dev = step_threshold_on_device(L, g, mode, st, &launches);
-  launch_select(B.scores, tau, !has_prev || mode == DARE_MODE_DENSE, g, B.idx, B.count, B.batch_off, B.delta, st, false,
-                tau_dev); ++launches;
-  inject_selection_error(L, g, st);
+  select_step(L, g, mode, tau, false, st, &launches);
   // K/V: Alg. 1 lines 6-9 (refresh set only) or Alg. 2 line 7 (all rows)
   const int* kv_idx = kv_sparse ? B.idx : nullptr;
   const int* kv_cnt = kv_sparse ? B.count : nullptr;
@@ -339,8 +340,7 @@ dare_status_t dare_score_kth(const float* scores, int64_t n_tokens, int64_t k, f
   if (!scores || !tau_out) return DARE_ERR_INVALID_ARG;
   if (n_tokens <= 0 || n_tokens > (int64_t)1 << 24) return DARE_ERR_SHAPE;
   const int kk = k < 0 ? 0 : (k > n_tokens ? (int)n_tokens : (int)k);
-  launch_kth_score(scores, (int)n_tokens, kk, tau_out, (cudaStream_t)cuda_stream);
-  CUDA_TRY(cudaGetLastError());
+  CUDA_TRY(launch_kth_score(scores, (int)n_tokens, kk, tau_out, (cudaStream_t)cuda_stream));
   return DARE_OK;
 }
 

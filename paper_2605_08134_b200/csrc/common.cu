@@ -277,72 +277,99 @@ template void launch_rmsnorm<__nv_bfloat16>(const __nv_bfloat16*, const float*, 
 // ---- the step's own threshold (Sec. 3.1 speaks of dynamic thresholding; the reuse-rate allocation turns a rate into
 // the matching quantile of the drift scores): tau_t = the k-th smallest score of this step, so that the k tokens that
 // drifted least are reused (and every token tied with the k-th).  Exact selection by four passes over the scores'
-// order-preserving 32-bit keys, eight bits at a time (histogram in shared memory, then the bin that holds rank k);
-// one CTA: a step has at most a few 10^4 tokens.  NaN scores sort last and are never reused.
+// order-preserving 32-bit keys, eight bits at a time.  NaN scores sort last and are never reused.
 // k <= 0: tau = -inf (nothing reused); k >= n or more than the scores that are numbers: +inf.
-__device__ __forceinline__ unsigned score_key(float s) {
-  if (s != s) return 0xffffffffu;
-  const unsigned u = __float_as_uint(s);
-  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
-__global__ void __launch_bounds__(1024) kth_score_kernel(const float* __restrict__ scores, int n, int k,
-                                                         float* __restrict__ tau_out) {
+// A step of at most kKthInCta tokens has the selection kernel do it: every CTA of that launch keeps all keys in
+// registers (16 per thread), so the passes touch shared memory only, and the step has no launch for it.  What bounds it
+// is the chain of the passes (histogram -> scan over 256 bins by one warp -> next digit), three barriers each.
+// (It was a launch of its own that read the scores once per pass and walked the bins with one thread.)
+constexpr int kKthInCta = 16384;
+constexpr int kKthPerThread = kKthInCta / 1024;
+template <int KPT>
+__device__ float kth_in_cta(const float* __restrict__ scores, int n, int k) {
   __shared__ int hist[256];
-  __shared__ unsigned s_prefix;
-  __shared__ int s_rank;
-  ptx::pdl_wait();
-  ptx::pdl_launch_dependents();
-  if (k <= 0 || k >= n) {
-    if (threadIdx.x == 0) *tau_out = __int_as_float(k <= 0 ? 0xff800000 : 0x7f800000);
-    return;
+  __shared__ int s_bin, s_rank;
+  if (k <= 0 || k >= n) return __int_as_float(k <= 0 ? 0xff800000 : 0x7f800000);
+  const int lane = threadIdx.x & 31;
+  unsigned key[KPT];
+#pragma unroll
+  for (int i = 0; i < KPT; ++i) {
+    const int t = i * 1024 + (int)threadIdx.x;
+    key[i] = t < n ? score_key(scores[t]) : kKeyNaN;
   }
   unsigned prefix = 0u, mask = 0u;
   int rank = k;                                       // rank (1-based) of the wanted key among the keys that match the prefix
+#pragma unroll 1
   for (int shift = 24; shift >= 0; shift -= 8) {
     if (threadIdx.x < 256) hist[threadIdx.x] = 0;
+    if (threadIdx.x == 0) s_bin = -1;
     __syncthreads();
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-      const unsigned key = score_key(scores[i]);
-      if ((key & mask) == prefix) atomicAdd(&hist[(key >> shift) & 255u], 1);
-    }
+#pragma unroll
+    for (int i = 0; i < KPT; ++i)
+      if (key[i] != kKeyNaN && (key[i] & mask) == prefix) atomicAdd(&hist[(key[i] >> shift) & 255u], 1);
     __syncthreads();
-    if (threadIdx.x == 0) {
-      int cum = 0, b = 0;
-      for (; b < 255; ++b) {
-        if (cum + hist[b] >= rank) break;
-        cum += hist[b];
+    if (threadIdx.x < 32) {
+      int c[8], mine = 0;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) { c[j] = hist[lane * 8 + j]; mine += c[j]; }
+      int inc = mine;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += v;
       }
-      s_prefix = prefix | ((unsigned)b << shift);
-      s_rank = rank - cum;
+      int cum = inc - mine;
+      if (cum < rank && rank <= inc) {                // exactly one lane, unless rank is past the scores that are numbers
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          if (cum < rank && rank <= cum + c[j]) { s_bin = lane * 8 + j; s_rank = rank - cum; }
+          cum += c[j];
+        }
+      }
     }
     __syncthreads();
-    prefix = s_prefix;
+    if (s_bin < 0) return __int_as_float(0x7f800000);             // rank k falls among the NaN scores: every number is reused
+    prefix |= (unsigned)s_bin << shift;
     rank = s_rank;
     mask |= 255u << shift;
+    __syncthreads();                                              // (s_bin is cleared for the next digit)
   }
-  if (threadIdx.x == 0) {
-    const unsigned u = (prefix & 0x80000000u) ? (prefix & 0x7fffffffu) : ~prefix;
-    float tau = __uint_as_float(u);
-    if (tau != tau) tau = __int_as_float(0x7f800000);         // rank k falls among the NaN scores: every number is reused
-    *tau_out = tau;
-  }
+  return key_score(prefix);
 }
-void launch_kth_score(const float* scores, int n, int k, float* tau_out, cudaStream_t st) {
-  launch_pdl(kth_score_kernel, dim3(1), dim3(1024), 0, st, 1, scores, n, k, tau_out);
+__global__ void __launch_bounds__(1024) kth_score_kernel(const float* __restrict__ scores, int n, int k,
+                                                         float* __restrict__ tau_out) {
+  ptx::pdl_wait();
+  ptx::pdl_launch_dependents();
+  const float tau = kth_in_cta<kKthPerThread>(scores, n, k);
+  if (threadIdx.x == 0) *tau_out = tau;
+}
+bool kth_score_in_select(int n) { return n <= kKthInCta; }
+cudaError_t launch_kth_score(const float* scores, int n, int k, float* tau_out, cudaStream_t st) {
+  if (n > kKthInCta) return launch_kth_score_large(scores, n, k, tau_out, st);
+  return launch_pdl(kth_score_kernel, dim3(1), dim3(1024), 0, st, 1, scores, n, k, tau_out);
 }
 
 constexpr int kSelPerThread = 4;
+constexpr int kSmallTokens = 2048;      // one token per thread and chunk up to here, four beyond
+// kKth: the threshold is the step's own reuse_count-th smallest score, worked out here and left at *tau_dev;
+// otherwise tau_dev (if given) is where an earlier launch left it.
+template <bool kKth>
 __global__ void __launch_bounds__(1024) select_kernel(const float* __restrict__ scores, float tau, int select_all,
                                                       StepGeom g, int* __restrict__ idx, int* __restrict__ count,
                                                       int* __restrict__ batch_off, int* __restrict__ delta,
-                                                      int wait_at_end, const float* __restrict__ tau_dev) {
+                                                      int wait_at_end, float* __restrict__ tau_dev, int reuse_count) {
   __shared__ int warp_tot[32];
   __shared__ int before_chunk;
   if (threadIdx.x == 0) before_chunk = 0;
   if (!wait_at_end) ptx::pdl_wait();
   ptx::pdl_launch_dependents();
-  if (tau_dev != nullptr) tau = *tau_dev;                // the threshold the step worked out itself
   const int T = g.tokens();
+  if (kKth) {
+    tau = kth_in_cta<kKthPerThread>(scores, T, reuse_count);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *tau_dev = tau;
+  } else if (tau_dev != nullptr) {
+    tau = *tau_dev;                                      // the threshold the step worked out itself
+  }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   constexpr int kChunk = 1024 * kSelPerThread;
   const int chunk0 = (int)blockIdx.x * kChunk;            // this CTA's chunk: tokens [chunk0, chunk0 + kChunk)
@@ -425,10 +452,11 @@ __global__ void __launch_bounds__(1024) select_kernel(const float* __restrict__ 
 
 // The same for short steps: one token per thread and chunk of 1024, warp ballot + popcount (less index arithmetic
 // per token, which is what a step of a few hundred tokens pays for).
+template <bool kKth>
 __global__ void __launch_bounds__(1024) select_small_kernel(const float* __restrict__ scores, float tau, int select_all,
                                                       StepGeom g, int* __restrict__ idx, int* __restrict__ count,
                                                       int* __restrict__ batch_off, int* __restrict__ delta,
-                                                      int wait_at_end, const float* __restrict__ tau_dev) {
+                                                      int wait_at_end, float* __restrict__ tau_dev, int reuse_count) {
   __shared__ int warp_excl[32];
   __shared__ int chunk_total;
   const int T = g.tokens();
@@ -436,7 +464,12 @@ __global__ void __launch_bounds__(1024) select_small_kernel(const float* __restr
   for (int t = threadIdx.x * 32; t < T; t += 1024 * 32) ptx::prefetch_l2(delta + g.cache_row(t));
   if (!wait_at_end) ptx::pdl_wait();
   ptx::pdl_launch_dependents();
-  if (tau_dev != nullptr) tau = *tau_dev;
+  if (kKth) {
+    tau = kth_in_cta<kSmallTokens / 1024>(scores, T, reuse_count);
+    if (threadIdx.x == 0) *tau_dev = tau;
+  } else if (tau_dev != nullptr) {
+    tau = *tau_dev;
+  }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int base = 0;
   for (int start = 0; start < T; start += 1024) {
@@ -481,16 +514,20 @@ __global__ void __launch_bounds__(1024) select_small_kernel(const float* __restr
 
 // beside_predecessor: the selection refreshes every token (it reads no scores) and nothing the kernel before it in the
 // stream touches, so it runs beside that kernel and waits for it only before it leaves.
+// reuse_count >= 0: the threshold is the reuse_count-th smallest score (left at *tau_dev); otherwise tau, or *tau_dev
+// if tau_dev is given.
 void launch_select(const float* scores, float tau, bool select_all, const StepGeom& g, int* idx, int* count,
-                   int* batch_off, int* delta, cudaStream_t st, bool beside_predecessor, const float* tau_dev) {
+                   int* batch_off, int* delta, cudaStream_t st, bool beside_predecessor, float* tau_dev, int reuse_count) {
   const int all = (select_all || scores == nullptr) ? 1 : 0;
   const int late = (beside_predecessor && all) ? 1 : 0;
-  if (g.tokens() <= 2048)
-    launch_pdl(select_small_kernel, dim3(1), dim3(1024), 0, st, 1, scores, tau, all, g, idx, count, batch_off, delta, late,
-               tau_dev);
+  const bool kth = !all && reuse_count >= 0;
+  if (g.tokens() <= kSmallTokens)
+    launch_pdl(kth ? select_small_kernel<true> : select_small_kernel<false>, dim3(1), dim3(1024), 0, st, 1, scores, tau, all, g,
+               idx, count, batch_off, delta, late, tau_dev, reuse_count);
   else
-    launch_pdl(select_kernel, dim3((g.tokens() + 1024 * kSelPerThread - 1) / (1024 * kSelPerThread)), dim3(1024), 0, st, 1,
-               scores, tau, all, g, idx, count, batch_off, delta, late, tau_dev);
+    launch_pdl(kth ? select_kernel<true> : select_kernel<false>,
+               dim3((g.tokens() + 1024 * kSelPerThread - 1) / (1024 * kSelPerThread)), dim3(1024), 0, st, 1, scores, tau, all, g,
+               idx, count, batch_off, delta, late, tau_dev, reuse_count);
 }
 
 // ------------------------------------------------------------------------------------------------ diagnostics

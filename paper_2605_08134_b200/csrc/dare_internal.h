@@ -40,6 +40,16 @@ __device__ __forceinline__ bool slice_ok(int lo, int hi, int cap, int* status) {
   flag_device_check(status);
   return false;
 }
+// Order-preserving 32-bit keys of scores; NaN (any) sorts last.
+constexpr unsigned kKeyNaN = 0xffffffffu;
+__device__ __forceinline__ unsigned score_key(float s) {
+  if (s != s) return kKeyNaN;
+  const unsigned u = __float_as_uint(s);
+  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+__device__ __forceinline__ float key_score(unsigned key) {
+  return __uint_as_float((key & 0x80000000u) ? (key & 0x7fffffffu) : ~key);
+}
 #endif
 
 // Geometry of one step, passed by value to kernels.
@@ -118,9 +128,14 @@ void launch_copy_reused_rows(const T* yc, T* y, const int* delta, const StepGeom
                              const int* gate_count = nullptr, int gate_hi = 0);   // leaves at once when *gate_count >= gate_hi
 void launch_select(const float* scores, float tau, bool select_all, const StepGeom& g, int* idx, int* count,
                    int* batch_off, int* delta, cudaStream_t st, bool beside_predecessor = false,
-                   const float* tau_dev = nullptr);   // tau_dev: read the threshold from device memory instead
-// *tau_out = the k-th smallest of n scores (see common.cu); one CTA
-void launch_kth_score(const float* scores, int n, int k, float* tau_out, cudaStream_t st);
+                   float* tau_dev = nullptr, int reuse_count = -1);
+// tau_dev alone: read the threshold from device memory; with reuse_count >= 0 (kth_score_in_select steps only) the
+// selection works it out from the scores and leaves it there
+bool kth_score_in_select(int n);
+// *tau_out = the k-th smallest of n scores: one CTA up to kth_score_in_select's limit (common.cu), one cluster beyond
+// (select_large.cu)
+cudaError_t launch_kth_score(const float* scores, int n, int k, float* tau_out, cudaStream_t st);
+cudaError_t launch_kth_score_large(const float* scores, int n, int k, float* tau_out, cudaStream_t st);
 template <typename T>
 void launch_gather_rows(const T* src, const int* idx, const int* count, T* dst, int max_rows, int d, cudaStream_t st);
 // dst[r, :] = src[idx[r] (or its cache row), :] for the rows of a step's refresh set

@@ -82,7 +82,8 @@ inline void prof_end(dare_layer* L, cudaStream_t st) {
   if (L->prof_on) cudaEventRecord(L->prof_ev[L->prof_n], st);
 }
 void inject_selection_error(dare_layer* L, const StepGeom& g, cudaStream_t st);
-const float* step_threshold_on_device(dare_layer* L, const StepGeom& g, int mode, cudaStream_t st, int* launches);
+void select_step(dare_layer* L, const StepGeom& g, int mode, float tau, bool beside_predecessor, cudaStream_t st,
+                 int* launches);
 dare_status_t tc_create(dare_layer* L);
 void tc_destroy(dare_layer* L);
 // add_input: y = x + W_O O instead of y = W_O O (the residual connection of a transformer block)

@@ -191,7 +191,161 @@ __global__ void __launch_bounds__(kTileWords) tile_scatter_kernel(const unsigned
   }
 }
 
+// ---- the k-th smallest of many scores, by ONE cluster of CTAs: exact radix selection over the order-preserving keys in
+// three passes (11 + 11 + 10 bits).  Every CTA counts its share of the scores into a histogram in its own shared memory;
+// the CTAs then add up one slice of the bins each over distributed shared memory and all of them pick the bin that
+// holds rank k.  A cluster (rather than a grid) because the call has no scratch memory to meet in: nothing is shared
+// between calls, whatever streams they run on.  Bound by what the cluster's SMs pull from the L2 (three reads of the
+// scores at about 0.1 TB/s an SM) and by shared-memory atomics in the first pass, where most scores fall into a few
+// bins: eight copies of the histogram, by lane, keep lanes of a warp apart.
+constexpr int kKthBins = 2048, kKthCopies = 8;
+constexpr int kKthSmem = (kKthBins * kKthCopies + kKthBins) * (int)sizeof(int);
+
+__global__ void __launch_bounds__(kThreads) kth_cluster_kernel(const float* __restrict__ scores, int n, int k,
+                                                               float* __restrict__ tau_out) {
+  extern __shared__ __align__(16) int kth_smem[];
+  int* hist = kth_smem;                               // [bin][copy]
+  int* sum = hist + kKthBins * kKthCopies;            // [bin], this CTA's copies added up
+  __shared__ int red[kKthBins], slice_total, s_bin, s_rank;   // red: this CTA's slice of the bins over the whole cluster
+  const int ctas = (int)gridDim.x, rank_cta = (int)ptx::cluster_ctarank(), lane = threadIdx.x & 31, tid = (int)threadIdx.x;
+  const int slice = kKthBins / ctas;
+  ptx::pdl_wait();
+  ptx::pdl_launch_dependents();
+  // 16-byte loads from the first aligned score on; the few before and after them are CTA 0's
+  const int head = min(n, (int)((16u - (unsigned)(reinterpret_cast<uintptr_t>(scores) & 15u)) & 15u) / 4);
+  const float4* body = reinterpret_cast<const float4*>(scores + head);
+  const int n4 = (n - head) / 4, tail0 = head + 4 * n4;
+  unsigned prefix = 0u, mask = 0u;
+  int rank = k;
+  bool numbers = true;                                // rank k falls among the scores that are numbers
+  for (int pass = 0; pass < 3 && numbers; ++pass) {
+    const int shift = pass == 0 ? 21 : (pass == 1 ? 10 : 0), bits = pass == 2 ? 10 : 11;
+    const unsigned dmask = (1u << bits) - 1u;
+    for (int i = tid; i < kKthBins * kKthCopies / 4; i += kThreads) reinterpret_cast<int4*>(hist)[i] = make_int4(0, 0, 0, 0);
+    if (tid == 0) s_bin = -1;
+    __syncthreads();
+    auto count = [&](float f) {
+      const unsigned key = score_key(f);
+      if (key != kKeyNaN && (key & mask) == prefix) atomicAdd(&hist[((key >> shift) & dmask) * kKthCopies + (lane & 7)], 1);
+    };
+    const int step = ctas * kThreads;
+    int i = rank_cta * kThreads + tid;
+    for (; i + 3 * step < n4; i += 4 * step) {
+      float4 v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) v[u] = body[i + u * step];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) { count(v[u].x); count(v[u].y); count(v[u].z); count(v[u].w); }
+    }
+    for (; i < n4; i += step) {
+      const float4 v = body[i];
+      count(v.x); count(v.y); count(v.z); count(v.w);
+    }
+    if (rank_cta == 0) {
+      if (tid < head) count(scores[tid]);
+      if (tid < n - tail0) count(scores[tail0 + tid]);
+    }
+    __syncthreads();
+    for (int b = tid; b < kKthBins; b += kThreads) {
+      const int4 c0 = reinterpret_cast<const int4*>(hist)[2 * b], c1 = reinterpret_cast<const int4*>(hist)[2 * b + 1];
+      sum[b] = (c0.x + c0.y) + (c0.z + c0.w) + (c1.x + c1.y) + (c1.z + c1.w);
+    }
+    if (tid == 0) slice_total = 0;
+    ptx::cluster_sync_all();
+    int mine = 0;
+    if (tid < slice) {                                // whole warps: a slice has 128 bins or more
+      for (int c = 0; c < ctas; ++c)
+        mine += (int)ptx::ld_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&sum[rank_cta * slice + tid]), (uint32_t)c));
+      red[tid] = mine;
+      mine = __reduce_add_sync(0xffffffffu, mine);
+      if (lane == 0) atomicAdd(&slice_total, mine);
+    }
+    ptx::cluster_sync_all();
+    if (tid < 32) {
+      // the slice that holds the rank, then the bin: `slice` bins, slice / 32 of them to a lane
+      auto scan = [&](int v) {
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int u = __shfl_up_sync(0xffffffffu, v, o);
+          if (lane >= o) v += u;
+        }
+        return v;
+      };
+      const int st = lane < ctas ? (int)ptx::ld_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&slice_total), (uint32_t)lane)) : 0;
+      const int inc = scan(st);
+      const unsigned hit = __ballot_sync(0xffffffffu, inc - st < rank && rank <= inc);
+      if (hit != 0u) {
+        const int sl = __ffs((int)hit) - 1;
+        const int before = __shfl_sync(0xffffffffu, inc - st, sl);
+        const int per = slice / 32;
+        int tot = 0;
+        for (int j = 0; j < per; ++j)
+          tot += (int)ptx::ld_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&red[lane * per + j]), (uint32_t)sl));
+        const int inc2 = before + scan(tot);
+        int cum = inc2 - tot;
+        if (cum < rank && rank <= inc2) {
+          for (int j = 0; j < per; ++j) {
+            const int c = (int)ptx::ld_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&red[lane * per + j]), (uint32_t)sl));
+            if (cum < rank && rank <= cum + c) { s_bin = sl * slice + lane * per + j; s_rank = rank - cum; }
+            cum += c;
+          }
+        }
+      }
+    }
+    __syncthreads();
+    numbers = s_bin >= 0;                             // (the same in every CTA)
+    if (numbers) {
+      prefix |= (unsigned)s_bin << shift;
+      rank = s_rank;
+      mask |= dmask << shift;
+    }
+    __syncthreads();
+  }
+  if (rank_cta == 0 && tid == 0) *tau_out = numbers ? key_score(prefix) : __int_as_float(0x7f800000);
+  ptx::cluster_sync_all();                            // nobody leaves while its bins are being read
+}
+__global__ void set_float_kernel(float* dst, float value) { *dst = value; }
 }  // namespace
+
+cudaError_t launch_kth_score_large(const float* scores, int n, int k, float* tau_out, cudaStream_t st) {
+  if (k <= 0 || k >= n) {
+    set_float_kernel<<<1, 1, 0, st>>>(tau_out, k <= 0 ? -INFINITY : INFINITY);
+    return cudaGetLastError();
+  }
+  // 16 CTAs where the device takes a cluster of that size (asked once per device), the portable 8 otherwise
+  static std::atomic<unsigned long long> asked{0}, wide{0};
+  int dev = 0;
+  if (cudaError_t e = cudaGetDevice(&dev); e != cudaSuccess) return e;
+  const unsigned long long bit = 1ull << (dev & 63);
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = kKthSmem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  if (!(asked.load(std::memory_order_acquire) & bit)) {
+    if (cudaError_t e = cudaFuncSetAttribute(kth_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kKthSmem); e != cudaSuccess) return e;
+    int clusters = 0;
+    cfg.gridDim = dim3(16);
+    attr[0].val.clusterDim.x = 16;
+    cfg.numAttrs = 1;
+    if (cudaFuncSetAttribute(kth_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&clusters, kth_cluster_kernel, &cfg) == cudaSuccess && clusters > 0)
+      wide.fetch_or(bit);
+    else
+      cudaGetLastError();
+    asked.fetch_or(bit, std::memory_order_release);
+  }
+  const unsigned ctas = (wide.load() & bit) ? 16u : 8u;
+  cfg.gridDim = dim3(ctas);
+  attr[0].val.clusterDim.x = ctas;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, kth_cluster_kernel, scores, n, k, tau_out);
+}
 
 int select_large_tiles(long long n) { return (int)((n + kTile - 1) / kTile); }
 size_t select_large_flag_bytes(long long n) { return (size_t)select_large_tiles(n) * kTileWords * sizeof(unsigned); }
