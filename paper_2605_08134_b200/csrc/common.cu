@@ -281,7 +281,8 @@ template void launch_rmsnorm<__nv_bfloat16>(const __nv_bfloat16*, const float*, 
 // k <= 0: tau = -inf (nothing reused); k >= n or more than the scores that are numbers: +inf.
 // A step of at most kKthInCta tokens has the selection kernel do it: every CTA of that launch keeps all keys in
 // registers (16 per thread), so the passes touch shared memory only, and the step has no launch for it.  What bounds it
-// is the chain of the passes (histogram -> scan over 256 bins by one warp -> next digit), three barriers each.
+// is the chain of the passes (histogram -> scan over 256 bins by one warp -> next digit); copies
+// of the histogram against lanes that meet in one bin made it slower (16384 scores: 9.7 -> 11.6 us a call).
 // (It was a launch of its own that read the scores once per pass and walked the bins with one thread.)
 constexpr int kKthInCta = 16384;
 constexpr int kKthPerThread = kKthInCta / 1024;
@@ -306,7 +307,7 @@ __device__ float kth_in_cta(const float* __restrict__ scores, int n, int k) {
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < KPT; ++i)
-      if (key[i] != kKeyNaN && (key[i] & mask) == prefix) atomicAdd(&hist[(key[i] >> shift) & 255u], 1);
+      if (key[i] != kKeyNaN && (key[i] & mask) == prefix) atomicAdd(&hist[((key[i] >> shift) & 255u) ], 1);
     __syncthreads();
     if (threadIdx.x < 32) {
       int c[8], mine = 0;

@@ -1,6 +1,6 @@
 // Stand-alone drift score and threshold/compaction for token counts far beyond one layer step (millions of rows):
 // the same arithmetic as inside the layer step, organised for HBM bandwidth.
-//   drift score (Sec. 3.1): one warp per row, 16-byte loads of both query rows, shuffle reduction
+//   drift score (Sec. 3.1): hd / 4 lanes per row, 16-byte loads of both query rows, shuffle reduction
 //   compaction (Eq. 2, complement): three passes over tiles of 16384 scores; the scores are read once
 //     (1) per-tile count of refreshed tokens and the decisions themselves, a plain bit array -> scratch
 //     (2) exclusive scan of the tile counts (one CTA) -> scratch, total -> *count
@@ -28,8 +28,54 @@ constexpr int kThreads = 1024, kVecs = 4;
 constexpr int kTile = kThreads * kVecs * 4;     // 16384 scores per CTA: four 16-byte vectors per thread
 constexpr int kTileWords = kTile / 32;          // 512 words of decision bits per tile
 
+// LPR lanes to a row (hd = 4 * LPR * VPL), so that every lane of a warp has work, and U rows of each lane group in
+// flight at once: the kernel is a stream of both query arrays, bound by how many bytes an SM keeps on their way (one row
+// a warp: 5.3 TB/s at 2^20 rows of 128).
+template <int LPR, int VPL, int U>
 __global__ void __launch_bounds__(256) drift_score_kernel(const float* __restrict__ a, const float* __restrict__ b,
-                                                          long long rows, int hd, float* __restrict__ scores) {
+                                                          long long rows, float* __restrict__ scores) {
+  constexpr int RPW = 32 / LPR * U, HD = 4 * LPR * VPL;      // rows a warp takes at once
+  const int lane = threadIdx.x & 31, sub = lane & (LPR - 1), grp = lane / LPR;
+  const long long warp0 = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
+  for (long long r0 = warp0 * RPW; r0 < rows; r0 += nwarps * RPW) {
+    float4 x[U][VPL], y[U][VPL];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const long long r = r0 + u * (32 / LPR) + grp, rc = r < rows ? r : rows - 1;
+#pragma unroll
+      for (int v = 0; v < VPL; ++v) {
+        x[u][v] = __ldcs(reinterpret_cast<const float4*>(a + rc * HD) + v * LPR + sub);
+        y[u][v] = __ldcs(reinterpret_cast<const float4*>(b + rc * HD) + v * LPR + sub);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      float dot = 0.f, n1 = 0.f, n2 = 0.f;
+#pragma unroll
+      for (int v = 0; v < VPL; ++v) {
+        const float4 p = x[u][v], q = y[u][v];
+        dot += p.x * q.x + p.y * q.y + p.z * q.z + p.w * q.w;
+        n1 += p.x * p.x + p.y * p.y + p.z * p.z + p.w * p.w;
+        n2 += q.x * q.x + q.y * q.y + q.z * q.z + q.w * q.w;
+      }
+#pragma unroll
+      for (int o = LPR / 2; o > 0; o >>= 1) {
+        dot += __shfl_xor_sync(0xffffffffu, dot, o);
+        n1 += __shfl_xor_sync(0xffffffffu, n1, o);
+        n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+      }
+      const long long r = r0 + u * (32 / LPR) + grp;
+      if (sub == 0 && r < rows) {
+        const float den = sqrtf(n1) * sqrtf(n2);
+        scores[r] = 1.f - (den > 0.f ? dot / den : 0.f);
+      }
+    }
+  }
+}
+// any other row length
+__global__ void __launch_bounds__(256) drift_score_any_kernel(const float* __restrict__ a, const float* __restrict__ b,
+                                                              long long rows, int hd, float* __restrict__ scores) {
   const int lane = threadIdx.x & 31;
   const long long warp0 = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
@@ -193,22 +239,20 @@ __global__ void __launch_bounds__(kTileWords) tile_scatter_kernel(const unsigned
 
 // ---- the k-th smallest of many scores, by ONE cluster of CTAs: exact radix selection over the order-preserving keys in
 // three passes (11 + 11 + 10 bits).  Every CTA counts its share of the scores into a histogram in its own shared memory;
-// the CTAs then add up one slice of the bins each over distributed shared memory and all of them pick the bin that
-// holds rank k.  A cluster (rather than a grid) because the call has no scratch memory to meet in: nothing is shared
-// between calls, whatever streams they run on.  Bound by what the cluster's SMs pull from the L2 (three reads of the
-// scores at about 0.1 TB/s an SM) and by shared-memory atomics in the first pass, where most scores fall into a few
-// bins: eight copies of the histogram, by lane, keep lanes of a warp apart.
-constexpr int kKthBins = 2048, kKthCopies = 8;
-constexpr int kKthSmem = (kKthBins * kKthCopies + kKthBins) * (int)sizeof(int);
+// the CTAs then add up one slice of the bins each over distributed shared memory, tell one another the slices' totals,
+// and all of them pick the bin that holds rank k.  A cluster (rather than a grid) because the call has no scratch memory
+// to meet in: nothing is shared between calls, whatever streams they run on.  Bound by what the cluster's SMs pull from
+// the L2 (three reads of the scores) and by the cluster-wide exchange of each pass: two cluster barriers and two remote
+// round trips.  (Copies of the histogram, to keep lanes that meet in one bin apart, changed nothing.)
+constexpr int kKthBins = 2048, kKthMaxCtas = 16;
 
 __global__ void __launch_bounds__(kThreads) kth_cluster_kernel(const float* __restrict__ scores, int n, int k,
                                                                float* __restrict__ tau_out) {
-  extern __shared__ __align__(16) int kth_smem[];
-  int* hist = kth_smem;                               // [bin][copy]
-  int* sum = hist + kKthBins * kKthCopies;            // [bin], this CTA's copies added up
-  __shared__ int red[kKthBins], slice_total, s_bin, s_rank;   // red: this CTA's slice of the bins over the whole cluster
+  __shared__ __align__(16) int hist[kKthBins];
+  __shared__ __align__(16) int red[kKthBins / 8];     // this CTA's slice of the bins over the whole cluster
+  __shared__ int part[kKthBins / 8 / 32], totals[kKthMaxCtas], s_bin, s_rank;
   const int ctas = (int)gridDim.x, rank_cta = (int)ptx::cluster_ctarank(), lane = threadIdx.x & 31, tid = (int)threadIdx.x;
-  const int slice = kKthBins / ctas;
+  const int slice = kKthBins / ctas;                  // 128 or 256: whole warps, four or eight bins to a lane
   ptx::pdl_wait();
   ptx::pdl_launch_dependents();
   // 16-byte loads from the first aligned score on; the few before and after them are CTA 0's
@@ -218,24 +262,33 @@ __global__ void __launch_bounds__(kThreads) kth_cluster_kernel(const float* __re
   unsigned prefix = 0u, mask = 0u;
   int rank = k;
   bool numbers = true;                                // rank k falls among the scores that are numbers
+  auto scan = [&](int v) {                            // inclusive, over the warp
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, v, o);
+      if (lane >= o) v += u;
+    }
+    return v;
+  };
   for (int pass = 0; pass < 3 && numbers; ++pass) {
-    const int shift = pass == 0 ? 21 : (pass == 1 ? 10 : 0), bits = pass == 2 ? 10 : 11;
-    const unsigned dmask = (1u << bits) - 1u;
-    for (int i = tid; i < kKthBins * kKthCopies / 4; i += kThreads) reinterpret_cast<int4*>(hist)[i] = make_int4(0, 0, 0, 0);
+    const int shift = pass == 0 ? 21 : (pass == 1 ? 10 : 0);
+    const unsigned dmask = pass == 2 ? 1023u : 2047u;
+    for (int b = tid; b < kKthBins; b += kThreads) hist[b] = 0;
     if (tid == 0) s_bin = -1;
     __syncthreads();
     auto count = [&](float f) {
       const unsigned key = score_key(f);
-      if (key != kKeyNaN && (key & mask) == prefix) atomicAdd(&hist[((key >> shift) & dmask) * kKthCopies + (lane & 7)], 1);
+      if (key != kKeyNaN && (key & mask) == prefix) atomicAdd(&hist[(key >> shift) & dmask], 1);
     };
+    constexpr int U = 8;                              // vectors a thread has in flight
     const int step = ctas * kThreads;
     int i = rank_cta * kThreads + tid;
-    for (; i + 3 * step < n4; i += 4 * step) {
-      float4 v[4];
+    for (; i + (U - 1) * step < n4; i += U * step) {
+      float4 v[U];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) v[u] = body[i + u * step];
+      for (int u = 0; u < U; ++u) v[u] = body[i + u * step];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) { count(v[u].x); count(v[u].y); count(v[u].z); count(v[u].w); }
+      for (int u = 0; u < U; ++u) { count(v[u].x); count(v[u].y); count(v[u].z); count(v[u].w); }
     }
     for (; i < n4; i += step) {
       const float4 v = body[i];
@@ -245,50 +298,42 @@ __global__ void __launch_bounds__(kThreads) kth_cluster_kernel(const float* __re
       if (tid < head) count(scores[tid]);
       if (tid < n - tail0) count(scores[tail0 + tid]);
     }
-    __syncthreads();
-    for (int b = tid; b < kKthBins; b += kThreads) {
-      const int4 c0 = reinterpret_cast<const int4*>(hist)[2 * b], c1 = reinterpret_cast<const int4*>(hist)[2 * b + 1];
-      sum[b] = (c0.x + c0.y) + (c0.z + c0.w) + (c1.x + c1.y) + (c1.z + c1.w);
-    }
-    if (tid == 0) slice_total = 0;
     ptx::cluster_sync_all();
-    int mine = 0;
-    if (tid < slice) {                                // whole warps: a slice has 128 bins or more
-      for (int c = 0; c < ctas; ++c)
-        mine += (int)ptx::ld_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&sum[rank_cta * slice + tid]), (uint32_t)c));
+    if (tid < slice) {
+      const uint32_t bin = ptx::smem_u32(&hist[rank_cta * slice + tid]);
+      int c[kKthMaxCtas], mine = 0;
+#pragma unroll
+      for (int j = 0; j < kKthMaxCtas; ++j) c[j] = j < ctas ? (int)ptx::ld_cluster_u32(ptx::map_to_cta(bin, (uint32_t)j)) : 0;
+#pragma unroll
+      for (int j = 0; j < kKthMaxCtas; ++j) mine += c[j];
       red[tid] = mine;
       mine = __reduce_add_sync(0xffffffffu, mine);
-      if (lane == 0) atomicAdd(&slice_total, mine);
+      if (lane == 0) part[tid >> 5] = mine;
+    }
+    __syncthreads();
+    if (tid < ctas) {                                 // the slice's total goes to every CTA
+      int tot = 0;
+      for (int w = 0; w < slice / 32; ++w) tot += part[w];
+      ptx::st_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&totals[rank_cta]), (uint32_t)tid), (uint32_t)tot);
     }
     ptx::cluster_sync_all();
     if (tid < 32) {
-      // the slice that holds the rank, then the bin: `slice` bins, slice / 32 of them to a lane
-      auto scan = [&](int v) {
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int u = __shfl_up_sync(0xffffffffu, v, o);
-          if (lane >= o) v += u;
-        }
-        return v;
-      };
-      const int st = lane < ctas ? (int)ptx::ld_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&slice_total), (uint32_t)lane)) : 0;
-      const int inc = scan(st);
+      const int st = lane < ctas ? totals[lane] : 0, inc = scan(st);
       const unsigned hit = __ballot_sync(0xffffffffu, inc - st < rank && rank <= inc);
       if (hit != 0u) {
-        const int sl = __ffs((int)hit) - 1;
+        const int sl = __ffs((int)hit) - 1, per = slice / 32;
         const int before = __shfl_sync(0xffffffffu, inc - st, sl);
-        const int per = slice / 32;
-        int tot = 0;
-        for (int j = 0; j < per; ++j)
-          tot += (int)ptx::ld_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&red[lane * per + j]), (uint32_t)sl));
-        const int inc2 = before + scan(tot);
-        int cum = inc2 - tot;
-        if (cum < rank && rank <= inc2) {
-          for (int j = 0; j < per; ++j) {
-            const int c = (int)ptx::ld_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&red[lane * per + j]), (uint32_t)sl));
-            if (cum < rank && rank <= cum + c) { s_bin = sl * slice + lane * per + j; s_rank = rank - cum; }
-            cum += c;
-          }
+        int c[8], tot = 0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          c[j] = j < per ? (int)ptx::ld_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&red[lane * per + j]), (uint32_t)sl)) : 0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) tot += c[j];
+        int cum = before + scan(tot) - tot;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          if (cum < rank && rank <= cum + c[j]) { s_bin = sl * slice + lane * per + j; s_rank = rank - cum; }
+          cum += c[j];
         }
       }
     }
@@ -320,7 +365,6 @@ cudaError_t launch_kth_score_large(const float* scores, int n, int k, float* tau
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[2];
   cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = kKthSmem;
   cfg.stream = st;
   cfg.attrs = attr;
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -328,7 +372,6 @@ cudaError_t launch_kth_score_large(const float* scores, int n, int k, float* tau
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   if (!(asked.load(std::memory_order_acquire) & bit)) {
-    if (cudaError_t e = cudaFuncSetAttribute(kth_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kKthSmem); e != cudaSuccess) return e;
     int clusters = 0;
     cfg.gridDim = dim3(16);
     attr[0].val.clusterDim.x = 16;
@@ -353,9 +396,15 @@ size_t select_large_flag_bytes(long long n) { return (size_t)select_large_tiles(
 cudaError_t launch_drift_scores(const float* a, const float* b, long long rows, int hd, float* scores,
                                 cudaStream_t st) {
   if (rows <= 0) return cudaSuccess;
-  long long blocks = (rows + 7) / 8;
-  if (blocks > 148 * 16) blocks = 148 * 16;
-  drift_score_kernel<<<(int)blocks, 256, 0, st>>>(a, b, rows, hd, scores);
+  auto blocks = [&](int rows_per_warp, int per_sm) {
+    const long long n = (rows + 8 * rows_per_warp - 1) / (8 * rows_per_warp);
+    return (int)(n < 148 * per_sm ? n : 148 * per_sm);
+  };
+  if (hd == 32) drift_score_kernel<8, 1, 4><<<blocks(16, 8), 256, 0, st>>>(a, b, rows, scores);
+  else if (hd == 64) drift_score_kernel<16, 1, 4><<<blocks(8, 8), 256, 0, st>>>(a, b, rows, scores);
+  else if (hd == 128) drift_score_kernel<32, 1, 4><<<blocks(4, 8), 256, 0, st>>>(a, b, rows, scores);
+  else if (hd == 256) drift_score_kernel<32, 2, 2><<<blocks(2, 8), 256, 0, st>>>(a, b, rows, scores);
+  else drift_score_any_kernel<<<blocks(1, 16), 256, 0, st>>>(a, b, rows, hd, scores);
   return cudaGetLastError();
 }
 
