@@ -79,7 +79,8 @@ typedef enum { DARE_F32 = 0, DARE_BF16 = 1 } dare_dtype_t;
 
 /* kernel_path: which kernel family the handle uses. */
 enum {
-  DARE_PATH_AUTO = 0,   /* tcgen05/TMEM tensor-core kernels when dtype = bf16 and head_dim = 128, else SIMT */
+  DARE_PATH_AUTO = 0,   /* tcgen05/TMEM tensor-core kernels when dtype = bf16, head_dim = 64 or 128 and d_model is a multiple
+                         * of 256, else SIMT */
   DARE_PATH_SIMT = 1,   /* plain fp32-accumulate CUDA-core kernels for every step (any supported geometry) */
   DARE_PATH_TENSOR = 2  /* tensor-core kernels or DARE_ERR_UNSUPPORTED */
 };
@@ -88,7 +89,7 @@ typedef struct {
   uint32_t struct_size; /* sizeof(dare_layer_config_t), checked */
   int32_t d_model;      /* = n_heads * head_dim; multiple of 8 */
   int32_t n_heads;
-  int32_t head_dim;     /* even; 32..256 for the SIMT path, 128 for the tensor-core path */
+  int32_t head_dim;     /* even; 32..256 for the SIMT path, 64 or 128 for the tensor-core path */
   int32_t max_batch;
   int32_t max_seq;
   float rope_theta;     /* rotary base (half-split pairing: element j rotates with j + head_dim/2) */

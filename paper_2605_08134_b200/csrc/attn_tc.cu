@@ -1,4 +1,4 @@
-// Bidirectional (no mask) softmax attention on tcgen05 tensor cores, head_dim = 128, bf16 operands, fp32 softmax.
+// Bidirectional (no mask) softmax attention on tcgen05 tensor cores, head_dim 128 or 64, bf16 operands, fp32 softmax.
 //   dense      : every query row of the step window                       (Alg. 1 line 10)
 //   row-sparse : only the query rows of the refresh set, gathered by index (Alg. 2 lines 6, 8; Eq. 4)
 // The result rows are written straight into the attention-output cache at their cache rows; rows that are not
@@ -38,18 +38,22 @@ namespace {
 
 constexpr int BQ = 128;    // query rows per CTA
 constexpr int BKV = 128;   // keys per block
-constexpr int HD = 128;
-
+// A CTA takes all of its SM's tensor memory, so two must never share an SM: the second would wait for the first, and
+// with clusters on both (key split) each could wait for the other.  Shared memory keeps them apart: more than half.
+constexpr int one_cta_per_sm(int bytes) { return bytes > 117 * 1024 ? bytes : 117 * 1024; }
+// Everything below is templated on the head width HD: 128, or 64 (one 64-column chunk per operand tile instead of two,
+// half of the products' steps and of the O columns).
+template <int HD>
 struct AttnSmem {
-  static constexpr int Q_BYTES = BQ * HD * 2;          // two 64-column chunks of [128 x 128 B]
-  static constexpr int K_BYTES = BKV * HD * 2;         // two chunks of [64 x 128 B]
+  static constexpr int Q_BYTES = BQ * HD * 2;          // HD / 64 64-column chunks of [128 x 128 B]
+  static constexpr int K_BYTES = BKV * HD * 2;         // the same chunks of a key block
   static constexpr int V_BYTES = BKV * HD * 2;
   static constexpr int Q_OFF = 0;
   static constexpr int K_OFF = Q_OFF + Q_BYTES;        // one buffer per stream
   static constexpr int V_OFF = K_OFF + 2 * K_BYTES;    // two buffers per stream: V(j) is wanted last in a block and
                                                        // its buffer is released last, so one buffer leaves no slack
   static constexpr int BAR_OFF = V_OFF + 4 * V_BYTES;
-  static constexpr int TOTAL = BAR_OFF + 256 + 1024;
+  static constexpr int TOTAL = one_cta_per_sm(BAR_OFF + 256 + 1024);
   // merge of the two streams: a stream's running maxima [128] and row sums [128] go to its first V buffer, idle
   // after its last product
   // after the key loop the operand buffers are idle; the merge of a key split reuses them:
@@ -57,7 +61,10 @@ struct AttnSmem {
   static constexpr int STAT_OFF = DUMP_OFF + BQ * HD * 4;   // running maximum [128], row sum [128]
   static constexpr int RECV_OFF = STAT_OFF + 2 * BQ * 4;    // up to 3 senders x (rows x 512 B + rows x 8 B)
 };
-static_assert(AttnSmem::TOTAL <= 232448, "shared memory");
+static_assert(AttnSmem<128>::TOTAL <= 232448, "shared memory");
+static_assert(AttnSmem<64>::RECV_OFF + 3 * (BQ / 4) * (64 * 4 + 8) <= AttnSmem<64>::BAR_OFF &&
+              AttnSmem<128>::RECV_OFF + 3 * (BQ / 4) * (128 * 4 + 8) <= AttnSmem<128>::BAR_OFF &&
+              AttnSmem<64>::RECV_OFF + (BQ / 2) * (64 * 4 + 8) <= AttnSmem<64>::BAR_OFF, "merge buffers");
 // (the key-split buffers may overlap the streams' statistics: they are filled after the statistics were read)
 
 // 2^x for x <= 0 on the special-function unit; results below the normal range flush to zero (they are softmax
@@ -77,18 +84,28 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
 
 constexpr int kThreads = 384;
 constexpr int kSoftmaxThreads = 256;
-// S of stream 0 / 1: columns [0, 128) / [128, 256), P over the first 64 of them; O: [256, 384) / [384, 512)
+// S of stream 0 / 1: columns [0, 128) / [128, 256), P over the first 64 of them; O: [256, 256 + HD) / behind it
 constexpr uint32_t kTmemCols = 512;
 constexpr int kPairMinDense = 128;      // dense launches with longer windows take the two-tile kernel
 constexpr int kPairMinSparse = 1024;    // row-sparse launches from this window length on
 constexpr float kRescaleStep = 8.f;     // log2 of the growth of the running maximum that triggers a rescale of O
 
+// The HD / 64 chunks of a key (or value) block, 64 columns of 128 rows each, counted on one barrier.
+template <int HD>
+__device__ __forceinline__ void load_block(uint8_t* dst, const CUtensorMap* tm, int h, int row, uint64_t* bar) {
+  mbar_arrive_expect_tx(bar, BKV * HD * 2);
+#pragma unroll
+  for (int c = 0; c < HD / 64; ++c) tma_load_2d(dst + c * (BKV * 128), tm, h * HD + c * 64, row, bar);
+}
+
 }  // namespace
 
+template <int HD>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                const AttnParams p) {
-  using S = AttnSmem;
+  using S = AttnSmem<HD>;
+  constexpr int UPR = HD / 8;                        // 16-byte units of a query row
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S::BAR_OFF);
@@ -206,12 +223,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       const int row = kv_row0 + (z + s2 * ksplit) * BKV;
       uint8_t* kd = smem + S::K_OFF + s2 * S::K_BYTES;
       uint8_t* vd = smem + S::V_OFF + 2 * s2 * S::V_BYTES;
-      mbar_arrive_expect_tx(&k_full[s2], S::K_BYTES);
-      tma_load_2d(kd, &tm_k, h * HD, row, &k_full[s2]);
-      tma_load_2d(kd + S::K_BYTES / 2, &tm_k, h * HD + 64, row, &k_full[s2]);
-      mbar_arrive_expect_tx(&v_full[2 * s2], S::V_BYTES);
-      tma_load_2d(vd, &tm_v, h * HD, row, &v_full[2 * s2]);
-      tma_load_2d(vd + S::V_BYTES / 2, &tm_v, h * HD + 64, row, &v_full[2 * s2]);
+      load_block<HD>(kd, &tm_k, h, row, &k_full[s2]);
+      load_block<HD>(vd, &tm_v, h, row, &v_full[2 * s2]);
     }
   }
   // ---- Q tile: gathered rows -> shared memory in the K-major 128-byte-swizzled layout (16-byte units), by the
@@ -219,29 +232,29 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   if (active && warp != 0) {
     uint8_t* qs = smem + S::Q_OFF;
     constexpr int kGather = kThreads - 32;
-    constexpr int QU = (BQ * 16 + kGather - 1) / kGather;     // 16-byte units per thread
+    constexpr int QU = (BQ * UPR + kGather - 1) / kGather;     // 16-byte units per thread
     const int u0 = (int)threadIdx.x - 32;
     int tok[QU];
     uint4 qv[QU];
     // all index loads first, then all row loads, then the stores: one memory round trip each instead of one per unit
 #pragma unroll
     for (int k = 0; k < QU; ++k) {
-      const int u = u0 + k * kGather, r = u >> 4;              // 16 units of 8 bf16 per row
+      const int u = u0 + k * kGather, r = u / UPR;              // units of 8 bf16
       tok[k] = -1;
-      if (u < BQ * 16 && r < rows_valid) tok[k] = p.idx ? __ldcg(p.idx + row0 + r) : row0 + r;
+      if (u < BQ * UPR && r < rows_valid) tok[k] = p.idx ? __ldcg(p.idx + row0 + r) : row0 + r;
       if (p.idx && tok[k] >= 0 && !token_ok(tok[k], g.tokens(), p.status)) tok[k] = -1;      // read as a row of zeros
     }
 #pragma unroll
     for (int k = 0; k < QU; ++k) {
-      const int unit = (u0 + k * kGather) & 15;
+      const int unit = (u0 + k * kGather) % UPR;
       qv[k] = make_uint4(0u, 0u, 0u, 0u);
       if (tok[k] >= 0) qv[k] = __ldcg(reinterpret_cast<const uint4*>(p.q + (size_t)tok[k] * g.d + h * HD + unit * 8));
     }
 #pragma unroll
     for (int k = 0; k < QU; ++k) {
-      const int u = u0 + k * kGather, r = u >> 4, unit = u & 15;
+      const int u = u0 + k * kGather, r = u / UPR, unit = u % UPR;
       const int chunk = unit >> 3, uc = unit & 7;
-      if (u < BQ * 16) *reinterpret_cast<uint4*>(qs + chunk * (BQ * 128) + r * 128 + ((uc ^ (r & 7)) << 4)) = qv[k];
+      if (u < BQ * UPR) *reinterpret_cast<uint4*>(qs + chunk * (BQ * 128) + r * 128 + ((uc ^ (r & 7)) << 4)) = qv[k];
     }
     fence_proxy_async_smem();
   }
@@ -271,18 +284,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       uint8_t* vd = smem + S::V_OFF + vb * S::V_BYTES;
       const int row = kv_row0 + (z + (2 * j + st) * ksplit) * BKV;
       mbar_wait(&k_empty[st], (j & 1) ^ 1, p.status);       // S(j-1) = Q K(j-1)^T has been computed
-      if (elect_one()) {
-        mbar_arrive_expect_tx(&k_full[st], S::K_BYTES);
-        tma_load_2d(kd, &tm_k, h * HD, row, &k_full[st]);
-        tma_load_2d(kd + S::K_BYTES / 2, &tm_k, h * HD + 64, row, &k_full[st]);
-      }
+      if (elect_one()) load_block<HD>(kd, &tm_k, h, row, &k_full[st]);
       __syncwarp();
       mbar_wait(&v_empty[vb], ((j >> 1) & 1) ^ 1, p.status);       // O += P(j-2) V(j-2) has been computed
-      if (elect_one()) {
-        mbar_arrive_expect_tx(&v_full[vb], S::V_BYTES);
-        tma_load_2d(vd, &tm_v, h * HD, row, &v_full[vb]);
-        tma_load_2d(vd + S::V_BYTES / 2, &tm_v, h * HD + 64, row, &v_full[vb]);
-      }
+      if (elect_one()) load_block<HD>(vd, &tm_v, h, row, &v_full[vb]);
       __syncwarp();
     }
   } else if (warp < 4) {
@@ -361,7 +366,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
             mbar_wait(&o_full[st], (j - 1) & 1, p.status);
             tc_fence_after();
 #pragma unroll 1
-            for (int ch = 0; ch < 4; ++ch) {
+            for (int ch = 0; ch < HD / 32; ++ch) {
               float o[32];
               tmem_ld_32x32(tmem_o + lane_addr + ch * 32, o);
 #pragma unroll
@@ -424,7 +429,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       tc_fence_after();
     }
     if (dbg && threadIdx.x == 128) p.debug[3] = globaltimer_ns();
-    // ---- merge the two streams: thread (stream st, row r) finishes columns [64 st, 64 st + 64) of the row
+    // ---- merge the two streams: thread (stream st, row r) finishes its half of the row's columns
+    constexpr int HC = HD / 2;
     float* stat_mine = reinterpret_cast<float*>(smem + S::V_OFF + 2 * st * S::V_BYTES);
     const float* stat_other = reinterpret_cast<const float*>(smem + S::V_OFF + 2 * (st ^ 1) * S::V_BYTES);
     stat_mine[r] = m;
@@ -437,11 +443,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     const float w_mine = n_st > 0 ? fast_exp2((m - m_all) * c) : 0.f;
     const float w_other = n_other > 0 ? fast_exp2((m_o - m_all) * c) : 0.f;
     const float l_row = w_mine * l + w_other * l_o;
-    const uint32_t t_mine = tmem_o + lane_addr + st * 64;
-    const uint32_t t_other = tmem_base + 2 * BKV + (st ^ 1) * HD + lane_addr + st * 64;
-    float acc[64];
+    const uint32_t t_mine = tmem_o + lane_addr + st * HC;
+    const uint32_t t_other = tmem_base + 2 * BKV + (st ^ 1) * HD + lane_addr + st * HC;
+    float acc[HC];
 #pragma unroll
-    for (int cgrp = 0; cgrp < 2; ++cgrp) {
+    for (int cgrp = 0; cgrp < HC / 32; ++cgrp) {
       float a[32];
       if (n_st > 0) {
         tmem_ld_32x32(t_mine + cgrp * 32, a);
@@ -463,19 +469,19 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       const int t = t_row;
       if (t >= 0 && (p.idx == nullptr ? (p.store_mask == nullptr || __ldcg(p.store_mask + g.cache_row(t)) == 0)
                                       : token_ok(t, g.tokens(), p.status))) {      // (else: no cache row to write)
-        __nv_bfloat16* dst = p.oc + (size_t)g.cache_row(t) * g.d + h * HD + st * 64;
+        __nv_bfloat16* dst = p.oc + (size_t)g.cache_row(t) * g.d + h * HD + st * HC;
 #pragma unroll
-        for (int i = 0; i < 64; ++i) acc[i] *= inv;
+        for (int i = 0; i < HC; ++i) acc[i] *= inv;
 #pragma unroll
-        for (int v = 0; v < 8; ++v) reinterpret_cast<uint4*>(dst)[v] = pack8_bf16(acc + 8 * v);
+        for (int v = 0; v < HC / 8; ++v) reinterpret_cast<uint4*>(dst)[v] = pack8_bf16(acc + 8 * v);
       }
     } else {
       // key split: leave the un-normalised row, its maximum and its sum in shared memory for the merge.  The
       // operand buffers those go to are idle: both streams' last products were complete before the barrier above.
       float* dump = reinterpret_cast<float*>(smem + S::DUMP_OFF) + (size_t)r * HD;
 #pragma unroll
-      for (int v = 0; v < 16; ++v) {
-        const int unit = st * 16 + v;                    // 32 sixteen-byte units per 512-byte row, XOR-swizzled
+      for (int v = 0; v < HC / 4; ++v) {
+        const int unit = st * (HC / 4) + v;              // HD / 4 sixteen-byte units per row, XOR-swizzled
         *reinterpret_cast<float4*>(dump + ((unit ^ (r & 7)) << 2)) =
             make_float4(acc[4 * v], acc[4 * v + 1], acc[4 * v + 2], acc[4 * v + 3]);
       }
@@ -511,7 +517,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     const float* stat = reinterpret_cast<const float*>(smem + S::STAT_OFF);
     const uint32_t slot_floats = (uint32_t)rows_own * (HD + 2);
     const float* recv = reinterpret_cast<const float*>(smem + S::RECV_OFF);
-    for (int rl = warp; rl < rows_own; rl += kThreads / 32) {
+    // (a warp per row of 128 columns, half a warp per row of 64; lane <-> 4 columns)
+    constexpr int LPR = HD / 4, RPW = 32 / LPR;
+    const int sub = lane & (LPR - 1);
+    for (int rl = warp * RPW + lane / LPR; rl < rows_own; rl += kThreads / 32 * RPW) {
       const int r = z * rows_own + rl;
       if (r >= rows_valid) break;
       float mz[4], lz[4];
@@ -523,7 +532,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         lz[s2 + 1] = sl[rows_own * HD + rows_own + rl];
         mx = fmaxf(mx, mz[s2 + 1]);
       }
-      const int off = ((lane ^ (r & 7)) << 2);           // this lane's 4 columns inside the swizzled row
+      const int off = ((sub ^ (r & 7)) << 2);            // this lane's 4 columns inside the swizzled row
       float w = exp2f((mz[0] - mx) * c);
       float4 o = *reinterpret_cast<const float4*>(dump + (size_t)r * HD + off);
       o.x *= w; o.y *= w; o.z *= w; o.w *= w;
@@ -538,7 +547,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       const int t = p.idx ? __ldcg(p.idx + row0 + r) : row0 + r;
       if (p.idx != nullptr && !token_ok(t, g.tokens(), p.status)) continue;        // no cache row to write
       if (p.idx == nullptr && p.store_mask != nullptr && __ldcg(p.store_mask + g.cache_row(t)) != 0) continue;   // a reused row
-      __nv_bfloat16* dst = p.oc + (size_t)g.cache_row(t) * g.d + h * HD + 4 * lane;
+      __nv_bfloat16* dst = p.oc + (size_t)g.cache_row(t) * g.d + h * HD + 4 * sub;
       __nv_bfloat162 lo2 = __floats2bfloat162_rn(o.x * inv, o.y * inv), hi2 = __floats2bfloat162_rn(o.z * inv, o.w * inv);
       uint2 packed;
       packed.x = *reinterpret_cast<uint32_t*>(&lo2);
@@ -575,6 +584,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
 // to rescale O or to read it out, on one of two barriers per stream (product h signals barrier h & 1) so that a
 // parity wait never has to tell more than two consecutive phases apart.
 namespace {
+template <int HD>
 struct PairSmem {
   static constexpr int Q_BYTES = BQ * HD * 2;
   static constexpr int KV_BYTES = BKV * HD * 2;
@@ -582,17 +592,19 @@ struct PairSmem {
   static constexpr int K_OFF = Q_OFF + 2 * Q_BYTES;      // ring of 2
   static constexpr int V_OFF = K_OFF + 2 * KV_BYTES;     // ring of 2
   static constexpr int BAR_OFF = V_OFF + 2 * KV_BYTES;
-  static constexpr int TOTAL = BAR_OFF + 256 + 1024;
+  static constexpr int TOTAL = one_cta_per_sm(BAR_OFF + 256 + 1024);
 };
-static_assert(PairSmem::TOTAL <= 232448, "shared memory");
+static_assert(PairSmem<128>::TOTAL <= 232448, "shared memory");
 constexpr int kPairRows = 2 * BQ;
 constexpr int kHalf = BKV / 2;     // keys per score buffer
 }  // namespace
 
+template <int HD>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                  const AttnParams p) {
-  using S = PairSmem;
+  using S = PairSmem<HD>;
+  constexpr int UPR = HD / 8;                        // 16-byte units of a query row
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S::BAR_OFF);
@@ -692,12 +704,8 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
     const int slot = i & 1, row = kv_row0 + i * BKV;
     uint8_t* kd = smem + S::K_OFF + slot * S::KV_BYTES;
     uint8_t* vd = smem + S::V_OFF + slot * S::KV_BYTES;
-    mbar_arrive_expect_tx(&k_full[slot], S::KV_BYTES);
-    tma_load_2d(kd, &tm_k, h * HD, row, &k_full[slot]);
-    tma_load_2d(kd + S::KV_BYTES / 2, &tm_k, h * HD + 64, row, &k_full[slot]);
-    mbar_arrive_expect_tx(&v_full[slot], S::KV_BYTES);
-    tma_load_2d(vd, &tm_v, h * HD, row, &v_full[slot]);
-    tma_load_2d(vd + S::KV_BYTES / 2, &tm_v, h * HD + 64, row, &v_full[slot]);
+    load_block<HD>(kd, &tm_k, h, row, &k_full[slot]);
+    load_block<HD>(vd, &tm_v, h, row, &v_full[slot]);
   };
   // the first two key blocks start as soon as the projection is complete, by the thread that initialised the
   // barriers: in flight during the Q gather
@@ -711,29 +719,29 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
   // ---- both Q tiles: gathered rows -> shared memory in the K-major 128-byte-swizzled layout (16-byte units)
   if (active && warp != 0) {
     constexpr int kGather = kThreads - 32;
-    constexpr int QU = (kPairRows * 16 + kGather - 1) / kGather;
+    constexpr int QU = (kPairRows * UPR + kGather - 1) / kGather;
     const int u0 = (int)threadIdx.x - 32;
     int tok[QU];
     uint4 qv[QU];
 #pragma unroll
     for (int k = 0; k < QU; ++k) {
-      const int u = u0 + k * kGather, r = u >> 4;
+      const int u = u0 + k * kGather, r = u / UPR;
       tok[k] = -1;
-      if (u < kPairRows * 16 && r < rows_all) tok[k] = idx ? __ldcg(idx + row0 + r) : row0 + r;
+      if (u < kPairRows * UPR && r < rows_all) tok[k] = idx ? __ldcg(idx + row0 + r) : row0 + r;
       if (idx && tok[k] >= 0 && !token_ok(tok[k], g.tokens(), p.status)) tok[k] = -1;      // read as a row of zeros
     }
 #pragma unroll
     for (int k = 0; k < QU; ++k) {
-      const int unit = (u0 + k * kGather) & 15;
+      const int unit = (u0 + k * kGather) % UPR;
       qv[k] = make_uint4(0u, 0u, 0u, 0u);
       if (tok[k] >= 0) qv[k] = __ldcg(reinterpret_cast<const uint4*>(p.q + (size_t)tok[k] * g.d + h * HD + unit * 8));
     }
 #pragma unroll
     for (int k = 0; k < QU; ++k) {
-      const int u = u0 + k * kGather, r = u >> 4, unit = u & 15;
+      const int u = u0 + k * kGather, r = u / UPR, unit = u % UPR;
       const int chunk = unit >> 3, uc = unit & 7, rt = r & (BQ - 1);
       uint8_t* qs = smem + S::Q_OFF + (r >> 7) * S::Q_BYTES;
-      if (u < kPairRows * 16) *reinterpret_cast<uint4*>(qs + chunk * (BQ * 128) + rt * 128 + ((uc ^ (rt & 7)) << 4)) = qv[k];
+      if (u < kPairRows * UPR) *reinterpret_cast<uint4*>(qs + chunk * (BQ * 128) + rt * 128 + ((uc ^ (rt & 7)) << 4)) = qv[k];
     }
     fence_proxy_async_smem();
   }
@@ -873,7 +881,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
           mbar_wait(&o_full[2 * st + ((hf - 1) & 1)], ((hf - 1) >> 1) & 1, p.status);
           tc_fence_after();
 #pragma unroll 1
-          for (int ch = 0; ch < 4; ++ch) {
+          for (int ch = 0; ch < HD / 32; ++ch) {
             float o[32];
             tmem_ld_32x32(tmem_o + lane_addr + ch * 32, o);
 #pragma unroll
@@ -915,7 +923,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
       if (idx == nullptr && store_mask != nullptr && ok && __ldcg(store_mask + g.cache_row(t)) != 0) ok = false;   // a reused row
       __nv_bfloat16* dst = p.oc + (size_t)g.cache_row(t) * g.d + h * HD;
 #pragma unroll 1
-      for (int ch = 0; ch < 4; ++ch) {
+      for (int ch = 0; ch < HD / 32; ++ch) {
         float o[32];
         tmem_ld_32x32(tmem_o + lane_addr + ch * 32, o);
 #pragma unroll
@@ -966,11 +974,12 @@ bool attention_tc_two_tiles(const StepGeom& g, bool row_sparse) {
   return pick_form(g, row_sparse, &ksplit);
 }
 
-cudaError_t launch_attention_tc(const CUtensorMap& tm_k, const CUtensorMap& tm_v, const AttnParams& p,
-                                cudaStream_t st) {
+template <int HD>
+static cudaError_t launch_attention_hd(const CUtensorMap& tm_k, const CUtensorMap& tm_v, const AttnParams& p,
+                                       cudaStream_t st) {
   static std::atomic<unsigned long long> attr_one{0}, attr_pair{0};
-  if (cudaError_t e = ensure_dyn_smem(attn_tc_kernel, AttnSmem::TOTAL, attr_one); e != cudaSuccess) return e;
-  if (cudaError_t e = ensure_dyn_smem(attn_pair_kernel, PairSmem::TOTAL, attr_pair); e != cudaSuccess) return e;
+  if (cudaError_t e = ensure_dyn_smem(attn_tc_kernel<HD>, AttnSmem<HD>::TOTAL, attr_one); e != cudaSuccess) return e;
+  if (cudaError_t e = ensure_dyn_smem(attn_pair_kernel<HD>, PairSmem<HD>::TOTAL, attr_pair); e != cudaSuccess) return e;
   const int tps = (p.g.seq_act + BQ - 1) / BQ;
   const int tps2 = (p.g.seq_act + kPairRows - 1) / kPairRows;
   int ksplit = 1;
@@ -978,11 +987,16 @@ cudaError_t launch_attention_tc(const CUtensorMap& tm_k, const CUtensorMap& tm_v
   if (pair) {
     dim3 grid(p.g.n_heads, p.g.batch * tps2, 1);
     if (grid.y == 0) return cudaSuccess;
-    return launch_pdl(attn_pair_kernel, grid, dim3(kThreads), PairSmem::TOTAL, st, 1, tm_k, tm_v, p);
+    return launch_pdl(attn_pair_kernel<HD>, grid, dim3(kThreads), PairSmem<HD>::TOTAL, st, 1, tm_k, tm_v, p);
   }
   dim3 grid(p.g.n_heads, p.g.batch * tps, ksplit);
   if (grid.y == 0) return cudaSuccess;
-  return launch_pdl(attn_tc_kernel, grid, dim3(kThreads), AttnSmem::TOTAL, st, ksplit, tm_k, tm_v, p);
+  return launch_pdl(attn_tc_kernel<HD>, grid, dim3(kThreads), AttnSmem<HD>::TOTAL, st, ksplit, tm_k, tm_v, p);
+}
+
+cudaError_t launch_attention_tc(const CUtensorMap& tm_k, const CUtensorMap& tm_v, const AttnParams& p,
+                                cudaStream_t st) {
+  return p.g.head_dim == 64 ? launch_attention_hd<64>(tm_k, tm_v, p, st) : launch_attention_hd<128>(tm_k, tm_v, p, st);
 }
 
 }  // namespace dare

@@ -35,7 +35,7 @@ namespace dare {
 using namespace ptx;
 
 namespace {
-constexpr int BM = 128, BN = 256, BK = 64, HD = 128;
+constexpr int BM = 128, BN = 256, BK = 64;
 constexpr int A_BYTES = BM * BK * 2;
 template <bool PAIR>
 struct Ring {
@@ -82,7 +82,8 @@ __device__ __forceinline__ TileGeom tile_geom(const GemmParams& p, int tile, int
 
 // GATHER: the rows of the launch are listed by an index list with a device-side count (row geometry and finishing
 // pass by token); A maps a compact copy of them.
-template <int EPI, bool GATHER, bool PAIR>
+// HDIM: head width, 128 (a chunk of the finishing pass is half of a head) or 64 (a whole head)
+template <int EPI, bool GATHER, bool PAIR, int HDIM>
 __global__ void __launch_bounds__(kWarps * 32, 1)
 gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b0,
                     const __grid_constant__ CUtensorMap tm_b1, const GemmParams p, const int n_tiles,
@@ -248,13 +249,13 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
         if ((unsigned)tok_first >= (unsigned)p.g.tokens()) tok_first = 0;
       }
       const bool rotate = (EPI == EPI_Q) || (EPI == EPI_KV && !t.is_b1);
-      const int head0 = t.n0 / HD;
-      const bool score_tile = (EPI == EPI_Q) && p.g.score_head >= head0 && p.g.score_head < head0 + BN / HD;
+      const int score_col = (EPI == EPI_Q) ? p.g.score_head * HDIM - t.n0 : -1;   // first column of the scoring head in this tile
       __nv_bfloat16* out = t.is_b1 ? p.out1 : p.out0;
 #pragma unroll 1
       for (int chunk = 0; chunk < 4; ++chunk) {
-        const int hh = chunk >> 1, half = chunk & 1;
-        const int c_lo = hh * HD + half * 32;            // tile columns [c_lo, c_lo + 32) and their partners + 64
+        const int half = HDIM == 128 ? chunk & 1 : 0;
+        // tile columns [c_lo, c_lo + 32) and their rotary partners + HDIM / 2
+        const int c_lo = HDIM == 128 ? (chunk >> 1) * 128 + half * 32 : chunk * 64;
         {
           float v[32];
           tmem_ld_32x32(t_lane + c_lo, v);
@@ -262,7 +263,7 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
           for (int u = 0; u < 8; ++u)
             asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(stg_w + (uint32_t)((u ^ (lane & 7)) << 4)),
                          "f"(v[4 * u]), "f"(v[4 * u + 1]), "f"(v[4 * u + 2]), "f"(v[4 * u + 3]) : "memory");
-          tmem_ld_32x32(t_lane + c_lo + HD / 2, v);
+          tmem_ld_32x32(t_lane + c_lo + HDIM / 2, v);
 #pragma unroll
           for (int u = 0; u < 8; ++u)
             asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(stg_w + 128u + (uint32_t)((u ^ (lane & 7)) << 4)),
@@ -277,7 +278,7 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
           }
         }
         __syncwarp();
-        const bool score_chunk = score_tile && head0 + hh == p.g.score_head;
+        const bool score_chunk = score_col >= 0 && c_lo - half * 32 == score_col;
         // 16 passes of two rows (one per half-warp), four passes at a time so that their table reads overlap
 #pragma unroll 1
         for (int i0 = 0; i0 < 16; i0 += 4) {
@@ -309,16 +310,16 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
             lo[k] = *reinterpret_cast<const float2*>(row + off);
             hi[k] = *reinterpret_cast<const float2*>(row + 128 + off);
             if (rotate)
-              cs[k] = *reinterpret_cast<const float4*>(p.rope + (size_t)pos * (HD / 2) + half * 32 + 2 * l16);
+              cs[k] = *reinterpret_cast<const float4*>(p.rope + (size_t)pos * (HDIM / 2) + half * 32 + 2 * l16);
             if (EPI == EPI_Q && score_chunk && p.has_prev) {
-              const float* qp = p.q_prev + crowr * HD + half * 32 + 2 * l16;
+              const float* qp = p.q_prev + crowr * HDIM + half * 32 + 2 * l16;
               qa[k] = *reinterpret_cast<const float2*>(qp);
-              qb[k] = *reinterpret_cast<const float2*>(qp + HD / 2);
+              qb[k] = *reinterpret_cast<const float2*>(qp + HDIM / 2);
             }
             if (EPI == EPI_OUT_RES) {
               const __nv_bfloat16* rs = p.resid + (size_t)tokr * p.ld_resid + t.n0 + c_lo + 2 * l16;
               ra[k] = *reinterpret_cast<const __nv_bfloat162*>(rs);
-              rb[k] = *reinterpret_cast<const __nv_bfloat162*>(rs + HD / 2);
+              rb[k] = *reinterpret_cast<const __nv_bfloat162*>(rs + HDIM / 2);
             }
           }
 #pragma unroll
@@ -329,7 +330,8 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
             float2 vlo = lo[k], vhi = hi[k];
             if (EPI == EPI_Q && score_chunk) {
               // Sec. 3.1 on the un-rotated query of the scoring head: 1 - cos(current, stored); this quarter of the
-              // head adds its part of the three sums, the second half of the head finishes the row
+              // head adds its part of the three sums, the second half of the head finishes the row (a head of
+              // 64 is one chunk: no sums to hand on)
               float dot = 0.f, n2 = 0.f;
               if (p.has_prev) {
                 dot = vlo.x * qa[k].x + vlo.y * qa[k].y + vhi.x * qb[k].x + vhi.y * qb[k].y;
@@ -343,15 +345,15 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
                 n2 += __shfl_xor_sync(0xffffffffu, n2, o);
               }
               if (ok[k]) {
-                float* qp = p.q_prev + crow * HD + half * 32 + 2 * l16;
+                float* qp = p.q_prev + crow * HDIM + half * 32 + 2 * l16;
                 *reinterpret_cast<float2*>(qp) = vlo;
-                *reinterpret_cast<float2*>(qp + HD / 2) = vhi;
+                *reinterpret_cast<float2*>(qp + HDIM / 2) = vhi;
               }
               if (l16 == 0) {
-                if (half == 0) {
+                if (HDIM == 128 && half == 0) {
                   sc_acc[3 * rr] = dot; sc_acc[3 * rr + 1] = n1; sc_acc[3 * rr + 2] = n2;
                 } else if (ok[k]) {
-                  dot += sc_acc[3 * rr]; n1 += sc_acc[3 * rr + 1]; n2 += sc_acc[3 * rr + 2];
+                  if (HDIM == 128) { dot += sc_acc[3 * rr]; n1 += sc_acc[3 * rr + 1]; n2 += sc_acc[3 * rr + 2]; }
                   float sc = __int_as_float(0x7f800000);   // +inf: nothing to compare with
                   if (p.has_prev) {
                     const float den = sqrtf(n1) * sqrtf(n2);
@@ -375,11 +377,11 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
             const __nv_bfloat162 o_lo = __floats2bfloat162_rn(vlo.x, vlo.y), o_hi = __floats2bfloat162_rn(vhi.x, vhi.y);
             __nv_bfloat16* dst = out + orow * p.ld_out + t.n0 + c_lo + 2 * l16;
             *reinterpret_cast<__nv_bfloat162*>(dst) = o_lo;
-            *reinterpret_cast<__nv_bfloat162*>(dst + HD / 2) = o_hi;
+            *reinterpret_cast<__nv_bfloat162*>(dst + HDIM / 2) = o_hi;
             if ((EPI == EPI_OUT || EPI == EPI_OUT_RES) && p.out1 != nullptr) {   // the projected-output cache
               __nv_bfloat16* dst2 = p.out1 + crow * p.ld_out + t.n0 + c_lo + 2 * l16;
               *reinterpret_cast<__nv_bfloat162*>(dst2) = o_lo;
-              *reinterpret_cast<__nv_bfloat162*>(dst2 + HD / 2) = o_hi;
+              *reinterpret_cast<__nv_bfloat162*>(dst2 + HDIM / 2) = o_hi;
             }
           }
         }
@@ -397,11 +399,11 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
   }
 }
 
-template <int EPI, bool GATHER, bool PAIR = false>
-static cudaError_t launch_persist(const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1, const GemmParams& p,
+template <int EPI, bool GATHER, bool PAIR, int HDIM>
+static cudaError_t launch_persist_hd(const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1, const GemmParams& p,
                                   int n_tiles, int m_tiles, cudaStream_t st) {
   static std::atomic<unsigned long long> attr_done{0};
-  auto kern = gemm_persist_kernel<EPI, GATHER, PAIR>;
+  auto kern = gemm_persist_kernel<EPI, GATHER, PAIR, HDIM>;
   if (cudaError_t e = ensure_dyn_smem(kern, SMEM_TOTAL, attr_done); e != cudaSuccess) return e;
   int dev = 0, sms = 0;
   if (cudaError_t e = cudaGetDevice(&dev); e != cudaSuccess) return e;
@@ -415,6 +417,15 @@ static cudaError_t launch_persist(const CUtensorMap& a, const CUtensorMap& b0, c
   }
   return launch_pdl(kern, dim3(total < sms ? total : sms), dim3(kWarps * 32), SMEM_TOTAL, st,
                     1, a, b0, b1, q, n_tiles, total);
+}
+
+template <int EPI, bool GATHER, bool PAIR = false>
+static cudaError_t launch_persist(const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1, const GemmParams& p,
+                                  int n_tiles, int m_tiles, cudaStream_t st) {
+  if constexpr (EPI == EPI_Q || EPI == EPI_KV) {
+    if (p.g.head_dim == 64) return launch_persist_hd<EPI, GATHER, PAIR, 64>(a, b0, b1, p, n_tiles, m_tiles, st);
+  }
+  return launch_persist_hd<EPI, GATHER, PAIR, 128>(a, b0, b1, p, n_tiles, m_tiles, st);
 }
 
 // 256-wide tiles, no reduction split; b0 / b1 are maps with 256-row boxes (128-row boxes with pair != 0).  Listed

@@ -34,7 +34,16 @@ using namespace ptx;
 namespace {
 constexpr int BM = 128, BK = 64;
 constexpr int A_BYTES = BM * BK * 2;
-constexpr int HD = 128;                              // head width the rotary/score epilogues assume
+constexpr int CH = 128;                              // columns of a tile that one warp-wide row access covers
+// Columns a lane finishes inside a CH-wide piece of a tile: (lo, lo + 1) and their rotary partners (lo + HDIM / 2, ...).
+// A piece is one head of 128 or two heads of 64 (half of the lanes each).
+template <int HDIM>
+struct Lanes {
+  static constexpr int HALF = HDIM / 2;
+  static_assert(HDIM == 128 || HDIM == 64, "head widths of the tensor-core path");
+  static __device__ __forceinline__ int lo(int lane) { return HDIM == 128 ? 2 * lane : (lane >> 4) * 64 + 2 * (lane & 15); }
+  static __device__ __forceinline__ int in_head(int lane) { return (2 * lane) & (HALF - 1); }   // the same inside its head
+};
 // PAIR: two CTAs (row tiles 2i, 2i + 1 of the same column tile and reduction slice) share one M = 256 MMA; each
 // keeps its own 128 rows of A and only half of the W tile's rows in shared memory: 32 KB instead of 48 KB per stage
 // and CTA come through the L2, which is what bounds the main loop of the projections.
@@ -67,14 +76,15 @@ struct RowBatch {
   size_t crow[RB];
   bool ok[RB];
   float4 cs[RB];          // (cos, sin) of the two rotary pairs this lane owns
-  float2 qa[RB], qb[RB];  // stored query of the scoring head: elements 2*lane.. and 64 + 2*lane..
+  float2 qa[RB], qb[RB];  // stored query of the scoring head: this lane's elements and their rotary partners
   __nv_bfloat162 res[RB][2][2];   // residual row (output projection of a transformer block): this lane's pairs per head
 };
 
-template <int EPI, int RB, int kWarps, int BN>
+template <int EPI, int RB, int kWarps, int BN, int HDIM>
 __device__ __forceinline__ void load_row_batch(RowBatch<RB>& rb, const GemmParams& p, int rl0, int z, int rows_per_cta,
                                                int rows_valid, int t0, int pos0, size_t crow0, bool rotate,
                                                bool score_tile, int lane, int n0) {
+  using L = Lanes<HDIM>;
 #pragma unroll
   for (int k = 0; k < RB; ++k) {
     const int rl = rl0 + kWarps * k;
@@ -94,27 +104,28 @@ __device__ __forceinline__ void load_row_batch(RowBatch<RB>& rb, const GemmParam
       rb.crow[k] = crow0 + rc;
     }
     // no instruction consumes these loads before the finishing pass, so they stay in flight across the exchange
-    if (rotate) rb.cs[k] = *reinterpret_cast<const float4*>(p.rope + (size_t)pos * (HD / 2) + 2 * lane);
+    if (rotate) rb.cs[k] = *reinterpret_cast<const float4*>(p.rope + (size_t)pos * L::HALF + L::in_head(lane));
     if (EPI == EPI_Q && score_tile && p.has_prev) {
-      rb.qa[k] = *reinterpret_cast<const float2*>(p.q_prev + rb.crow[k] * HD + 2 * lane);
-      rb.qb[k] = *reinterpret_cast<const float2*>(p.q_prev + rb.crow[k] * HD + HD / 2 + 2 * lane);
+      rb.qa[k] = *reinterpret_cast<const float2*>(p.q_prev + rb.crow[k] * HDIM + L::in_head(lane));
+      rb.qb[k] = *reinterpret_cast<const float2*>(p.q_prev + rb.crow[k] * HDIM + L::HALF + L::in_head(lane));
     }
     if (EPI == EPI_OUT_RES) {
       const __nv_bfloat16* rs = p.resid + (size_t)rb.tok[k] * p.ld_resid + n0;
 #pragma unroll
-      for (int hh = 0; hh < BN / HD; ++hh) {
-        rb.res[k][hh][0] = *reinterpret_cast<const __nv_bfloat162*>(rs + hh * HD + 2 * lane);
-        rb.res[k][hh][1] = *reinterpret_cast<const __nv_bfloat162*>(rs + hh * HD + HD / 2 + 2 * lane);
+      for (int hh = 0; hh < BN / CH; ++hh) {
+        rb.res[k][hh][0] = *reinterpret_cast<const __nv_bfloat162*>(rs + hh * CH + 2 * lane);
+        rb.res[k][hh][1] = *reinterpret_cast<const __nv_bfloat162*>(rs + hh * CH + CH / 2 + 2 * lane);
       }
     }
   }
 }
 
-template <int EPI, int BN, bool PAIR>
+template <int EPI, int BN, bool PAIR, int HDIM>
 __global__ void __launch_bounds__(Warps<BN>::N * 32, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b0,
                const __grid_constant__ CUtensorMap tm_b1, const GemmParams p) {
   using C = Cfg<BN, PAIR>;
+  using L = Lanes<HDIM>;
   constexpr int STAGES = C::STAGES, STAGE_BYTES = C::STAGE_BYTES;
   constexpr int kWarps = Warps<BN>::N, RB = Warps<BN>::RB;
   constexpr int PROW_BYTES = C::PROW_BYTES, RECV_OFFSET = C::RECV_OFFSET;
@@ -269,8 +280,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
   const int nkb = KB / splits;                    // k-blocks this CTA walks for the tile
   const int quarter = warp & 3;                   // TMEM lanes a warp may touch: 32*quarter .. +31
   const bool rotate = (EPI == EPI_Q) || (EPI == EPI_KV && !is_b1);
-  const int head0 = n0 / HD;
-  const bool score_tile = (EPI == EPI_Q) && p.g.score_head >= head0 && p.g.score_head < head0 + BN / HD;
+  const int score_col = (EPI == EPI_Q) ? p.g.score_head * HDIM - n0 : -1;       // first column of the scoring head in this tile
+  const bool score_tile = score_col >= 0 && score_col < BN;
   RowBatch<RB> rb;
 
   if (active) {
@@ -346,13 +357,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     }
   } else {
     // While the main loop runs, pull the table rows the finishing pass of this CTA will read into the L2
-    // (dense tiles; 512 bytes = 4 lines per row and table).
+    // (dense tiles; 4 * HDIM bytes = LINES lines per row and table).
     if (p.idx == nullptr) {
-      for (int i = threadIdx.x - 64; i < rows_per_cta * 4; i += (kWarps - 2) * 32) {
-        const int r = z * rows_per_cta + (i >> 2);
+      constexpr int LINES = HDIM / 32;
+      for (int i = threadIdx.x - 64; i < rows_per_cta * LINES; i += (kWarps - 2) * 32) {
+        const int r = z * rows_per_cta + i / LINES;
         if (r >= rows_valid) break;
-        if (rotate) prefetch_l2(p.rope + (size_t)(pos0 + r) * (HD / 2) + (i & 3) * 16);
-        if (score_tile && p.has_prev) prefetch_l2(p.q_prev + (crow0 + r) * HD + (i & 3) * 32);
+        if (rotate) prefetch_l2(p.rope + (size_t)(pos0 + r) * L::HALF + (i % LINES) * 16);
+        if (score_tile && p.has_prev) prefetch_l2(p.q_prev + (crow0 + r) * HDIM + (i % LINES) * 32);
       }
     }
     // the table reads of this warp's first rows of the finishing pass: in flight for the whole main loop
@@ -363,7 +375,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       tok_own = p.idx[t0 + r_own];
       if (!token_ok(tok_own, p.g.tokens(), p.status)) tok_own = -1;      // read as a row of zeros
     }
-    load_row_batch<EPI, RB, kWarps, BN>(rb, p, warp, z, rows_per_cta, rows_valid, t0, pos0, crow0, rotate, score_tile, lane, n0);
+    load_row_batch<EPI, RB, kWarps, BN, HDIM>(rb, p, warp, z, rows_per_cta, rows_valid, t0, pos0, crow0, rotate, score_tile, lane, n0);
     if (gather && warp < 6) {
       // One stage of the A tile = 128 rows x 128 bytes (64 k-elements).  A warp takes 32 rows; one of its copy
       // instructions covers four rows, eight consecutive lanes fetching the eight 16-byte units of a row, so every
@@ -410,7 +422,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
 
   // The table reads of the first rows the producer and MMA warps will finish start now (those of the other warps
   // started before the main loop) and land during the exchange below.
-  if (warp < 2) load_row_batch<EPI, RB, kWarps, BN>(rb, p, warp, z, rows_per_cta, rows_valid, t0, pos0, crow0, rotate, score_tile, lane, n0);
+  if (warp < 2) load_row_batch<EPI, RB, kWarps, BN, HDIM>(rb, p, warp, z, rows_per_cta, rows_valid, t0, pos0, crow0, rotate, score_tile, lane, n0);
 
   // ---- every CTA of the cluster has finished its main loop: the rings are free to receive partial rows
   tc_fence_before();
@@ -463,22 +475,22 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
   if (splits > 1) mbar_wait(recv_bar, 0, p.status);     // the partner's rows have landed
   if (dbg && threadIdx.x == 64) p.debug[4] = globaltimer_ns();
 
-  // ---- finish the owned rows: one warp per row, lane <-> pairs (2*lane, 2*lane+1) of each head of the tile.
+  // ---- finish the owned rows: one warp per row, lane <-> column pairs of each piece of the tile.
   // Rows are taken four at a time so that their table reads are in flight together.
   {
     __nv_bfloat16* out = is_b1 ? p.out1 : p.out0;
 #pragma unroll 1
     for (int rl0 = warp; rl0 < rows_per_cta; rl0 += kWarps * RB) {
-      if (rl0 != warp) load_row_batch<EPI, RB, kWarps, BN>(rb, p, rl0, z, rows_per_cta, rows_valid, t0, pos0, crow0, rotate, score_tile, lane, n0);
+      if (rl0 != warp) load_row_batch<EPI, RB, kWarps, BN, HDIM>(rb, p, rl0, z, rows_per_cta, rows_valid, t0, pos0, crow0, rotate, score_tile, lane, n0);
       if (dbg && EPI == EPI_Q && threadIdx.x == 64) p.debug[34 + (rl0 - warp) / (kWarps * RB) * 2] = globaltimer_ns();
-      // (1) combine the partial rows: lane <-> pairs (2*lane, 2*lane+1) of each head
-      float2 vlo[RB][BN / HD], vhi[RB][BN / HD];
+      // (1) combine the partial rows: lane <-> a pair of columns of each piece and its rotary partners
+      float2 vlo[RB][BN / CH], vhi[RB][BN / CH];
 #pragma unroll
       for (int k = 0; k < RB; ++k) {
         const int rl = rb.ok[k] ? rl0 + kWarps * k : warp;     // rows that do not exist re-read an existing one
 #pragma unroll
-        for (int hh = 0; hh < BN / HD; ++hh) {
-          const int c_lo = hh * HD + 2 * lane, c_hi = c_lo + HD / 2;
+        for (int hh = 0; hh < BN / CH; ++hh) {
+          const int c_lo = hh * CH + L::lo(lane), c_hi = c_lo + L::HALF;
           // (unit of the column inside its 32-column chunk, swizzled by the row; rows_per_cta is a multiple of 8)
           const uint32_t in_lo = (uint32_t)(((((c_lo >> 2) & 7) ^ (rl & 7)) << 4) | ((c_lo & 3) << 2));
           const uint32_t in_hi = (uint32_t)(((((c_hi >> 2) & 7) ^ (rl & 7)) << 4) | ((c_hi & 3) << 2));
@@ -498,20 +510,22 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       //     reduced across the lanes together; lane k finishes row k.  Then the current query is stored.
       if (EPI == EPI_Q && score_tile) {
         float dot[RB], n1[RB], n2[RB];
+        const bool mine = HDIM == CH || (lane >> 4) == ((score_col / HDIM) & 1);   // this lane holds columns of the scoring head
 #pragma unroll
         for (int k = 0; k < RB; ++k) {
           float2 lo = vlo[k][0], hi = vhi[k][0];
 #pragma unroll
-          for (int hh = 1; hh < BN / HD; ++hh)
-            if (head0 + hh == p.g.score_head) { lo = vlo[k][hh]; hi = vhi[k][hh]; }
+          for (int hh = 1; hh < BN / CH; ++hh)
+            if (score_col / CH == hh) { lo = vlo[k][hh]; hi = vhi[k][hh]; }
           const float2 a = rb.qa[k], b = rb.qb[k];
           dot[k] = lo.x * a.x + lo.y * a.y + hi.x * b.x + hi.y * b.y;
           n1[k] = lo.x * lo.x + lo.y * lo.y + hi.x * hi.x + hi.y * hi.y;
           n2[k] = a.x * a.x + a.y * a.y + b.x * b.x + b.y * b.y;
-          if (rb.ok[k]) {
-            float* qp = p.q_prev + rb.crow[k] * HD;
-            *reinterpret_cast<float2*>(qp + 2 * lane) = lo;
-            *reinterpret_cast<float2*>(qp + HD / 2 + 2 * lane) = hi;
+          if (!mine) { dot[k] = 0.f; n1[k] = 0.f; n2[k] = 0.f; }
+          if (rb.ok[k] && mine) {
+            float* qp = p.q_prev + rb.crow[k] * HDIM + L::in_head(lane);
+            *reinterpret_cast<float2*>(qp) = lo;
+            *reinterpret_cast<float2*>(qp + L::HALF) = hi;
           }
         }
 #pragma unroll
@@ -544,19 +558,19 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         const size_t orow = p.out_is_cache == 1 ? rb.crow[k] : (p.out_is_cache == 2 ? (size_t)rb.row[k] : (size_t)rb.tok[k]);
         if (EPI == EPI_SWIGLU) {
           // columns [0, 128) of a 256-wide tile are the gate, [128, 256) the up projection of the same 128 outputs
-          const float2 g_lo = vlo[k][0], g_hi = vhi[k][0], u_lo = vlo[k][BN / HD - 1], u_hi = vhi[k][BN / HD - 1];
+          const float2 g_lo = vlo[k][0], g_hi = vhi[k][0], u_lo = vlo[k][BN / CH - 1], u_hi = vhi[k][BN / CH - 1];
           __nv_bfloat16* dst = out + orow * p.ld_out + n0;
           auto act = [](float g, float u) { return g / (1.f + __expf(-g)) * u; };
           *reinterpret_cast<__nv_bfloat162*>(dst + 2 * lane) = __floats2bfloat162_rn(act(g_lo.x, u_lo.x), act(g_lo.y, u_lo.y));
-          *reinterpret_cast<__nv_bfloat162*>(dst + HD / 2 + 2 * lane) =
+          *reinterpret_cast<__nv_bfloat162*>(dst + CH / 2 + 2 * lane) =
               __floats2bfloat162_rn(act(g_hi.x, u_hi.x), act(g_hi.y, u_hi.y));
           continue;
         }
         __nv_bfloat16* dst = out + orow * p.ld_out + n0;
 #pragma unroll
-        for (int hh = 0; hh < BN / HD; ++hh) {
+        for (int hh = 0; hh < BN / CH; ++hh) {
           float2 lo = vlo[k][hh], hi = vhi[k][hh];
-          const int c_lo = hh * HD + 2 * lane, c_hi = c_lo + HD / 2;
+          const int c_lo = hh * CH + L::lo(lane), c_hi = c_lo + L::HALF;
           if (rotate) {
             const float a0 = lo.x, b0 = hi.x, a1 = lo.y, b1 = hi.y;
             lo.x = a0 * rb.cs[k].x - b0 * rb.cs[k].y; hi.x = a0 * rb.cs[k].y + b0 * rb.cs[k].x;
@@ -618,11 +632,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
   }
 }
 
-template <int EPI, int BN, bool PAIR>
-static cudaError_t launch_one(const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1, const GemmParams& p,
+template <int EPI, int BN, bool PAIR, int HDIM>
+static cudaError_t launch_hd(const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1, const GemmParams& p,
                               int n_tiles, int m_tiles, int splits, cudaStream_t st) {
   static std::atomic<unsigned long long> attr_done{0};
-  auto kern = gemm_tc_kernel<EPI, BN, PAIR>;
+  auto kern = gemm_tc_kernel<EPI, BN, PAIR, HDIM>;
   constexpr int SMEM_TOTAL = Cfg<BN, PAIR>::SMEM_TOTAL;
   if (cudaError_t e = ensure_dyn_smem(kern, SMEM_TOTAL, attr_done); e != cudaSuccess) return e;
   GemmParams q = p;
@@ -632,6 +646,15 @@ static cudaError_t launch_one(const CUtensorMap& a, const CUtensorMap& b0, const
                          splits, a, b0, b1, q);
   return launch_pdl_xz(kern, dim3(n_tiles, m_tiles, splits), dim3(Warps<BN>::N * 32), SMEM_TOTAL, st, 1, splits, a, b0, b1,
                        q);
+}
+// (only the epilogues that rotate and score know heads; to the others the lane map is any map)
+template <int EPI, int BN, bool PAIR>
+static cudaError_t launch_one(const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1, const GemmParams& p,
+                              int n_tiles, int m_tiles, int splits, cudaStream_t st) {
+  if constexpr (EPI == EPI_Q || EPI == EPI_KV) {
+    if (p.g.head_dim == 64) return launch_hd<EPI, BN, PAIR, 64>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
+  }
+  return launch_hd<EPI, BN, PAIR, 128>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
 }
 
 // pair != 0: the launch uses two-CTA MMAs (256-wide tiles, A through the tensor map); b0 / b1 must then be maps with
