@@ -119,39 +119,31 @@ namespace {
 template <typename T>
 dare_status_t step_simt(dare_layer_t* L, const T* x, const StepGeom& g, int mode, float tau, T* y, cudaStream_t st) {
   const Buffers& B = L->buf;
-  const int T_ = g.tokens(), d = g.d;
-  const bool has_prev = L->has_prev;
-  const bool kv_sparse = has_prev && (mode & DARE_MODE_KV);
-  const bool o_sparse = has_prev && (mode & DARE_MODE_O);
+  const bool kv_sparse = L->has_prev && (mode & DARE_MODE_KV);
+  const bool o_sparse = L->has_prev && (mode & DARE_MODE_O);
+  const SimtStep s = {g, B.rope_cs, B.q_prev, B.scores, B.tmp, L->has_prev ? 1 : 0, B.status};
   int launches = 0;
   prof_begin(L);
   // Alg. 1/2 line 1
   prof_mark(L, SLOT_NORM, st);
-  launch_rmsnorm<T>(x, L->w.rms_gain, (T*)B.xn, T_, d, L->cfg.rms_eps, st); ++launches;
-  // line 2: dense Q projection
+  launch_rmsnorm<T>(x, L->w.rms_gain, (T*)B.xn, g.tokens(), g.d, L->cfg.rms_eps, st); ++launches;
+  // line 2: dense Q projection; line 3 + stored-query update + rotary embedding
   prof_mark(L, SLOT_Q_GEMM, st);
-  launch_gemm_simt<T>((const T*)B.xn, nullptr, nullptr, (const T*)L->w.w_q, B.tmp, T_, d, d, d, st); ++launches;
-  // line 3 + stored-query update + rotary embedding
-  prof_mark(L, SLOT_Q_POST, st);
-  launch_q_post_simt<T>(B.tmp, d, B.rope_cs, B.q_prev, B.scores, has_prev, (T*)B.q, g, st); ++launches;
+  CUDA_TRY(launch_q_simt<T>(s, (const T*)B.xn, (const T*)L->w.w_q, (T*)B.q, st, &launches));
   // lines 4-5: refresh set as a compacted index list; Sec. 4 staleness
   prof_mark(L, SLOT_SELECT, st);
   select_step(L, g, mode, tau, false, st, &launches);
   // K/V: Alg. 1 lines 6-9 (refresh set only) or Alg. 2 line 7 (all rows)
-  const int* kv_idx = kv_sparse ? B.idx : nullptr;
-  const int* kv_cnt = kv_sparse ? B.count : nullptr;
   prof_mark(L, SLOT_KV_GEMM, st);
-  launch_gemm_simt<T>((const T*)B.xn, kv_idx, kv_cnt, (const T*)L->w.w_k, B.tmp, T_, d, d, 2 * d, st, T_, B.status); ++launches;
-  launch_gemm_simt<T>((const T*)B.xn, kv_idx, kv_cnt, (const T*)L->w.w_v, B.tmp + d, T_, d, d, 2 * d, st, T_, B.status); ++launches;
-  prof_mark(L, SLOT_KV_POST, st);
-  launch_kv_post_simt<T>(B.tmp, 2 * d, kv_idx, kv_cnt, B.rope_cs, (T*)B.kc, (T*)B.vc, g, st, B.status); ++launches;
+  CUDA_TRY(launch_kv_simt<T>(s, (const T*)B.xn, kv_sparse ? B.idx : nullptr, kv_sparse ? B.count : nullptr,
+                             (const T*)L->w.w_k, (const T*)L->w.w_v, (T*)B.kc, (T*)B.vc, st)); ++launches;
   // attention: Alg. 1 line 10 (all rows) or Alg. 2 lines 6, 8-10 (refresh set rows, others keep the cache)
   prof_mark(L, SLOT_ATTN, st);
-  launch_attention_simt<T>((const T*)B.q, (const T*)B.kc, (const T*)B.vc, o_sparse ? B.idx : nullptr,
-                           o_sparse ? B.count : nullptr, (T*)B.oc, g, st, B.status); ++launches;
+  CUDA_TRY(launch_attention_simt<T>(s, (const T*)B.q, (const T*)B.kc, (const T*)B.vc, o_sparse ? B.idx : nullptr,
+                                    o_sparse ? B.batch_off : nullptr, (T*)B.oc, st)); ++launches;
   // last line: output projection of every row
   prof_mark(L, SLOT_OUT_GEMM, st);
-  launch_out_proj_simt<T>((const T*)B.oc, (const T*)L->w.w_o, B.tmp, y, g, st); ++launches;
+  CUDA_TRY(launch_out_simt<T>(s, (const T*)B.oc, (const T*)L->w.w_o, y, st)); ++launches;
   prof_end(L, st);
   L->last_launches = launches;
   CUDA_TRY(cudaGetLastError());

@@ -155,28 +155,32 @@ cudaError_t launch_select_large(const float* scores, long long n, float tau, int
 size_t select_large_flag_bytes(long long n);   // bytes of the decision words for n scores
 
 // ---- SIMT path (simt.cu) ----------------------------------------------------------------------------------
-// C[m, n] (fp32, ld = ldc) = sum_k A[arow(m), k] * W[n, k];  arow(m) = a_idx ? a_idx[m] : m;
-// rows m >= *count (when count != nullptr) are skipped.
+// What the kernels of one CUDA-core step share.
+struct SimtStep {
+  StepGeom g;
+  const float* rope_cs;
+  float* q_prev;
+  float* scores;
+  float* tmp;            // fp32 scratch [T, 2d]
+  int has_prev;
+  int* status;
+};
+// Q projection with its tail: score of the scoring head against q_prev (fp32, cache rows), q_prev update, rotary
+// embedding, store in the layer dtype (heads wider than 64: the score is a launch of its own).
 template <typename T>
-void launch_gemm_simt(const T* a, const int* a_idx, const int* count, const T* w, float* c, int m_max, int n, int k,
-                      int ldc, cudaStream_t st, int a_rows = 0, int* status = nullptr);   // a_rows: rows of a that a_idx may name
-// Q post-pass: score of the scoring head against q_prev (fp32, cache rows), q_prev update, rotary embedding,
-// store Q in the layer dtype.
+cudaError_t launch_q_simt(const SimtStep& s, const T* xn, const T* w_q, T* q, cudaStream_t st, int* launches);
+// K/V projection of the refresh set's rows (or all rows, idx == nullptr): rotary embedding on K, store to cache rows.
 template <typename T>
-void launch_q_post_simt(const float* qf, int ldq, const float* rope_cs, float* q_prev, float* scores, bool has_prev,
-                        T* q, const StepGeom& g, cudaStream_t st);
-// K/V post-pass: rows r < *count (or all when idx == nullptr): rotary embedding on K, store K and V to cache rows.
+cudaError_t launch_kv_simt(const SimtStep& s, const T* xn, const int* idx, const int* count, const T* w_k, const T* w_v,
+                           T* kc, T* vc, cudaStream_t st);
+// Attention: query rows = the refresh set (idx, sliced per sequence by batch_off) or all rows (idx == nullptr); output
+// rows go to the O cache.
 template <typename T>
-void launch_kv_post_simt(const float* kvf, int ld, const int* idx, const int* count, const float* rope_cs, T* kc,
-                         T* vc, const StepGeom& g, cudaStream_t st, int* status = nullptr);
-// Attention: query rows = idx[0..count) (or all rows when idx == nullptr), one warp per (row, head);
-// output rows go to the O cache.
-template <typename T>
-void launch_attention_simt(const T* q, const T* kc, const T* vc, const int* idx, const int* count, T* oc,
-                           const StepGeom& g, cudaStream_t st, int* status = nullptr);
+cudaError_t launch_attention_simt(const SimtStep& s, const T* q, const T* kc, const T* vc, const int* idx,
+                                  const int* batch_off, T* oc, cudaStream_t st);
 // y[t, :] = W_O oc[cache_row(t), :]
 template <typename T>
-void launch_out_proj_simt(const T* oc, const T* w_o, float* tmp, T* y, const StepGeom& g, cudaStream_t st);
+cudaError_t launch_out_simt(const SimtStep& s, const T* oc, const T* w_o, T* y, cudaStream_t st);
 
 // ---- tensor-core path (gemm_tc.cu, attn_tc.cu) -----------------------------------------------------------
 struct TcLayerMaps;  // tensor maps and launch state, owned by the handle
