@@ -31,13 +31,16 @@ __device__ __forceinline__ void fetch4(float* dst, const __nv_bfloat16* src, boo
 }
 
 // ------------------------------------------------------------------------------------------------ projections
-// C[m, n] = sum_k A[arow(m), k] * W[n, k]  (W stored [out, in]: Alg. 1 line 2).  A tile has 8 * RM rows and 64 columns:
-// 32 rotary pairs, columns (j, j + head_dim / 2) of the heads they belong to, so that the rotary embedding (and, with
-// heads of at most 64, the drift score) happens on the accumulators.  128 threads own RM x 4 results each; KG such groups
-// share the tile, each taking 32 of every 32 * KG k-elements.  Operands lie in shared memory row by row with k innermost
-// (pitch = 4 mod 32 words: the rows a quarter-warp reads start on different banks), three stages deep by cp.async; a
-// thread reads four k at a time and multiplies two of them per packed instruction (fma.f32x2), even and odd k in
-// accumulators of their own.  Bound by the FMA pipe and by shared-memory reads, 12 16-byte reads per 128 FMAs at RM = 8.
+// C[m, n] = sum_k A[arow(m), k] * W[n, k]  (W stored [out, in]: Alg. 1 line 2).  A tile has BM rows and 64 columns: 32
+// rotary pairs, columns (j, j + head_dim / 2) of the heads they belong to, so that the rotary embedding (and, with heads
+// of at most 64, the drift score) happens on the accumulators.  A CTA has 512 threads, 16 warps, and an SM to itself:
+// KG groups of 2 x WM warps share the tile, each taking 32 of every 32 * KG k-elements, and a thread owns RM x 4 results
+// (BM = 4 * RM * WM).  Operands lie in shared memory row by row with k innermost (pitch = 4 mod 32 words: the rows a
+// quarter-warp reads start on different banks), three stages deep by cp.async; a thread reads four k at a time and
+// multiplies two of them per packed instruction (fma.f32x2), even and odd k in accumulators of their own.
+// Bound by the FMA pipe and the registers that feed it: the inner loop alone reaches 53 TFLOP/s at RM = 6, 48 at RM = 4,
+// 30 at RM = 2.  (Two CTAs of 256 threads an SM were slower: a launch of one wave filled SMs two by two and left the
+// others idle.)
 enum { SG_Q = 0, SG_KV = 1, SG_OUT = 2 };
 struct SgemmParams {
   const void* a;
@@ -57,21 +60,25 @@ struct SgemmParams {
   int has_prev;
   int* status;
 };
-constexpr int kStages = 3, kGroup = 128;
+constexpr int kStages = 3, kSgThreads = 512;
 
-template <int RM, int KG>
+template <int RM, int WM, int KG>
 struct Sg {
-  static constexpr int BM = 8 * RM, BN = 64, BK = 32 * KG, PITCH = BK + 4, THREADS = kGroup * KG;
+  static constexpr int GROUP = 64 * WM;                               // threads of a k-group
+  static_assert(GROUP * KG == kSgThreads, "16 warps");
+  static constexpr int BM = 4 * RM * WM, BN = 64, BK = 32 * KG, PITCH = BK + 4, THREADS = kSgThreads;
   static constexpr int STAGE = (BN + BM) * PITCH;                     // floats: W rows, then A rows
   static constexpr int CHUNKS = (BN + BM) * (BK / 4) / THREADS, W_CHUNKS = BN * (BK / 4) / THREADS;
-  static_assert(W_CHUNKS == 4, "16 rows per chunk index");
-  static constexpr int SMEM = kStages * STAGE * 4;
+  static constexpr int ROWS = THREADS / (BK / 4);                     // rows per chunk index
+  static_assert(W_CHUNKS * ROWS == BN && CHUNKS * ROWS == BN + BM, "whole rows per chunk index");
+  static constexpr int SMEM = kStages * STAGE * 4 > 116 * 1024 ? kStages * STAGE * 4 : 116 * 1024;   // one CTA an SM
   static_assert((KG - 1) * BM * BN <= kStages * STAGE, "group sums fit the ring");
 };
 
-template <typename T, int EPI, int RM, int KG>
-__global__ void __launch_bounds__(kGroup* KG) sgemm_kernel(const SgemmParams p) {
-  using S = Sg<RM, KG>;
+template <typename T, int EPI, int RM, int WM, int KG>
+__global__ void __launch_bounds__(kSgThreads, 1) sgemm_kernel(const SgemmParams p) {
+  using S = Sg<RM, WM, KG>;
+  constexpr int kGroup = S::GROUP;
   constexpr int BM = S::BM, PITCH = S::PITCH;
   extern __shared__ __align__(16) float ring[];
   __shared__ int s_tok[BM];                      // token of a row, -1: no such row
@@ -89,7 +96,7 @@ __global__ void __launch_bounds__(kGroup* KG) sgemm_kernel(const SgemmParams p) 
   const T* w = reinterpret_cast<const T*>(second ? p.w1 : p.w0);
 #pragma unroll
   for (int i = 0; i < S::W_CHUNKS; ++i) {
-    const int n = i * 16 + row_of, pair = pair0 + (n & 31);
+    const int n = i * S::ROWS + row_of, pair = pair0 + (n & 31);
     ok[i] = pair < n_pairs;
     src[i] = w + (size_t)(ok[i] ? column(pair, n >> 5) : 0) * K + kc;
   }
@@ -100,7 +107,7 @@ __global__ void __launch_bounds__(kGroup* KG) sgemm_kernel(const SgemmParams p) 
     for (int i = 0; i < S::CHUNKS; ++i) {
       if (i < i0 || i >= i1) continue;
       const bool in = ok[i] && kb * S::BK + kc < K;
-      fetch4(st + (i * 16 + row_of) * PITCH + kc, src[i] + (in ? kb * S::BK : -kc), in);
+      fetch4(st + (i * S::ROWS + row_of) * PITCH + kc, src[i] + (in ? kb * S::BK : -kc), in);
     }
   };
   // the weights do not depend on the kernel before: their first stages are on their way while it drains
@@ -130,7 +137,7 @@ __global__ void __launch_bounds__(kGroup* KG) sgemm_kernel(const SgemmParams p) 
   __syncthreads();
 #pragma unroll
   for (int i = S::W_CHUNKS; i < S::CHUNKS; ++i) {
-    const int t = s_tok[(i - S::W_CHUNKS) * 16 + row_of];
+    const int t = s_tok[(i - S::W_CHUNKS) * S::ROWS + row_of];
     ok[i] = t >= 0;
     const size_t row = t < 0 ? 0 : (p.a_cache_rows ? (size_t)p.g.cache_row(t) : (size_t)t);
     src[i] = reinterpret_cast<const T*>(p.a) + row * K + kc;
@@ -141,15 +148,15 @@ __global__ void __launch_bounds__(kGroup* KG) sgemm_kernel(const SgemmParams p) 
     cp_async_commit();                           // (the first group holds every stage's W chunks as well)
   }
 
-  const int grp = tid / kGroup, wp = (tid >> 5) & 3, lane = tid & 31;
+  const int grp = tid / kGroup, wp = (tid % kGroup) >> 5, lane = tid & 31;
   const int wm = wp >> 1, wn = wp & 1, tx = lane & 7, ty = lane >> 3;
-  // rows wm * BM/2 + ty + 4 i; columns 16 wn + tx + {0, 8} and their partners + 32
+  // rows wm * 4 RM + ty + 4 i; columns 16 wn + tx + {0, 8} and their partners + 32
   float2 acc[RM][4];
 #pragma unroll
   for (int i = 0; i < RM; ++i)
 #pragma unroll
     for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
-  const int w_at = (16 * wn + tx) * PITCH + grp * 32, a_at = (64 + wm * (BM / 2) + ty) * PITCH + grp * 32;
+  const int w_at = (16 * wn + tx) * PITCH + grp * 32, a_at = (64 + wm * (4 * RM) + ty) * PITCH + grp * 32;
   for (int kb = 0; kb < nk; ++kb) {
     cp_async_wait<kStages - 2>();
     __syncthreads();
@@ -193,15 +200,31 @@ __global__ void __launch_bounds__(kGroup* KG) sgemm_kernel(const SgemmParams p) 
       for (int e = 0; e < RM * 4; ++e) v[e >> 2][e & 3] += ring[(gi * RM * 4 + e) * kGroup + tid];
   }
 
-  // ---- the projection's own tail
+  // ---- the projection's own tail.  All table reads first: one memory round trip for the rows of this thread.
   const int pair = pair0 + 16 * wn + tx;         // and pair + 8
   const bool score_tile = EPI == SG_Q && half <= 32 && ((p.g.score_head * half) >> 5) == pair0 >> 5;
+  const bool rotate = EPI == SG_Q || (EPI == SG_KV && !second);
   T* out = reinterpret_cast<T*>(second ? p.out1 : p.out0);
+  float2 cs[RM][2], old[RM][2];
 #pragma unroll
   for (int i = 0; i < RM; ++i) {
-    const int r = wm * (BM / 2) + ty + 4 * i, t = s_tok[r];
+    const int t = s_tok[wm * (4 * RM) + ty + 4 * i];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int pj = pair + 8 * j, jj = pj & (half - 1);
+      cs[i][j] = old[i][j] = make_float2(0.f, 0.f);
+      if (t < 0 || pj >= n_pairs) continue;
+      if (rotate) cs[i][j] = p.rope[(size_t)p.g.position(t) * half + jj];
+      if (score_tile && p.has_prev && (pj >> lh) == p.g.score_head) {
+        const float* qp = p.q_prev + (size_t)p.g.cache_row(t) * (2 * half) + jj;
+        old[i][j] = make_float2(qp[0], qp[half]);
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < RM; ++i) {
+    const int r = wm * (4 * RM) + ty + 4 * i, t = s_tok[r];
     const bool row_ok = t >= 0;
-    const int pos = row_ok ? p.g.position(t) : 0;
     const size_t cr = row_ok ? (size_t)p.g.cache_row(t) : 0;
     float dot = 0.f, n1 = 0.f, n2 = 0.f;
 #pragma unroll
@@ -213,20 +236,17 @@ __global__ void __launch_bounds__(kGroup* KG) sgemm_kernel(const SgemmParams p) 
       if (EPI == SG_Q && (pj >> lh) == p.g.score_head) {
         // Sec. 3.1 on the un-rotated query; the current one is kept for the next step (Sec. 3.2)
         if (score_tile) {
+          const float2 o = old[i][j];
+          dot = fmaf(a, o.x, fmaf(b, o.y, dot)); n1 = fmaf(a, a, fmaf(b, b, n1)); n2 = fmaf(o.x, o.x, fmaf(o.y, o.y, n2));
           float* qp = p.q_prev + cr * (2 * half) + jj;
-          if (p.has_prev) {
-            const float pa = qp[0], pb = qp[half];
-            dot = fmaf(a, pa, fmaf(b, pb, dot)); n1 = fmaf(a, a, fmaf(b, b, n1)); n2 = fmaf(pa, pa, fmaf(pb, pb, n2));
-          }
           qp[0] = a; qp[half] = b;
         } else {
           float* qr = p.q_raw + (size_t)t * (2 * half) + jj;
           qr[0] = a; qr[half] = b;
         }
       }
-      if (EPI == SG_Q || (EPI == SG_KV && !second)) {
-        const float2 cs = p.rope[(size_t)pos * half + jj];
-        const float ra = a * cs.x - b * cs.y, rb = a * cs.y + b * cs.x;
+      if (rotate) {
+        const float ra = a * cs[i][j].x - b * cs[i][j].y, rb = a * cs[i][j].y + b * cs[i][j].x;
         a = ra; b = rb;
       }
       T* dst = out + (EPI == SG_KV ? cr : (size_t)t) * K + c;
@@ -286,11 +306,11 @@ __global__ void __launch_bounds__(256) score_kernel(const float* __restrict__ q_
   }
 }
 
-template <typename T, int EPI, int RM, int KG>
+template <typename T, int EPI, int RM, int WM, int KG>
 cudaError_t launch_sgemm_as(const SgemmParams& p, int n_tiles, cudaStream_t st) {
-  using S = Sg<RM, KG>;
+  using S = Sg<RM, WM, KG>;
   static std::atomic<unsigned long long> attr_done{0};
-  auto kern = sgemm_kernel<T, EPI, RM, KG>;
+  auto kern = sgemm_kernel<T, EPI, RM, WM, KG>;
   if (cudaError_t e = ensure_dyn_smem(kern, S::SMEM, attr_done); e != cudaSuccess) return e;
   return launch_pdl(kern, dim3(n_tiles, (p.rows + S::BM - 1) / S::BM), dim3(S::THREADS), S::SMEM, st, 1, p);
 }
@@ -299,25 +319,35 @@ template <typename T, int EPI>
 cudaError_t launch_sgemm(const SgemmParams& p, int rows_likely, cudaStream_t st) {
   if (p.rows <= 0) return cudaSuccess;
   const int n_tiles = (p.g.d / 2 + 31) / 32 * (EPI == SG_KV ? 2 : 1);
-  auto tiles = [&](int bm) { return n_tiles * ((rows_likely + bm - 1) / bm); };
-  // The taller tile reads less shared memory per FMA (measured rate 1 : 1.25 : 1.9), the shorter ones spread few rows over
-  // more SMs: whichever leaves the busiest SM the least to do.
-  auto cost = [&](int bm, float f) { return (float)((tiles(bm) + 147) / 148 * bm) * f; };
-  const float c64 = cost(64, 1.f), c32 = cost(32, 1.25f), c16 = cost(16, 1.9f);
-  if (c16 < c32 && c16 < c64) return launch_sgemm_as<T, EPI, 2, 4>(p, n_tiles, st);
-  if (c32 < c64) return launch_sgemm_as<T, EPI, 4, 2>(p, n_tiles, st);
-  return launch_sgemm_as<T, EPI, 8, 1>(p, n_tiles, st);
+  // What a launch takes is its waves of 148 tiles times the tile height over the rate of its inner loop (above), plus what
+  // a tile costs whatever its height (first operands, finishing: measured as about 12 rows).
+  auto cost = [&](int bm, float f) {
+    return (float)((n_tiles * ((rows_likely + bm - 1) / bm) + 147) / 148) * (12.f + (float)bm * f);
+  };
+  const float c[5] = {cost(96, 1.f), cost(64, 1.1f), cost(48, 1.f), cost(32, 1.1f), cost(16, 1.8f)};
+  int best = 0;
+  for (int i = 1; i < 5; ++i)
+    if (c[i] < c[best]) best = i;
+  switch (best) {
+    case 0: return launch_sgemm_as<T, EPI, 6, 4, 2>(p, n_tiles, st);
+    case 1: return launch_sgemm_as<T, EPI, 4, 4, 2>(p, n_tiles, st);
+    case 2: return launch_sgemm_as<T, EPI, 6, 2, 4>(p, n_tiles, st);
+    case 3: return launch_sgemm_as<T, EPI, 4, 2, 4>(p, n_tiles, st);
+    default: return launch_sgemm_as<T, EPI, 2, 2, 4>(p, n_tiles, st);
+  }
 }
 }  // namespace
 
 // ------------------------------------------------------------------------------------------------ attention
 // Eq. 4 / Alg. 2 line 8 (row-sparse) and Alg. 1 line 10 (all rows): bidirectional softmax attention, no mask, fp32.
-// One CTA = one head x 32 query rows of one sequence.  Two groups of 128 threads take alternate key blocks, each with
-// its own double-buffered K and V tiles (cp.async), running maxima, sums and accumulators, merged at the end.  A thread
-// owns 4 rows: scores of BKV / 16 keys each, then HD / 16 output columns each; the 16 lanes of a half-warp share their
-// rows, so the softmax is shuffles and the probabilities pass through shared memory within the half-warp only.
-// Bound by the FMA pipe and shared-memory reads like the projections (8 16-byte reads per 64 FMAs).  The result row is
-// written into the O cache; rows that are not computed keep what they hold (Alg. 2 lines 9-10).
+// One CTA = one head x 32 * RG query rows of one sequence, RG x KG groups of 128 threads: a group has 32 of the rows and
+// every KG-th key block.  The RG groups of a key group share its K and V tile (cp.async: the next K block arrives while
+// P V is computed, V while S is); KG partial results are merged at the end.  A thread owns 4 rows: scores of BKV / 16 keys
+// each, then HD / 16 output columns each; the 16 lanes of a half-warp share their rows, so the softmax is shuffles and the
+// probabilities pass through shared memory within the half-warp only.
+// Bound by the FMA pipe and shared-memory reads like the projections (8 16-byte reads per 64 FMAs).  Row groups re-read
+// the keys least, key groups leave more SMs with work when rows are few (launch rule below).  The result row is written
+// into the O cache; rows that are not computed keep what they hold (Alg. 2 lines 9-10).
 // (One warp per row and head, a key at a time, was bound by the latency of its five-step reduction per key: 2 x 384 rows
 // of 16 heads x 64 over 384 keys took about 300 us.)
 namespace {
@@ -331,25 +361,28 @@ struct SattnParams {
   StepGeom g;
   int* status;
 };
-template <int HD>
+template <int HD, int RG, int KG>
 struct Sa {
-  static constexpr int BQ = 32, BKV = HD <= 64 ? 64 : (HD == 128 ? 32 : 16), JN = BKV / 16;
+  static constexpr int BQ = 32 * RG, BKV = HD == 256 ? 16 : (HD == 128 || KG > 2 ? 32 : 64), JN = BKV / 16;
+  static constexpr int THREADS = 128 * RG * KG;
   static constexpr int KP = HD + 4, PP = BKV + 4;                       // pitches of K / Q rows and of the probabilities
   static constexpr int VW = HD >= 64 ? 4 : 2, NC = HD / (16 * VW);      // a lane's output columns: NC vectors of VW
   static constexpr int BUF = BKV * KP + BKV * HD;                       // K and V of one block (floats)
-  static constexpr int Q_OFF = 0, P_OFF = BQ * KP, KV_OFF = P_OFF + 2 * BQ * PP, FLOATS = KV_OFF + 2 * 2 * BUF;
+  static constexpr int Q_OFF = 0, P_OFF = BQ * KP, KV_OFF = P_OFF + KG * BQ * PP, FLOATS = KV_OFF + KG * BUF;
+  static constexpr int PART = BQ * HD + 2 * BQ;                         // a key group's part in the merge, over Q, P, K, V
   static constexpr int SMEM = FLOATS * 4;
-  static_assert(SMEM <= 226 * 1024 && BQ * HD + 2 * BQ <= 2 * BUF, "shared memory, merge buffer");
+  static_assert(SMEM <= 226 * 1024 && (KG - 1) * PART <= FLOATS, "shared memory, merge buffer");
 };
 
-template <typename T, int HD>
-__global__ void __launch_bounds__(256) sattn_kernel(const SattnParams p) {
-  using S = Sa<HD>;
+template <typename T, int HD, int RG, int KG>
+__global__ void __launch_bounds__(128 * RG * KG, 1) sattn_kernel(const SattnParams p) {
+  using S = Sa<HD, RG, KG>;
   constexpr int BQ = S::BQ, BKV = S::BKV, JN = S::JN, KP = S::KP, PP = S::PP, VW = S::VW, NC = S::NC;
   extern __shared__ __align__(16) float sm[];
   __shared__ int s_tok[BQ];
   const StepGeom& g = p.g;
-  const int tid = threadIdx.x, grp = tid >> 7, gt = tid & 127, tx = gt & 15, ty = gt >> 4;
+  const int tid = threadIdx.x, grp = tid / (128 * RG), lt = tid % (128 * RG), tx = tid & 15, ty = lt >> 4;   // key group; row
+  const int r0 = (ty >> 3) * 32 + (ty & 7);                             // this thread's rows: r0 + 8 i
   const int h = blockIdx.x, b = blockIdx.y, tile = blockIdx.z, d = g.d;
   pdl_wait();
   pdl_launch_dependents();
@@ -366,30 +399,31 @@ __global__ void __launch_bounds__(256) sattn_kernel(const SattnParams p) {
   const T* kbase = reinterpret_cast<const T*>(p.kc) + (size_t)b * g.max_seq * d + h * HD;
   const T* vbase = reinterpret_cast<const T*>(p.vc) + (size_t)b * g.max_seq * d + h * HD;
   const int n_blocks = (g.kv_len + BKV - 1) / BKV;
-  float* kv = sm + S::KV_OFF + grp * 2 * S::BUF;
-  auto fetch_block = [&](int blk, int buf) {       // keys past the last: zeros
-    float* kd = kv + buf * S::BUF;
-    float* vd = kd + BKV * KP;
-    for (int c = gt; c < BKV * (HD / 4); c += 128) {
-      const int r = c / (HD / 4), e = (c % (HD / 4)) * 4, key = blk * BKV + r;
-      const bool ok = key < g.kv_len;
-      const size_t off = (size_t)(ok ? key : 0) * d + e;
-      fetch4(kd + r * KP + e, kbase + off, ok);
-      fetch4(vd + r * HD + e, vbase + off, ok);
+  float* kd = sm + S::KV_OFF + grp * S::BUF;
+  float* vd = kd + BKV * KP;
+  auto fetch_block = [&](float* dst, int pitch, const T* base, int blk) {       // keys past the last: zeros
+    if (blk < n_blocks) {
+#pragma unroll 4
+      for (int c = lt; c < BKV * (HD / 4); c += 128 * RG) {
+        const int r = c / (HD / 4), e = (c % (HD / 4)) * 4, key = blk * BKV + r;
+        const bool ok = key < g.kv_len;
+        fetch4(dst + r * pitch + e, base + (size_t)(ok ? key : 0) * d + e, ok);
+      }
     }
+    cp_async_commit();                             // (empty past the last block: the group count stays uniform)
   };
-  if (grp < n_blocks) fetch_block(grp, 0);
   if (tid < BQ) {
     int t = tid < n_rows ? (p.idx ? p.idx[row0 + tid] : row0 + tid) : -1;
     if (p.idx && t != -1 && !token_ok(t, g.tokens(), p.status)) t = -1;   // neither a query row to read nor a cache row to write
     s_tok[tid] = t;
   }
   __syncthreads();
-  for (int c = tid; c < BQ * (HD / 4); c += 256) {
+  for (int c = tid; c < BQ * (HD / 4); c += S::THREADS) {
     const int r = c / (HD / 4), e = (c % (HD / 4)) * 4, t = s_tok[r];
     fetch4(sm + S::Q_OFF + r * KP + e, reinterpret_cast<const T*>(p.q) + (size_t)(t < 0 ? 0 : t) * d + h * HD + e, t >= 0);
   }
-  cp_async_commit();
+  fetch_block(kd, KP, kbase, grp);                 // (one group with Q)
+  fetch_block(vd, HD, vbase, grp);
   const float c = rsqrtf((float)HD) * 1.4426950408889634f;              // softmax scale folded into the exp2 argument
   float m[4], l[4], acc[4][NC][VW];
 #pragma unroll
@@ -400,16 +434,18 @@ __global__ void __launch_bounds__(256) sattn_kernel(const SattnParams p) {
 #pragma unroll
       for (int e = 0; e < VW; ++e) acc[i][n][e] = 0.f;
   }
-  const float* qs = sm + S::Q_OFF + ty * KP;                            // rows ty + 8 i
-  float* ps = sm + S::P_OFF + grp * BQ * PP + ty * PP;
-  cp_async_wait<0>();
-  __syncthreads();                                                      // Q is both groups'
-  int buf = 0;
-  for (int blk = grp; blk < n_blocks; blk += 2, buf ^= 1) {
-    if (blk + 2 < n_blocks) fetch_block(blk + 2, buf ^ 1);
-    cp_async_commit();
-    const float* ks = kv + buf * S::BUF + tx * KP;                      // keys tx + 16 j
-    const float* vs = kv + buf * S::BUF + BKV * KP + tx * VW;
+  const float* qs = sm + S::Q_OFF + r0 * KP;
+  float* ps = sm + S::P_OFF + (grp * BQ + r0) * PP;
+  const float* ks = kd + tx * KP;                                       // keys tx + 16 j
+  const float* vs = vd + tx * VW;
+  auto group_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(128 * RG) : "memory"); };
+  cp_async_wait<1>();
+  __syncthreads();                                                      // Q is every group's
+  for (int blk = grp; blk < n_blocks; blk += KG) {
+    if (blk != grp) {
+      cp_async_wait<1>();                                               // this K block; its V may still be on its way
+      group_sync();
+    }
     float2 s2[4][JN];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
@@ -430,6 +466,8 @@ __global__ void __launch_bounds__(256) sattn_kernel(const SattnParams p) {
           s2[i][j] = __ffma2_rn(make_float2(qf[i].z, qf[i].w), make_float2(kf[j].z, kf[j].w), s2[i][j]);
         }
     }
+    group_sync();                                                       // everybody is done with the K block
+    fetch_block(kd, KP, kbase, blk + KG);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       float s[JN], mx = m[i];
@@ -455,7 +493,8 @@ __global__ void __launch_bounds__(256) sattn_kernel(const SattnParams p) {
 #pragma unroll
         for (int e = 0; e < VW; ++e) acc[i][n][e] *= corr;
     }
-    __syncwarp();
+    cp_async_wait<1>();                                                 // this V block
+    group_sync();                                                       // (and the half-warp's probabilities)
 #pragma unroll 2
     for (int k = 0; k < BKV; k += 4) {
       float4 pf[4];
@@ -486,49 +525,85 @@ __global__ void __launch_bounds__(256) sattn_kernel(const SattnParams p) {
           }
         }
     }
-    cp_async_wait<0>();
-    asm volatile("bar.sync %0, 128;" ::"r"(1 + grp) : "memory");        // the group is done with this buffer; the next has landed
+    group_sync();
+    fetch_block(vd, HD, vbase, blk + KG);
   }
+  cp_async_wait<0>();
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
     for (int o = 8; o > 0; o >>= 1) l[i] += __shfl_xor_sync(0xffffffffu, l[i], o);
-  // group 1 hands its part over through its own (idle) K/V buffers
-  float* part = sm + S::KV_OFF + 2 * S::BUF;                            // accumulators [BQ][HD], then maxima, then sums
-  if (grp == 1) {
+  // key groups hand their parts to the first one through shared memory, idle once all are past their blocks
+  if (KG > 1) {
+    __syncthreads();
+    float* part = sm + (grp - 1) * S::PART;                             // accumulators [BQ][HD], then maxima, then sums
+    if (grp > 0) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int r = ty + 8 * i;
+      for (int i = 0; i < 4; ++i) {
+        const int r = r0 + 8 * i;
 #pragma unroll
-      for (int n = 0; n < NC; ++n)
+        for (int n = 0; n < NC; ++n)
 #pragma unroll
-        for (int e = 0; e < VW; ++e) part[r * HD + n * 16 * VW + tx * VW + e] = acc[i][n][e];
-      if (tx == 0) { part[BQ * HD + r] = m[i]; part[BQ * HD + BQ + r] = l[i]; }
+          for (int e = 0; e < VW; ++e) part[r * HD + n * 16 * VW + tx * VW + e] = acc[i][n][e];
+        if (tx == 0) { part[BQ * HD + r] = m[i]; part[BQ * HD + BQ + r] = l[i]; }
+      }
     }
+    __syncthreads();
+    if (grp > 0) return;
   }
-  __syncthreads();
-  if (grp == 1) return;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const int r = ty + 8 * i, t = s_tok[r];
+    const int r = r0 + 8 * i, t = s_tok[r];
     if (t < 0) continue;
-    const float mo = part[BQ * HD + r], lo = part[BQ * HD + BQ + r], mx = fmaxf(m[i], mo);
-    const float wa = exp2f(m[i] - mx), wb = exp2f(mo - mx), inv = 1.f / (wa * l[i] + wb * lo);
+    float w[KG], mx = m[i], sum = 0.f;
+#pragma unroll
+    for (int k = 1; k < KG; ++k) mx = fmaxf(mx, sm[(k - 1) * S::PART + BQ * HD + r]);
+    w[0] = exp2f(m[i] - mx);
+    sum = w[0] * l[i];
+#pragma unroll
+    for (int k = 1; k < KG; ++k) {
+      const float* pk = sm + (k - 1) * S::PART + BQ * HD;
+      w[k] = exp2f(pk[r] - mx);
+      sum = fmaf(w[k], pk[BQ + r], sum);
+    }
+    const float inv = 1.f / sum;
     T* dst = reinterpret_cast<T*>(p.oc) + (size_t)g.cache_row(t) * d + h * HD + tx * VW;
 #pragma unroll
     for (int n = 0; n < NC; ++n)
 #pragma unroll
-      for (int e = 0; e < VW; ++e)
-        dst[n * 16 * VW + e] = from_f<T>((wa * acc[i][n][e] + wb * part[r * HD + n * 16 * VW + tx * VW + e]) * inv);
+      for (int e = 0; e < VW; ++e) {
+        float o = w[0] * acc[i][n][e];
+#pragma unroll
+        for (int k = 1; k < KG; ++k) o = fmaf(w[k], sm[(k - 1) * S::PART + r * HD + n * 16 * VW + tx * VW + e], o);
+        dst[n * 16 * VW + e] = from_f<T>(o * inv);
+      }
   }
 }
 
+template <typename T, int HD, int RG, int KG>
+cudaError_t launch_sattn_as(const SattnParams& p, cudaStream_t st) {
+  using S = Sa<HD, RG, KG>;
+  static std::atomic<unsigned long long> attr_done{0};
+  auto kern = sattn_kernel<T, HD, RG, KG>;
+  if (cudaError_t e = ensure_dyn_smem(kern, S::SMEM, attr_done); e != cudaSuccess) return e;
+  return launch_pdl(kern, dim3(p.g.n_heads, p.g.batch, (p.g.seq_act + S::BQ - 1) / S::BQ), dim3(S::THREADS), S::SMEM, st, 1,
+                    p);
+}
 template <typename T, int HD>
 cudaError_t launch_sattn_hd(const SattnParams& p, cudaStream_t st) {
-  static std::atomic<unsigned long long> attr_done{0};
-  auto kern = sattn_kernel<T, HD>;
-  if (cudaError_t e = ensure_dyn_smem(kern, Sa<HD>::SMEM, attr_done); e != cudaSuccess) return e;
-  return launch_pdl(kern, dim3(p.g.n_heads, p.g.batch, (p.g.seq_act + 31) / 32), dim3(256), Sa<HD>::SMEM, st, 1, p);
+  // rows a sequence is likely to have (a refresh set's size is known to the device only: a quarter of the window)
+  const int rows = p.idx ? (p.g.seq_act + 3) / 4 : p.g.seq_act;
+  // waves of 148 CTAs, times the rows of one, times the key blocks its slowest group takes
+  auto cost = [&](int bq, int kg, int bkv, float f) {
+    const int tiles = p.g.n_heads * p.g.batch * ((rows + bq - 1) / bq), blocks = (p.g.kv_len + bkv - 1) / bkv;
+    return (float)((tiles + 147) / 148) * (float)bq * (float)((blocks + kg - 1) / kg * kg * bkv) * f;
+  };
+  const int b1 = Sa<HD, 1, 4>::BKV, b2 = Sa<HD, 2, 2>::BKV, b3 = Sa<HD, 3, 1>::BKV;
+  const float c1 = cost(32, 4, b1, 1.15f), c2 = cost(64, 2, b2, 1.f), c3 = cost(96, 1, b3, 1.05f), c4 = cost(128, 1, b3, 1.f);
+  if (c1 <= c2 && c1 <= c3 && c1 <= c4) return launch_sattn_as<T, HD, 1, 4>(p, st);
+  if (c2 <= c3 && c2 <= c4) return launch_sattn_as<T, HD, 2, 2>(p, st);
+  if (c3 <= c4) return launch_sattn_as<T, HD, 3, 1>(p, st);
+  return launch_sattn_as<T, HD, 4, 1>(p, st);
 }
 }  // namespace
 
