@@ -25,7 +25,9 @@
 // traffic (ncu: tensor pipe 87 % active).  Both CTAs' TMA loads complete on the even CTA's barriers, stages and
 // accumulators are released to both by one commit each, and the finishing warps of both CTAs hand an accumulator
 // back by arriving on the even CTA's barrier.
-// No reduction split, epilogues Q, K/V, OUT, OUT_RES.
+// No reduction split, epilogues Q, K/V, OUT, OUT_RES, SWIGLU (a tile then holds the gate and the up projection of the same
+// 128 outputs, and a finishing chunk 32 columns of each: eight row tiles of 4096 x 2 x 12288 took 251 us in the
+// one-tile-per-CTA kernel, 6 waves of CTAs that each fill and drain on their own, and 175 us here).
 #include "layer.h"
 #include "tc.h"
 #include "tc_ptx.cuh"
@@ -63,7 +65,7 @@ __device__ __forceinline__ TileGeom tile_geom(const GemmParams& p, int tile, int
   t.nt = tile % n_tiles;
   t.mt = tile / n_tiles;
   t.is_b1 = t.nt >= p.n_split;
-  t.n0 = (t.is_b1 ? t.nt - p.n_split : t.nt) * BN;
+  t.n0 = p.b_pair ? t.nt * (BN / 2) : (t.is_b1 ? t.nt - p.n_split : t.nt) * BN;
   if (gather) {                      // rows t0 .. of the index list; position and cache row come from the tokens
     t.t0 = t.mt * BM;
     t.rows_valid = min(BM, n_rows - t.t0);
@@ -176,11 +178,17 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
             const uint32_t fb = map_to_cta(smem_u32(&full_bar[s]), 0);
             if (pr == 0) mbar_arrive_expect_tx(&full_bar[s], 2u * STAGE_BYTES);
             tma_load_2d_pair(dst, &tm_a, kb * BK, t.a_row, fb);
-            tma_load_2d_pair(dst + A_BYTES, tm_b, kb * BK, t.n0 + pr * (BN / 2), fb);
+            if (EPI == EPI_SWIGLU) tma_load_2d_pair(dst + A_BYTES, pr == 0 ? &tm_b0 : &tm_b1, kb * BK, t.n0, fb);
+            else tma_load_2d_pair(dst + A_BYTES, tm_b, kb * BK, t.n0 + pr * (BN / 2), fb);
           } else {
             mbar_arrive_expect_tx(&full_bar[s], (uint32_t)STAGE_BYTES);
             tma_load_2d(dst, &tm_a, kb * BK, t.a_row, &full_bar[s]);
-            tma_load_2d(dst + A_BYTES, tm_b, kb * BK, t.n0, &full_bar[s]);
+            if (EPI == EPI_SWIGLU) {
+              tma_load_2d(dst + A_BYTES, &tm_b0, kb * BK, t.n0, &full_bar[s]);
+              tma_load_2d(dst + A_BYTES + B_BYTES / 2, &tm_b1, kb * BK, t.n0, &full_bar[s]);
+            } else {
+              tma_load_2d(dst + A_BYTES, tm_b, kb * BK, t.n0, &full_bar[s]);
+            }
           }
         }
         __syncwarp();
@@ -254,8 +262,9 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
 #pragma unroll 1
       for (int chunk = 0; chunk < 4; ++chunk) {
         const int half = HDIM == 128 ? chunk & 1 : 0;
-        // tile columns [c_lo, c_lo + 32) and their rotary partners + HDIM / 2
-        const int c_lo = HDIM == 128 ? (chunk >> 1) * 128 + half * 32 : chunk * 64;
+        // tile columns [c_lo, c_lo + 32) and their partners + PART: of the rotary embedding, or gate and up
+        constexpr int PART = EPI == EPI_SWIGLU ? BN / 2 : HDIM / 2;
+        const int c_lo = EPI == EPI_SWIGLU ? chunk * 32 : (HDIM == 128 ? (chunk >> 1) * 128 + half * 32 : chunk * 64);
         {
           float v[32];
           tmem_ld_32x32(t_lane + c_lo, v);
@@ -263,7 +272,7 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
           for (int u = 0; u < 8; ++u)
             asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(stg_w + (uint32_t)((u ^ (lane & 7)) << 4)),
                          "f"(v[4 * u]), "f"(v[4 * u + 1]), "f"(v[4 * u + 2]), "f"(v[4 * u + 3]) : "memory");
-          tmem_ld_32x32(t_lane + c_lo + HDIM / 2, v);
+          tmem_ld_32x32(t_lane + c_lo + PART, v);
 #pragma unroll
           for (int u = 0; u < 8; ++u)
             asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(stg_w + 128u + (uint32_t)((u ^ (lane & 7)) << 4)),
@@ -374,6 +383,12 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
               vlo.x += fa.x; vlo.y += fa.y; vhi.x += fb.x; vhi.y += fb.y;
             }
             const size_t orow = p.out_is_cache == 1 ? crow : (p.out_is_cache == 2 ? (size_t)(t.t0 + r) : (size_t)tok);
+            if (EPI == EPI_SWIGLU) {
+              auto act = [](float gate, float up) { return gate / (1.f + __expf(-gate)) * up; };
+              *reinterpret_cast<__nv_bfloat162*>(out + orow * p.ld_out + t.n0 + c_lo + 2 * l16) =
+                  __floats2bfloat162_rn(act(vlo.x, vhi.x), act(vlo.y, vhi.y));
+              continue;
+            }
             const __nv_bfloat162 o_lo = __floats2bfloat162_rn(vlo.x, vlo.y), o_hi = __floats2bfloat162_rn(vhi.x, vhi.y);
             __nv_bfloat16* dst = out + orow * p.ld_out + t.n0 + c_lo + 2 * l16;
             *reinterpret_cast<__nv_bfloat162*>(dst) = o_lo;
@@ -428,13 +443,13 @@ static cudaError_t launch_persist(const CUtensorMap& a, const CUtensorMap& b0, c
   return launch_persist_hd<EPI, GATHER, PAIR, 128>(a, b0, b1, p, n_tiles, m_tiles, st);
 }
 
-// 256-wide tiles, no reduction split; b0 / b1 are maps with 256-row boxes (128-row boxes with pair != 0).  Listed
+// 256-wide tiles, no reduction split; b0 / b1 are maps with 256-row boxes (128-row boxes with pair != 0, and for SWIGLU).  Listed
 // launches (idx and count set, gather_src not; m_tiles = capacity of the row list in tiles): `a` maps a compact copy of
 // the listed rows (row r of the list = row r of the copy).
 cudaError_t launch_gemm_persist(int epi, const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1,
                                 const GemmParams& p, int n_tiles, int m_tiles, cudaStream_t st, int pair) {
   if (m_tiles <= 0 || n_tiles <= 0) return cudaSuccess;
-  if (p.b_pair || p.K % BK != 0) return cudaErrorInvalidValue;
+  if ((p.b_pair != 0) != (epi == EPI_SWIGLU) || p.K % BK != 0) return cudaErrorInvalidValue;
   const bool listed = p.idx != nullptr, gather = p.gather_src != nullptr;
   if (listed != (p.count != nullptr) || (gather && !listed)) return cudaErrorInvalidValue;
   if (epi == EPI_OUT && p.resid != nullptr) epi = EPI_OUT_RES;
@@ -454,12 +469,14 @@ cudaError_t launch_gemm_persist(int epi, const CUtensorMap& a, const CUtensorMap
     if (epi == EPI_KV) return launch_persist<EPI_KV, false, true>(a, b0, b1, p, n_tiles, m_tiles, st);
     if (epi == EPI_OUT) return launch_persist<EPI_OUT, false, true>(a, b0, b1, p, n_tiles, m_tiles, st);
     if (epi == EPI_OUT_RES) return launch_persist<EPI_OUT_RES, false, true>(a, b0, b1, p, n_tiles, m_tiles, st);
+    if (epi == EPI_SWIGLU) return launch_persist<EPI_SWIGLU, false, true>(a, b0, b1, p, n_tiles, m_tiles, st);
     return cudaErrorInvalidValue;
   }
   if (epi == EPI_Q) return launch_persist<EPI_Q, false>(a, b0, b1, p, n_tiles, m_tiles, st);
   if (epi == EPI_KV) return launch_persist<EPI_KV, false>(a, b0, b1, p, n_tiles, m_tiles, st);
   if (epi == EPI_OUT) return launch_persist<EPI_OUT, false>(a, b0, b1, p, n_tiles, m_tiles, st);
   if (epi == EPI_OUT_RES) return launch_persist<EPI_OUT_RES, false>(a, b0, b1, p, n_tiles, m_tiles, st);
+  if (epi == EPI_SWIGLU) return launch_persist<EPI_SWIGLU, false>(a, b0, b1, p, n_tiles, m_tiles, st);
   return cudaErrorInvalidValue;
 }
 

@@ -289,6 +289,10 @@ dare_status_t forward(dare_stack* S, const int* tokens, int batch, int seq_total
         q.nt0 = full; q.wait_at_end = 1;
         if (launch_gemm_tc(EPI_SWIGLU, 256, S->a_n2, S->maps[l].w_gate, S->maps[l].w_up, q, rest, m_tiles, 2, st, 1) != cudaSuccess)
           return DARE_ERR_CUDA;
+      } else if (m_tiles > 2 && persist_pays(n_tiles, m_tiles, sp)) {
+        if (launch_gemm_persist(EPI_SWIGLU, S->a_n2, S->maps[l].w_gate, S->maps[l].w_up, p, n_tiles, m_tiles, st,
+                                persist_pairs_pay(n_tiles, m_tiles) ? 1 : 0) != cudaSuccess)
+          return DARE_ERR_CUDA;
       } else if (launch_gemm_tc(EPI_SWIGLU, 256, S->a_n2, S->maps[l].w_gate, S->maps[l].w_up, p, n_tiles, m_tiles, sp, st,
                                 pairs ? 1 : 0) != cudaSuccess) {
         return DARE_ERR_CUDA;
@@ -304,6 +308,10 @@ dare_status_t forward(dare_stack* S, const int* tokens, int batch, int seq_total
       if (narrow_pairs_pay(d, m_tiles, f / 64)) {
         if (launch_gemm_tc(EPI_OUT, 128, S->a_act, S->maps[l].w_down64, S->maps[l].w_down64, p, d / 128, m_tiles, 2, st,
                            1) != cudaSuccess) return DARE_ERR_CUDA;
+      } else if (persist_pays(n_tiles, m_tiles, sp)) {
+        const int pp = persist_pairs_pay(n_tiles, m_tiles) ? 1 : 0;
+        const CUtensorMap& wd = pp ? S->maps[l].w_down128 : S->maps[l].w_down;
+        if (launch_gemm_persist(EPI_OUT, S->a_act, wd, wd, p, n_tiles, m_tiles, st, pp) != cudaSuccess) return DARE_ERR_CUDA;
       } else {
         const CUtensorMap& wd = pair ? S->maps[l].w_down128 : S->maps[l].w_down;
         if (launch_gemm_tc(EPI_OUT, 256, S->a_act, wd, wd, p, n_tiles, m_tiles, sp, st, pair ? 1 : 0) != cudaSuccess)

@@ -20,7 +20,6 @@ namespace {
 bool use_pairs(int n_tiles, int m_tiles, int splits) { return pairs_pay(n_tiles, m_tiles, splits); }
 // units (column tile x pair of row tiles) from which the two-CTA form of a listed launch runs: two rounds of the 74 clusters
 constexpr int kPairUnitGate = 148;
-bool use_persist(int n_tiles, int m_tiles, int splits) { return persist_pays(n_tiles, m_tiles, splits); }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
@@ -142,8 +141,11 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
     const int sp = pick_splits(n_tiles * m_tiles_dense, kblocks);
     if (narrow_pairs_pay(d, m_tiles_dense, kblocks))
       e = launch_gemm_tc(EPI_Q, 128, S.a_xn, S.w_q64, S.w_q64, p, d / 128, m_tiles_dense, 2, st, 1);
-    else if (use_persist(n_tiles, m_tiles_dense, sp))
-      e = launch_gemm_persist(EPI_Q, S.a_xn, S.w_q128, S.w_q128, p, n_tiles, m_tiles_dense, st, 1);
+    else if (persist_pays(n_tiles, m_tiles_dense, sp)) {
+      const int pair = persist_pairs_pay(n_tiles, m_tiles_dense) ? 1 : 0;
+      const CUtensorMap& wq = pair ? S.w_q128 : S.w_q;
+      e = launch_gemm_persist(EPI_Q, S.a_xn, wq, wq, p, n_tiles, m_tiles_dense, st, pair);
+    }
     else if (use_pairs(n_tiles, m_tiles_dense, sp))
       e = launch_gemm_tc(EPI_Q, 256, S.a_xn, S.w_q128, S.w_q128, p, n_tiles, m_tiles_dense, sp, st, 1);
     else
@@ -156,7 +158,9 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
   // kernels decide) it is issued right behind the Q projection and runs beside it: the two launches are one fused
   // Q/K/V projection of the step's rows, spread over two grids because the Q tiles take a split reduction and the
   // K/V tiles do not.  The selection then follows both.
-  const bool kv_beside_q = !kv_sparse && m_tiles_dense <= 8;
+  // (not where the K/V tiles are more than one wave and take the persistent kernel)
+  const bool kv_beside_q = !kv_sparse && m_tiles_dense <= 8 &&
+                           !persist_pays(2 * d / 256, m_tiles_dense, pick_splits(2 * d / 256 * m_tiles_dense, kblocks));
   // lines 4-5 + Sec. 4
   const bool select_all = !has_prev || mode == DARE_MODE_DENSE;
   auto select_now = [&]() {
@@ -187,11 +191,11 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
                            pick_splits(n_tiles128, kblocks), st); ++launches;
       } else {
         // Many tokens: even a small refreshed fraction fills the GPU with 256-wide tiles, which re-read the least.
-        if (use_persist(n_tiles, m_tiles, 1) && compact_ok) {
+        if (persist_pays_listed(n_tiles, m_tiles) && compact_ok) {
           // a compact copy of the refresh set's rows first (a stream of n x d elements), then the projection with
           // every operand through TMA and two-CTA MMAs; beyond gate_kv refreshed tokens the dense form instead: every
           // row of the step projected, the rows of the refresh set stored (the others keep their cached K and V)
-          const bool dense_form = use_persist(n_tiles, m_tiles_dense, 1);
+          const bool dense_form = persist_pays_listed(n_tiles, m_tiles_dense);
           const int hi = dense_form ? gate_kv : 1 << 30;
           launch_gather_step_rows((const bf16*)B.xn, B.idx, B.count, (bf16*)B.x_stage, g, false, st, B.status, hi); ++launches;
           p.gather_src = nullptr;
@@ -214,8 +218,11 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
       prof_mark(L, SLOT_KV_GEMM, st);
       p.wait_at_end = kv_beside_q ? 1 : 0;
       const int sp = pick_splits(n_tiles * m_tiles_dense, kblocks);
-      if (use_persist(n_tiles, m_tiles_dense, sp))
-        e = launch_gemm_persist(EPI_KV, S.a_xn, S.w_k128, S.w_v128, p, n_tiles, m_tiles_dense, st, 1);
+      if (persist_pays(n_tiles, m_tiles_dense, sp)) {
+        const int pair = persist_pairs_pay(n_tiles, m_tiles_dense) ? 1 : 0;
+        e = launch_gemm_persist(EPI_KV, S.a_xn, pair ? S.w_k128 : S.w_k, pair ? S.w_v128 : S.w_v, p, n_tiles, m_tiles_dense,
+                                st, pair);
+      }
       else if (use_pairs(n_tiles, m_tiles_dense, sp))
         e = launch_gemm_tc(EPI_KV, 256, S.a_xn, S.w_k128, S.w_v128, p, n_tiles, m_tiles_dense, sp, st, 1);
       else
@@ -238,7 +245,7 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
     p.gate_count = nullptr; p.gate_lo = 0; p.gate_hi = 1 << 30; p.store_mask = nullptr;
     // a long row-sparse step is issued in both forms: over the refresh set's rows, and dense with only the refreshed
     // rows stored (tiles without one skipped); the size of the set decides on the device which of them runs
-    const bool both_forms = o_sparse && m_tiles_dense > 8 && use_persist(d / 256, m_tiles_dense, 1);
+    const bool both_forms = o_sparse && m_tiles_dense > 8 && persist_pays_listed(d / 256, m_tiles_dense);
     // (one launch carries both when both take the kernel with two query tiles per CTA: its CTAs pick the form; a
     // launch that only looks at the count and leaves still costs a wave of CTAs per 148 of them)
     const bool one_launch = both_forms && attention_tc_two_tiles(g, true) && attention_tc_two_tiles(g, false);
@@ -276,9 +283,9 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
     if (y_sparse) {
       p.idx = B.idx; p.count = B.count; p.gather_src = (const bf16*)B.oc; p.gather_cache_rows = 1;
       bool dense_form = false;
-      if (use_persist(n_tiles, (T_ + 127) / 128, 1) && compact_ok) {
+      if (persist_pays_listed(n_tiles, (T_ + 127) / 128) && compact_ok) {
         // (beyond gate_o refreshed tokens the dense projection of every row instead: Alg. 2 line 11 as written)
-        dense_form = use_persist(n_tiles, m_tiles_dense, 1);
+        dense_form = persist_pays_listed(n_tiles, m_tiles_dense);
         const int hi = dense_form ? gate_o : 1 << 30;
         launch_gather_step_rows((const bf16*)B.oc, B.idx, B.count, (bf16*)B.x_stage, g, true, st, B.status, hi); ++launches;
         p.gather_src = nullptr;
@@ -302,8 +309,11 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
       const int sp = pick_splits(n_tiles * m_tiles_dense, kblocks);
       if (narrow_pairs_pay(d, m_tiles_dense, kblocks))
         e = launch_gemm_tc(EPI_OUT, 128, S.a_oc, S.w_o64, S.w_o64, p, d / 128, m_tiles_dense, 2, st, 1);
-      else if (use_persist(n_tiles, m_tiles_dense, sp))
-        e = launch_gemm_persist(EPI_OUT, S.a_oc, S.w_o128, S.w_o128, p, n_tiles, m_tiles_dense, st, 1);
+      else if (persist_pays(n_tiles, m_tiles_dense, sp)) {
+        const int pair = persist_pairs_pay(n_tiles, m_tiles_dense) ? 1 : 0;
+        const CUtensorMap& wo = pair ? S.w_o128 : S.w_o;
+        e = launch_gemm_persist(EPI_OUT, S.a_oc, wo, wo, p, n_tiles, m_tiles_dense, st, pair);
+      }
       else if (use_pairs(n_tiles, m_tiles_dense, sp))
         e = launch_gemm_tc(EPI_OUT, 256, S.a_oc, S.w_o128, S.w_o128, p, n_tiles, m_tiles_dense, sp, st, 1);
       else

@@ -118,7 +118,16 @@ cudaError_t launch_gemm_tc(int epi, int bn, const CUtensorMap& a, const CUtensor
 // pair != 0 (dense launches only): two-CTA MMAs over pairs of row tiles, b0 / b1 with 128-row boxes.
 cudaError_t launch_gemm_persist(int epi, const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1,
                                 const GemmParams& p, int n_tiles, int m_tiles, cudaStream_t st, int pair = 0);
-// ... pays from about two waves of tiles on.
-inline bool persist_pays(int n_tiles, int m_tiles, int splits) { return splits == 1 && n_tiles * m_tiles >= 296; }
+// ... pays as soon as the tiles are more than one wave: from there on a tile's set-up, pipeline fill and finishing pass
+// hide behind the next tile's main loop.
+inline bool persist_pays(int n_tiles, int m_tiles, int splits) { return splits == 1 && n_tiles * m_tiles > 148; }
+// A listed launch comes with a compact copy of its rows and a second form that only looks at the count: from two waves.
+inline bool persist_pays_listed(int n_tiles, int m_tiles) { return n_tiles * m_tiles >= 296; }
+// Two-CTA MMAs in it, or single CTAs?  A k-block takes a pair 0.93 of the time it takes a single CTA (644 against 667-690
+// cycles), but pairs walk in waves of 74 units of two row tiles, an odd row tile being padded to a pair.
+inline bool persist_pairs_pay(int n_tiles, int m_tiles) {
+  const int units = n_tiles * ((m_tiles + 1) / 2), tiles = n_tiles * m_tiles;
+  return 0.93f * (float)((units + 73) / 74) <= (float)((tiles + 147) / 148);
+}
 
 }  // namespace dare
