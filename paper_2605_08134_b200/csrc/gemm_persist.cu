@@ -5,11 +5,13 @@
 //              across tile boundaries
 //   warp 1     one elected lane issues tcgen05.mma (M = 128, N = 256, K = 16) into one of TWO 128 x 256 fp32
 //              accumulators in tensor memory (all 512 columns), alternating per tile
-//   warps 2-5  finishing pass, one warp per TMEM lane quarter (32 rows), independent of one another: a quarter of
-//              a head at a time (32 + 32 columns whose rotary partners they are) goes tensor memory -> registers
-//              (thread <-> row) -> the warp's own 8 KB of shared memory -> registers (half-warp <-> row, lane <->
-//              two column pairs), where the fused tail runs (score, stored query, rotary embedding, residual) and
-//              the row segments are stored; the accumulator is handed back after the last read of tensor memory
+//   warps 2-9  finishing pass, two warps per TMEM lane quarter (32 rows), half of the tile's columns each (one head of
+//              128), independent of one another: 16 columns and their 16 rotary partners at a time go tensor memory ->
+//              registers (thread <-> row) -> the warp's own 4 KB of shared memory -> registers (quarter-warp <-> row,
+//              lane <-> two column pairs), where the fused tail runs (score, stored query, rotary embedding, residual)
+//              and the row segments are stored; the accumulator is handed back after the last read of tensor memory.
+//              The pass is a chain of table reads and shared-memory round trips: with four warps it took about 13 us a
+//              tile with the rotary embedding, longer than the main loop over a reduction of 2048
 // In the one-tile-per-CTA kernel of gemm_tc.cu a tile costs set-up + pipeline fill + finishing pass + the gap to the
 // next CTA on top of its main loop (about 30 % at these sizes, measured); here the main loops follow one another.
 // Listed launches (the rows of a refresh set, Alg. 1 line 6 / the gathered output projection, given by an index list
@@ -45,14 +47,15 @@ struct Ring {
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr int STAGES = PAIR ? 6 : 4;
 };
-constexpr int STG_OFFSET = Ring<false>::STAGES * Ring<false>::STAGE_BYTES;   // finishing warps' staging: 4 x (32 rows x 64 fp32)
+constexpr int STG_OFFSET = Ring<false>::STAGES * Ring<false>::STAGE_BYTES;   // finishing warps' staging: 8 x (32 rows x 32 fp32)
 static_assert(Ring<true>::STAGES * Ring<true>::STAGE_BYTES == STG_OFFSET, "both rings end where the staging begins");
-constexpr int STG_ROW_BYTES = 64 * 4, STG_WARP_BYTES = 32 * STG_ROW_BYTES;
-constexpr int ACC_OFFSET = STG_OFFSET + 4 * STG_WARP_BYTES;   // partial score sums: [128 rows][3] fp32
+constexpr int STG_ROW_BYTES = 32 * 4, STG_WARP_BYTES = 32 * STG_ROW_BYTES;
+constexpr int kFinish = 8;                           // finishing warps
+constexpr int ACC_OFFSET = STG_OFFSET + kFinish * STG_WARP_BYTES;   // partial score sums: [128 rows][3] fp32
 constexpr int BAR_OFFSET = ACC_OFFSET + BM * 12;
 static_assert(BAR_OFFSET + 256 + 1024 <= 227 * 1024, "shared memory of one CTA");
 constexpr int SMEM_TOTAL = BAR_OFFSET + 256 + 1024;  // barriers + slack for 1024-byte alignment
-constexpr int kWarps = 6;
+constexpr int kWarps = 2 + kFinish;
 
 struct TileGeom {
   int nt, mt, n0, is_b1;
@@ -109,7 +112,7 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
-    for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], PAIR ? 8 : 4); }
+    for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], PAIR ? 2 * kFinish : kFinish); }
     fence_mbar_init();
     prefetch_tmap(&tm_a);
     prefetch_tmap(&tm_b0);
@@ -233,12 +236,15 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
   } else if (warp == 1) {
     // (the odd CTA of a pair issues nothing)
   } else {
-    // ---- finishing warps: quarter q of the TMEM lanes = rows 32q .. 32q + 31 of every tile
-    const int q = warp & 3;
-    uint8_t* stg = smem + STG_OFFSET + q * STG_WARP_BYTES;
-    float* sc_acc = reinterpret_cast<float*>(smem + ACC_OFFSET) + q * 32 * 3;
+    // ---- finishing warps: quarter q of the TMEM lanes = rows 32q .. 32q + 31 of every tile, half `sub` of its columns
+    const int q = warp & 3, sub = (warp - 2) >> 2;
+    uint8_t* stg = smem + STG_OFFSET + (warp - 2) * STG_WARP_BYTES;
+    float* sc_acc = reinterpret_cast<float*>(smem + ACC_OFFSET) + q * 32 * 3;   // (the one warp with the scoring head)
+    // 16-byte units of a staging row: 0-3 the columns, 4-7 their partners; swizzled so that neither eight rows written at
+    // one unit nor two rows read at four units meet in a bank
+    auto unit_at = [](int row, int u) { return (uint32_t)((u ^ (((row & 1) << 2) | ((row >> 1) & 3))) << 4); };
     const uint32_t stg_w = smem_u32(stg) + (uint32_t)lane * STG_ROW_BYTES;    // this thread's row when it writes
-    const int half_id = lane >> 4, l16 = lane & 15;
+    const int row_id = lane >> 3, l8 = lane & 7;
     uint32_t tcount = 0;
     for (int tile = walker; tile < total_tiles; tile += n_walkers, ++tcount) {
       const TileGeom t = tile_of(tile);
@@ -261,21 +267,20 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
       __nv_bfloat16* out = t.is_b1 ? p.out1 : p.out0;
 #pragma unroll 1
       for (int chunk = 0; chunk < 4; ++chunk) {
-        const int half = HDIM == 128 ? chunk & 1 : 0;
-        // tile columns [c_lo, c_lo + 32) and their partners + PART: of the rotary embedding, or gate and up
+        // tile columns [c_lo, c_lo + 16) and their partners + PART: of the rotary embedding (h_col: the columns' place in
+        // the first half of their head), or gate and up
         constexpr int PART = EPI == EPI_SWIGLU ? BN / 2 : HDIM / 2;
-        const int c_lo = EPI == EPI_SWIGLU ? chunk * 32 : (HDIM == 128 ? (chunk >> 1) * 128 + half * 32 : chunk * 64);
+        const int h_col = EPI == EPI_SWIGLU ? 0 : (HDIM == 128 ? chunk * 16 : (chunk & 1) * 16);
+        const int head_col = EPI == EPI_SWIGLU ? 0 : (HDIM == 128 ? sub * 128 : sub * 128 + (chunk >> 1) * 64);
+        const int c_lo = EPI == EPI_SWIGLU ? sub * 64 + chunk * 16 : head_col + h_col;
         {
           float v[32];
-          tmem_ld_32x32(t_lane + c_lo, v);
+          tmem_ld_32x16_nowait(t_lane + c_lo, v);
+          tmem_ld_32x16_nowait(t_lane + c_lo + PART, v + 16);
+          tmem_ld_wait();
 #pragma unroll
           for (int u = 0; u < 8; ++u)
-            asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(stg_w + (uint32_t)((u ^ (lane & 7)) << 4)),
-                         "f"(v[4 * u]), "f"(v[4 * u + 1]), "f"(v[4 * u + 2]), "f"(v[4 * u + 3]) : "memory");
-          tmem_ld_32x32(t_lane + c_lo + PART, v);
-#pragma unroll
-          for (int u = 0; u < 8; ++u)
-            asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(stg_w + 128u + (uint32_t)((u ^ (lane & 7)) << 4)),
+            asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(stg_w + unit_at(lane, u)),
                          "f"(v[4 * u]), "f"(v[4 * u + 1]), "f"(v[4 * u + 2]), "f"(v[4 * u + 3]) : "memory");
         }
         if (chunk == 3) {                                // the accumulator is free for the tile after next
@@ -287,10 +292,11 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
           }
         }
         __syncwarp();
-        const bool score_chunk = score_col >= 0 && c_lo - half * 32 == score_col;
-        // 16 passes of two rows (one per half-warp), four passes at a time so that their table reads overlap
+        const bool score_chunk = score_col >= 0 && head_col == score_col;
+        const bool score_first = h_col == 0, score_last = h_col == HDIM / 2 - 16;
+        // 8 passes of four rows (one per quarter-warp), four passes at a time so that their table reads overlap
 #pragma unroll 1
-        for (int i0 = 0; i0 < 16; i0 += 4) {
+        for (int i0 = 0; i0 < 8; i0 += 4) {
           float2 lo[4], hi[4];
           float4 cs[4];
           float2 qa[4], qb[4];
@@ -300,7 +306,7 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
           size_t crow_k[4];
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
-            const int rr = 2 * (i0 + k) + half_id, r = q * 32 + rr;
+            const int rr = 4 * (i0 + k) + row_id, r = q * 32 + rr;
             ok[k] = r < t.rows_valid;
             const int rc = ok[k] ? r : 0;                // rows past the end read row 0's tables and are dropped
             int pos = t.pos0 + rc, tokr = t.t0 + rc;
@@ -314,33 +320,31 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
             }
             tok_k[k] = tokr; crow_k[k] = crowr;
             if (!GATHER && EPI == EPI_KV && p.store_mask != nullptr && ok[k] && p.store_mask[crowr] != 0) ok[k] = false;
-            const uint8_t* row = stg + rr * STG_ROW_BYTES;
-            const uint32_t off = (uint32_t)((((l16 >> 1) ^ (rr & 7)) << 4) | ((l16 & 1) << 3));
-            lo[k] = *reinterpret_cast<const float2*>(row + off);
-            hi[k] = *reinterpret_cast<const float2*>(row + 128 + off);
+            const uint8_t* row = stg + rr * STG_ROW_BYTES + (l8 & 1) * 8;
+            lo[k] = *reinterpret_cast<const float2*>(row + unit_at(rr, l8 >> 1));
+            hi[k] = *reinterpret_cast<const float2*>(row + unit_at(rr, 4 + (l8 >> 1)));
             if (rotate)
-              cs[k] = *reinterpret_cast<const float4*>(p.rope + (size_t)pos * (HDIM / 2) + half * 32 + 2 * l16);
+              cs[k] = *reinterpret_cast<const float4*>(p.rope + (size_t)pos * (HDIM / 2) + h_col + 2 * l8);
             if (EPI == EPI_Q && score_chunk && p.has_prev) {
-              const float* qp = p.q_prev + crowr * HDIM + half * 32 + 2 * l16;
+              const float* qp = p.q_prev + crowr * HDIM + h_col + 2 * l8;
               qa[k] = *reinterpret_cast<const float2*>(qp);
               qb[k] = *reinterpret_cast<const float2*>(qp + HDIM / 2);
             }
             if (EPI == EPI_OUT_RES) {
-              const __nv_bfloat16* rs = p.resid + (size_t)tokr * p.ld_resid + t.n0 + c_lo + 2 * l16;
+              const __nv_bfloat16* rs = p.resid + (size_t)tokr * p.ld_resid + t.n0 + c_lo + 2 * l8;
               ra[k] = *reinterpret_cast<const __nv_bfloat162*>(rs);
               rb[k] = *reinterpret_cast<const __nv_bfloat162*>(rs + HDIM / 2);
             }
           }
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
-            const int rr = 2 * (i0 + k) + half_id, r = q * 32 + rr;
+            const int rr = 4 * (i0 + k) + row_id, r = q * 32 + rr;
             const int tok = tok_k[k];
             const size_t crow = crow_k[k];
             float2 vlo = lo[k], vhi = hi[k];
             if (EPI == EPI_Q && score_chunk) {
-              // Sec. 3.1 on the un-rotated query of the scoring head: 1 - cos(current, stored); this quarter of the
-              // head adds its part of the three sums, the second half of the head finishes the row (a head of
-              // 64 is one chunk: no sums to hand on)
+              // Sec. 3.1 on the un-rotated query of the scoring head: 1 - cos(current, stored); each chunk of the head
+              // adds its part of the three sums, the last one finishes the row
               float dot = 0.f, n2 = 0.f;
               if (p.has_prev) {
                 dot = vlo.x * qa[k].x + vlo.y * qa[k].y + vhi.x * qb[k].x + vhi.y * qb[k].y;
@@ -348,21 +352,21 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
               }
               float n1 = vlo.x * vlo.x + vlo.y * vlo.y + vhi.x * vhi.x + vhi.y * vhi.y;
 #pragma unroll
-              for (int o = 8; o > 0; o >>= 1) {          // over the 16 lanes of the row
+              for (int o = 4; o > 0; o >>= 1) {          // over the 8 lanes of the row
                 dot += __shfl_xor_sync(0xffffffffu, dot, o);
                 n1 += __shfl_xor_sync(0xffffffffu, n1, o);
                 n2 += __shfl_xor_sync(0xffffffffu, n2, o);
               }
               if (ok[k]) {
-                float* qp = p.q_prev + crow * HDIM + half * 32 + 2 * l16;
+                float* qp = p.q_prev + crow * HDIM + h_col + 2 * l8;
                 *reinterpret_cast<float2*>(qp) = vlo;
                 *reinterpret_cast<float2*>(qp + HDIM / 2) = vhi;
               }
-              if (l16 == 0) {
-                if (HDIM == 128 && half == 0) {
+              if (l8 == 0) {
+                if (!score_first) { dot += sc_acc[3 * rr]; n1 += sc_acc[3 * rr + 1]; n2 += sc_acc[3 * rr + 2]; }
+                if (!score_last) {
                   sc_acc[3 * rr] = dot; sc_acc[3 * rr + 1] = n1; sc_acc[3 * rr + 2] = n2;
                 } else if (ok[k]) {
-                  if (HDIM == 128) { dot += sc_acc[3 * rr]; n1 += sc_acc[3 * rr + 1]; n2 += sc_acc[3 * rr + 2]; }
                   float sc = __int_as_float(0x7f800000);   // +inf: nothing to compare with
                   if (p.has_prev) {
                     const float den = sqrtf(n1) * sqrtf(n2);
@@ -385,16 +389,16 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
             const size_t orow = p.out_is_cache == 1 ? crow : (p.out_is_cache == 2 ? (size_t)(t.t0 + r) : (size_t)tok);
             if (EPI == EPI_SWIGLU) {
               auto act = [](float gate, float up) { return gate / (1.f + __expf(-gate)) * up; };
-              *reinterpret_cast<__nv_bfloat162*>(out + orow * p.ld_out + t.n0 + c_lo + 2 * l16) =
+              *reinterpret_cast<__nv_bfloat162*>(out + orow * p.ld_out + t.n0 + c_lo + 2 * l8) =
                   __floats2bfloat162_rn(act(vlo.x, vhi.x), act(vlo.y, vhi.y));
               continue;
             }
             const __nv_bfloat162 o_lo = __floats2bfloat162_rn(vlo.x, vlo.y), o_hi = __floats2bfloat162_rn(vhi.x, vhi.y);
-            __nv_bfloat16* dst = out + orow * p.ld_out + t.n0 + c_lo + 2 * l16;
+            __nv_bfloat16* dst = out + orow * p.ld_out + t.n0 + c_lo + 2 * l8;
             *reinterpret_cast<__nv_bfloat162*>(dst) = o_lo;
             *reinterpret_cast<__nv_bfloat162*>(dst + HDIM / 2) = o_hi;
             if ((EPI == EPI_OUT || EPI == EPI_OUT_RES) && p.out1 != nullptr) {   // the projected-output cache
-              __nv_bfloat16* dst2 = p.out1 + crow * p.ld_out + t.n0 + c_lo + 2 * l16;
+              __nv_bfloat16* dst2 = p.out1 + crow * p.ld_out + t.n0 + c_lo + 2 * l8;
               *reinterpret_cast<__nv_bfloat162*>(dst2) = o_lo;
               *reinterpret_cast<__nv_bfloat162*>(dst2 + HDIM / 2) = o_hi;
             }
