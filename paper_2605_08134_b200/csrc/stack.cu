@@ -26,7 +26,10 @@ constexpr int kMaxCand = 128;       // candidates per decoding step: batch * blo
 
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 
-struct BlockMaps { CUtensorMap w_gate, w_up, w_down, w_down128, w_down64; };   // w_down: 256-row boxes, w_down64: 64, the others 128
+struct BlockMaps {
+  CUtensorMap w_gate, w_up, w_down, w_down128, w_down64;   // w_down: 256-row boxes, w_down64: 64, the others 128
+  CUtensorMap w_gate1, w_up1, w_gate2, w_up2;              // SwiGLU of at most 128 / 256 rows: boxes of a CTA's part of the tile
+};
 
 // x[t, :] = emb[tokens[b, pos_begin + i], :]   (t = b*seq_act + i)
 __global__ void __launch_bounds__(256) embed_kernel(const int* __restrict__ tokens, int seq_total, int seq_act,
@@ -222,7 +225,7 @@ struct dare_stack {
   const void* emb;
   const float* final_gain;
   StackBuffers buf;
-  int sm_count;               // SMs of the device the stack was created on
+  int width1, width2;         // SwiGLU of at most 128 / 256 rows: outputs of a tile (the device's SMs decide)
   int capture_layer;          // test hook: copy this layer's input and output of every pass (-1 = off)
   void* capture_x;
   void* capture_h;
@@ -242,8 +245,9 @@ GemmParams base_params(const dare_stack* S, int batch, int seq_act, int pos_begi
   const dare_layer_config_t& lc = S->cfg.layer;
   p.g.batch = batch; p.g.seq_act = seq_act; p.g.pos_begin = pos_begin; p.g.max_seq = lc.max_seq; p.g.kv_len = lc.max_seq;
   p.g.d = lc.d_model; p.g.n_heads = lc.n_heads; p.g.head_dim = lc.head_dim; p.g.score_head = 0;
-  p.K = lc.d_model; p.m_total = batch * seq_act; p.seq_act = seq_act; p.tiles_per_seq = (seq_act + 127) / 128;
-  p.a_seq_stride = seq_act; p.a_row0 = 0; p.n_split = 1 << 30; p.ld_out = lc.d_model;
+  // (every operand of the MLP is compact over the window: row tiles run on across sequences)
+  p.K = lc.d_model; p.m_total = batch * seq_act; p.seq_act = p.m_total; p.tiles_per_seq = (p.m_total + 127) / 128;
+  p.a_seq_stride = p.m_total; p.a_row0 = 0; p.n_split = 1 << 30; p.ld_out = lc.d_model;
   p.status = S->layers[0]->buf.status;
   return p;
 }
@@ -257,7 +261,8 @@ dare_status_t forward(dare_stack* S, const int* tokens, int batch, int seq_total
   const StackBuffers& B = S->buf;
   embed_kernel<<<T_, 256, 0, st>>>(tokens, seq_total, seq_act, pos_begin, (const uint4*)S->emb, (uint4*)B.xa, d / 8,
                                    S->cfg.vocab);
-  const int m_tiles = batch * ((seq_act + 127) / 128);
+  const int m_tiles = (T_ + 127) / 128;
+  const int width = T_ <= 128 ? S->width1 : S->width2;
   for (int l = 0; l < S->cfg.n_layers; ++l) {
     // h = x + DARE attention
     if (l == S->capture_layer && S->capture_x)
@@ -274,29 +279,20 @@ dare_status_t forward(dare_stack* S, const int* tokens, int batch, int seq_total
       p.b_pair = 1; p.out0 = B.act; p.ld_out = f;
       const int n_tiles = f / 128;
       const int sp = pick_splits(n_tiles * m_tiles, d / 64);
-      const bool pairs = pairs_pay(n_tiles, m_tiles, sp);
-      // Pair tiles over the whole reduction fill the SM pairs in waves; a last wave that is less than half full (96
-      // tiles on 74 pairs) is issued as a launch of its own with the reduction split in two, which puts twice as many
-      // SM pairs on it for half as long.  It needs nothing from the launch before it and runs behind it as SMs come
-      // free (it waits for its predecessors only before it leaves).
-      const int wave = S->sm_count / 2;
-      const int rest = pairs && sp == 1 && m_tiles == 2 && wave > 0 ? n_tiles % wave : 0;
-      if (rest > 0 && n_tiles > wave && 2 * rest <= wave) {
-        const int full = n_tiles - rest;
-        if (launch_gemm_tc(EPI_SWIGLU, 256, S->a_n2, S->maps[l].w_gate, S->maps[l].w_up, p, full, m_tiles, 1, st, 1) != cudaSuccess)
-          return DARE_ERR_CUDA;
-        GemmParams q = p;
-        q.nt0 = full; q.wait_at_end = 1;
-        if (launch_gemm_tc(EPI_SWIGLU, 256, S->a_n2, S->maps[l].w_gate, S->maps[l].w_up, q, rest, m_tiles, 2, st, 1) != cudaSuccess)
-          return DARE_ERR_CUDA;
-      } else if (m_tiles > 2 && persist_pays(n_tiles, m_tiles, sp)) {
-        if (launch_gemm_persist(EPI_SWIGLU, S->a_n2, S->maps[l].w_gate, S->maps[l].w_up, p, n_tiles, m_tiles, st,
-                                persist_pairs_pay(n_tiles, m_tiles) ? 1 : 0) != cudaSuccess)
-          return DARE_ERR_CUDA;
-      } else if (launch_gemm_tc(EPI_SWIGLU, 256, S->a_n2, S->maps[l].w_gate, S->maps[l].w_up, p, n_tiles, m_tiles, sp, st,
-                                pairs ? 1 : 0) != cudaSuccess) {
-        return DARE_ERR_CUDA;
+      cudaError_t e;
+      if (m_tiles <= 2) {
+        // few rows: a stream of both matrices, one wave of tiles as wide as the device needs
+        const BlockMaps& m = S->maps[l];
+        e = launch_swiglu(S->a_n2, m_tiles == 2 ? m.w_gate2 : m.w_gate1, m_tiles == 2 ? m.w_up2 : m.w_up1, width, T_, f, d, B.act,
+                          p.status, st);
+      } else if (persist_pays(n_tiles, m_tiles, sp)) {
+        e = launch_gemm_persist(EPI_SWIGLU, S->a_n2, S->maps[l].w_gate, S->maps[l].w_up, p, n_tiles, m_tiles, st,
+                                persist_pairs_pay(n_tiles, m_tiles) ? 1 : 0);
+      } else {
+        e = launch_gemm_tc(EPI_SWIGLU, 256, S->a_n2, S->maps[l].w_gate, S->maps[l].w_up, p, n_tiles, m_tiles, sp, st,
+                           pairs_pay(n_tiles, m_tiles, sp) ? 1 : 0);
       }
+      if (e != cudaSuccess) return DARE_ERR_CUDA;
     }
     // x_next = h + W_D act
     {
@@ -356,10 +352,10 @@ dare_status_t dare_stack_create(const dare_stack_config_t* cfg, const dare_stack
   S->cfg = *cfg;
   {
     int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
-      S->sm_count = sms;
-    else
-      S->sm_count = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      sms = 148;
+    S->width1 = swiglu_width(cfg->d_ff, sms, false);
+    S->width2 = swiglu_width(cfg->d_ff, sms, true);
   }
   S->cfg.layer.kernel_path = DARE_PATH_TENSOR;
   S->emb = w->emb;
@@ -382,7 +378,9 @@ dare_status_t dare_stack_create(const dare_stack_config_t* cfg, const dare_stack
     BlockMaps m;
     if (!make_map(&m.w_gate, bw.w_gate, f, d, 128) || !make_map(&m.w_up, bw.w_up, f, d, 128) ||
         !make_map(&m.w_down, bw.w_down, d, f, 256) || !make_map(&m.w_down128, bw.w_down, d, f, 128) ||
-        !make_map(&m.w_down64, bw.w_down, d, f, 64))
+        !make_map(&m.w_down64, bw.w_down, d, f, 64) || !make_map(&m.w_gate1, bw.w_gate, f, d, S->width1) ||
+        !make_map(&m.w_up1, bw.w_up, f, d, S->width1) || !make_map(&m.w_gate2, bw.w_gate, f, d, S->width2 / 2) ||
+        !make_map(&m.w_up2, bw.w_up, f, d, S->width2 / 2))
       st = DARE_ERR_CUDA;
     S->maps.push_back(m);
   }

@@ -54,7 +54,6 @@ struct GemmParams {
   const int* gate_count;
   int gate_lo, gate_hi;
   const int* store_mask;
-  int nt0;               // first column tile of this launch (a projection issued as two launches over its column tiles)
   int loop_rows;         // gathered launch with ONE row of CTAs in the grid: each takes the refresh set's row tiles in turn
   int wait_at_end;       // 1: the launch reads nothing its predecessor in the stream writes and writes nothing that one
                          // reads, so it runs beside it: its CTAs start as soon as the predecessor's have passed their own
@@ -112,6 +111,12 @@ inline bool narrow_pairs_pay(int d_out, int m_tiles, int kblocks) {
 cudaError_t launch_gemm_tc(int epi, int bn, const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1,
                            const GemmParams& p, int n_tiles, int m_tiles, int splits, cudaStream_t st, int pair = 0);
 
+
+// SwiGLU of at most 256 rows (gemm_swiglu.cu): x maps the rows with 128-row boxes, gate / up the matrices with boxes of
+// `width` rows (rows <= 128) or width / 2 (two-CTA form, beyond); width = swiglu_width(..., rows > 128).
+int swiglu_width(int d_ff, int sms, bool pair);
+cudaError_t launch_swiglu(const CUtensorMap& x, const CUtensorMap& gate, const CUtensorMap& up, int width, int rows, int d_ff,
+                          int K, __nv_bfloat16* act, int* status, cudaStream_t st);
 
 // Persistent form for launches of many row tiles (dense rows, 256-wide tiles, no reduction split, epilogues Q, K/V,
 // OUT): one CTA per SM walks the tiles, finishing pass overlapped with the next tile's main loop.
