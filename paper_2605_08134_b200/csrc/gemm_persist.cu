@@ -165,7 +165,8 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
     return t;
   };
   if (warp == 0) {
-    // ---- producer
+    // ---- producer (p.a_piece: A in boxes of 32 rows, each in one sequence of the cache; rows past the end are dropped later)
+    auto piece_row = [&](int tok) { const int T = p.g.tokens(); return p.g.cache_row(tok < T ? tok : T - 32); };
     uint32_t it = 0;
     for (int tile = walker; tile < total_tiles; tile += n_walkers) {
       const TileGeom t = tile_of(tile);
@@ -180,12 +181,14 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
             // of the W tile's rows
             const uint32_t fb = map_to_cta(smem_u32(&full_bar[s]), 0);
             if (pr == 0) mbar_arrive_expect_tx(&full_bar[s], 2u * STAGE_BYTES);
-            tma_load_2d_pair(dst, &tm_a, kb * BK, t.a_row, fb);
+            if (p.a_piece) for (int q = 0; q < BM / 32; ++q) tma_load_2d_pair(dst + q * (32 * BK * 2), &tm_a, kb * BK, piece_row(t.t0 + 32 * q), fb);
+            else tma_load_2d_pair(dst, &tm_a, kb * BK, t.a_row, fb);
             if (EPI == EPI_SWIGLU) tma_load_2d_pair(dst + A_BYTES, pr == 0 ? &tm_b0 : &tm_b1, kb * BK, t.n0, fb);
             else tma_load_2d_pair(dst + A_BYTES, tm_b, kb * BK, t.n0 + pr * (BN / 2), fb);
           } else {
             mbar_arrive_expect_tx(&full_bar[s], (uint32_t)STAGE_BYTES);
-            tma_load_2d(dst, &tm_a, kb * BK, t.a_row, &full_bar[s]);
+            if (p.a_piece) for (int q = 0; q < BM / 32; ++q) tma_load_2d(dst + q * (32 * BK * 2), &tm_a, kb * BK, piece_row(t.t0 + 32 * q), &full_bar[s]);
+            else tma_load_2d(dst, &tm_a, kb * BK, t.a_row, &full_bar[s]);
             if (EPI == EPI_SWIGLU) {
               tma_load_2d(dst + A_BYTES, &tm_b0, kb * BK, t.n0, &full_bar[s]);
               tma_load_2d(dst + A_BYTES + B_BYTES / 2, &tm_b1, kb * BK, t.n0, &full_bar[s]);
@@ -262,6 +265,7 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
         tok_first = t.rows_valid > 0 ? p.idx[t.t0] : 0;  // a row that exists, for the table reads of rows that do not
         if ((unsigned)tok_first >= (unsigned)p.g.tokens()) tok_first = 0;
       }
+      const FlatRows fr(p.g, t.t0, p.flat != 0);
       const bool rotate = (EPI == EPI_Q) || (EPI == EPI_KV && !t.is_b1);
       const int score_col = (EPI == EPI_Q) ? p.g.score_head * HDIM - t.n0 : -1;   // first column of the scoring head in this tile
       __nv_bfloat16* out = t.is_b1 ? p.out1 : p.out0;
@@ -317,6 +321,8 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
               tokr = ok[k] ? tk : tok_first;
               pos = p.g.position(tokr);
               crowr = (size_t)p.g.cache_row(tokr);
+            } else if (p.flat) {
+              fr.at(rc, &pos, &crowr);
             }
             tok_k[k] = tokr; crow_k[k] = crowr;
             if (!GATHER && EPI == EPI_KV && p.store_mask != nullptr && ok[k] && p.store_mask[crowr] != 0) ok[k] = false;

@@ -9,11 +9,11 @@
 //   warps 2-7 wait for the accumulator (warps 2-5 are also the A-operand producers of a gathered launch); afterwards
 //             all warps finish rows, and move the accumulator out of tensor memory first (thread <-> row; with eight
 //             warps the two warps of a TMEM lane quarter take half of the columns each)
-// Split-K: when a launch has too few tiles to fill the GPU, the two CTAs of a thread-block cluster share a tile, each
-// over half of the reduction.  Every CTA first moves its fp32 accumulator from tensor memory into its own shared
+// Split-K: when a launch has too few tiles to fill the GPU, the two (128-wide tiles: up to four) CTAs of a thread-block
+// cluster share a tile, each over its part of the reduction.  Every CTA first moves its fp32 accumulator from tensor memory into its own shared
 // memory (the operand ring is idle by then).  The halves are then combined by a reduce-scatter over distributed
-// shared memory: CTA k owns 64 rows of the tile and receives the partner's partial of those rows by one bulk copy
-// per warp (32 KB, completion counted on an mbarrier of the receiver).  Each CTA finishes the rows it owns with all
+// shared memory: CTA k owns 64 (32) rows of the tile and receives the partners' partials of those rows by bulk copies
+// (completion counted on an mbarrier of the receiver).  Each CTA finishes the rows it owns with all
 // of its warps: one warp per row, lane <-> column pairs, so that table reads and output stores are contiguous.
 // The fused epilogue work is thereby spread over both CTAs as well.
 // Fused epilogues:
@@ -59,7 +59,7 @@ struct Cfg {
 };
 // After the main loop the ring is reused: [0, 128 KB) this CTA's fp32 partial tile, [row][256 columns], 1 KB per row,
 // the 16-byte units of a row XOR-swizzled with the row index (bank-conflict-free for row-per-thread writes and for
-// row-per-warp reads); [128 KB, 192 KB) the partner's partial of the 64 rows this CTA owns (split-K only).
+// row-per-warp reads); behind it the partners' partials of the rows this CTA owns, one slot per partner (split-K only).
 }  // namespace
 
 // Finishing pass, per warp: RB rows at a time (rows rl0, rl0 + #warps, ...); their table reads are issued together.
@@ -80,10 +80,10 @@ struct RowBatch {
   __nv_bfloat162 res[RB][2][2];   // residual row (output projection of a transformer block): this lane's pairs per head
 };
 
-template <int EPI, int RB, int kWarps, int BN, int HDIM>
+template <int EPI, int RB, int kWarps, int BN, int HDIM, bool FLAT>
 __device__ __forceinline__ void load_row_batch(RowBatch<RB>& rb, const GemmParams& p, int rl0, int z, int rows_per_cta,
-                                               int rows_valid, int t0, int pos0, size_t crow0, bool rotate,
-                                               bool score_tile, int lane, int n0) {
+                                               int rows_valid, int t0, int pos0, size_t crow0,
+                                               const FlatRows& fr, bool rotate, bool score_tile, int lane, int n0) {
   using L = Lanes<HDIM>;
 #pragma unroll
   for (int k = 0; k < RB; ++k) {
@@ -98,6 +98,9 @@ __device__ __forceinline__ void load_row_batch(RowBatch<RB>& rb, const GemmParam
       if (!token_ok(rb.tok[k], p.g.tokens(), p.status)) { rb.tok[k] = 0; rb.ok[k] = false; }   // no row to write
       pos = p.g.position(rb.tok[k]);
       rb.crow[k] = (size_t)p.g.cache_row(rb.tok[k]);
+    } else if (FLAT) {
+      rb.tok[k] = t0 + rc;
+      fr.at(rc, &pos, &rb.crow[k]);
     } else {
       rb.tok[k] = t0 + rc;
       pos = pos0 + rc;
@@ -120,7 +123,10 @@ __device__ __forceinline__ void load_row_batch(RowBatch<RB>& rb, const GemmParam
   }
 }
 
-template <int EPI, int BN, bool PAIR, int HDIM>
+// FLAT: row tiles run on across sequences (p.flat, p.a_piece); a kernel of its own because the row mapping sits on the
+// critical path of every tile (0.5-1 us a launch when all launches carried it).
+// FOUR: the reduction is split in four (for the same reason).
+template <int EPI, int BN, bool PAIR, int HDIM, bool FLAT, bool FOUR>
 __global__ void __launch_bounds__(Warps<BN>::N * 32, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b0,
                const __grid_constant__ CUtensorMap tm_b1, const GemmParams p) {
@@ -181,6 +187,21 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     pdl_wait();
     if (mt * BM >= checked_count(*p.count, p.m_total, p.status)) return;     // uniform over the cluster
   }
+  // One k-block of the A tile: one box of 128 rows, or (p.a_piece) four boxes of 32, each of which lies in one sequence of
+  // a row space the tile's rows are not consecutive in.
+  auto load_a = [&](uint8_t* dst, int x, int a_row, uint64_t* bar) {
+    if (!FLAT || !p.a_piece) {
+      if (PAIR) tma_load_2d_pair(dst, &tm_a, x, a_row, map_to_cta(smem_u32(bar), lead));
+      else tma_load_2d(dst, &tm_a, x, a_row, bar);
+      return;
+    }
+    const int T = p.g.tokens();
+    for (int q = 0; q < BM / 32; ++q) {
+      const int t = a_row + 32 * q, row = p.g.cache_row(t < T ? t : T - 32);      // (past the end: any rows, dropped later)
+      if (PAIR) tma_load_2d_pair(dst + q * (32 * BK * 2), &tm_a, x, row, map_to_cta(smem_u32(bar), lead));
+      else tma_load_2d(dst + q * (32 * BK * 2), &tm_a, x, row, bar);
+    }
+  };
   // Gathered A operand: the four epilogue warps fetch the rows of the refresh set themselves, 16 bytes at a time,
   // into the swizzled tile layout (the TMA producer then only brings the W tiles); each of them arrives on a stage
   // once its rows of that stage have landed.
@@ -196,7 +217,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     mbar_init(accum_bar, 1);
     mbar_init(recv_bar, 1);
     fence_mbar_init();
-    if (cl_splits > 1) mbar_arrive_expect_tx(recv_bar, (uint32_t)(BM / 2) * PROW_BYTES);   // the partner's 64 rows (if split)
+    if (cl_splits > 1) mbar_arrive_expect_tx(recv_bar, (uint32_t)((cl_splits - 1) * (BM / cl_splits)) * PROW_BYTES);   // the partners' rows (if split)
     prefetch_tmap(&tm_a);
     prefetch_tmap(tm_b);
   }
@@ -251,11 +272,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
   if (p.count != nullptr) {
     const int n = checked_count(*p.count, p.m_total, p.status);
     if (p.loop_rows) {
-      // The cluster's two CTAs share one row tile (half of the reduction each, partial tiles exchanged) while there is
-      // only one left; with two or more left each takes a row tile of its own over the whole reduction: one pass
-      // over the weights for two tiles instead of two, and nothing to exchange.
+      // The cluster's CTAs share one row tile (a part of the reduction each, partial tiles exchanged) while fewer tiles are
+      // left than CTAs; otherwise each takes a row tile of its own over the whole reduction: one pass over the weights
+      // for all of them, and nothing to exchange.
       const int tiles_left = (n + BM - 1) / BM - tiles_done;
-      if (!PAIR && cl_splits == 2 && tiles_left >= 2) { mt = tiles_done + cl_z; splits = 1; z = 0; tile_step = 2; }
+      if (!PAIR && cl_splits > 1 && tiles_left >= cl_splits) { mt = tiles_done + cl_z; splits = 1; z = 0; tile_step = cl_splits; }
       else mt = tiles_done;
     }
     t0 = mt * BM;
@@ -275,8 +296,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     crow0 = (size_t)b * p.g.max_seq + pos0;
   }
 
+  const FlatRows fr(p.g, FLAT ? t0 : 0, FLAT);
+
   // epilogue geometry
   const int rows_per_cta = BM / splits;           // rows of the tile this CTA finishes
+  constexpr int slot_rows = FOUR ? BM / 4 : BM / 2;
   const int nkb = KB / splits;                    // k-blocks this CTA walks for the tile
   const int quarter = warp & 3;                   // TMEM lanes a warp may touch: 32*quarter .. +31
   const bool rotate = (EPI == EPI_Q) || (EPI == EPI_KV && !is_b1);
@@ -290,10 +314,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
   if (warp == 0) {
     if (!gather && elect_one()) {
       for (int i = 0; i < n_early; ++i) {        // the W halves of these stages are already on their way
-        if (PAIR)
-          tma_load_2d_pair(smem + i * STAGE_BYTES, &tm_a, kb_of(i) * BK, a_row, map_to_cta(smem_u32(&full_bar[i]), lead));
-        else
-          tma_load_2d(smem + i * STAGE_BYTES, &tm_a, kb_of(i) * BK, a_row, &full_bar[i]);
+        load_a(smem + i * STAGE_BYTES, kb_of(i) * BK, a_row, &full_bar[i]);
       }
     }
     __syncwarp();
@@ -305,12 +326,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         if (PAIR) {
           const uint32_t fb = map_to_cta(smem_u32(&full_bar[s]), lead);
           if (pr == 0) mbar_arrive_expect_tx(&full_bar[s], 2 * STAGE_BYTES);
-          tma_load_2d_pair(a_dst, &tm_a, kb_of(i) * BK, a_row, fb);
+          load_a(a_dst, kb_of(i) * BK, a_row, &full_bar[s]);
           tma_load_2d_pair(a_dst + A_BYTES, p.b_pair ? (pr == 0 ? &tm_b0 : &tm_b1) : tm_b, kb_of(i) * BK,
                            p.b_pair ? n0 : n0 + pr * (BN / 2), fb);
         } else {
           mbar_arrive_expect_tx(&full_bar[s], tx_bytes);
-          if (!gather) tma_load_2d(a_dst, &tm_a, kb_of(i) * BK, a_row, &full_bar[s]);
+          if (!gather) load_a(a_dst, kb_of(i) * BK, a_row, &full_bar[s]);
           if (p.b_pair) {
             tma_load_2d(a_dst + A_BYTES, &tm_b0, kb_of(i) * BK, n0, &full_bar[s]);
             tma_load_2d(a_dst + A_BYTES + C::B_BYTES / 2, &tm_b1, kb_of(i) * BK, n0, &full_bar[s]);
@@ -358,13 +379,16 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
   } else {
     // While the main loop runs, pull the table rows the finishing pass of this CTA will read into the L2
     // (dense tiles; 4 * HDIM bytes = LINES lines per row and table).
-    if (p.idx == nullptr) {
+    if (p.idx == nullptr && (rotate || (score_tile && p.has_prev))) {
       constexpr int LINES = HDIM / 32;
       for (int i = threadIdx.x - 64; i < rows_per_cta * LINES; i += (kWarps - 2) * 32) {
         const int r = z * rows_per_cta + i / LINES;
         if (r >= rows_valid) break;
-        if (rotate) prefetch_l2(p.rope + (size_t)(pos0 + r) * L::HALF + (i % LINES) * 16);
-        if (score_tile && p.has_prev) prefetch_l2(p.q_prev + (crow0 + r) * HDIM + (i % LINES) * 32);
+        int pos = pos0 + r;
+        size_t crow = crow0 + r;
+        if (FLAT) fr.at(r, &pos, &crow);
+        if (rotate) prefetch_l2(p.rope + (size_t)pos * L::HALF + (i % LINES) * 16);
+        if (score_tile && p.has_prev) prefetch_l2(p.q_prev + crow * HDIM + (i % LINES) * 32);
       }
     }
     // the table reads of this warp's first rows of the finishing pass: in flight for the whole main loop
@@ -375,7 +399,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       tok_own = p.idx[t0 + r_own];
       if (!token_ok(tok_own, p.g.tokens(), p.status)) tok_own = -1;      // read as a row of zeros
     }
-    load_row_batch<EPI, RB, kWarps, BN, HDIM>(rb, p, warp, z, rows_per_cta, rows_valid, t0, pos0, crow0, rotate, score_tile, lane, n0);
+    load_row_batch<EPI, RB, kWarps, BN, HDIM, FLAT>(rb, p, warp, z, rows_per_cta, rows_valid, t0, pos0, crow0, fr, rotate, score_tile, lane, n0);
     if (gather && warp < 6) {
       // One stage of the A tile = 128 rows x 128 bytes (64 k-elements).  A warp takes 32 rows; one of its copy
       // instructions covers four rows, eight consecutive lanes fetching the eight 16-byte units of a row, so every
@@ -422,7 +446,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
 
   // The table reads of the first rows the producer and MMA warps will finish start now (those of the other warps
   // started before the main loop) and land during the exchange below.
-  if (warp < 2) load_row_batch<EPI, RB, kWarps, BN, HDIM>(rb, p, warp, z, rows_per_cta, rows_valid, t0, pos0, crow0, rotate, score_tile, lane, n0);
+  if (warp < 2) load_row_batch<EPI, RB, kWarps, BN, HDIM, FLAT>(rb, p, warp, z, rows_per_cta, rows_valid, t0, pos0, crow0, fr, rotate, score_tile, lane, n0);
 
   // ---- every CTA of the cluster has finished its main loop: the rings are free to receive partial rows
   tc_fence_before();
@@ -446,7 +470,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     const bool send = splits > 1 && owner != z;
     const int rl0 = quarter * 32 - owner * rows_per_cta;
     const uint32_t rbar = send ? map_to_cta(smem_u32(recv_bar), rank_of_slice(owner)) : 0u;
-    const uint32_t rbase = send ? map_to_cta(smem_u32(smem + RECV_OFFSET), rank_of_slice(owner)) : 0u;
+    const int slot = z < owner ? z : z - 1;                          // this CTA's slot at the owner
+    const uint32_t rbase = send ? map_to_cta(smem_u32(smem + RECV_OFFSET) + (uint32_t)(FOUR ? slot * slot_rows : 0) * PROW_BYTES,
+                                             rank_of_slice(owner)) : 0u;
     // (the next chunk's tensor-memory load is in flight while this chunk is written and sent)
     float va[32], vb[32];
     tmem_ld_32x32_nowait(t_lane + ch0 * 32, va);
@@ -465,7 +491,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0)
-          bulk_copy_to_cta(rbase + (uint32_t)ch * (uint32_t)((BM / 2) * 128) + (uint32_t)rl0 * 128u,
+          bulk_copy_to_cta(rbase + (uint32_t)ch * (uint32_t)(slot_rows * 128) + (uint32_t)rl0 * 128u,
                            smem_u32(smem) + (uint32_t)ch * (uint32_t)(BM * 128) + (uint32_t)(quarter * 32) * 128u, 32 * 128, rbar);
       }
     }
@@ -481,7 +507,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     __nv_bfloat16* out = is_b1 ? p.out1 : p.out0;
 #pragma unroll 1
     for (int rl0 = warp; rl0 < rows_per_cta; rl0 += kWarps * RB) {
-      if (rl0 != warp) load_row_batch<EPI, RB, kWarps, BN, HDIM>(rb, p, rl0, z, rows_per_cta, rows_valid, t0, pos0, crow0, rotate, score_tile, lane, n0);
+      if (rl0 != warp) load_row_batch<EPI, RB, kWarps, BN, HDIM, FLAT>(rb, p, rl0, z, rows_per_cta, rows_valid, t0, pos0, crow0, fr, rotate, score_tile, lane, n0);
       if (dbg && EPI == EPI_Q && threadIdx.x == 64) p.debug[34 + (rl0 - warp) / (kWarps * RB) * 2] = globaltimer_ns();
       // (1) combine the partial rows: lane <-> a pair of columns of each piece and its rotary partners
       float2 vlo[RB][BN / CH], vhi[RB][BN / CH];
@@ -497,12 +523,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
           const uint8_t* mine = smem + (size_t)(z * rows_per_cta + rl) * 128;             // this CTA's partial
           float2 lo = *reinterpret_cast<const float2*>(mine + (size_t)(c_lo >> 5) * (BM * 128) + in_lo);
           float2 hi = *reinterpret_cast<const float2*>(mine + (size_t)(c_hi >> 5) * (BM * 128) + in_hi);
-          if (splits > 1) {
-            const uint8_t* theirs = smem + RECV_OFFSET + (size_t)rl * 128;                // the partner's partial
-            const float2 a = *reinterpret_cast<const float2*>(theirs + (size_t)(c_lo >> 5) * ((BM / 2) * 128) + in_lo);
-            const float2 b = *reinterpret_cast<const float2*>(theirs + (size_t)(c_hi >> 5) * ((BM / 2) * 128) + in_hi);
+          auto add_slot = [&](int s2) {                                                   // a partner's partial
+            const uint8_t* theirs = smem + RECV_OFFSET + (size_t)(s2 * slot_rows) * PROW_BYTES + (size_t)rl * 128;
+            const float2 a = *reinterpret_cast<const float2*>(theirs + (size_t)((c_lo >> 5) * slot_rows) * 128 + in_lo);
+            const float2 b = *reinterpret_cast<const float2*>(theirs + (size_t)((c_hi >> 5) * slot_rows) * 128 + in_hi);
             lo.x += a.x; lo.y += a.y; hi.x += b.x; hi.y += b.y;
-          }
+          };
+          if (splits > 1) add_slot(0);
+          if (FOUR && splits == 4) { add_slot(1); add_slot(2); }
           vlo[k][hh] = lo; vhi[k][hh] = hi;
         }
       }
@@ -632,11 +660,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
   }
 }
 
-template <int EPI, int BN, bool PAIR, int HDIM>
-static cudaError_t launch_hd(const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1, const GemmParams& p,
+template <int EPI, int BN, bool PAIR, int HDIM, bool FLAT, bool FOUR>
+static cudaError_t launch_as(const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1, const GemmParams& p,
                               int n_tiles, int m_tiles, int splits, cudaStream_t st) {
   static std::atomic<unsigned long long> attr_done{0};
-  auto kern = gemm_tc_kernel<EPI, BN, PAIR, HDIM>;
+  auto kern = gemm_tc_kernel<EPI, BN, PAIR, HDIM, FLAT, FOUR>;
   constexpr int SMEM_TOTAL = Cfg<BN, PAIR>::SMEM_TOTAL;
   if (cudaError_t e = ensure_dyn_smem(kern, SMEM_TOTAL, attr_done); e != cudaSuccess) return e;
   GemmParams q = p;
@@ -646,6 +674,22 @@ static cudaError_t launch_hd(const CUtensorMap& a, const CUtensorMap& b0, const 
                          splits, a, b0, b1, q);
   return launch_pdl_xz(kern, dim3(n_tiles, m_tiles, splits), dim3(Warps<BN>::N * 32), SMEM_TOTAL, st, 1, splits, a, b0, b1,
                        q);
+}
+template <int EPI, int BN, bool PAIR, int HDIM, bool FLAT>
+static cudaError_t launch_split(const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1, const GemmParams& p,
+                                int n_tiles, int m_tiles, int splits, cudaStream_t st) {
+  if constexpr (BN == 128) {
+    if (splits == 4) return launch_as<EPI, BN, PAIR, HDIM, FLAT, true>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
+  }
+  return launch_as<EPI, BN, PAIR, HDIM, FLAT, false>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
+}
+template <int EPI, int BN, bool PAIR, int HDIM>
+static cudaError_t launch_hd(const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1, const GemmParams& p,
+                             int n_tiles, int m_tiles, int splits, cudaStream_t st) {
+  if constexpr (EPI != EPI_SWIGLU && EPI != EPI_F32) {
+    if (p.flat && p.idx == nullptr) return launch_split<EPI, BN, PAIR, HDIM, true>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
+  }
+  return launch_split<EPI, BN, PAIR, HDIM, false>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
 }
 // (only the epilogues that rotate and score know heads; to the others the lane map is any map)
 template <int EPI, int BN, bool PAIR>
@@ -663,7 +707,7 @@ cudaError_t launch_gemm_tc(int epi, int bn, const CUtensorMap& a, const CUtensor
                            const GemmParams& p, int n_tiles, int m_tiles, int splits, cudaStream_t st, int pair) {
   if (m_tiles <= 0 || n_tiles <= 0) return cudaSuccess;
   if (epi == EPI_OUT && p.resid != nullptr) epi = EPI_OUT_RES;
-  if ((splits != 1 && splits != 2) || splits > p.K / BK) return cudaErrorInvalidValue;
+  if ((splits != 1 && splits != 2 && (splits != 4 || bn != 128)) || p.K / BK % splits != 0) return cudaErrorInvalidValue;
   if (pair && bn == 128) {
     // narrow pair tiles (256 rows x 128 columns per pair; b0 / b1 with 64-row boxes): twice the CTAs of the wide ones
     // for launches of two row tiles, whose main loops are bound by what one SM can pull from the L2
@@ -691,7 +735,12 @@ cudaError_t launch_gemm_tc(int epi, int bn, const CUtensorMap& a, const CUtensor
     if (epi == EPI_OUT_RES) return launch_one<EPI_OUT_RES, 256, false>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
     return launch_one<EPI_OUT, 256, false>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
   }
-  if (bn == 128 && epi == EPI_KV) return launch_one<EPI_KV, 128, false>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
+  if (bn == 128 && !p.b_pair) {
+    if (epi == EPI_KV) return launch_one<EPI_KV, 128, false>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
+    if (epi == EPI_Q) return launch_one<EPI_Q, 128, false>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
+    if (epi == EPI_OUT) return launch_one<EPI_OUT, 128, false>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
+    if (epi == EPI_OUT_RES) return launch_one<EPI_OUT_RES, 128, false>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
+  }
   return cudaErrorInvalidValue;
 }
 

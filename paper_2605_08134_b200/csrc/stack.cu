@@ -299,19 +299,16 @@ dare_status_t forward(dare_stack* S, const int* tokens, int batch, int seq_total
       GemmParams p = base_params(S, batch, seq_act, pos_begin);
       p.K = f; p.out0 = B.xa; p.resid = B.hb; p.ld_resid = d;
       const int n_tiles = d / 256;
-      const int sp = pick_splits(n_tiles * m_tiles, f / 64);
-      const bool pair = pairs_pay(n_tiles, m_tiles, sp);
-      if (narrow_pairs_pay(d, m_tiles, f / 64)) {
-        if (launch_gemm_tc(EPI_OUT, 128, S->a_act, S->maps[l].w_down64, S->maps[l].w_down64, p, d / 128, m_tiles, 2, st,
-                           1) != cudaSuccess) return DARE_ERR_CUDA;
-      } else if (persist_pays(n_tiles, m_tiles, sp)) {
+      TileForm t;
+      if (pick_one_wave(d, m_tiles, f / 64, &t)) {
+        const int box = t.pair ? t.bn / 2 : t.bn;
+        const CUtensorMap& wd = box == 256 ? S->maps[l].w_down : (box == 128 ? S->maps[l].w_down128 : S->maps[l].w_down64);
+        if (launch_gemm_tc(EPI_OUT, t.bn, S->a_act, wd, wd, p, d / t.bn, m_tiles, t.splits, st, t.pair) != cudaSuccess)
+          return DARE_ERR_CUDA;
+      } else {
         const int pp = persist_pairs_pay(n_tiles, m_tiles) ? 1 : 0;
         const CUtensorMap& wd = pp ? S->maps[l].w_down128 : S->maps[l].w_down;
         if (launch_gemm_persist(EPI_OUT, S->a_act, wd, wd, p, n_tiles, m_tiles, st, pp) != cudaSuccess) return DARE_ERR_CUDA;
-      } else {
-        const CUtensorMap& wd = pair ? S->maps[l].w_down128 : S->maps[l].w_down;
-        if (launch_gemm_tc(EPI_OUT, 256, S->a_act, wd, wd, p, n_tiles, m_tiles, sp, st, pair ? 1 : 0) != cudaSuccess)
-          return DARE_ERR_CUDA;
       }
     }
   }

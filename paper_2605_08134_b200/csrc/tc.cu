@@ -8,6 +8,7 @@ namespace dare {
 
 struct TcState {
   CUtensorMap a_xn, a_oc;                  // A operands, box 64 x 128 rows
+  CUtensorMap a_oc32;                      // ... box 64 x 32 rows, for row tiles that run on across sequences
   CUtensorMap a_xg;                        // compact copy of a refresh set's rows (the input staging buffer, idle after RMSNorm)
   CUtensorMap w_q, w_k, w_v, w_o;          // weights, box 64 x 256 rows
   CUtensorMap w_k128, w_v128, w_q128, w_o128;   // weights, box 64 x 128 rows
@@ -17,7 +18,6 @@ struct TcState {
 
 namespace {
 
-bool use_pairs(int n_tiles, int m_tiles, int splits) { return pairs_pay(n_tiles, m_tiles, splits); }
 // units (column tile x pair of row tiles) from which the two-CTA form of a listed launch runs: two rounds of the 74 clusters
 constexpr int kPairUnitGate = 148;
 
@@ -43,6 +43,12 @@ int pick_splits(int tiles, int kblocks) {
   int s = 1;
   while (s < 2 && tiles * s * 2 <= 160 && s * 2 <= kblocks) s *= 2;
   return s;
+}
+
+// ... of narrow K/V tiles: up to four over one row tile (two row tiles are better off with a CTA of a pair each)
+int kv_splits(int tiles, int kblocks, bool one_row_tile) {
+  int s = pick_splits(tiles, kblocks);
+  return s == 2 && one_row_tile && tiles * 4 <= 128 && kblocks % 4 == 0 && kblocks >= 16 ? 4 : s;
 }
 
 }  // namespace
@@ -71,7 +77,7 @@ dare_status_t tc_create(dare_layer* L) {
   if (!s) return DARE_ERR_INVALID_ARG;
   const uint64_t Tm = (uint64_t)L->cfg.max_batch * L->cfg.max_seq, d = L->cfg.d_model;
   bool ok = make_map(&s->a_xn, L->buf.xn, Tm, d, 128) && make_map(&s->a_xg, L->buf.x_stage, Tm, d, 128) &&
-            make_map(&s->a_oc, L->buf.oc, Tm, d, 128) && make_map(&s->w_q, L->w.w_q, d, d, 256) &&
+            make_map(&s->a_oc, L->buf.oc, Tm, d, 128) && make_map(&s->a_oc32, L->buf.oc, Tm, d, 32) && make_map(&s->w_q, L->w.w_q, d, d, 256) &&
             make_map(&s->w_k, L->w.w_k, d, d, 256) && make_map(&s->w_v, L->w.w_v, d, d, 256) &&
             make_map(&s->w_o, L->w.w_o, d, d, 256) && make_map(&s->w_k128, L->w.w_k, d, d, 128) &&
             make_map(&s->w_v128, L->w.w_v, d, d, 128) && make_map(&s->w_q128, L->w.w_q, d, d, 128) &&
@@ -100,15 +106,23 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
   // the input staging buffer doubles as the compact copy of a refresh set's rows once x has been normalised; not
   // when x is still needed later (the residual of a transformer block reads it in the output projection)
   const bool compact_ok = !add_input || x != B.x_stage;
-  const int tiles_per_seq = (g.seq_act + 127) / 128;
-  const int m_tiles_dense = g.batch * tiles_per_seq;
+  // Row tiles of the projections run on across sequences: x_norm is compact over the step's tokens, and the O cache is
+  // too where the step covers all of every sequence, or can be fetched in boxes of 32 rows.  Otherwise a sequence's last
+  // tile may be partly filled (eight windows of 32 rows are two tiles, not eight).
+  const int tiles_per_seq = (g.seq_act + 127) / 128, m_tiles_seq = g.batch * tiles_per_seq;
+  const bool run_on = (T_ + 127) / 128 < m_tiles_seq;
+  const int m_tiles_dense = run_on ? (T_ + 127) / 128 : m_tiles_seq;
+  const bool oc_compact = g.seq_act == g.max_seq, oc_flat = run_on && (oc_compact || g.seq_act % 32 == 0);
+  const int m_tiles_out = oc_flat ? m_tiles_dense : m_tiles_seq;
   const int kblocks = d / 64;
   int launches = 0;
   cudaError_t e;
 
   GemmParams base;
   base.K = d; base.m_total = T_; base.seq_act = g.seq_act; base.tiles_per_seq = tiles_per_seq;
-  base.a_seq_stride = g.seq_act; base.a_row0 = 0; base.idx = nullptr; base.count = nullptr; base.g = g;
+  base.a_seq_stride = g.seq_act; base.a_row0 = 0; base.flat = 0; base.a_piece = 0;
+  if (run_on) { base.seq_act = base.a_seq_stride = T_; base.tiles_per_seq = m_tiles_dense; base.flat = 1; }
+  base.idx = nullptr; base.count = nullptr; base.g = g;
   base.gather_src = nullptr; base.gather_cache_rows = 0; base.unit_gate = 0;
   base.n_split = 1 << 30; base.out0 = nullptr; base.out1 = nullptr; base.ld_out = d;
   base.out_is_cache = 0; base.resid = nullptr; base.ld_resid = 0; base.out_f32 = nullptr; base.b_pair = 0;
@@ -136,20 +150,17 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
     GemmParams p = base;
     p.out0 = (bf16*)B.q;
     p.debug = dbg;
-    const int n_tiles = d / 256;
     prof_mark(L, SLOT_Q_GEMM, st);
-    const int sp = pick_splits(n_tiles * m_tiles_dense, kblocks);
-    if (narrow_pairs_pay(d, m_tiles_dense, kblocks))
-      e = launch_gemm_tc(EPI_Q, 128, S.a_xn, S.w_q64, S.w_q64, p, d / 128, m_tiles_dense, 2, st, 1);
-    else if (persist_pays(n_tiles, m_tiles_dense, sp)) {
-      const int pair = persist_pairs_pay(n_tiles, m_tiles_dense) ? 1 : 0;
+    TileForm f;
+    if (pick_one_wave(d, m_tiles_dense, kblocks, &f)) {
+      const int box = f.pair ? f.bn / 2 : f.bn;
+      const CUtensorMap& wq = box == 256 ? S.w_q : (box == 128 ? S.w_q128 : S.w_q64);
+      e = launch_gemm_tc(EPI_Q, f.bn, S.a_xn, wq, wq, p, d / f.bn, m_tiles_dense, f.splits, st, f.pair);
+    } else {
+      const int pair = persist_pairs_pay(d / 256, m_tiles_dense) ? 1 : 0;
       const CUtensorMap& wq = pair ? S.w_q128 : S.w_q;
-      e = launch_gemm_persist(EPI_Q, S.a_xn, wq, wq, p, n_tiles, m_tiles_dense, st, pair);
+      e = launch_gemm_persist(EPI_Q, S.a_xn, wq, wq, p, d / 256, m_tiles_dense, st, pair);
     }
-    else if (use_pairs(n_tiles, m_tiles_dense, sp))
-      e = launch_gemm_tc(EPI_Q, 256, S.a_xn, S.w_q128, S.w_q128, p, n_tiles, m_tiles_dense, sp, st, 1);
-    else
-      e = launch_gemm_tc(EPI_Q, 256, S.a_xn, S.w_q, S.w_q, p, n_tiles, m_tiles_dense, sp, st);
     ++launches;
     if (e != cudaSuccess) return DARE_ERR_CUDA;
   }
@@ -187,8 +198,8 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
         p.n_split = d / 128;
         const int n_tiles128 = 2 * d / 128;
         p.loop_rows = 1;                         // one row of CTAs: no CTA that only looks at the count and leaves
-        e = launch_gemm_tc(EPI_KV, 128, S.a_xn, S.w_k128, S.w_v128, p, n_tiles128, 1,
-                           pick_splits(n_tiles128, kblocks), st); ++launches;
+        e = launch_gemm_tc(EPI_KV, 128, S.a_xn, S.w_k128, S.w_v128, p, n_tiles128, 1, kv_splits(n_tiles128, kblocks, T_ <= 128), st);
+        ++launches;
       } else {
         // Many tokens: even a small refreshed fraction fills the GPU with 256-wide tiles, which re-read the least.
         if (persist_pays_listed(n_tiles, m_tiles) && compact_ok) {
@@ -223,7 +234,11 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
         e = launch_gemm_persist(EPI_KV, S.a_xn, pair ? S.w_k128 : S.w_k, pair ? S.w_v128 : S.w_v, p, n_tiles, m_tiles_dense,
                                 st, pair);
       }
-      else if (use_pairs(n_tiles, m_tiles_dense, sp))
+      else if (m_tiles_dense == 1) {             // few rows: a stream of the weights, narrow tiles put twice as many CTAs on it
+        p.n_split = d / 128;
+        e = launch_gemm_tc(EPI_KV, 128, S.a_xn, S.w_k128, S.w_v128, p, 2 * d / 128, 1, kv_splits(2 * d / 128, kblocks, true), st);
+      }
+      else if (pairs_pay(n_tiles, m_tiles_dense, sp))
         e = launch_gemm_tc(EPI_KV, 256, S.a_xn, S.w_k128, S.w_v128, p, n_tiles, m_tiles_dense, sp, st, 1);
       else
         e = launch_gemm_tc(EPI_KV, 256, S.a_xn, S.w_k, S.w_v, p, n_tiles, m_tiles_dense, sp, st);
@@ -271,9 +286,14 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
   // copies the others.  With few tokens the projection is a stream of W_O whatever the row count, and stays dense.
   {
     const bool many = m_tiles_dense > 8 && !add_input;
+    const CUtensorMap& a_oc = oc_flat && !oc_compact ? S.a_oc32 : S.a_oc;
     const bool y_sparse = o_sparse && many && L->yc_valid;
     GemmParams p = base;
-    p.a_seq_stride = g.max_seq; p.a_row0 = g.pos_begin;
+    if (oc_flat) {
+      p.a_piece = oc_compact ? 0 : 1;
+    } else {
+      p.seq_act = g.seq_act; p.tiles_per_seq = tiles_per_seq; p.a_seq_stride = g.max_seq; p.a_row0 = g.pos_begin; p.flat = 0;
+    }
     p.out0 = (bf16*)y;
     if (many) p.out1 = (bf16*)B.yc;                                   // kept by cache row for later steps
     if (add_input) { p.resid = (const bf16*)x; p.ld_resid = d; }      // y = x + W_O O (residual block)
@@ -281,11 +301,12 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
     const int n_tiles = d / 256;
     prof_mark(L, SLOT_OUT_GEMM, st);
     if (y_sparse) {
-      p.idx = B.idx; p.count = B.count; p.gather_src = (const bf16*)B.oc; p.gather_cache_rows = 1;
+      const int a_piece = p.a_piece;
+      p.idx = B.idx; p.count = B.count; p.gather_src = (const bf16*)B.oc; p.gather_cache_rows = 1; p.a_piece = 0;
       bool dense_form = false;
       if (persist_pays_listed(n_tiles, (T_ + 127) / 128) && compact_ok) {
         // (beyond gate_o refreshed tokens the dense projection of every row instead: Alg. 2 line 11 as written)
-        dense_form = persist_pays_listed(n_tiles, m_tiles_dense);
+        dense_form = persist_pays_listed(n_tiles, m_tiles_out);
         const int hi = dense_form ? gate_o : 1 << 30;
         launch_gather_step_rows((const bf16*)B.oc, B.idx, B.count, (bf16*)B.x_stage, g, true, st, B.status, hi); ++launches;
         p.gather_src = nullptr;
@@ -295,10 +316,10 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
         if (e == cudaSuccess) e = launch_gemm_persist(EPI_OUT, S.a_xg, S.w_o, S.w_o, p, n_tiles, (T_ + 127) / 128, st, 0);
         if (dense_form && e == cudaSuccess) {
           GemmParams pd = p;
-          pd.idx = nullptr; pd.count = nullptr; pd.unit_gate = 0; pd.gather_cache_rows = 0;
+          pd.idx = nullptr; pd.count = nullptr; pd.unit_gate = 0; pd.gather_cache_rows = 0; pd.a_piece = a_piece;
           pd.gate_lo = gate_o; pd.gate_hi = 1 << 30;
           ++launches;
-          e = launch_gemm_persist(EPI_OUT, S.a_oc, S.w_o128, S.w_o128, pd, n_tiles, m_tiles_dense, st, 1);
+          e = launch_gemm_persist(EPI_OUT, a_oc, S.w_o128, S.w_o128, pd, n_tiles, m_tiles_out, st, 1);
         }
       } else
         e = launch_gemm_tc(EPI_OUT, 256, S.a_oc, S.w_o, S.w_o, p, n_tiles, (T_ + 127) / 128, 1, st);
@@ -306,18 +327,16 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
       if (e != cudaSuccess) return DARE_ERR_CUDA;
       launch_copy_reused_rows((const bf16*)B.yc, (bf16*)y, B.delta, g, st, dense_form ? B.count : nullptr, gate_o); ++launches;
     } else {
-      const int sp = pick_splits(n_tiles * m_tiles_dense, kblocks);
-      if (narrow_pairs_pay(d, m_tiles_dense, kblocks))
-        e = launch_gemm_tc(EPI_OUT, 128, S.a_oc, S.w_o64, S.w_o64, p, d / 128, m_tiles_dense, 2, st, 1);
-      else if (persist_pays(n_tiles, m_tiles_dense, sp)) {
-        const int pair = persist_pairs_pay(n_tiles, m_tiles_dense) ? 1 : 0;
+      TileForm f;
+      if (pick_one_wave(d, m_tiles_out, kblocks, &f)) {
+        const int box = f.pair ? f.bn / 2 : f.bn;
+        const CUtensorMap& wo = box == 256 ? S.w_o : (box == 128 ? S.w_o128 : S.w_o64);
+        e = launch_gemm_tc(EPI_OUT, f.bn, a_oc, wo, wo, p, d / f.bn, m_tiles_out, f.splits, st, f.pair);
+      } else {
+        const int pair = persist_pairs_pay(n_tiles, m_tiles_out) ? 1 : 0;
         const CUtensorMap& wo = pair ? S.w_o128 : S.w_o;
-        e = launch_gemm_persist(EPI_OUT, S.a_oc, wo, wo, p, n_tiles, m_tiles_dense, st, pair);
+        e = launch_gemm_persist(EPI_OUT, a_oc, wo, wo, p, n_tiles, m_tiles_out, st, pair);
       }
-      else if (use_pairs(n_tiles, m_tiles_dense, sp))
-        e = launch_gemm_tc(EPI_OUT, 256, S.a_oc, S.w_o128, S.w_o128, p, n_tiles, m_tiles_dense, sp, st, 1);
-      else
-        e = launch_gemm_tc(EPI_OUT, 256, S.a_oc, S.w_o, S.w_o, p, n_tiles, m_tiles_dense, sp, st);
       ++launches;
       if (e != cudaSuccess) return DARE_ERR_CUDA;
       // the cache is complete once a dense projection has covered every cached row, and stays so while every

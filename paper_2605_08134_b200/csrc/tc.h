@@ -18,6 +18,9 @@ struct GemmParams {
   int tiles_per_seq;     // ... and 128-row tiles per sequence
   int a_seq_stride;      // rows between sequences in A's row space
   int a_row0;            // first row of the window in A's row space
+  int flat;              // dense row tiles run on across sequences (one "sequence" of all the step's tokens in the mapping
+                         // above): positions and cache rows come from the tokens
+  int a_piece;           // ... and A is addressed by cache row, in boxes of 32 rows (windows of a multiple of 32 rows)
   const int* idx;        // gathered: token of each A row (ascending refresh set), else nullptr
   const int* count;      // gathered: device count of rows, else nullptr
   const __nv_bfloat16* gather_src;  // gathered: the matrix [*, K] whose rows idx[] the kernel fetches itself as its A
@@ -61,6 +64,28 @@ struct GemmParams {
                          // only before they leave, which keeps completion transitive along the stream
 };
 
+#ifdef __CUDACC__
+// Position and cache row of the rows of a tile that runs on across sequences (GemmParams::flat): row r of the tile is the
+// step's token t0 + r.  One integer division per tile; per row a multiplication, exact because the quotient is small (a
+// tile spans at most 128 sequences) and (i + 0.5) / seq_act stays 0.5 / seq_act away from an integer.
+struct FlatRows {
+  int b0, i0, seq_act, pos_begin, max_seq;
+  float inv;
+  __device__ __forceinline__ FlatRows(const StepGeom& g, int t0, bool used) {
+    if (!used) return;
+    b0 = t0 / g.seq_act;
+    i0 = t0 - b0 * g.seq_act;
+    seq_act = g.seq_act; pos_begin = g.pos_begin; max_seq = g.max_seq;
+    inv = 1.f / (float)g.seq_act;
+  }
+  __device__ __forceinline__ void at(int r, int* pos, size_t* crow) const {
+    const int i = i0 + r, b = (int)(((float)i + 0.5f) * inv);
+    *pos = pos_begin + i - b * seq_act;
+    *crow = (size_t)(b0 + b) * max_seq + *pos;
+  }
+};
+#endif
+
 struct AttnParams {
   const __nv_bfloat16* q;   // [T, d] rotated queries of the step (flat token rows)
   __nv_bfloat16* oc;        // attention-output cache
@@ -86,9 +111,9 @@ bool attention_tc_two_tiles(const StepGeom& g, bool row_sparse);
 cudaError_t launch_attention_tc(const CUtensorMap& tm_k, const CUtensorMap& tm_v, const AttnParams& p,
                                 cudaStream_t st);
 
-// grid = (n_tiles of bn columns, m_tiles of 128 rows, splits of the reduction dimension = cluster size: 1 or 2);
-// bn = 256 (least re-reading per flop) or 128 (more CTAs for the weight-streaming K/V projection of a small refresh
-// set).
+// grid = (n_tiles of bn columns, m_tiles of 128 rows, splits of the reduction dimension = cluster size: 1, 2, or 4 with
+// bn = 128);
+// bn = 256 (least re-reading per flop) or 128 (more CTAs where few rows make the launch a stream of the weights).
 // The W tensor maps must have a box of bn rows.
 // Row-major bf16 matrix [rows, cols] as a TMA tensor map with a box of 64 columns x box_rows rows, 128-byte swizzle.
 bool make_map(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows);
@@ -102,10 +127,25 @@ inline bool pairs_pay(int n_tiles, int m_tiles, int splits) {
   return m_tiles >= 2 && (ctas <= 160 || m_tiles <= 4);
 }
 
-// ... and with exactly two row tiles (a window of up to 256 rows) the narrow pair tiles (256 x 128 per pair, reduction
-// split in two) put twice as many CTAs on the launch: d/128 column tiles x 2 x 2 CTAs, if that still is one wave.
-inline bool narrow_pairs_pay(int d_out, int m_tiles, int kblocks) {
-  return m_tiles == 2 && kblocks >= 4 && (d_out / 128) * 2 * 2 <= 160;
+// The form of a dense projection that is one wave of CTAs: tile width, two-CTA MMAs or not, reduction splits.  What a CTA
+// takes is its k-blocks times what one takes it (bound by the operand bytes an SM pulls from the L2: 48, 32, 32 and 24 KB
+// for wide, wide pair, narrow and narrow pair tiles) plus the exchange of partial tiles; few row tiles want narrow tiles
+// and more splits (one row tile of 4096 x 4096: 32 CTAs of 32 k-blocks -> 128 of 16), more of them wide ones.  Clusters of
+// four and more CTAs do not cover all 148 SMs.  false: no form is one wave.
+struct TileForm { int bn, pair, splits; };
+inline bool pick_one_wave(int d_out, int m_tiles, int kblocks, TileForm* best) {
+  float best_us = 1e30f;
+  for (int pair = 0; pair < 2; ++pair)
+    for (int bn = 128; bn <= 256; bn += 128)
+      for (int s = 1; s <= (bn == 128 ? 4 : 2); s *= 2) {
+        const int cluster = (pair + 1) * s, ctas = d_out / bn * (pair ? (m_tiles + 1) / 2 * 2 : m_tiles) * s;
+        if (d_out % bn != 0 || ctas > (cluster >= 4 ? 128 : 148) || kblocks % s != 0 || kblocks / s < 2) continue;
+        if (pair && m_tiles < 2) continue;
+        const float us = (float)(kblocks / s) * (bn == 256 ? (pair ? 0.33f : 0.36f) : (pair ? 0.25f : 0.31f)) +
+                         (s == 1 ? 0.f : (s == 2 ? 2.5f : 3.2f)) + (pair ? 0.3f : 0.f);
+        if (us < best_us) { best_us = us; *best = TileForm{bn, pair, s}; }
+      }
+  return best_us < 1e29f;
 }
 
 cudaError_t launch_gemm_tc(int epi, int bn, const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1,
