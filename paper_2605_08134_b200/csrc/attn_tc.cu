@@ -125,7 +125,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const int ksplit = gridDim.z;                      // = cluster size along z
   const int z = ksplit > 1 ? (int)cluster_ctarank() : 0;
-  const int rows_own = BQ / ksplit;                   // rows of the tile this CTA writes out
   const bool dbg = p.debug != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0;
   if (dbg && threadIdx.x == 0) p.debug[0] = globaltimer_ns();
   const StepGeom& g = p.g;
@@ -175,7 +174,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     }
     mbar_init(recv_bar, 1);
     fence_mbar_init();
-    if (ksplit > 1) mbar_arrive_expect_tx(recv_bar, (uint32_t)((ksplit - 1) * rows_own * (HD * 4 + 8)));
     prefetch_tmap(&tm_k);
     prefetch_tmap(&tm_v);
   }
@@ -209,6 +207,12 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       active = __syncthreads_or(mine) != 0;
     }
   }
+  // Key split: the rows that exist are shared out evenly (in fours: the copies of their statistics are whole 16-byte
+  // units); a CTA past them owns none, and nothing is merged for rows that do not exist.
+  const int rows_own = ksplit > 1 ? ((rows_valid + ksplit - 1) / ksplit + 3) & ~3 : BQ;
+  const bool owns = active && z * rows_own < rows_valid;
+  if (ksplit > 1 && threadIdx.x == 0 && owns)
+    mbar_arrive_expect_tx(recv_bar, (uint32_t)((ksplit - 1) * rows_own * (HD * 4 + 8)));
   const int n_blocks_all = (g.kv_len + BKV - 1) / BKV;
   const int n_blocks = n_blocks_all > z ? (n_blocks_all - z + ksplit - 1) / ksplit : 0;   // blocks z, z + ksplit, ...
   const int kv_row0 = b * g.max_seq;
@@ -345,7 +349,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       mbar_wait(&s_full[st], j & 1, p.status);
       tc_fence_after();
       if (dbg && j == 0 && threadIdx.x == 128) p.debug[2] = globaltimer_ns();
-      if (!warp_has_rows && ksplit == 1) {
+      if (!warp_has_rows) {
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&p_full[st]);
@@ -429,6 +433,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       tc_fence_after();
     }
     if (dbg && threadIdx.x == 128) p.debug[3] = globaltimer_ns();
+    // (a warp without rows has nothing to merge or store, but takes part in the barrier)
     // ---- merge the two streams: thread (stream st, row r) finishes its half of the row's columns
     constexpr int HC = HD / 2;
     float* stat_mine = reinterpret_cast<float*>(smem + S::V_OFF + 2 * st * S::V_BYTES);
@@ -438,6 +443,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     tc_fence_before();
     asm volatile("bar.sync 1, %0;" ::"n"(kSoftmaxThreads) : "memory");
     tc_fence_after();
+    if (warp_has_rows) {
     const float m_o = n_other > 0 ? stat_other[r] : -INFINITY, l_o = n_other > 0 ? stat_other[BQ + r] : 0.f;
     const float m_all = fmaxf(m, m_o);
     const float w_mine = n_st > 0 ? fast_exp2((m - m_all) * c) : 0.f;
@@ -492,6 +498,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       }
       fence_proxy_async_smem();
     }
+    }  // warp_has_rows
   }
   if (ksplit > 1) {
     // ---- merge of the key split (all warps)
@@ -499,7 +506,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     tc_fence_before();
     cluster_sync_relaxed();                              // every CTA of the cluster is past its key loop
     tc_fence_after();
-    if (warp == 4 && lane < ksplit && lane != z) {
+    if (warp == 4 && lane < ksplit && lane != z && lane * rows_own < rows_valid) {
       // hand the rows owned by CTA `lane` to it: the rows, their maxima, their sums
       const int k = lane;
       const int slot = z < k ? z : z - 1;
@@ -511,7 +518,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       bulk_copy_to_cta(dst + rows_own * HD * 4 + rows_own * 4, smem_u32(smem + S::STAT_OFF + (BQ + k * rows_own) * 4),
                        rows_own * 4, bar);
     }
-    mbar_wait(recv_bar, 0, p.status);
+    if (owns) mbar_wait(recv_bar, 0, p.status);
     const float c = rsqrtf((float)HD) * 1.4426950408889634f;
     const float* dump = reinterpret_cast<const float*>(smem + S::DUMP_OFF);
     const float* stat = reinterpret_cast<const float*>(smem + S::STAT_OFF);

@@ -286,6 +286,34 @@ template void launch_rmsnorm<__nv_bfloat16>(const __nv_bfloat16*, const float*, 
 // (It was a launch of its own that read the scores once per pass and walked the bins with one thread.)
 constexpr int kKthInCta = 16384;
 constexpr int kKthPerThread = kKthInCta / 1024;
+// At most kKthCount tokens: every token's rank is counted instead, against all keys in shared memory (1024 / n threads to
+// a token), which is one pass with one barrier on each side (64 tokens: selection 6.0 -> 3.5 us).
+constexpr int kKthCount = 512;
+__device__ float kth_by_count(const float* __restrict__ scores, int n, int k) {
+  __shared__ __align__(16) unsigned keys[kKthCount];
+  __shared__ float s_tau;
+  if (k <= 0 || k >= n) return __int_as_float(k <= 0 ? 0xff800000 : 0x7f800000);
+  const int tid = threadIdx.x;
+  if (tid < kKthCount) keys[tid] = tid < n ? score_key(scores[tid]) : kKeyNaN;    // (missing tokens sort last, as NaN)
+  if (tid == 0) s_tau = __int_as_float(0x7f800000);                              // stays: rank k falls among the NaN scores
+  __syncthreads();
+  const int per = n <= 32 ? 32 : (n <= 64 ? 16 : (n <= 128 ? 8 : (n <= 256 ? 4 : 2)));   // threads to a token
+  const int t = tid / per, part = tid % per;
+  const unsigned mine = t < kKthCount ? keys[t] : kKeyNaN;
+  int less = 0, same = 0;
+  for (int i = part * 4; i < n; i += per * 4) {                                  // (up to 3 past n: they read as NaN)
+    const uint4 v = *reinterpret_cast<const uint4*>(keys + i);
+    less += (v.x < mine) + (v.y < mine) + (v.z < mine) + (v.w < mine);
+    same += (v.x == mine) + (v.y == mine) + (v.z == mine) + (v.w == mine);
+  }
+  for (int o = per / 2; o > 0; o >>= 1) {
+    less += __shfl_xor_sync(0xffffffffu, less, o);
+    same += __shfl_xor_sync(0xffffffffu, same, o);
+  }
+  if (t < n && mine != kKeyNaN && less < k && k <= less + same) s_tau = key_score(mine);   // (tied tokens write the same value)
+  __syncthreads();
+  return s_tau;
+}
 template <int KPT>
 __device__ float kth_in_cta(const float* __restrict__ scores, int n, int k) {
   __shared__ int hist[256];
@@ -341,7 +369,7 @@ __global__ void __launch_bounds__(1024) kth_score_kernel(const float* __restrict
                                                          float* __restrict__ tau_out) {
   ptx::pdl_wait();
   ptx::pdl_launch_dependents();
-  const float tau = kth_in_cta<kKthPerThread>(scores, n, k);
+  const float tau = n <= kKthCount ? kth_by_count(scores, n, k) : kth_in_cta<kKthPerThread>(scores, n, k);
   if (threadIdx.x == 0) *tau_out = tau;
 }
 bool kth_score_in_select(int n) { return n <= kKthInCta; }
@@ -466,7 +494,7 @@ __global__ void __launch_bounds__(1024) select_small_kernel(const float* __restr
   if (!wait_at_end) ptx::pdl_wait();
   ptx::pdl_launch_dependents();
   if (kKth) {
-    tau = kth_in_cta<kSmallTokens / 1024>(scores, T, reuse_count);
+    tau = T <= kKthCount ? kth_by_count(scores, T, reuse_count) : kth_in_cta<kSmallTokens / 1024>(scores, T, reuse_count);
     if (threadIdx.x == 0) *tau_dev = tau;
   } else if (tau_dev != nullptr) {
     tau = *tau_dev;

@@ -179,6 +179,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
   // leaves free only to look at the count and leave, and the next kernel cannot start before the last of them has).
   for (int iter = 0;; ++iter) {
   int mt = mt_first + iter;
+  int grp2 = -1;                                // (two CTAs a tile in a cluster of four: which of the two tiles)
   int splits = cl_splits, z = cl_z, tile_step = 1;   // (settled below, once the size of the refresh set is known)
   // Row tiles past the first one of a gathered launch are usually empty (the refresh set is small): they look at
   // the count before spending anything on set-up.  The others set up first and wait for the previous kernel later.
@@ -217,7 +218,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     mbar_init(accum_bar, 1);
     mbar_init(recv_bar, 1);
     fence_mbar_init();
-    if (cl_splits > 1) mbar_arrive_expect_tx(recv_bar, (uint32_t)((cl_splits - 1) * (BM / cl_splits)) * PROW_BYTES);   // the partners' rows (if split)
     prefetch_tmap(&tm_a);
     prefetch_tmap(tm_b);
   }
@@ -272,11 +272,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
   if (p.count != nullptr) {
     const int n = checked_count(*p.count, p.m_total, p.status);
     if (p.loop_rows) {
-      // The cluster's CTAs share one row tile (a part of the reduction each, partial tiles exchanged) while fewer tiles are
-      // left than CTAs; otherwise each takes a row tile of its own over the whole reduction: one pass over the weights
-      // for all of them, and nothing to exchange.
+      // The cluster's CTAs share one row tile (a part of the reduction each, partial tiles exchanged) while there is only
+      // one left; with as many left as CTAs each takes a row tile of its own over the whole reduction: one pass over the
+      // weights for all of them, and nothing to exchange.  Four CTAs and two or three tiles: two CTAs a tile, half of the
+      // reduction each (CTAs 0, 2 and 1, 3: the k-blocks a CTA has asked for early are the start of its half).
       const int tiles_left = (n + BM - 1) / BM - tiles_done;
       if (!PAIR && cl_splits > 1 && tiles_left >= cl_splits) { mt = tiles_done + cl_z; splits = 1; z = 0; tile_step = cl_splits; }
+      else if (FOUR && tiles_left >= 2) { grp2 = cl_z & 1; mt = tiles_done + grp2; splits = 2; z = cl_z >> 1; tile_step = 2; }
       else mt = tiles_done;
     }
     t0 = mt * BM;
@@ -300,7 +302,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
 
   // epilogue geometry
   const int rows_per_cta = BM / splits;           // rows of the tile this CTA finishes
-  constexpr int slot_rows = FOUR ? BM / 4 : BM / 2;
+  if (threadIdx.x == 0 && splits > 1)             // the partners' rows (they start to arrive behind the cluster barrier below)
+    mbar_arrive_expect_tx(recv_bar, (uint32_t)((splits - 1) * rows_per_cta) * PROW_BYTES);
+  const int slot_rows = FOUR ? rows_per_cta : BM / 2;
   const int nkb = KB / splits;                    // k-blocks this CTA walks for the tile
   const int quarter = warp & 3;                   // TMEM lanes a warp may touch: 32*quarter .. +31
   const bool rotate = (EPI == EPI_Q) || (EPI == EPI_KV && !is_b1);
@@ -469,10 +473,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     const int owner = r / rows_per_cta;                              // (uniform over the warp: 32 | rows_per_cta)
     const bool send = splits > 1 && owner != z;
     const int rl0 = quarter * 32 - owner * rows_per_cta;
-    const uint32_t rbar = send ? map_to_cta(smem_u32(recv_bar), rank_of_slice(owner)) : 0u;
+    const uint32_t owner_rank = FOUR && grp2 >= 0 ? (uint32_t)(grp2 + 2 * owner) : rank_of_slice(owner);
+    const uint32_t rbar = send ? map_to_cta(smem_u32(recv_bar), owner_rank) : 0u;
     const int slot = z < owner ? z : z - 1;                          // this CTA's slot at the owner
     const uint32_t rbase = send ? map_to_cta(smem_u32(smem + RECV_OFFSET) + (uint32_t)(FOUR ? slot * slot_rows : 0) * PROW_BYTES,
-                                             rank_of_slice(owner)) : 0u;
+                                             owner_rank) : 0u;
     // (the next chunk's tensor-memory load is in flight while this chunk is written and sent)
     float va[32], vb[32];
     tmem_ld_32x32_nowait(t_lane + ch0 * 32, va);

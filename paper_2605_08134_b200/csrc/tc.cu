@@ -45,10 +45,10 @@ int pick_splits(int tiles, int kblocks) {
   return s;
 }
 
-// ... of narrow K/V tiles: up to four over one row tile (two row tiles are better off with a CTA of a pair each)
-int kv_splits(int tiles, int kblocks, bool one_row_tile) {
+// ... of narrow K/V tiles: up to four
+int kv_splits(int tiles, int kblocks) {
   int s = pick_splits(tiles, kblocks);
-  return s == 2 && one_row_tile && tiles * 4 <= 128 && kblocks % 4 == 0 && kblocks >= 16 ? 4 : s;
+  return s == 2 && tiles * 4 <= 128 && kblocks % 4 == 0 && kblocks >= 16 ? 4 : s;
 }
 
 }  // namespace
@@ -198,7 +198,7 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
         p.n_split = d / 128;
         const int n_tiles128 = 2 * d / 128;
         p.loop_rows = 1;                         // one row of CTAs: no CTA that only looks at the count and leaves
-        e = launch_gemm_tc(EPI_KV, 128, S.a_xn, S.w_k128, S.w_v128, p, n_tiles128, 1, kv_splits(n_tiles128, kblocks, T_ <= 128), st);
+        e = launch_gemm_tc(EPI_KV, 128, S.a_xn, S.w_k128, S.w_v128, p, n_tiles128, 1, kv_splits(n_tiles128, kblocks), st);
         ++launches;
       } else {
         // Many tokens: even a small refreshed fraction fills the GPU with 256-wide tiles, which re-read the least.
@@ -236,7 +236,7 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
       }
       else if (m_tiles_dense == 1) {             // few rows: a stream of the weights, narrow tiles put twice as many CTAs on it
         p.n_split = d / 128;
-        e = launch_gemm_tc(EPI_KV, 128, S.a_xn, S.w_k128, S.w_v128, p, 2 * d / 128, 1, kv_splits(2 * d / 128, kblocks, true), st);
+        e = launch_gemm_tc(EPI_KV, 128, S.a_xn, S.w_k128, S.w_v128, p, 2 * d / 128, 1, kv_splits(2 * d / 128, kblocks), st);
       }
       else if (pairs_pay(n_tiles, m_tiles_dense, sp))
         e = launch_gemm_tc(EPI_KV, 256, S.a_xn, S.w_k128, S.w_v128, p, n_tiles, m_tiles_dense, sp, st, 1);
