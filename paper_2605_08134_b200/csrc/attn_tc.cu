@@ -100,7 +100,8 @@ __device__ __forceinline__ void load_block(uint8_t* dst, const CUtensorMap* tm, 
 
 }  // namespace
 
-template <int HD>
+// SPLIT: the keys are split over a cluster (a kernel of its own: the unsplit one has no registers to spare)
+template <int HD, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                const AttnParams p) {
@@ -123,8 +124,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   // the warp index through a shuffle, so that the compiler knows it (and every role decision and shared-memory
   // descriptor derived from it) to be uniform over the warp
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
-  const int ksplit = gridDim.z;                      // = cluster size along z
-  const int z = ksplit > 1 ? (int)cluster_ctarank() : 0;
+  const int ksplit = SPLIT ? (int)gridDim.z : 1;     // = cluster size along z
+  const int z = SPLIT ? (int)cluster_ctarank() : 0;
   const bool dbg = p.debug != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0;
   if (dbg && threadIdx.x == 0) p.debug[0] = globaltimer_ns();
   const StepGeom& g = p.g;
@@ -207,12 +208,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       active = __syncthreads_or(mine) != 0;
     }
   }
-  // Key split: the rows that exist are shared out evenly (in fours: the copies of their statistics are whole 16-byte
-  // units); a CTA past them owns none, and nothing is merged for rows that do not exist.
-  const int rows_own = ksplit > 1 ? ((rows_valid + ksplit - 1) / ksplit + 3) & ~3 : BQ;
-  const bool owns = active && z * rows_own < rows_valid;
-  if (ksplit > 1 && threadIdx.x == 0 && owns)
-    mbar_arrive_expect_tx(recv_bar, (uint32_t)((ksplit - 1) * rows_own * (HD * 4 + 8)));
   const int n_blocks_all = (g.kv_len + BKV - 1) / BKV;
   const int n_blocks = n_blocks_all > z ? (n_blocks_all - z + ksplit - 1) / ksplit : 0;   // blocks z, z + ksplit, ...
   const int kv_row0 = b * g.max_seq;
@@ -469,7 +464,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         for (int i = 0; i < 32; ++i) acc[cgrp * 32 + i] = fmaf(a[i], w_other, acc[cgrp * 32 + i]);
       }
     }
-    if (ksplit == 1) {
+    if (!SPLIT) {
       // normalise, store
       const float inv = 1.f / l_row;
       const int t = t_row;
@@ -500,8 +495,12 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     }
     }  // warp_has_rows
   }
-  if (ksplit > 1) {
-    // ---- merge of the key split (all warps)
+  if (SPLIT) {
+    // ---- merge of the key split (all warps).  The rows that exist are shared out evenly (in fours: the copies of their
+    // statistics are whole 16-byte units); a CTA past them owns none, and nothing is merged for rows that do not exist.
+    const int rows_own = ((rows_valid + ksplit - 1) / ksplit + 3) & ~3;
+    const bool owns = z * rows_own < rows_valid;
+    if (threadIdx.x == 0 && owns) mbar_arrive_expect_tx(recv_bar, (uint32_t)((ksplit - 1) * rows_own * (HD * 4 + 8)));
     __syncthreads();
     tc_fence_before();
     cluster_sync_relaxed();                              // every CTA of the cluster is past its key loop
@@ -565,7 +564,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   }  // active
   tc_fence_before();
   // nobody leaves while a copy out of its shared memory may still be in flight (its receiver has seen it land)
-  if (ksplit > 1) cluster_sync_relaxed(); else __syncthreads();
+  if (SPLIT) cluster_sync_relaxed(); else __syncthreads();
   if (dbg && threadIdx.x == 0) p.debug[4] = globaltimer_ns();
   if (p.debug != nullptr && threadIdx.x == 0) {      // latest end over the CTAs that had work, and their number
     atomicMax(&p.debug[6], globaltimer_ns());
@@ -984,8 +983,9 @@ bool attention_tc_two_tiles(const StepGeom& g, bool row_sparse) {
 template <int HD>
 static cudaError_t launch_attention_hd(const CUtensorMap& tm_k, const CUtensorMap& tm_v, const AttnParams& p,
                                        cudaStream_t st) {
-  static std::atomic<unsigned long long> attr_one{0}, attr_pair{0};
-  if (cudaError_t e = ensure_dyn_smem(attn_tc_kernel<HD>, AttnSmem<HD>::TOTAL, attr_one); e != cudaSuccess) return e;
+  static std::atomic<unsigned long long> attr_one{0}, attr_split{0}, attr_pair{0};
+  if (cudaError_t e = ensure_dyn_smem(attn_tc_kernel<HD, false>, AttnSmem<HD>::TOTAL, attr_one); e != cudaSuccess) return e;
+  if (cudaError_t e = ensure_dyn_smem(attn_tc_kernel<HD, true>, AttnSmem<HD>::TOTAL, attr_split); e != cudaSuccess) return e;
   if (cudaError_t e = ensure_dyn_smem(attn_pair_kernel<HD>, PairSmem<HD>::TOTAL, attr_pair); e != cudaSuccess) return e;
   const int tps = (p.g.seq_act + BQ - 1) / BQ;
   const int tps2 = (p.g.seq_act + kPairRows - 1) / kPairRows;
@@ -998,7 +998,7 @@ static cudaError_t launch_attention_hd(const CUtensorMap& tm_k, const CUtensorMa
   }
   dim3 grid(p.g.n_heads, p.g.batch * tps, ksplit);
   if (grid.y == 0) return cudaSuccess;
-  return launch_pdl(attn_tc_kernel<HD>, grid, dim3(kThreads), AttnSmem<HD>::TOTAL, st, ksplit, tm_k, tm_v, p);
+  return launch_pdl(ksplit > 1 ? attn_tc_kernel<HD, true> : attn_tc_kernel<HD, false>, grid, dim3(kThreads), AttnSmem<HD>::TOTAL, st, ksplit, tm_k, tm_v, p);
 }
 
 cudaError_t launch_attention_tc(const CUtensorMap& tm_k, const CUtensorMap& tm_v, const AttnParams& p,

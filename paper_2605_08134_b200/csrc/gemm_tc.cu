@@ -218,6 +218,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     mbar_init(accum_bar, 1);
     mbar_init(recv_bar, 1);
     fence_mbar_init();
+    // the partner's 64 rows (if split; with up to four CTAs a tile the number is settled below)
+    if (!FOUR && cl_splits > 1) mbar_arrive_expect_tx(recv_bar, (uint32_t)(BM / 2) * PROW_BYTES);
     prefetch_tmap(&tm_a);
     prefetch_tmap(tm_b);
   }
@@ -302,7 +304,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
 
   // epilogue geometry
   const int rows_per_cta = BM / splits;           // rows of the tile this CTA finishes
-  if (threadIdx.x == 0 && splits > 1)             // the partners' rows (they start to arrive behind the cluster barrier below)
+  if (FOUR && threadIdx.x == 96 && splits > 1)    // the partners' rows (they start to arrive behind the cluster barrier below)
     mbar_arrive_expect_tx(recv_bar, (uint32_t)((splits - 1) * rows_per_cta) * PROW_BYTES);
   const int slot_rows = FOUR ? rows_per_cta : BM / 2;
   const int nkb = KB / splits;                    // k-blocks this CTA walks for the tile
