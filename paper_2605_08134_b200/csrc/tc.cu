@@ -140,6 +140,20 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
   // (no clearing between steps: a copy or memset in the stream would break the kernels' launch overlap; the stamps
   // are plain stores or maxima of a clock that only grows)
 
+  // A dense K/V projection (Alg. 2 line 7, or the full forward of Appendix E.2) needs nothing from the Q projection
+  // or the selection.  On a short step (launches of about one wave, where fixed costs and the hand-off between
+  // kernels decide) it is issued right behind the Q projection and runs beside it: the two launches are one fused
+  // Q/K/V projection of the step's rows, spread over two grids because the Q tiles take a split reduction and the
+  // K/V tiles do not.  The selection then follows both.
+  // (K/V tiles that are more than one wave may be better off in the persistent kernel behind the Q projection: a round of
+  // CTAs of both launches takes about 9 us + 0.36 us a k-block, the persistent kernel 0.33 us a k-block and round of pairs)
+  bool kv_beside_q = !kv_sparse && m_tiles_dense <= 8;
+  if (kv_beside_q && persist_pays(2 * d / 256, m_tiles_dense, pick_splits(2 * d / 256 * m_tiles_dense, kblocks))) {
+    const int q_ctas = d / 256 * ((m_tiles_dense + 1) / 2 * 2), units = 2 * d / 256 * ((m_tiles_dense + 1) / 2);
+    const float beside = (float)((q_ctas + 2 * d / 256 * m_tiles_dense + 147) / 148) * (9.f + 0.36f * (float)kblocks);
+    const float behind = 20.f + 0.33f * (float)(kblocks * (1 + (units + 73) / 74));
+    kv_beside_q = beside < behind;
+  }
   prof_begin(L);
   // Alg. 1/2 line 1
   prof_mark(L, SLOT_NORM, st);
@@ -152,7 +166,17 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
     p.debug = dbg;
     prof_mark(L, SLOT_Q_GEMM, st);
     TileForm f;
-    if (pick_one_wave(d, m_tiles_dense, kblocks, &f)) {
+    // (a K/V projection beside it: both launches resident at once where they fit and this one does not become the longer)
+    int kv_ctas = 0;
+    float kv_us = 0.f;
+    if (kv_beside_q) {
+      const int n_kv = 2 * d / 256, sp = pick_splits(n_kv * m_tiles_dense, kblocks);
+      kv_ctas = m_tiles_dense == 1 ? 2 * n_kv * kv_splits(2 * n_kv, kblocks)
+                                   : n_kv * (pairs_pay(n_kv, m_tiles_dense, sp) ? (m_tiles_dense + 1) / 2 * 2 : m_tiles_dense) * sp;
+      kv_us = 0.33f * (float)(kblocks / sp) + 6.f;
+    }
+    if ((kv_ctas > 0 && pick_one_wave(d, m_tiles_dense, kblocks, &f, kv_ctas, kv_us)) ||
+        pick_one_wave(d, m_tiles_dense, kblocks, &f)) {
       const int box = f.pair ? f.bn / 2 : f.bn;
       const CUtensorMap& wq = box == 256 ? S.w_q : (box == 128 ? S.w_q128 : S.w_q64);
       e = launch_gemm_tc(EPI_Q, f.bn, S.a_xn, wq, wq, p, d / f.bn, m_tiles_dense, f.splits, st, f.pair);
@@ -164,14 +188,6 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
     ++launches;
     if (e != cudaSuccess) return DARE_ERR_CUDA;
   }
-  // A dense K/V projection (Alg. 2 line 7, or the full forward of Appendix E.2) needs nothing from the Q projection
-  // or the selection.  On a short step (launches of about one wave, where fixed costs and the hand-off between
-  // kernels decide) it is issued right behind the Q projection and runs beside it: the two launches are one fused
-  // Q/K/V projection of the step's rows, spread over two grids because the Q tiles take a split reduction and the
-  // K/V tiles do not.  The selection then follows both.
-  // (not where the K/V tiles are more than one wave and take the persistent kernel)
-  const bool kv_beside_q = !kv_sparse && m_tiles_dense <= 8 &&
-                           !persist_pays(2 * d / 256, m_tiles_dense, pick_splits(2 * d / 256 * m_tiles_dense, kblocks));
   // lines 4-5 + Sec. 4
   const bool select_all = !has_prev || mode == DARE_MODE_DENSE;
   auto select_now = [&]() {
@@ -229,7 +245,7 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
       prof_mark(L, SLOT_KV_GEMM, st);
       p.wait_at_end = kv_beside_q ? 1 : 0;
       const int sp = pick_splits(n_tiles * m_tiles_dense, kblocks);
-      if (persist_pays(n_tiles, m_tiles_dense, sp)) {
+      if (!kv_beside_q && persist_pays(n_tiles, m_tiles_dense, sp)) {
         const int pair = persist_pairs_pay(n_tiles, m_tiles_dense) ? 1 : 0;
         e = launch_gemm_persist(EPI_KV, S.a_xn, pair ? S.w_k128 : S.w_k, pair ? S.w_v128 : S.w_v, p, n_tiles, m_tiles_dense,
                                 st, pair);

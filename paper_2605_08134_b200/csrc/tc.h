@@ -129,23 +129,31 @@ inline bool pairs_pay(int n_tiles, int m_tiles, int splits) {
 
 // The form of a dense projection that is one wave of CTAs: tile width, two-CTA MMAs or not, reduction splits.  What a CTA
 // takes is its k-blocks times what one takes it (bound by the operand bytes an SM pulls from the L2: 48, 32, 32 and 24 KB
-// for wide, wide pair, narrow and narrow pair tiles) plus the exchange of partial tiles; few row tiles want narrow tiles
-// and more splits (one row tile of 4096 x 4096: 32 CTAs of 32 k-blocks -> 128 of 16), more of them wide ones.  Clusters of
-// four and more CTAs do not cover all 148 SMs.  false: no form is one wave.
+// for wide, wide pair, narrow and narrow pair tiles), the read-out of the accumulator with the exchange of partial tiles,
+// and the finishing pass over its share of the tile (measured by the kernels' own stamps).  Few row tiles want narrow
+// tiles and more splits (one row tile of 4096 x 4096: 32 CTAs of 32 k-blocks -> 128 of 16), more of them wide ones.
+// Clusters of four CTAs do not cover all 148 SMs, and clusters of eight wait for eight free SMs of one GPC behind the
+// kernel before (a 240-row pass of a 2048-wide stack took 29 % longer with them), so there are none.
+// `beside`: CTAs of a launch that runs at the same time and should find SMs free; such a form is taken if it takes no
+// longer than `limit_us`, that launch itself.  false: no form.
 struct TileForm { int bn, pair, splits; };
-inline bool pick_one_wave(int d_out, int m_tiles, int kblocks, TileForm* best) {
+inline bool pick_one_wave(int d_out, int m_tiles, int kblocks, TileForm* best, int beside = 0,
+                          float limit_us = 1e29f) {
+  const float sms = 148.f - (float)beside;
   float best_us = 1e30f;
   for (int pair = 0; pair < 2; ++pair)
     for (int bn = 128; bn <= 256; bn += 128)
-      for (int s = 1; s <= (bn == 128 ? 4 : 2); s *= 2) {
+      for (int s = 1; s <= (bn == 128 && !pair ? 4 : 2); s *= 2) {
         const int cluster = (pair + 1) * s, ctas = d_out / bn * (pair ? (m_tiles + 1) / 2 * 2 : m_tiles) * s;
-        if (d_out % bn != 0 || ctas > (cluster >= 4 ? 128 : 148) || kblocks % s != 0 || kblocks / s < 2) continue;
+        if (d_out % bn != 0 || (float)ctas > (cluster >= 4 ? 0.87f : 1.f) * sms || kblocks % s != 0 || kblocks / s < 2) continue;
         if (pair && m_tiles < 2) continue;
-        const float us = (float)(kblocks / s) * (bn == 256 ? (pair ? 0.33f : 0.36f) : (pair ? 0.25f : 0.31f)) +
-                         (s == 1 ? 0.f : (s == 2 ? 2.5f : 3.2f)) + (pair ? 0.3f : 0.f);
+        const float main_loop = (float)(kblocks / s) * (bn == 256 ? (pair ? 0.33f : 0.36f) : (pair ? 0.25f : 0.31f));
+        const float exchange = s == 1 ? 1.f : (bn == 256 ? 2.5f : (s == 2 ? 2.f : 2.2f));
+        const float finish = 1.1f + 0.5f * (float)(4 / s * (bn / 128));
+        const float us = main_loop + exchange + finish + (pair ? 0.3f : 0.f);
         if (us < best_us) { best_us = us; *best = TileForm{bn, pair, s}; }
       }
-  return best_us < 1e29f;
+  return best_us < limit_us;
 }
 
 cudaError_t launch_gemm_tc(int epi, int bn, const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1,
