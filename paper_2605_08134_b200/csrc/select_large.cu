@@ -237,20 +237,28 @@ __global__ void __launch_bounds__(kTileWords) tile_scatter_kernel(const unsigned
   }
 }
 
-// ---- the k-th smallest of many scores, by ONE cluster of CTAs: exact radix selection over the order-preserving keys in
-// three passes (11 + 11 + 10 bits).  Every CTA counts its share of the scores into a histogram in its own shared memory;
-// the CTAs then add up one slice of the bins each over distributed shared memory, tell one another the slices' totals,
-// and all of them pick the bin that holds rank k.  A cluster (rather than a grid) because the call has no scratch memory
-// to meet in: nothing is shared between calls, whatever streams they run on.  Bound by what the cluster's SMs pull from
-// the L2 (three reads of the scores) and by the cluster-wide exchange of each pass: two cluster barriers and two remote
-// round trips.  (Copies of the histogram, to keep lanes that meet in one bin apart, changed nothing.)
-constexpr int kKthBins = 2048, kKthMaxCtas = 16;
+// ---- the k-th smallest of many scores, by ONE cluster of CTAs: exact selection by narrowing a range of order-preserving
+// keys, 2048 bins at a time.  Every CTA counts its share of the scores that lie in the range into a histogram in its own
+// shared memory; the CTAs then send one another slices of the bins (bulk copies), add up their own, tell one another the
+// slices' totals, and all of them pick the bin that holds rank k: the next range.  All keys are three such passes.  A
+// shared-memory atomic takes a cycle a lane whatever it meets, so the first pass costs a cycle a score of the CTA's share
+// (copies of the histogram changed nothing): with many scores the range starts as a bracket around rank k from a sample of
+// 256 of them, which most scores lie outside; a bracket that turns out not to hold the rank is given up for all keys.
+// A cluster (rather than a grid) because the call has no scratch memory to meet in: nothing is shared between calls,
+// whatever streams they run on.
+constexpr int kKthBins = 2048, kKthMaxCtas = 16, kKthSample = 256;
+constexpr int kKthBracket = 1 << 19;        // the sample costs about 4 us: from this many scores on
+constexpr unsigned kKeyMinusInf = 0x007fffffu, kKeyPlusInf = 0xff800000u;
 
 __global__ void __launch_bounds__(kThreads) kth_cluster_kernel(const float* __restrict__ scores, int n, int k,
                                                                float* __restrict__ tau_out) {
   __shared__ __align__(16) int hist[kKthBins];
+  __shared__ __align__(16) int recv[kKthBins];        // [sender][bin of this CTA's slice]
+  __shared__ uint64_t recv_bar;
   __shared__ __align__(16) int red[kKthBins / 8];     // this CTA's slice of the bins over the whole cluster
-  __shared__ int part[kKthBins / 8 / 32], totals[kKthMaxCtas], s_bin, s_rank;
+  __shared__ __align__(16) unsigned sample[kKthSample];
+  __shared__ int part[kKthBins / 8 / 32], totals[kKthMaxCtas], below[kKthMaxCtas], s_below, s_bin, s_rank;
+  __shared__ unsigned s_lo, s_hi;
   const int ctas = (int)gridDim.x, rank_cta = (int)ptx::cluster_ctarank(), lane = threadIdx.x & 31, tid = (int)threadIdx.x;
   const int slice = kKthBins / ctas;                  // 128 or 256: whole warps, four or eight bins to a lane
   ptx::pdl_wait();
@@ -259,9 +267,6 @@ __global__ void __launch_bounds__(kThreads) kth_cluster_kernel(const float* __re
   const int head = min(n, (int)((16u - (unsigned)(reinterpret_cast<uintptr_t>(scores) & 15u)) & 15u) / 4);
   const float4* body = reinterpret_cast<const float4*>(scores + head);
   const int n4 = (n - head) / 4, tail0 = head + 4 * n4;
-  unsigned prefix = 0u, mask = 0u;
-  int rank = k;
-  bool numbers = true;                                // rank k falls among the scores that are numbers
   auto scan = [&](int v) {                            // inclusive, over the warp
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -270,56 +275,116 @@ __global__ void __launch_bounds__(kThreads) kth_cluster_kernel(const float* __re
     }
     return v;
   };
-  for (int pass = 0; pass < 3 && numbers; ++pass) {
-    const int shift = pass == 0 ? 21 : (pass == 1 ? 10 : 0);
-    const unsigned dmask = pass == 2 ? 1023u : 2047u;
+  // ---- the bracket, the same in every CTA: the sample's keys four standard deviations of its rank either side of k
+  const bool bracket = n >= kKthBracket;
+  if (bracket && tid < kKthSample) sample[tid] = score_key(scores[(int)(((long long)tid * n) / kKthSample)]);
+  if (tid == 0) {
+    s_lo = kKeyMinusInf; s_hi = kKeyPlusInf;
+    ptx::mbar_init(&recv_bar, 1);
+    ptx::fence_mbar_init();
+  }
+  __syncthreads();
+  if (bracket) {
+    const float p = (float)k / (float)n;
+    const int c = (int)(p * kKthSample), w = (int)(4.f * sqrtf(p * (1.f - p) * kKthSample)) + 2;
+    const int me = tid >> 2;                          // four threads to a sample key
+    const unsigned mine = sample[me];
+    int r = 0;
+    for (int i = (tid & 3) * 4; i < kKthSample; i += 16) {
+      const uint4 v = *reinterpret_cast<const uint4*>(sample + i);
+      r += (v.x < mine || (v.x == mine && i < me)) + (v.y < mine || (v.y == mine && i + 1 < me)) +
+           (v.z < mine || (v.z == mine && i + 2 < me)) + (v.w < mine || (v.w == mine && i + 3 < me));
+    }
+    r += __shfl_xor_sync(0xffffffffu, r, 1);
+    r += __shfl_xor_sync(0xffffffffu, r, 2);
+    if ((tid & 3) == 0) {
+      if (r == c - w && mine != kKeyNaN) s_lo = mine;
+      if (r == c + w && mine != kKeyNaN) s_hi = mine;
+    }
+  }
+  __syncthreads();
+  unsigned lo = s_lo, hi = s_hi;                      // keys in [lo, hi]
+  int rank = k;                                       // of the wanted key: among all of them, then among those in the range
+  bool found = false, numbers = true;                 // numbers: rank k falls among the scores that are numbers
+  ptx::cluster_sync_all();                            // every CTA's barrier is set up
+  uint32_t phase = 0;
+  for (bool first = true, whole = lo == kKeyMinusInf && hi == kKeyPlusInf; !found && numbers; ) {
+    const unsigned range = hi - lo;
+    const int shift = range < (unsigned)kKthBins ? 0 : 21 - __clz((int)range);
     for (int b = tid; b < kKthBins; b += kThreads) hist[b] = 0;
-    if (tid == 0) s_bin = -1;
+    if (tid == 0) { s_bin = -1; s_below = 0; }
     __syncthreads();
-    auto count = [&](float f) {
-      const unsigned key = score_key(f);
-      if (key != kKeyNaN && (key & mask) == prefix) atomicAdd(&hist[(key >> shift) & dmask], 1);
+    int under = 0;
+    auto walk = [&](auto count) {
+      constexpr int U = 8;                            // vectors a thread has in flight
+      const int step = ctas * kThreads;
+      int i = rank_cta * kThreads + tid;
+      for (; i + (U - 1) * step < n4; i += U * step) {
+        float4 v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) v[u] = body[i + u * step];
+#pragma unroll
+        for (int u = 0; u < U; ++u) { count(v[u].x); count(v[u].y); count(v[u].z); count(v[u].w); }
+      }
+      for (; i < n4; i += step) {
+        const float4 v = body[i];
+        count(v.x); count(v.y); count(v.z); count(v.w);
+      }
+      if (rank_cta == 0) {
+        if (tid < head) count(scores[tid]);
+        if (tid < n - tail0) count(scores[tail0 + tid]);
+      }
     };
-    constexpr int U = 8;                              // vectors a thread has in flight
-    const int step = ctas * kThreads;
-    int i = rank_cta * kThreads + tid;
-    for (; i + (U - 1) * step < n4; i += U * step) {
-      float4 v[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u) v[u] = body[i + u * step];
-#pragma unroll
-      for (int u = 0; u < U; ++u) { count(v[u].x); count(v[u].y); count(v[u].z); count(v[u].w); }
+    auto raw_key = [](float f) {                      // score_key of a number; NaN goes below -inf or above +inf
+      const unsigned u = __float_as_uint(f);
+      return u ^ ((unsigned)((int)u >> 31) | 0x80000000u);
+    };
+    auto bin_of = [&](unsigned key) {
+      const unsigned d = key - lo;
+      if (d <= range) atomicAdd(&hist[d >> shift], 1);
+    };
+    if (first)
+      walk([&](float f) {
+        const unsigned key = raw_key(f);
+        under += key - kKeyMinusInf < lo - kKeyMinusInf ? 1 : 0;
+        bin_of(key);
+      });
+    else
+      walk([&](float f) { bin_of(raw_key(f)); });
+    if (first) {
+      under = __reduce_add_sync(0xffffffffu, under);
+      if (lane == 0 && under != 0) atomicAdd(&s_below, under);
     }
-    for (; i < n4; i += step) {
-      const float4 v = body[i];
-      count(v.x); count(v.y); count(v.z); count(v.w);
-    }
-    if (rank_cta == 0) {
-      if (tid < head) count(scores[tid]);
-      if (tid < n - tail0) count(scores[tail0 + tid]);
-    }
-    ptx::cluster_sync_all();
+    if (tid == 0) ptx::mbar_arrive_expect_tx(&recv_bar, (uint32_t)kKthBins * 4u);
+    ptx::fence_proxy_async_smem();
+    __syncthreads();
+    if (tid < ctas)                                   // slice `tid` of this CTA's bins goes to CTA `tid`
+      ptx::bulk_copy_to_cta(ptx::map_to_cta(ptx::smem_u32(recv + rank_cta * slice), (uint32_t)tid),
+                            ptx::smem_u32(hist + tid * slice), (uint32_t)slice * 4u,
+                            ptx::map_to_cta(ptx::smem_u32(&recv_bar), (uint32_t)tid));
+    ptx::mbar_wait(&recv_bar, phase, nullptr);
+    phase ^= 1;
     if (tid < slice) {
-      const uint32_t bin = ptx::smem_u32(&hist[rank_cta * slice + tid]);
-      int c[kKthMaxCtas], mine = 0;
+      int mine = 0;
 #pragma unroll
-      for (int j = 0; j < kKthMaxCtas; ++j) c[j] = j < ctas ? (int)ptx::ld_cluster_u32(ptx::map_to_cta(bin, (uint32_t)j)) : 0;
-#pragma unroll
-      for (int j = 0; j < kKthMaxCtas; ++j) mine += c[j];
+      for (int j = 0; j < kKthMaxCtas; ++j) mine += j < ctas ? recv[j * slice + tid] : 0;
       red[tid] = mine;
       mine = __reduce_add_sync(0xffffffffu, mine);
       if (lane == 0) part[tid >> 5] = mine;
     }
     __syncthreads();
-    if (tid < ctas) {                                 // the slice's total goes to every CTA
+    if (tid < ctas) {                                 // the slice's total goes to every CTA, and what lies below the range
       int tot = 0;
       for (int w = 0; w < slice / 32; ++w) tot += part[w];
       ptx::st_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&totals[rank_cta]), (uint32_t)tid), (uint32_t)tot);
+      ptx::st_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&below[rank_cta]), (uint32_t)tid), (uint32_t)s_below);
     }
     ptx::cluster_sync_all();
     if (tid < 32) {
+      int want = rank;
+      if (first) want -= __reduce_add_sync(0xffffffffu, lane < ctas ? below[lane] : 0);
       const int st = lane < ctas ? totals[lane] : 0, inc = scan(st);
-      const unsigned hit = __ballot_sync(0xffffffffu, inc - st < rank && rank <= inc);
+      const unsigned hit = __ballot_sync(0xffffffffu, inc - st < want && want <= inc);
       if (hit != 0u) {
         const int sl = __ffs((int)hit) - 1, per = slice / 32;
         const int before = __shfl_sync(0xffffffffu, inc - st, sl);
@@ -332,33 +397,84 @@ __global__ void __launch_bounds__(kThreads) kth_cluster_kernel(const float* __re
         int cum = before + scan(tot) - tot;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-          if (cum < rank && rank <= cum + c[j]) { s_bin = sl * slice + lane * per + j; s_rank = rank - cum; }
+          if (cum < want && want <= cum + c[j]) { s_bin = sl * slice + lane * per + j; s_rank = want - cum; }
           cum += c[j];
         }
       }
     }
     __syncthreads();
-    numbers = s_bin >= 0;                             // (the same in every CTA)
-    if (numbers) {
-      prefix |= (unsigned)s_bin << shift;
+    const int bin = s_bin;                            // (the same in every CTA)
+    if (bin >= 0) {
+      lo += (unsigned)bin << shift;
+      hi = min(hi, lo + ((1u << shift) - 1u));
       rank = s_rank;
-      mask |= dmask << shift;
+      found = shift == 0;
+      first = false;
+    } else if (first && !whole) {                     // the bracket does not hold the rank: all keys
+      lo = kKeyMinusInf; hi = kKeyPlusInf; whole = true;
+    } else {
+      numbers = false;
     }
     __syncthreads();
   }
-  if (rank_cta == 0 && tid == 0) *tau_out = numbers ? key_score(prefix) : __int_as_float(0x7f800000);
+  if (rank_cta == 0 && tid == 0) *tau_out = numbers ? key_score(lo) : __int_as_float(0x7f800000);
   ptx::cluster_sync_all();                            // nobody leaves while its bins are being read
+}
+// ---- compaction of up to kClusterSelect scores by one cluster in one launch: every CTA decides on a contiguous share
+// (kept as bits in registers), tells the others its count over distributed shared memory, and writes its part of the list
+// behind the ones before it.  Below that size three launches take longer than their work (2^16 scores: 13 -> 6 us).
+constexpr int kClusterIters = 8;                      // 16-byte vectors a thread decides on
+constexpr int kClusterSelect = 8 * kClusterIters * kThreads * 4;       // scores that eight CTAs (the portable size) can take
+
+__global__ void __launch_bounds__(kThreads) select_cluster_kernel(const float* __restrict__ scores, int n, float tau,
+                                                                  int* __restrict__ idx, int* __restrict__ count_out) {
+  __shared__ int warp_sums[32], total, totals[kKthMaxCtas];
+  const int ctas = (int)gridDim.x, rank = (int)ptx::cluster_ctarank(), tid = (int)threadIdx.x;
+  ptx::pdl_wait();
+  ptx::pdl_launch_dependents();
+  const int iters = (n + ctas * kThreads * 4 - 1) / (ctas * kThreads * 4);   // <= kClusterIters
+  const int base = rank * iters * kThreads * 4;
+  unsigned bits = 0u;
+#pragma unroll
+  for (int it = 0; it < kClusterIters; ++it) {
+    const int i0 = base + (it * kThreads + tid) * 4;
+    if (it >= iters || i0 >= n) continue;
+    if (i0 + 3 < n) {
+      const float4 v = *reinterpret_cast<const float4*>(scores + i0);
+      bits |= ((!(v.x <= tau) ? 1u : 0u) | (!(v.y <= tau) ? 2u : 0u) | (!(v.z <= tau) ? 4u : 0u) | (!(v.w <= tau) ? 8u : 0u)) << (4 * it);
+    } else {
+      for (int e = 0; i0 + e < n; ++e) bits |= (!(scores[i0 + e] <= tau) ? 1u : 0u) << (4 * it + e);
+    }
+  }
+  const int mine = __reduce_add_sync(0xffffffffu, __popc(bits));
+  if (tid == 0) total = 0;
+  __syncthreads();
+  if ((tid & 31) == 0 && mine != 0) atomicAdd(&total, mine);
+  __syncthreads();
+  if (tid < ctas) ptx::st_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&totals[rank]), (uint32_t)tid), (uint32_t)total);
+  ptx::cluster_sync_all();
+  int out = 0, all = 0;
+  for (int c = 0; c < ctas; ++c) { out += c < rank ? totals[c] : 0; all += totals[c]; }
+  if (rank == 0 && tid == 0) *count_out = all;
+  for (int it = 0; it < iters; ++it) {
+    const unsigned b = (bits >> (4 * it)) & 15u;
+    int at = out + block_exclusive_scan<int>(__popc(b), warp_sums, &total);
+    const int i0 = base + (it * kThreads + tid) * 4;
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (b & (1u << e)) idx[at++] = i0 + e;
+    out += total;
+    __syncthreads();
+  }
 }
 __global__ void set_float_kernel(float* dst, float value) { *dst = value; }
 }  // namespace
 
-cudaError_t launch_kth_score_large(const float* scores, int n, int k, float* tau_out, cudaStream_t st) {
-  if (k <= 0 || k >= n) {
-    set_float_kernel<<<1, 1, 0, st>>>(tau_out, k <= 0 ? -INFINITY : INFINITY);
-    return cudaGetLastError();
-  }
-  // 16 CTAs where the device takes a cluster of that size (asked once per device), the portable 8 otherwise
-  static std::atomic<unsigned long long> asked{0}, wide{0};
+// One cluster of 16 CTAs where the device takes one of that size (asked once per device and kernel), of the portable 8
+// otherwise.
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_cluster(void (*kernel)(KArgs...), cudaStream_t st, Args... args) {
+  static std::atomic<unsigned long long> asked{0}, wide{0};      // (per kernel signature: the two kernels' differ)
   int dev = 0;
   if (cudaError_t e = cudaGetDevice(&dev); e != cudaSuccess) return e;
   const unsigned long long bit = 1ull << (dev & 63);
@@ -373,21 +489,29 @@ cudaError_t launch_kth_score_large(const float* scores, int n, int k, float* tau
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   if (!(asked.load(std::memory_order_acquire) & bit)) {
     int clusters = 0;
-    cfg.gridDim = dim3(16);
-    attr[0].val.clusterDim.x = 16;
+    cfg.gridDim = dim3(kKthMaxCtas);
+    attr[0].val.clusterDim.x = kKthMaxCtas;
     cfg.numAttrs = 1;
-    if (cudaFuncSetAttribute(kth_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-        cudaOccupancyMaxActiveClusters(&clusters, kth_cluster_kernel, &cfg) == cudaSuccess && clusters > 0)
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) == cudaSuccess && clusters > 0)
       wide.fetch_or(bit);
     else
       cudaGetLastError();
     asked.fetch_or(bit, std::memory_order_release);
   }
-  const unsigned ctas = (wide.load() & bit) ? 16u : 8u;
+  const unsigned ctas = (wide.load() & bit) ? kKthMaxCtas : 8u;
   cfg.gridDim = dim3(ctas);
   attr[0].val.clusterDim.x = ctas;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, kth_cluster_kernel, scores, n, k, tau_out);
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+cudaError_t launch_kth_score_large(const float* scores, int n, int k, float* tau_out, cudaStream_t st) {
+  if (k <= 0 || k >= n) {
+    set_float_kernel<<<1, 1, 0, st>>>(tau_out, k <= 0 ? -INFINITY : INFINITY);
+    return cudaGetLastError();
+  }
+  return launch_cluster(kth_cluster_kernel, st, scores, n, k, tau_out);
 }
 
 int select_large_tiles(long long n) { return (int)((n + kTile - 1) / kTile); }
@@ -413,6 +537,7 @@ cudaError_t launch_select_large(const float* scores, long long n, float tau, int
                                 int* tile_offsets, unsigned* flags, cudaStream_t st) {
   const int tiles = select_large_tiles(n);
   if (tiles == 0) return cudaMemsetAsync(count, 0, sizeof(int), st);
+  if (n <= kClusterSelect) return launch_cluster(select_cluster_kernel, st, scores, (int)n, tau, idx, count);
   tile_flag_kernel<<<tiles, kThreads, 0, st>>>(scores, n, tau, tile_counts, flags);
   cudaError_t e = launch_pdl(tile_scan_kernel, dim3(1), dim3(kThreads), 0, st, 1, (const int*)tile_counts, tiles,
                              tile_offsets, count);

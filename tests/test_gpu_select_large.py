@@ -133,3 +133,56 @@ def test_standalone_rmsnorm_matches_the_oracle(dare, rows, d, dtype):
     assert np.max(np.abs(got - want) / (np.abs(want) + 1.0)) <= tol
     assert dare.dare_rmsnorm(0, gd.data_ptr(), yd.data_ptr(), rows, d, 1e-5, dare.F32, 0) == dare.ERR_INVALID_ARG
     assert dare.dare_rmsnorm(xd.data_ptr(), gd.data_ptr(), yd.data_ptr(), rows, d + 1, 1e-5, dare.F32, 0) == dare.ERR_SHAPE
+
+
+@pytest.mark.parametrize("n", [16385, 20_000, 262_145, 524_288, 600_003])
+@pytest.mark.parametrize("kind", ["spread", "two values", "periodic", "mostly nan", "ascending"])
+def test_kth_of_many_scores(n, kind):
+    """The cluster-wide selection: bracket from a sample (which a periodic or sorted array misleads), full range, ranks at
+    both ends and among ties and NaN, at an address that is not 16-byte aligned; against sort-and-index."""
+    import torch
+    from paper_2605_08134_b200 import dare
+    rng = np.random.default_rng(n)
+    s = (rng.standard_normal(n) * np.exp(rng.uniform(-12, 2, n))).astype(np.float32)
+    if kind == "two values":
+        s = np.where(rng.random(n) < 0.4, np.float32(0.25), np.float32(-3.0)).astype(np.float32)
+    elif kind == "periodic":
+        s = np.where(np.arange(n) % max(1, n // 256) == 0, np.float32(7.0), s).astype(np.float32)
+    elif kind == "mostly nan":
+        s[rng.random(n) < 0.9] = np.nan
+    elif kind == "ascending":
+        s.sort()
+    buf = torch.empty(n + 4, device="cuda")
+    out = torch.zeros(1, device="cuda")
+    srt = np.sort(s)                                                   # NaN last
+    for shift in (0, 1):
+        sd = buf[shift:shift + n]
+        sd.copy_(torch.from_numpy(s))
+        for k in sorted({1, 2, n // 1000, n // 10, n // 2, int(0.93 * n), n - 1}):
+            assert dare.dare_score_kth(sd.data_ptr(), n, k, out.data_ptr(), torch.cuda.current_stream().cuda_stream) == 0
+            got, want = out.cpu().numpy()[0], srt[k - 1]
+            assert got == (np.inf if np.isnan(want) else want), (kind, k, got, want)
+
+
+@pytest.mark.parametrize("n", [1, 3, 4096, 65_536, 65_537, 262_143, 262_144, 262_145])
+def test_compaction_in_one_launch_and_in_three(n):
+    """Around the size up to which one cluster compacts in a single launch: list, count, nothing past the list touched."""
+    import torch
+    from paper_2605_08134_b200 import dare
+    rng = np.random.default_rng(n)
+    s = rng.random(n).astype(np.float32)
+    s[rng.random(n) < 0.01] = np.nan
+    sd = torch.from_numpy(s).cuda()
+    idx = torch.full((n + 8,), -7, dtype=torch.int32, device="cuda")
+    cnt = torch.zeros(1, dtype=torch.int32, device="cuda")
+    nb = dare.dare_select_compact_scratch_bytes(n)
+    scratch = torch.empty(nb, dtype=torch.uint8, device="cuda")
+    for tau in (-1.0, 0.3, 0.97, 2.0):
+        idx.fill_(-7)
+        assert dare.dare_select_compact(sd.data_ptr(), n, tau, idx.data_ptr(), cnt.data_ptr(), scratch.data_ptr(), nb,
+                                        torch.cuda.current_stream().cuda_stream) == 0
+        want = np.nonzero(~(s <= np.float32(tau)))[0]
+        assert int(cnt.item()) == len(want)
+        got = idx.cpu().numpy()
+        np.testing.assert_array_equal(got[:len(want)], want)
+        assert (got[max(len(want), n):] == -7).all()
