@@ -4,16 +4,19 @@
 // The result rows are written straight into the attention-output cache at their cache rows; rows that are not
 // computed keep their cached value (Alg. 2 lines 9-10).
 //
-// One CTA = one head x one tile of up to 128 query rows of one sequence, walking the keys in blocks of 128.  The key
+// One CTA = one head x one tile of up to 128 query rows of one sequence, walking the keys in blocks of 64.  The key
 // blocks alternate between two independent streams (even blocks: stream 0, odd blocks: stream 1); each stream has
 // its own running maximum, row sum and accumulator, and the two are merged at the end like the partials of a key
 // split.  While one stream's softmax warps are busy on the special-function unit the other stream's are moving
 // data, so both the tensor pipe and the exponentials stay busy.  Per stream:
-//   warp s       TMA producer: K block and V block of the cache (two 64-column boxes each, 128-byte swizzle)
-//   warp 2+s     one lane issues S = Q K^T (M128 N128 K16 x 8, both operands in shared memory) and O += P V
-//                (M128 N128 K16 x 8, P read from tensor memory, V from shared memory as an MN-major operand)
+//   warp s       TMA producer: K and V blocks of the cache (64-column boxes, 128-byte swizzle) into rings of three
+//   warp 2+s     one lane issues S = Q K^T (M128 N64 K16, both operands in shared memory) and O += P V (K = 64 keys, P
+//                read from tensor memory, V from shared memory as an MN-major operand).  Two score buffers: S(j + 1)
+//                is computed while the softmax warps are on S(j), so they go from one block to the next without waiting
+//                for the tensor core (blocks of 128 with one score buffer: 2.5 us a block and stream, most of it the
+//                chain S -> softmax -> P V -> S)
 //   warps 4+4s.. four softmax warps, thread <-> query row: reads its row of S from tensor memory, exponentiates, and
-//                writes P as bf16 over the first 64 columns of S (two keys per 32-bit column, the layout of a
+//                writes P as bf16 over the first 32 columns of S (two keys per 32-bit column, the layout of a
 //                tensor-memory A operand), so P never passes through shared memory.  O accumulates in tensor
 //                memory; it is rescaled in place only when the running maximum has grown by more than 2^8 (the
 //                exponentials are taken against the older maximum until then, which changes nothing in exact
@@ -37,7 +40,9 @@ using namespace ptx;
 namespace {
 
 constexpr int BQ = 128;    // query rows per CTA
-constexpr int BKV = 128;   // keys per block
+constexpr int BKV = 128;   // keys per block of the two-tile kernel
+constexpr int BK1 = 64;    // ... of the one-tile kernel
+constexpr int kRing1 = 3;  // its K and V blocks per stream
 // A CTA takes all of its SM's tensor memory, so two must never share an SM: the second would wait for the first, and
 // with clusters on both (key split) each could wait for the other.  Shared memory keeps them apart: more than half.
 constexpr int one_cta_per_sm(int bytes) { return bytes > 117 * 1024 ? bytes : 117 * 1024; }
@@ -46,14 +51,13 @@ constexpr int one_cta_per_sm(int bytes) { return bytes > 117 * 1024 ? bytes : 11
 template <int HD>
 struct AttnSmem {
   static constexpr int Q_BYTES = BQ * HD * 2;          // HD / 64 64-column chunks of [128 x 128 B]
-  static constexpr int K_BYTES = BKV * HD * 2;         // the same chunks of a key block
-  static constexpr int V_BYTES = BKV * HD * 2;
+  static constexpr int K_BYTES = BK1 * HD * 2;         // the same chunks of a key block
+  static constexpr int V_BYTES = BK1 * HD * 2;
   static constexpr int Q_OFF = 0;
-  static constexpr int K_OFF = Q_OFF + Q_BYTES;        // one buffer per stream
-  static constexpr int V_OFF = K_OFF + 2 * K_BYTES;    // two buffers per stream: V(j) is wanted last in a block and
-                                                       // its buffer is released last, so one buffer leaves no slack
-  static constexpr int BAR_OFF = V_OFF + 4 * V_BYTES;
-  static constexpr int TOTAL = one_cta_per_sm(BAR_OFF + 256 + 1024);
+  static constexpr int K_OFF = Q_OFF + Q_BYTES;        // a ring per stream
+  static constexpr int V_OFF = K_OFF + 2 * kRing1 * K_BYTES;
+  static constexpr int BAR_OFF = V_OFF + 2 * kRing1 * V_BYTES;
+  static constexpr int TOTAL = one_cta_per_sm(BAR_OFF + 512 + 1024);
   // merge of the two streams: a stream's running maxima [128] and row sums [128] go to its first V buffer, idle
   // after its last product
   // after the key loop the operand buffers are idle; the merge of a key split reuses them:
@@ -84,18 +88,19 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
 
 constexpr int kThreads = 384;
 constexpr int kSoftmaxThreads = 256;
-// S of stream 0 / 1: columns [0, 128) / [128, 256), P over the first 64 of them; O: [256, 256 + HD) / behind it
+// Scores of stream 0 / 1: columns [0, 128) / [128, 256), two buffers of 64 each, P over the first 32 of a buffer; O:
+// [256, 256 + HD) / behind it
 constexpr uint32_t kTmemCols = 512;
 constexpr int kPairMinDense = 128;      // dense launches with longer windows take the two-tile kernel
 constexpr int kPairMinSparse = 1024;    // row-sparse launches from this window length on
 constexpr float kRescaleStep = 8.f;     // log2 of the growth of the running maximum that triggers a rescale of O
 
-// The HD / 64 chunks of a key (or value) block, 64 columns of 128 rows each, counted on one barrier.
-template <int HD>
+// The HD / 64 chunks of a key (or value) block, 64 columns of KEYS rows each, counted on one barrier.
+template <int HD, int KEYS>
 __device__ __forceinline__ void load_block(uint8_t* dst, const CUtensorMap* tm, int h, int row, uint64_t* bar) {
-  mbar_arrive_expect_tx(bar, BKV * HD * 2);
+  mbar_arrive_expect_tx(bar, KEYS * HD * 2);
 #pragma unroll
-  for (int c = 0; c < HD / 64; ++c) tma_load_2d(dst + c * (BKV * 128), tm, h * HD + c * 64, row, bar);
+  for (int c = 0; c < HD / 64; ++c) tma_load_2d(dst + c * (KEYS * 128), tm, h * HD + c * 64, row, bar);
 }
 
 }  // namespace
@@ -110,16 +115,15 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S::BAR_OFF);
-  // one of each per stream
-  uint64_t* k_full = bars;          // [2]
-  uint64_t* k_empty = bars + 2;     // [2]
-  uint64_t* s_full = bars + 4;      // [2]
-  uint64_t* p_full = bars + 6;      // [2]
-  uint64_t* o_full = bars + 8;      // [2]
-  uint64_t* v_full = bars + 10;     // [2 streams][2 buffers]
-  uint64_t* v_empty = bars + 14;    // [2 streams][2 buffers]
-  uint64_t* recv_bar = bars + 18;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 19);
+  uint64_t* k_full = bars;                     // [2 streams][ring]
+  uint64_t* k_empty = k_full + 2 * kRing1;
+  uint64_t* v_full = k_empty + 2 * kRing1;
+  uint64_t* v_empty = v_full + 2 * kRing1;
+  uint64_t* s_full = v_empty + 2 * kRing1;     // [2 streams][2 score buffers]
+  uint64_t* p_full = s_full + 4;               // [2 streams][2 score buffers]
+  uint64_t* o_full = p_full + 4;               // [2 streams][2]: product j signals o_full[stream][j & 1]
+  uint64_t* recv_bar = o_full + 4;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(recv_bar + 1);
 
   // the warp index through a shuffle, so that the compiler knows it (and every role decision and shared-memory
   // descriptor derived from it) to be uniform over the warp
@@ -166,10 +170,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     if (__ldcg(p.batch_off + b) + tile * BQ >= __ldcg(p.batch_off + b + 1)) return;
   }
   if (threadIdx.x == 0) {
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < 2 * kRing1; ++i) {
       mbar_init(&k_full[i], 1); mbar_init(&k_empty[i], 1);
-      mbar_init(&v_full[2 * i], 1); mbar_init(&v_full[2 * i + 1], 1);
-      mbar_init(&v_empty[2 * i], 1); mbar_init(&v_empty[2 * i + 1], 1);
+      mbar_init(&v_full[i], 1); mbar_init(&v_empty[i], 1);
+    }
+    for (int i = 0; i < 4; ++i) {
       mbar_init(&s_full[i], 1); mbar_init(&o_full[i], 1);
       mbar_init(&p_full[i], kSoftmaxThreads / 64);     // one arrival per softmax warp of the stream
     }
@@ -208,22 +213,20 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       active = __syncthreads_or(mine) != 0;
     }
   }
-  const int n_blocks_all = (g.kv_len + BKV - 1) / BKV;
+  const int n_blocks_all = (g.kv_len + BK1 - 1) / BK1;
   const int n_blocks = n_blocks_all > z ? (n_blocks_all - z + ksplit - 1) / ksplit : 0;   // blocks z, z + ksplit, ...
   const int kv_row0 = b * g.max_seq;
-  // The first K and V block of each stream start as soon as the projection is complete, by the thread that
+  // The first K and V blocks of each stream start as soon as the projection is complete, by the thread that
   // initialised the barriers, so that they are in flight while the Q tile is gathered.
   if (warp == 0) {
     pdl_wait();
     pdl_launch_dependents();
   }
   if (threadIdx.x == 0 && active) {
-    for (int s2 = 0; s2 < 2 && s2 < n_blocks; ++s2) {
-      const int row = kv_row0 + (z + s2 * ksplit) * BKV;
-      uint8_t* kd = smem + S::K_OFF + s2 * S::K_BYTES;
-      uint8_t* vd = smem + S::V_OFF + 2 * s2 * S::V_BYTES;
-      load_block<HD>(kd, &tm_k, h, row, &k_full[s2]);
-      load_block<HD>(vd, &tm_v, h, row, &v_full[2 * s2]);
+    for (int i = 0; i < 2 * kRing1 && i < n_blocks; ++i) {     // local block i: stream i & 1, ring slot i >> 1
+      const int row = kv_row0 + (z + i * ksplit) * BK1, slot = (i & 1) * kRing1 + (i >> 1);
+      load_block<HD, BK1>(smem + S::K_OFF + slot * S::K_BYTES, &tm_k, h, row, &k_full[slot]);
+      load_block<HD, BK1>(smem + S::V_OFF + slot * S::V_BYTES, &tm_v, h, row, &v_full[slot]);
     }
   }
   // ---- Q tile: gathered rows -> shared memory in the K-major 128-byte-swizzled layout (16-byte units), by the
@@ -273,58 +276,60 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   const int st = warp < 4 ? (warp & 1) : ((warp - 4) >> 2);
   const int n_st = (n_blocks - st + 1) / 2;
   const int n_other = n_blocks - n_st;
-  const uint32_t tmem_s = tmem_base + st * BKV, tmem_o = tmem_base + 2 * BKV + st * HD;
+  const uint32_t tmem_s = tmem_base + st * 2 * BK1, tmem_o = tmem_base + 4 * BK1 + st * HD;
   // The producer and issuer warps run their loops converged (every lane polls the barriers); one elected lane
   // issues the copies and the MMAs.  Their operands are then warp-uniform values, which is what those instructions take.
   if (warp < 2) {
-    uint8_t* kd = smem + S::K_OFF + st * S::K_BYTES;
-    for (int j = 1; j < n_st; ++j) {                        // block 0 of the stream was started before the Q gather
-      const int vb = 2 * st + (j & 1);
-      uint8_t* vd = smem + S::V_OFF + vb * S::V_BYTES;
-      const int row = kv_row0 + (z + (2 * j + st) * ksplit) * BKV;
-      mbar_wait(&k_empty[st], (j & 1) ^ 1, p.status);       // S(j-1) = Q K(j-1)^T has been computed
-      if (elect_one()) load_block<HD>(kd, &tm_k, h, row, &k_full[st]);
+    for (int j = kRing1; j < n_st; ++j) {                   // the first blocks of the stream were started before the Q gather
+      const int slot = st * kRing1 + j % kRing1, row = kv_row0 + (z + (2 * j + st) * ksplit) * BK1;
+      const uint32_t freed = ((j / kRing1) & 1) ^ 1;
+      mbar_wait(&k_empty[slot], freed, p.status);           // S(j - kRing1) has been computed
+      if (elect_one()) load_block<HD, BK1>(smem + S::K_OFF + slot * S::K_BYTES, &tm_k, h, row, &k_full[slot]);
       __syncwarp();
-      mbar_wait(&v_empty[vb], ((j >> 1) & 1) ^ 1, p.status);       // O += P(j-2) V(j-2) has been computed
-      if (elect_one()) load_block<HD>(vd, &tm_v, h, row, &v_full[vb]);
+      mbar_wait(&v_empty[slot], freed, p.status);           // O += P(j - kRing1) V(j - kRing1) has been computed
+      if (elect_one()) load_block<HD, BK1>(smem + S::V_OFF + slot * S::V_BYTES, &tm_v, h, row, &v_full[slot]);
       __syncwarp();
     }
   } else if (warp < 4) {
-    constexpr uint32_t idesc_qk = idesc_bf16(BQ, BKV, false);
+    constexpr uint32_t idesc_qk = idesc_bf16(BQ, BK1, false);
     constexpr uint32_t idesc_pv = idesc_bf16(BQ, HD, true);
     const uint64_t q_desc = smem_desc_k_sw128(smem_u32(smem + S::Q_OFF));
-    const uint64_t k_desc = smem_desc_k_sw128(smem_u32(smem + S::K_OFF + st * S::K_BYTES));
-    const uint64_t v_desc0 = smem_desc_mn_sw128(smem_u32(smem + S::V_OFF + 2 * st * S::V_BYTES), BKV * 128);
+    const uint64_t k_desc0 = smem_desc_k_sw128(smem_u32(smem + S::K_OFF + st * kRing1 * S::K_BYTES));
+    const uint64_t v_desc0 = smem_desc_mn_sw128(smem_u32(smem + S::V_OFF + st * kRing1 * S::V_BYTES), BK1 * 128);
     auto issue_qk = [&](int j) {
-      mbar_wait(&k_full[st], j & 1, p.status);
+      const int rs = j % kRing1;
+      mbar_wait(&k_full[st * kRing1 + rs], (j / kRing1) & 1, p.status);
       tc_fence_after();
       if (elect_one()) {
+        const uint64_t k_desc = k_desc0 + (uint64_t)(rs * (S::K_BYTES >> 4));
 #pragma unroll
         for (int kk = 0; kk < HD / 16; ++kk)
-          umma_ss(tmem_s, q_desc + (((kk >> 2) * (BQ * 128) + (kk & 3) * 32) >> 4),
-                  k_desc + (((kk >> 2) * (BKV * 128) + (kk & 3) * 32) >> 4), idesc_qk, kk != 0 ? 1u : 0u);
-        umma_commit(&s_full[st]);
-        umma_commit(&k_empty[st]);
+          umma_ss(tmem_s + (j & 1) * BK1, q_desc + (((kk >> 2) * (BQ * 128) + (kk & 3) * 32) >> 4),
+                  k_desc + (((kk >> 2) * (BK1 * 128) + (kk & 3) * 32) >> 4), idesc_qk, kk != 0 ? 1u : 0u);
+        umma_commit(&s_full[2 * st + (j & 1)]);
+        umma_commit(&k_empty[st * kRing1 + rs]);
       }
       __syncwarp();
     };
     if (n_st > 0) issue_qk(0);
+    if (n_st > 1) issue_qk(1);
     for (int j = 0; j < n_st; ++j) {
-      mbar_wait(&p_full[st], j & 1, p.status);      // P(j) has replaced S(j) in tensor memory
-      const int vb = 2 * st + (j & 1);
-      mbar_wait(&v_full[vb], (j >> 1) & 1, p.status);
+      const int rs = j % kRing1;
+      mbar_wait(&p_full[2 * st + (j & 1)], (j >> 1) & 1, p.status);      // P(j) has replaced S(j) in tensor memory
+      mbar_wait(&v_full[st * kRing1 + rs], (j / kRing1) & 1, p.status);
       tc_fence_after();
       if (elect_one()) {
-        const uint64_t v_desc = v_desc0 + (uint64_t)((j & 1) * (S::V_BYTES >> 4));
+        const uint64_t v_desc = v_desc0 + (uint64_t)(rs * (S::V_BYTES >> 4));
 #pragma unroll
-        for (int ks = 0; ks < BKV / 16; ++ks)       // 16 keys of P = 8 columns
-          umma_ts(tmem_o, tmem_s + ks * 8, v_desc + ((ks * (16 * 128)) >> 4), idesc_pv, (j | ks) != 0 ? 1u : 0u);
-        umma_commit(&o_full[st]);
-        umma_commit(&v_empty[vb]);
+        for (int ks = 0; ks < BK1 / 16; ++ks)       // 16 keys of P = 8 columns
+          umma_ts(tmem_o, tmem_s + (j & 1) * BK1 + ks * 8, v_desc + ((ks * (16 * 128)) >> 4), idesc_pv,
+                  (j | ks) != 0 ? 1u : 0u);
+        umma_commit(&o_full[2 * st + (j & 1)]);
+        umma_commit(&v_empty[st * kRing1 + rs]);
       }
       __syncwarp();
-      // the tensor pipe runs MMAs in issue order: the next scores overwrite P(j) only after the product above read it
-      if (j + 1 < n_st) issue_qk(j + 1);
+      // the tensor pipe runs MMAs in issue order: S(j + 2) overwrites P(j) only after the product above read it
+      if (j + 2 < n_st) issue_qk(j + 2);
     }
   } else {
     // ---- softmax of this stream's blocks: thread <-> query row
@@ -341,51 +346,24 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     // and O are whatever the score buffer held, belong to no token and are never stored
     const bool warp_has_rows = quarter * 32 < rows_valid;
     for (int j = 0; j < n_st; ++j) {
-      mbar_wait(&s_full[st], j & 1, p.status);
+      const uint32_t sbuf = tmem_s + (j & 1) * BK1 + lane_addr;         // scores of block j, then its P
+      mbar_wait(&s_full[2 * st + (j & 1)], (j >> 1) & 1, p.status);
       tc_fence_after();
       if (dbg && j == 0 && threadIdx.x == 128) p.debug[2] = globaltimer_ns();
       if (!warp_has_rows) {
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&p_full[st]);
+        if (lane == 0) mbar_arrive(&p_full[2 * st + (j & 1)]);
         continue;
       }
-      const int key0 = (z + (2 * j + st) * ksplit) * BKV;
-      const int n_keys = min(BKV, g.kv_len - key0);   // the last block may be ragged: keys past kv_len do not exist
-      // O and the row sum move to a new maximum only when it grew by more than kRescaleStep (in log2 units); the
-      // product that last wrote O has to be complete before O is rescaled in place
-      auto settle_max = [&](float m_new) {
-        if (j == 0) {
-          m = m_new;
-        } else {
-          const bool grow = (m_new - m) * c > kRescaleStep;
-          if (__any_sync(0xffffffffu, grow)) {
-            const float alpha = grow ? fast_exp2((m - m_new) * c) : 1.f;
-            if (grow) { m = m_new; l *= alpha; }
-            mbar_wait(&o_full[st], (j - 1) & 1, p.status);
-            tc_fence_after();
-#pragma unroll 1
-            for (int ch = 0; ch < HD / 32; ++ch) {
-              float o[32];
-              tmem_ld_32x32(tmem_o + lane_addr + ch * 32, o);
-#pragma unroll
-              for (int i = 0; i < 32; ++i) o[i] *= alpha;
-              tmem_st_32x32(tmem_o + lane_addr + ch * 32, o);
-            }
-          }
-        }
-      };
-      float sum4[4] = {0.f, 0.f, 0.f, 0.f};
-      // the row of S: four loads in flight together
-      float v[128];
-      tmem_ld_32x32_nowait(tmem_s + lane_addr, v);
-      tmem_ld_32x32_nowait(tmem_s + lane_addr + 32, v + 32);
-      tmem_ld_32x32_nowait(tmem_s + lane_addr + 64, v + 64);
-      tmem_ld_32x32_nowait(tmem_s + lane_addr + 96, v + 96);
+      const int n_keys = g.kv_len - (z + (2 * j + st) * ksplit) * BK1;   // the last block may be ragged: keys past kv_len do not exist
+      float v[BK1];
+      tmem_ld_32x32_nowait(sbuf, v);
+      tmem_ld_32x32_nowait(sbuf + 32, v + 32);
       tmem_ld_wait();
-      if (n_keys < BKV) {
+      if (n_keys < BK1) {
 #pragma unroll
-        for (int i = 0; i < 128; ++i)
+        for (int i = 0; i < BK1; ++i)
           if (i >= n_keys) v[i] = -INFINITY;
       }
       // row maximum: four independent chains of three-input maxima
@@ -393,20 +371,41 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
 #pragma unroll
       for (int k = 0; k < 4; ++k) mx4[k] = fmaxf(v[k], v[4 + k]);
 #pragma unroll
-      for (int i = 8; i < 128; i += 8) {
+      for (int i = 8; i < BK1; i += 8) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) mx4[k] = fmax3(mx4[k], v[i + k], v[i + 4 + k]);
       }
-      settle_max(fmax3(m, fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])));
+      const float m_new = fmax3(m, fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
+      // O and the row sum move to a new maximum only when it grew by more than kRescaleStep (in log2 units); the
+      // product that last wrote O has to be complete before O is rescaled in place.  (The softmax warps may be two
+      // products ahead of the tensor core, and a parity wait tells apart only two consecutive phases: hence one barrier
+      // per parity of j, each of which these warps are at most one phase behind.)
+      if (j == 0) {
+        m = m_new;
+      } else {
+        const bool grow = (m_new - m) * c > kRescaleStep;
+        if (__any_sync(0xffffffffu, grow)) {
+          const float alpha = grow ? fast_exp2((m - m_new) * c) : 1.f;
+          if (grow) { m = m_new; l *= alpha; }
+          mbar_wait(&o_full[2 * st + ((j - 1) & 1)], ((j - 1) >> 1) & 1, p.status);
+          tc_fence_after();
+#pragma unroll 1
+          for (int ch = 0; ch < HD / 32; ++ch) {
+            float o[32];
+            tmem_ld_32x32(tmem_o + lane_addr + ch * 32, o);
+#pragma unroll
+            for (int i = 0; i < 32; ++i) o[i] *= alpha;
+            tmem_st_32x32(tmem_o + lane_addr + ch * 32, o);
+          }
+        }
+      }
       // exponentials against m (masked keys: 2^-inf = 0) and the row sum, the scaling and the sum two keys per
       // instruction (packed fp32)
       const float2 c2 = make_float2(c, c), nmc2 = make_float2(-m * c, -m * c);
       float2 sum2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-      // P as bf16 over the first 64 columns of this row of S: column i = keys (2i, 2i+1); packed as it is produced,
-      // so that the scores leave the register file pair by pair
-      float pk[64];
+      float pk[BK1 / 2];                            // P as bf16: column i = keys (2i, 2i+1)
 #pragma unroll
-      for (int i = 0; i < 128; i += 2) {
+      for (int i = 0; i < BK1; i += 2) {
         float2 e = __ffma2_rn(make_float2(v[i], v[i + 1]), c2, nmc2);
         e.x = fast_exp2(e.x);
         e.y = fast_exp2(e.y);
@@ -414,25 +413,22 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         __nv_bfloat162 h2 = __floats2bfloat162_rn(e.x, e.y);
         pk[i >> 1] = __uint_as_float(*reinterpret_cast<uint32_t*>(&h2));
       }
-      sum4[0] = sum2[0].x; sum4[1] = sum2[0].y; sum4[2] = sum2[1].x; sum4[3] = sum2[1].y;
-      tmem_st_32x32_nowait(tmem_s + lane_addr, pk);
-      tmem_st_32x32_nowait(tmem_s + lane_addr + 32, pk + 32);
+      tmem_st_32x32_nowait(sbuf, pk);
       tmem_st_wait();
-      l += (sum4[0] + sum4[1]) + (sum4[2] + sum4[3]);
+      l += (sum2[0].x + sum2[0].y) + (sum2[1].x + sum2[1].y);
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&p_full[st]);
+      if (lane == 0) mbar_arrive(&p_full[2 * st + (j & 1)]);
     }
-    if (n_st > 0) {
-      mbar_wait(&o_full[st], (n_st - 1) & 1, p.status);
-      tc_fence_after();
-    }
+    for (int j = max(0, n_st - 2); j < n_st; ++j)              // the last two products
+      mbar_wait(&o_full[2 * st + (j & 1)], (j >> 1) & 1, p.status);
+    tc_fence_after();
     if (dbg && threadIdx.x == 128) p.debug[3] = globaltimer_ns();
     // (a warp without rows has nothing to merge or store, but takes part in the barrier)
     // ---- merge the two streams: thread (stream st, row r) finishes its half of the row's columns
     constexpr int HC = HD / 2;
-    float* stat_mine = reinterpret_cast<float*>(smem + S::V_OFF + 2 * st * S::V_BYTES);
-    const float* stat_other = reinterpret_cast<const float*>(smem + S::V_OFF + 2 * (st ^ 1) * S::V_BYTES);
+    float* stat_mine = reinterpret_cast<float*>(smem + S::V_OFF + kRing1 * st * S::V_BYTES);
+    const float* stat_other = reinterpret_cast<const float*>(smem + S::V_OFF + kRing1 * (st ^ 1) * S::V_BYTES);
     stat_mine[r] = m;
     stat_mine[BQ + r] = l;
     tc_fence_before();
@@ -445,7 +441,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     const float w_other = n_other > 0 ? fast_exp2((m_o - m_all) * c) : 0.f;
     const float l_row = w_mine * l + w_other * l_o;
     const uint32_t t_mine = tmem_o + lane_addr + st * HC;
-    const uint32_t t_other = tmem_base + 2 * BKV + (st ^ 1) * HD + lane_addr + st * HC;
+    const uint32_t t_other = tmem_base + 4 * BK1 + (st ^ 1) * HD + lane_addr + st * HC;
     float acc[HC];
 #pragma unroll
     for (int cgrp = 0; cgrp < HC / 32; ++cgrp) {
@@ -710,8 +706,8 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
     const int slot = i & 1, row = kv_row0 + i * BKV;
     uint8_t* kd = smem + S::K_OFF + slot * S::KV_BYTES;
     uint8_t* vd = smem + S::V_OFF + slot * S::KV_BYTES;
-    load_block<HD>(kd, &tm_k, h, row, &k_full[slot]);
-    load_block<HD>(vd, &tm_v, h, row, &v_full[slot]);
+    load_block<HD, BKV>(kd, &tm_k, h, row, &k_full[slot]);
+    load_block<HD, BKV>(vd, &tm_v, h, row, &v_full[slot]);
   };
   // the first two key blocks start as soon as the projection is complete, by the thread that initialised the
   // barriers: in flight during the Q gather
@@ -961,7 +957,7 @@ bool pick_form(const StepGeom& g, bool row_sparse, int* ksplit_out) {
   // CTAs expected to have work: every row tile (dense) or one row tile per sequence (row-sparse, small refresh set)
   const int expected = g.n_heads * g.batch * (row_sparse ? 1 : tps);
   const int n_blocks = (g.kv_len + BKV - 1) / BKV;
-  // The merge of a key split costs about as much as four key blocks (three cluster-wide barriers and the copies), so
+  // (blocks of 128 keys here.)  The merge of a key split costs about as much as four key blocks (three cluster-wide barriers and the copies), so
   // the keys are split only when every CTA still keeps at least four blocks.
   int ksplit = 1;
   while (ksplit < 4 && expected * ksplit * 2 <= 160 && ksplit * 2 * 4 <= n_blocks) ksplit *= 2;
@@ -981,8 +977,7 @@ bool attention_tc_two_tiles(const StepGeom& g, bool row_sparse) {
 }
 
 template <int HD>
-static cudaError_t launch_attention_hd(const CUtensorMap& tm_k, const CUtensorMap& tm_v, const AttnParams& p,
-                                       cudaStream_t st) {
+static cudaError_t launch_attention_hd(const KvMaps& maps, const AttnParams& p, cudaStream_t st) {
   static std::atomic<unsigned long long> attr_one{0}, attr_split{0}, attr_pair{0};
   if (cudaError_t e = ensure_dyn_smem(attn_tc_kernel<HD, false>, AttnSmem<HD>::TOTAL, attr_one); e != cudaSuccess) return e;
   if (cudaError_t e = ensure_dyn_smem(attn_tc_kernel<HD, true>, AttnSmem<HD>::TOTAL, attr_split); e != cudaSuccess) return e;
@@ -994,16 +989,16 @@ static cudaError_t launch_attention_hd(const CUtensorMap& tm_k, const CUtensorMa
   if (pair) {
     dim3 grid(p.g.n_heads, p.g.batch * tps2, 1);
     if (grid.y == 0) return cudaSuccess;
-    return launch_pdl(attn_pair_kernel<HD>, grid, dim3(kThreads), PairSmem<HD>::TOTAL, st, 1, tm_k, tm_v, p);
+    return launch_pdl(attn_pair_kernel<HD>, grid, dim3(kThreads), PairSmem<HD>::TOTAL, st, 1, maps.k128, maps.v128, p);
   }
   dim3 grid(p.g.n_heads, p.g.batch * tps, ksplit);
   if (grid.y == 0) return cudaSuccess;
-  return launch_pdl(ksplit > 1 ? attn_tc_kernel<HD, true> : attn_tc_kernel<HD, false>, grid, dim3(kThreads), AttnSmem<HD>::TOTAL, st, ksplit, tm_k, tm_v, p);
+  return launch_pdl(ksplit > 1 ? attn_tc_kernel<HD, true> : attn_tc_kernel<HD, false>, grid, dim3(kThreads), AttnSmem<HD>::TOTAL, st, ksplit, maps.k64,
+                    maps.v64, p);
 }
 
-cudaError_t launch_attention_tc(const CUtensorMap& tm_k, const CUtensorMap& tm_v, const AttnParams& p,
-                                cudaStream_t st) {
-  return p.g.head_dim == 64 ? launch_attention_hd<64>(tm_k, tm_v, p, st) : launch_attention_hd<128>(tm_k, tm_v, p, st);
+cudaError_t launch_attention_tc(const KvMaps& maps, const AttnParams& p, cudaStream_t st) {
+  return p.g.head_dim == 64 ? launch_attention_hd<64>(maps, p, st) : launch_attention_hd<128>(maps, p, st);
 }
 
 }  // namespace dare

@@ -13,7 +13,7 @@ struct TcState {
   CUtensorMap w_q, w_k, w_v, w_o;          // weights, box 64 x 256 rows
   CUtensorMap w_k128, w_v128, w_q128, w_o128;   // weights, box 64 x 128 rows
   CUtensorMap w_q64, w_o64;                // weights, box 64 x 64 rows (narrow pair tiles)
-  CUtensorMap kc64, vc64;                  // K/V caches as attention operands, box 64 x 128 rows (keys)
+  KvMaps kv;                               // K/V caches as attention operands
 };
 
 namespace {
@@ -82,8 +82,9 @@ dare_status_t tc_create(dare_layer* L) {
             make_map(&s->w_o, L->w.w_o, d, d, 256) && make_map(&s->w_k128, L->w.w_k, d, d, 128) &&
             make_map(&s->w_v128, L->w.w_v, d, d, 128) && make_map(&s->w_q128, L->w.w_q, d, d, 128) &&
             make_map(&s->w_o128, L->w.w_o, d, d, 128) && make_map(&s->w_q64, L->w.w_q, d, d, 64) &&
-            make_map(&s->w_o64, L->w.w_o, d, d, 64) && make_map(&s->kc64, L->buf.kc, Tm, d, 128) &&
-            make_map(&s->vc64, L->buf.vc, Tm, d, 128);
+            make_map(&s->w_o64, L->w.w_o, d, d, 64) && make_map(&s->kv.k128, L->buf.kc, Tm, d, 128) &&
+            make_map(&s->kv.v128, L->buf.vc, Tm, d, 128) && make_map(&s->kv.k64, L->buf.kc, Tm, d, 64) &&
+            make_map(&s->kv.v64, L->buf.vc, Tm, d, 64);
   if (!ok) { delete s; return DARE_ERR_CUDA; }
   L->tc = s;
   return DARE_OK;
@@ -286,12 +287,12 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
       if (one_launch) { p.dense_from = gate_o; p.dense_mask = B.delta; }
       else p.gate_hi = gate_o;
     }
-    e = launch_attention_tc(S.kc64, S.vc64, p, st); ++launches;
+    e = launch_attention_tc(S.kv, p, st); ++launches;
     if (both_forms && !one_launch && e == cudaSuccess) {
       AttnParams pd = p;
       pd.idx = nullptr; pd.batch_off = nullptr; pd.debug = nullptr;
       pd.gate_lo = gate_o; pd.gate_hi = 1 << 30; pd.store_mask = B.delta;
-      e = launch_attention_tc(S.kc64, S.vc64, pd, st); ++launches;
+      e = launch_attention_tc(S.kv, pd, st); ++launches;
     }
     if (e != cudaSuccess) return DARE_ERR_CUDA;
   }

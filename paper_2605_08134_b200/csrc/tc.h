@@ -108,8 +108,9 @@ struct AttnParams {
 // does a launch of this geometry take the kernel with two query tiles per CTA?
 bool attention_tc_two_tiles(const StepGeom& g, bool row_sparse);
 
-cudaError_t launch_attention_tc(const CUtensorMap& tm_k, const CUtensorMap& tm_v, const AttnParams& p,
-                                cudaStream_t st);
+// K and V caches as attention operands: boxes of 64 columns x 128 or 64 rows (keys).
+struct KvMaps { CUtensorMap k128, v128, k64, v64; };
+cudaError_t launch_attention_tc(const KvMaps& maps, const AttnParams& p, cudaStream_t st);
 
 // grid = (n_tiles of bn columns, m_tiles of 128 rows, splits of the reduction dimension = cluster size: 1, 2, or 4 with
 // bn = 128);
