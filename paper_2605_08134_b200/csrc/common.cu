@@ -289,12 +289,12 @@ constexpr int kKthPerThread = kKthInCta / 1024;
 // At most kKthCount tokens: every token's rank is counted instead, against all keys in shared memory (1024 / n threads to
 // a token), which is one pass with one barrier on each side (64 tokens: selection 6.0 -> 3.5 us).
 constexpr int kKthCount = 512;
-__device__ float kth_by_count(const float* __restrict__ scores, int n, int k) {
+__device__ float kth_by_count(float score, int n, int k) {      // score: thread t's is token t's
   __shared__ __align__(16) unsigned keys[kKthCount];
   __shared__ float s_tau;
   if (k <= 0 || k >= n) return __int_as_float(k <= 0 ? 0xff800000 : 0x7f800000);
   const int tid = threadIdx.x;
-  if (tid < kKthCount) keys[tid] = tid < n ? score_key(scores[tid]) : kKeyNaN;    // (missing tokens sort last, as NaN)
+  if (tid < kKthCount) keys[tid] = tid < n ? score_key(score) : kKeyNaN;    // (missing tokens sort last, as NaN)
   if (tid == 0) s_tau = __int_as_float(0x7f800000);                              // stays: rank k falls among the NaN scores
   __syncthreads();
   const int per = n <= 32 ? 32 : (n <= 64 ? 16 : (n <= 128 ? 8 : (n <= 256 ? 4 : 2)));   // threads to a token
@@ -369,7 +369,8 @@ __global__ void __launch_bounds__(1024) kth_score_kernel(const float* __restrict
                                                          float* __restrict__ tau_out) {
   ptx::pdl_wait();
   ptx::pdl_launch_dependents();
-  const float tau = n <= kKthCount ? kth_by_count(scores, n, k) : kth_in_cta<kKthPerThread>(scores, n, k);
+  const float tau = n <= kKthCount ? kth_by_count((int)threadIdx.x < n ? scores[threadIdx.x] : 0.f, n, k)
+                                     : kth_in_cta<kKthPerThread>(scores, n, k);
   if (threadIdx.x == 0) *tau_out = tau;
 }
 bool kth_score_in_select(int n) { return n <= kKthInCta; }
@@ -493,8 +494,12 @@ __global__ void __launch_bounds__(1024) select_small_kernel(const float* __restr
   for (int t = threadIdx.x * 32; t < T; t += 1024 * 32) ptx::prefetch_l2(delta + g.cache_row(t));
   if (!wait_at_end) ptx::pdl_wait();
   ptx::pdl_launch_dependents();
+  // the first chunk's loads, all in flight together and ahead of the threshold's own work
+  const int cr0 = (int)threadIdx.x < T ? g.cache_row(threadIdx.x) : 0;
+  const int stale0 = (int)threadIdx.x < T ? delta[cr0] : 0;
+  const float score0 = (int)threadIdx.x < T && !select_all ? scores[threadIdx.x] : 0.f;
   if (kKth) {
-    tau = T <= kKthCount ? kth_by_count(scores, T, reuse_count) : kth_in_cta<kSmallTokens / 1024>(scores, T, reuse_count);
+    tau = T <= kKthCount ? kth_by_count(score0, T, reuse_count) : kth_in_cta<kSmallTokens / 1024>(scores, T, reuse_count);
     if (threadIdx.x == 0) *tau_dev = tau;
   } else if (tau_dev != nullptr) {
     tau = *tau_dev;
@@ -505,10 +510,10 @@ __global__ void __launch_bounds__(1024) select_small_kernel(const float* __restr
     const int t = start + threadIdx.x;
     const bool valid = t < T;
     // both loads of the token first (score and staleness counter): one memory round trip instead of two
-    const int cr = valid ? g.cache_row(t) : 0;
-    const int stale = valid ? delta[cr] : 0;
+    const int cr = start == 0 ? cr0 : (valid ? g.cache_row(t) : 0);
+    const int stale = start == 0 ? stale0 : (valid ? delta[cr] : 0);
     bool sel = false;
-    if (valid) sel = select_all ? true : !(scores[t] <= tau);
+    if (valid) sel = select_all ? true : !((start == 0 ? score0 : scores[t]) <= tau);
     const unsigned bal = __ballot_sync(0xffffffffu, sel);
     const int lane_prefix = __popc(bal & ((1u << lane) - 1u));
     if (lane == 0) warp_excl[warp] = __popc(bal);
