@@ -614,28 +614,7 @@ template void launch_copy_reused_rows<__nv_bfloat16>(const __nv_bfloat16*, __nv_
                                                      cudaStream_t, const int*, int);
 
 // ------------------------------------------------------------------------------------------------ row gather
-// dst[r, :] = src[idx[r], :] for r < *count (Alg. 1 line 6: x_norm restricted to the refresh set).
-template <typename T>
-__global__ void __launch_bounds__(256) gather_rows_kernel(const T* __restrict__ src, const int* __restrict__ idx,
-                                                          const int* __restrict__ count, T* __restrict__ dst,
-                                                          int max_rows, int d) {
-  const int n = min(*count, max_rows);
-  constexpr int N = 16 / sizeof(T);
-  const int nvec = d / N;
-  for (int r = blockIdx.x; r < n; r += gridDim.x) {
-    const uint4* s = reinterpret_cast<const uint4*>(src + (size_t)idx[r] * d);
-    uint4* o = reinterpret_cast<uint4*>(dst + (size_t)r * d);
-    for (int v = threadIdx.x; v < nvec; v += blockDim.x) o[v] = s[v];
-  }
-}
-
-template <typename T>
-void launch_gather_rows(const T* src, const int* idx, const int* count, T* dst, int max_rows, int d, cudaStream_t st) {
-  if (max_rows <= 0) return;
-  int grid = max_rows < 148 * 8 ? max_rows : 148 * 8;
-  gather_rows_kernel<T><<<grid, 256, 0, st>>>(src, idx, count, dst, max_rows, d);
-}
-// The same for the rows of a step's refresh set, by flat token index or (by_cache_row) by cache row: a stream of
+// dst[r, :] = src[idx[r], :] for the rows of a step's refresh set (Alg. 1 line 6), by flat token index or (by_cache_row) by cache row: a stream of
 // n * d elements, chained with programmatic dependent launch.
 template <typename T>
 __global__ void __launch_bounds__(256) gather_step_rows_kernel(const T* __restrict__ src, const int* __restrict__ idx,
@@ -667,8 +646,5 @@ void launch_gather_step_rows(const T* src, const int* idx, const int* count, T* 
 }
 template void launch_gather_step_rows<__nv_bfloat16>(const __nv_bfloat16*, const int*, const int*, __nv_bfloat16*,
                                                      const StepGeom&, bool, cudaStream_t, int*, int);
-template void launch_gather_rows<float>(const float*, const int*, const int*, float*, int, int, cudaStream_t);
-template void launch_gather_rows<__nv_bfloat16>(const __nv_bfloat16*, const int*, const int*, __nv_bfloat16*, int, int,
-                                                cudaStream_t);
 
 }  // namespace dare

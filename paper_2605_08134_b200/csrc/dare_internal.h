@@ -136,8 +136,6 @@ bool kth_score_in_select(int n);
 // (select_large.cu)
 cudaError_t launch_kth_score(const float* scores, int n, int k, float* tau_out, cudaStream_t st);
 cudaError_t launch_kth_score_large(const float* scores, int n, int k, float* tau_out, cudaStream_t st);
-template <typename T>
-void launch_gather_rows(const T* src, const int* idx, const int* count, T* dst, int max_rows, int d, cudaStream_t st);
 // dst[r, :] = src[idx[r] (or its cache row), :] for the rows of a step's refresh set
 template <typename T>
 void launch_gather_step_rows(const T* src, const int* idx, const int* count, T* dst, const StepGeom& g, bool by_cache_row,

@@ -27,7 +27,7 @@
 // traffic (ncu: tensor pipe 87 % active).  Both CTAs' TMA loads complete on the even CTA's barriers, stages and
 // accumulators are released to both by one commit each, and the finishing warps of both CTAs hand an accumulator
 // back by arriving on the even CTA's barrier.
-// No reduction split, epilogues Q, K/V, OUT, OUT_RES, SWIGLU (a tile then holds the gate and the up projection of the same
+// No reduction split, epilogues Q, K/V, OUT, OUT_RES, F32 (logits of listed rows), SWIGLU (a tile then holds the gate and the up projection of the same
 // 128 outputs, and a finishing chunk 32 columns of each: eight row tiles of 4096 x 2 x 12288 took 251 us in the
 // one-tile-per-CTA kernel, 6 waves of CTAs that each fill and drain on their own, and 175 us here).
 #include "layer.h"
@@ -393,6 +393,12 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
               vlo.x += fa.x; vlo.y += fa.y; vhi.x += fb.x; vhi.y += fb.y;
             }
             const size_t orow = p.out_is_cache == 1 ? crow : (p.out_is_cache == 2 ? (size_t)(t.t0 + r) : (size_t)tok);
+            if (EPI == EPI_F32) {
+              float* d32 = p.out_f32 + orow * p.ld_out + t.n0 + c_lo + 2 * l8;
+              *reinterpret_cast<float2*>(d32) = vlo;
+              *reinterpret_cast<float2*>(d32 + HDIM / 2) = vhi;
+              continue;
+            }
             if (EPI == EPI_SWIGLU) {
               auto act = [](float gate, float up) { return gate / (1.f + __expf(-gate)) * up; };
               *reinterpret_cast<__nv_bfloat162*>(out + orow * p.ld_out + t.n0 + c_lo + 2 * l8) =
@@ -471,6 +477,7 @@ cudaError_t launch_gemm_persist(int epi, const CUtensorMap& a, const CUtensorMap
     } else {
       if (epi == EPI_KV) return launch_persist<EPI_KV, true, false>(a, b0, b1, p, n_tiles, m_tiles, st);
       if (epi == EPI_OUT) return launch_persist<EPI_OUT, true, false>(a, b0, b1, p, n_tiles, m_tiles, st);
+      if (epi == EPI_F32) return launch_persist<EPI_F32, true, false>(a, b0, b1, p, n_tiles, m_tiles, st);
     }
     return cudaErrorInvalidValue;
   }

@@ -22,7 +22,6 @@
 //   K/V  rotary embedding of K, scatter of both rows into the caches at the refresh-set rows (Eq. 3)
 //   OUT  bf16 store of y (OUT_RES: plus a residual row, read together with the row's tables)
 //   SWIGLU  silu(gate) * up of a tile that holds both projections of the same 128 outputs (MLP of a stack)
-//   F32  fp32 store (logits of a stack's LM head)
 #include "layer.h"
 #include "tc.h"
 #include "tc_ptx.cuh"
@@ -611,12 +610,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
             lo.x = a0 * rb.cs[k].x - b0 * rb.cs[k].y; hi.x = a0 * rb.cs[k].y + b0 * rb.cs[k].x;
             lo.y = a1 * rb.cs[k].z - b1 * rb.cs[k].w; hi.y = a1 * rb.cs[k].w + b1 * rb.cs[k].z;
           }
-          if (EPI == EPI_F32) {
-            float* d32 = p.out_f32 + orow * p.ld_out + n0;
-            *reinterpret_cast<float2*>(d32 + c_lo) = lo;
-            *reinterpret_cast<float2*>(d32 + c_hi) = hi;
-            continue;
-          }
           if (EPI == EPI_OUT_RES) {                                  // (read with the row's tables, long before)
             const float2 ra = __bfloat1622float2(rb.res[k][hh][0]), rb2 = __bfloat1622float2(rb.res[k][hh][1]);
             lo.x += ra.x; lo.y += ra.y; hi.x += rb2.x; hi.y += rb2.y;
@@ -693,7 +686,7 @@ static cudaError_t launch_split(const CUtensorMap& a, const CUtensorMap& b0, con
 template <int EPI, int BN, bool PAIR, int HDIM>
 static cudaError_t launch_hd(const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1, const GemmParams& p,
                              int n_tiles, int m_tiles, int splits, cudaStream_t st) {
-  if constexpr (EPI != EPI_SWIGLU && EPI != EPI_F32) {
+  if constexpr (EPI != EPI_SWIGLU) {
     if (p.flat && p.idx == nullptr) return launch_split<EPI, BN, PAIR, HDIM, true>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
   }
   return launch_split<EPI, BN, PAIR, HDIM, false>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
@@ -738,7 +731,6 @@ cudaError_t launch_gemm_tc(int epi, int bn, const CUtensorMap& a, const CUtensor
     if (epi == EPI_Q) return launch_one<EPI_Q, 256, false>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
     if (epi == EPI_KV) return launch_one<EPI_KV, 256, false>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
     if (epi == EPI_SWIGLU) return launch_one<EPI_SWIGLU, 256, false>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
-    if (epi == EPI_F32) return launch_one<EPI_F32, 256, false>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
     if (epi == EPI_OUT_RES) return launch_one<EPI_OUT_RES, 256, false>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
     return launch_one<EPI_OUT, 256, false>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
   }

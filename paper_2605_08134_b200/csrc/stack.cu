@@ -9,6 +9,7 @@
 #include "dare_stack.h"
 #include "layer.h"
 #include "tc.h"
+#include "tc_ptx.cuh"
 
 using namespace dare;
 
@@ -35,6 +36,8 @@ struct BlockMaps {
 __global__ void __launch_bounds__(256) embed_kernel(const int* __restrict__ tokens, int seq_total, int seq_act,
                                                     int pos_begin, const uint4* __restrict__ emb, uint4* __restrict__ x,
                                                     int row_vecs, int vocab) {
+  ptx::pdl_wait();                     // (the step before writes its token into the buffer)
+  ptx::pdl_launch_dependents();
   const int t = blockIdx.x;
   const int b = t / seq_act, i = t - b * seq_act;
   int id = tokens[(size_t)b * seq_total + pos_begin + i];
@@ -45,36 +48,52 @@ __global__ void __launch_bounds__(256) embed_kernel(const int* __restrict__ toke
 }
 
 // Masked positions of the active block, ascending per sequence: cand_row = row of the window's hidden states,
-// cand_pos = position, cand_off[b] = start of sequence b's slice.  One warp per sequence (block <= 32).
-__global__ void cand_kernel(const int* __restrict__ tokens, int batch, int seq_total, int lo, int hi, int mask_id,
-                            int pos_begin, int seq_act, int* __restrict__ cand_row, int* __restrict__ cand_pos,
-                            int* __restrict__ cand_off, int* __restrict__ cand_count) {
-  __shared__ int cnt[32];
-  const int b = threadIdx.x >> 5, lane = threadIdx.x & 31;
+// cand_pos = position, cand_off[b] = start of sequence b's slice; and the candidates' rows of the hidden states, compact.
+// One CTA per possible candidate, each works the list out for itself (a warp per sequence, block <= 32; a launch less than
+// list and copy apart), CTA 0 writes it.
+__global__ void __launch_bounds__(1024) cand_kernel(const int* __restrict__ tokens, int batch, int seq_total, int lo, int hi,
+                                                    int mask_id, int pos_begin, int seq_act, int* __restrict__ cand_row,
+                                                    int* __restrict__ cand_pos, int* __restrict__ cand_off,
+                                                    int* __restrict__ cand_count, const uint4* __restrict__ hidden,
+                                                    uint4* __restrict__ lm_a, int row_vecs) {
+  __shared__ int off[33], mine;
+  ptx::pdl_wait();
+  ptx::pdl_launch_dependents();
+  const int b = threadIdx.x >> 5, lane = threadIdx.x & 31, r = blockIdx.x;
   const int pos = lo + lane;
   const bool is = b < batch && pos < hi && tokens[(size_t)b * seq_total + pos] == mask_id;
   const unsigned bal = __ballot_sync(0xffffffffu, is);
-  if (lane == 0 && b < 32) cnt[b] = __popc(bal);
+  if (lane == 0) off[b + 1] = __popc(bal);
   __syncthreads();
-  int off = 0;
-  for (int k = 0; k < b; ++k) off += cnt[k];
+  if (b == 0) {
+    int v = off[lane + 1];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, v, o);
+      if (lane >= o) v += u;
+    }
+    off[lane + 1] = v;
+    if (lane == 0) off[0] = 0;
+  }
+  __syncthreads();
+  const int total = off[32];
   if (is) {
-    const int o = off + __popc(bal & ((1u << lane) - 1u));
-    cand_row[o] = b * seq_act + pos - pos_begin;
-    cand_pos[o] = pos;
+    const int o = off[b] + __popc(bal & ((1u << lane) - 1u)), row = b * seq_act + pos - pos_begin;
+    if (o == r) mine = row;
+    if (r == 0) { cand_row[o] = row; cand_pos[o] = pos; }
   }
-  if (lane == 0 && b < batch) cand_off[b] = off;
-  if (threadIdx.x == 0) {
-    int tot = 0;
-    for (int k = 0; k < batch; ++k) tot += cnt[k];
-    cand_off[batch] = tot;
-    *cand_count = tot;
-  }
+  if (r == 0 && (int)threadIdx.x <= batch) cand_off[threadIdx.x] = off[threadIdx.x];
+  if (r == 0 && threadIdx.x == 0) *cand_count = total;
+  if (r >= total) return;
+  __syncthreads();
+  for (int v = threadIdx.x; v < row_vecs; v += blockDim.x) lm_a[(size_t)r * row_vecs + v] = hidden[(size_t)mine * row_vecs + v];
 }
 
 // Per candidate row of the logits: argmax (lowest index on ties, the mask id excluded) and its softmax probability.
 // One pass over the row: every thread keeps a running maximum (with its index) and the sum of exp(v - maximum),
-// rescaled when the maximum moves; the triples are then merged over the warp and the CTA.
+// rescaled when the maximum moves; the triples are then merged over the warp and the CTA.  A row is shared by kSlices
+// CTAs (there are few candidates, and one SM needs 25 us for 126464 logits); pick_kernel merges their triples.
+constexpr int kSlices = 16;
 struct RowStat {
   float m, s;
   int arg;
@@ -94,71 +113,75 @@ __device__ __forceinline__ void stat_merge(RowStat& a, float om, float os, int o
   a.s = sa + sb; a.m = M;
   if (take) a.arg = oa;
 }
-__global__ void __launch_bounds__(1024) rowstats_kernel(const float* __restrict__ logits, const int* __restrict__ count,
-                                                        int vocab, int mask_id, int* __restrict__ tok,
-                                                        float* __restrict__ prob) {
-  __shared__ float s_max[32], s_sum[32];
-  __shared__ int s_arg[32];
-  const int r = blockIdx.x;
-  if (r >= *count) return;
-  const float* row = logits + (size_t)r * vocab;
-  RowStat a{-INFINITY, 0.f, 0x7fffffff};
-  if ((vocab & 3) == 0) {                                   // rows then start on 16-byte boundaries
-    const float4* row4 = reinterpret_cast<const float4*>(row);
-    for (int j4 = threadIdx.x; j4 < vocab / 4; j4 += blockDim.x) {
-      const float4 v = row4[j4];
-      const int j = 4 * j4;
-      if (j != mask_id) stat_add(a, v.x, j);
-      if (j + 1 != mask_id) stat_add(a, v.y, j + 1);
-      if (j + 2 != mask_id) stat_add(a, v.z, j + 2);
-      if (j + 3 != mask_id) stat_add(a, v.w, j + 3);
-    }
-  } else {
-    for (int j = threadIdx.x; j < vocab; j += blockDim.x)
-      if (j != mask_id) stat_add(a, row[j], j);
-  }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+__device__ __forceinline__ void stat_merge_warp(RowStat& a) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     const float om = __shfl_xor_sync(0xffffffffu, a.m, o), os = __shfl_xor_sync(0xffffffffu, a.s, o);
     const int oa = __shfl_xor_sync(0xffffffffu, a.arg, o);
     stat_merge(a, om, os, oa);
   }
-  if (lane == 0) { s_max[warp] = a.m; s_sum[warp] = a.s; s_arg[warp] = a.arg; }
+}
+__global__ void __launch_bounds__(512) rowstats_kernel(const float* __restrict__ logits, const int* __restrict__ count,
+                                                       int vocab, int mask_id, RowStat* __restrict__ parts) {
+  __shared__ RowStat s_part[16];
+  ptx::pdl_wait();
+  ptx::pdl_launch_dependents();
+  const int r = blockIdx.y, slice = blockIdx.x;
+  if (r >= *count) return;
+  const float4* row = reinterpret_cast<const float4*>(logits + (size_t)r * vocab);      // (vocab is a multiple of 256)
+  const int n4 = vocab / 4, per = (n4 + kSlices - 1) / kSlices, end = min(n4, (slice + 1) * per);
+  RowStat a{-INFINITY, 0.f, 0x7fffffff};
+  for (int j4 = slice * per + (int)threadIdx.x; j4 < end; j4 += blockDim.x) {
+    const float4 v = row[j4];
+    const int j = 4 * j4;
+    if (j != mask_id) stat_add(a, v.x, j);
+    if (j + 1 != mask_id) stat_add(a, v.y, j + 1);
+    if (j + 2 != mask_id) stat_add(a, v.z, j + 2);
+    if (j + 3 != mask_id) stat_add(a, v.w, j + 3);
+  }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  stat_merge_warp(a);
+  if (lane == 0) s_part[warp] = a;
   __syncthreads();
   if (warp == 0) {
-    a.m = s_max[lane]; a.s = s_sum[lane]; a.arg = s_arg[lane];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float om = __shfl_xor_sync(0xffffffffu, a.m, o), os = __shfl_xor_sync(0xffffffffu, a.s, o);
-      const int oa = __shfl_xor_sync(0xffffffffu, a.arg, o);
-      stat_merge(a, om, os, oa);
-    }
-    if (lane == 0) {
-      tok[r] = a.arg;
-      prob[r] = 1.f / a.s;                                  // exp(max - max) / sum
-    }
+    a = lane < 16 ? s_part[lane] : RowStat{-INFINITY, 0.f, 0x7fffffff};
+    stat_merge_warp(a);
+    if (lane == 0) parts[r * kSlices + slice] = a;
   }
 }
 
-// Per sequence: the candidate with the largest probability (first one on ties); its token goes into the buffer
-// unless a forced (position, token) is given.
-__global__ void pick_kernel(const int* __restrict__ cand_off, const int* __restrict__ cand_pos,
-                            const int* __restrict__ tok, const float* __restrict__ prob, int batch, int seq_total,
-                            int* __restrict__ tokens, const int* __restrict__ forced_pos,
-                            const int* __restrict__ forced_tok, int* __restrict__ pos_out, int* __restrict__ tok_out,
-                            float* __restrict__ prob_out) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+// Per sequence (one warp): the candidate with the largest probability (first one on ties); its token goes into the buffer
+// unless a forced (position, token) is given.  Lane <-> candidate of the sequence (block <= 32).
+__global__ void __launch_bounds__(1024) pick_kernel(const int* __restrict__ cand_off, const int* __restrict__ cand_pos,
+                                                    const RowStat* __restrict__ parts, int batch, int seq_total,
+                                                    int* __restrict__ tokens, const int* __restrict__ forced_pos,
+                                                    const int* __restrict__ forced_tok, int* __restrict__ pos_out,
+                                                    int* __restrict__ tok_out, float* __restrict__ prob_out) {
+  ptx::pdl_wait();
+  ptx::pdl_launch_dependents();
+  const int b = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (b >= batch) return;
-  int best = -1;
-  float bp = -1.f;
-  for (int i = cand_off[b]; i < cand_off[b + 1]; ++i)
-    if (prob[i] > bp) { bp = prob[i]; best = i; }
-  int p_ = -1, t_ = -1;
-  if (best >= 0) { p_ = cand_pos[best]; t_ = tok[best]; }
+  const int i = cand_off[b] + lane, n = cand_off[b + 1] - cand_off[b];
+  RowStat a{-INFINITY, 0.f, 0x7fffffff};
+  float prob = -1.f;
+  if (lane < n) {
+    for (int s = 0; s < kSlices; ++s) {
+      const RowStat o = parts[i * kSlices + s];
+      stat_merge(a, o.m, o.s, o.arg);
+    }
+    prob = 1.f / a.s;                                       // exp(max - max) / sum
+  }
+  float bp = prob;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) bp = fmaxf(bp, __shfl_xor_sync(0xffffffffu, bp, o));
+  const unsigned hit = __ballot_sync(0xffffffffu, lane < n && prob == bp);
+  const int best = hit != 0u ? __ffs((int)hit) - 1 : 0;
+  const int tok = __shfl_sync(0xffffffffu, a.arg, best);
+  if (lane != 0) return;
+  const int p_ = hit != 0u ? cand_pos[cand_off[b] + best] : -1, t_ = hit != 0u ? tok : -1;
   if (pos_out) pos_out[b] = p_;
   if (tok_out) tok_out[b] = t_;
-  if (prob_out) prob_out[b] = best >= 0 ? bp : 0.f;
+  if (prob_out) prob_out[b] = hit != 0u ? bp : 0.f;
   int wp = p_, wt = t_;
   if (forced_pos != nullptr) { wp = forced_pos[b]; wt = forced_tok[b]; }
   if (wp >= 0 && wp < seq_total) tokens[(size_t)b * seq_total + wp] = wt;
@@ -167,8 +190,8 @@ __global__ void pick_kernel(const int* __restrict__ cand_off, const int* __restr
 struct StackBuffers {
   bf16 *xa, *hb, *n2, *act, *hidden, *lm_a;
   float* logits;
-  int *cand_row, *cand_pos, *cand_off, *cand_count, *cand_tok, *forced;
-  float* cand_prob;
+  int *cand_row, *cand_pos, *cand_off, *cand_count, *forced;
+  RowStat* cand_parts;
 };
 
 size_t carve_stack(const dare_stack_config_t* c, char* base, StackBuffers* b, std::vector<void*>* layer_ws,
@@ -193,8 +216,7 @@ size_t carve_stack(const dare_stack_config_t* c, char* base, StackBuffers* b, st
   B.cand_pos = (int*)take(kMaxCand * sizeof(int));
   B.cand_off = (int*)take(64 * sizeof(int));
   B.cand_count = (int*)take(sizeof(int));
-  B.cand_tok = (int*)take(kMaxCand * sizeof(int));
-  B.cand_prob = (float*)take(kMaxCand * sizeof(float));
+  B.cand_parts = (RowStat*)take(kMaxCand * kSlices * sizeof(RowStat));
   B.forced = (int*)take(2 * 64 * sizeof(int));
   for (int l = 0; l < c->n_layers; ++l) {
     void* p = take(layer_bytes);
@@ -259,8 +281,8 @@ dare_status_t forward(dare_stack* S, const int* tokens, int batch, int seq_total
   const dare_layer_config_t& lc = S->cfg.layer;
   const int T_ = batch * seq_act, d = lc.d_model, f = S->cfg.d_ff;
   const StackBuffers& B = S->buf;
-  embed_kernel<<<T_, 256, 0, st>>>(tokens, seq_total, seq_act, pos_begin, (const uint4*)S->emb, (uint4*)B.xa, d / 8,
-                                   S->cfg.vocab);
+  if (launch_pdl(embed_kernel, dim3(T_), dim3(256), 0, st, 1, tokens, seq_total, seq_act, pos_begin, (const uint4*)S->emb,
+                 (uint4*)B.xa, d / 8, S->cfg.vocab) != cudaSuccess) return DARE_ERR_CUDA;
   const int m_tiles = (T_ + 127) / 128;
   const int width = T_ <= 128 ? S->width1 : S->width2;
   for (int l = 0; l < S->cfg.n_layers; ++l) {
@@ -470,17 +492,19 @@ dare_status_t dare_stack_decode_step(dare_stack_t* S, int32_t* tokens, int batch
   if (s != DARE_OK) return s;
   const StackBuffers& B = S->buf;
   const int d = S->cfg.layer.d_model, V = S->cfg.vocab;
-  cand_kernel<<<1, 32 * 32, 0, st>>>(tokens, batch, seq_total, lo, hi, S->cfg.mask_id, pos_begin, seq_act, B.cand_row,
-                                     B.cand_pos, B.cand_off, B.cand_count);
-  launch_gather_rows<bf16>(B.hidden, B.cand_row, B.cand_count, B.lm_a, kMaxCand, d, st);
+  if (launch_pdl(cand_kernel, dim3(S->cfg.layer.max_batch * blk), dim3(1024), 0, st, 1, (const int*)tokens, batch, seq_total, lo,
+                 hi, S->cfg.mask_id, pos_begin, seq_act, B.cand_row, B.cand_pos, B.cand_off, B.cand_count,
+                 (const uint4*)B.hidden, (uint4*)B.lm_a, d / 8) != cudaSuccess) return DARE_ERR_CUDA;
   {
     GemmParams p = base_params(S, batch, seq_act, pos_begin);
     p.idx = B.cand_row; p.count = B.cand_count; p.m_total = kMaxCand;
     p.out_f32 = B.logits; p.ld_out = V; p.out_is_cache = 2;
-    if (launch_gemm_tc(EPI_F32, 256, S->a_lm, S->w_head, S->w_head, p, V / 256, 1, 1, st) != cudaSuccess)
+    // (a stream of the head's rows: one persistent CTA per SM, its ring running on from tile to tile)
+    if (launch_gemm_persist(EPI_F32, S->a_lm, S->w_head, S->w_head, p, V / 256, 1, st, 0) != cudaSuccess)
       return DARE_ERR_CUDA;
   }
-  rowstats_kernel<<<kMaxCand, 1024, 0, st>>>(B.logits, B.cand_count, V, S->cfg.mask_id, B.cand_tok, B.cand_prob);
+  if (launch_pdl(rowstats_kernel, dim3(kSlices, S->cfg.layer.max_batch * blk), dim3(512), 0, st, 1, (const float*)B.logits,
+                 (const int*)B.cand_count, V, S->cfg.mask_id, B.cand_parts) != cudaSuccess) return DARE_ERR_CUDA;
   const int* fpos = nullptr;
   const int* ftok = nullptr;
   if (forced_pos_host) {
@@ -489,8 +513,9 @@ dare_status_t dare_stack_decode_step(dare_stack_t* S, int32_t* tokens, int batch
       return DARE_ERR_CUDA;
     fpos = B.forced; ftok = B.forced + 64;
   }
-  pick_kernel<<<1, 32, 0, st>>>(B.cand_off, B.cand_pos, B.cand_tok, B.cand_prob, batch, seq_total, tokens, fpos, ftok,
-                                pos_out, tok_out, prob_out);
+  if (launch_pdl(pick_kernel, dim3(1), dim3(32 * batch), 0, st, 1, (const int*)B.cand_off, (const int*)B.cand_pos,
+                 (const RowStat*)B.cand_parts, batch, seq_total, tokens, fpos, ftok, pos_out, tok_out, prob_out) != cudaSuccess)
+    return DARE_ERR_CUDA;
   if (cudaGetLastError() != cudaSuccess) return DARE_ERR_CUDA;
   return DARE_OK;
 }
