@@ -24,7 +24,7 @@ __device__ __forceinline__ __nv_bfloat16 from_f<__nv_bfloat16>(float v) { return
 __device__ __forceinline__ void fetch4(float* dst, const float* src, bool ok) { cp_async_16(smem_u32(dst), src, ok ? 16u : 0u); }
 __device__ __forceinline__ void fetch4(float* dst, const __nv_bfloat16* src, bool ok) {
   uint2 raw = make_uint2(0u, 0u);
-  if (ok) raw = *reinterpret_cast<const uint2*>(src);
+  if (ok) raw = __ldcg(reinterpret_cast<const uint2*>(src));
   const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&raw.x));
   const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&raw.y));
   *reinterpret_cast<float4*>(dst) = make_float4(a.x, a.y, b.x, b.y);
@@ -150,6 +150,33 @@ __global__ void __launch_bounds__(kSgThreads, 1) sgemm_kernel(const SgemmParams 
 
   const int grp = tid / kGroup, wp = (tid % kGroup) >> 5, lane = tid & 31;
   const int wm = wp >> 1, wn = wp & 1, tx = lane & 7, ty = lane >> 3;
+  // All table reads of the tail together, one memory round trip for the rows of this thread; the shortest tiles, whose launches
+  // are short chains of round trips, have the registers to start them ahead of the main loop.  (The stored query is this
+  // layer's previous step's, the tables are constant.)
+  constexpr bool kEarlyTables = RM == 2;
+  const int pair = pair0 + 16 * wn + tx;         // and pair + 8
+  const bool score_tile = EPI == SG_Q && half <= 32 && ((p.g.score_head * half) >> 5) == pair0 >> 5;
+  const bool rotate = EPI == SG_Q || (EPI == SG_KV && !second);
+  T* out = reinterpret_cast<T*>(second ? p.out1 : p.out0);
+  float2 cs[RM][2], old[RM][2];
+  auto read_tables = [&]() {
+#pragma unroll
+    for (int i = 0; i < RM; ++i) {
+      const int t = s_tok[wm * (4 * RM) + ty + 4 * i];
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const int pj = pair + 8 * j, jj = pj & (half - 1);
+        cs[i][j] = old[i][j] = make_float2(0.f, 0.f);
+        if (t < 0 || pj >= n_pairs) continue;
+        if (rotate) cs[i][j] = p.rope[(size_t)p.g.position(t) * half + jj];
+        if (score_tile && p.has_prev && (pj >> lh) == p.g.score_head) {
+          const float* qp = p.q_prev + (size_t)p.g.cache_row(t) * (2 * half) + jj;
+          old[i][j] = make_float2(qp[0], qp[half]);
+        }
+      }
+    }
+  };
+  if (kEarlyTables && grp == 0) read_tables();
   // rows wm * 4 RM + ty + 4 i; columns 16 wn + tx + {0, 8} and their partners + 32
   float2 acc[RM][4];
 #pragma unroll
@@ -200,27 +227,8 @@ __global__ void __launch_bounds__(kSgThreads, 1) sgemm_kernel(const SgemmParams 
       for (int e = 0; e < RM * 4; ++e) v[e >> 2][e & 3] += ring[(gi * RM * 4 + e) * kGroup + tid];
   }
 
-  // ---- the projection's own tail.  All table reads first: one memory round trip for the rows of this thread.
-  const int pair = pair0 + 16 * wn + tx;         // and pair + 8
-  const bool score_tile = EPI == SG_Q && half <= 32 && ((p.g.score_head * half) >> 5) == pair0 >> 5;
-  const bool rotate = EPI == SG_Q || (EPI == SG_KV && !second);
-  T* out = reinterpret_cast<T*>(second ? p.out1 : p.out0);
-  float2 cs[RM][2], old[RM][2];
-#pragma unroll
-  for (int i = 0; i < RM; ++i) {
-    const int t = s_tok[wm * (4 * RM) + ty + 4 * i];
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const int pj = pair + 8 * j, jj = pj & (half - 1);
-      cs[i][j] = old[i][j] = make_float2(0.f, 0.f);
-      if (t < 0 || pj >= n_pairs) continue;
-      if (rotate) cs[i][j] = p.rope[(size_t)p.g.position(t) * half + jj];
-      if (score_tile && p.has_prev && (pj >> lh) == p.g.score_head) {
-        const float* qp = p.q_prev + (size_t)p.g.cache_row(t) * (2 * half) + jj;
-        old[i][j] = make_float2(qp[0], qp[half]);
-      }
-    }
-  }
+  // ---- the projection's own tail
+  if (!kEarlyTables) read_tables();
 #pragma unroll
   for (int i = 0; i < RM; ++i) {
     const int r = wm * (4 * RM) + ty + 4 * i, t = s_tok[r];
@@ -384,12 +392,12 @@ __global__ void __launch_bounds__(128 * RG * KG, 1) sattn_kernel(const SattnPara
   const int tid = threadIdx.x, grp = tid / (128 * RG), lt = tid % (128 * RG), tx = tid & 15, ty = lt >> 4;   // key group; row
   const int r0 = (ty >> 3) * 32 + (ty & 7);                             // this thread's rows: r0 + 8 i
   const int h = blockIdx.x, b = blockIdx.y, tile = blockIdx.z, d = g.d;
-  pdl_wait();
-  pdl_launch_dependents();
+  // The kernel before (the K/V projection) writes the caches only; queries and refresh set come from kernels further back,
+  // complete by the time any CTA of this grid runs: they are read, through the L2, ahead of the wait.
   int row0, n_rows;
   if (p.idx) {
-    const int lo = p.batch_off[b], hi = p.batch_off[b + 1];
-    if (!slice_ok(lo, hi, g.tokens(), p.status) || lo + tile * BQ >= hi) return;
+    const int lo = __ldcg(p.batch_off + b), hi = __ldcg(p.batch_off + b + 1);
+    if (!slice_ok(lo, hi, g.tokens(), p.status) || lo + tile * BQ >= hi) { pdl_wait(); return; }
     row0 = lo + tile * BQ;
     n_rows = min(BQ, hi - row0);
   } else {
@@ -413,7 +421,7 @@ __global__ void __launch_bounds__(128 * RG * KG, 1) sattn_kernel(const SattnPara
     cp_async_commit();                             // (empty past the last block: the group count stays uniform)
   };
   if (tid < BQ) {
-    int t = tid < n_rows ? (p.idx ? p.idx[row0 + tid] : row0 + tid) : -1;
+    int t = tid < n_rows ? (p.idx ? __ldcg(p.idx + row0 + tid) : row0 + tid) : -1;
     if (p.idx && t != -1 && !token_ok(t, g.tokens(), p.status)) t = -1;   // neither a query row to read nor a cache row to write
     s_tok[tid] = t;
   }
@@ -422,6 +430,8 @@ __global__ void __launch_bounds__(128 * RG * KG, 1) sattn_kernel(const SattnPara
     const int r = c / (HD / 4), e = (c % (HD / 4)) * 4, t = s_tok[r];
     fetch4(sm + S::Q_OFF + r * KP + e, reinterpret_cast<const T*>(p.q) + (size_t)(t < 0 ? 0 : t) * d + h * HD + e, t >= 0);
   }
+  pdl_wait();
+  pdl_launch_dependents();
   fetch_block(kd, KP, kbase, grp);                 // (one group with Q)
   fetch_block(vd, HD, vbase, grp);
   const float c = rsqrtf((float)HD) * 1.4426950408889634f;              // softmax scale folded into the exp2 argument
