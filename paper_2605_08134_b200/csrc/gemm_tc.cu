@@ -261,8 +261,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       }
     }
   }
-  if (!p.wait_at_end) pdl_wait();
-  pdl_launch_dependents();
+  if (!p.wait_at_end && !p.late_wait) pdl_wait();
+  if (!p.late_wait) pdl_launch_dependents();
   if (dbg && threadIdx.x == 0) p.debug[1] = globaltimer_ns();
 
   // ---- which rows does this tile cover? (uniform over the cluster; a tile past the refresh set has nothing to do)
@@ -453,6 +453,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
   // started before the main loop) and land during the exchange below.
   if (warp < 2) load_row_batch<EPI, RB, kWarps, BN, HDIM, FLAT>(rb, p, warp, z, rows_per_cta, rows_valid, t0, pos0, crow0, fr, rotate, score_tile, lane, n0);
 
+  if (EPI == EPI_KV && p.late_wait) {
+    pdl_wait();
+    pdl_launch_dependents();
+  }
   // ---- every CTA of the cluster has finished its main loop: the rings are free to receive partial rows
   tc_fence_before();
   if (splits > 1) cluster_sync_relaxed(); else __syncthreads();
@@ -514,6 +518,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
 #pragma unroll 1
     for (int rl0 = warp; rl0 < rows_per_cta; rl0 += kWarps * RB) {
       if (rl0 != warp) load_row_batch<EPI, RB, kWarps, BN, HDIM, FLAT>(rb, p, rl0, z, rows_per_cta, rows_valid, t0, pos0, crow0, fr, rotate, score_tile, lane, n0);
+      // (a masked store keeps the rows this step's selection refreshed: Eq. 3, every other row keeps its cached K and V)
+      if (EPI == EPI_KV && p.store_mask != nullptr) {
+#pragma unroll
+        for (int k = 0; k < RB; ++k) rb.ok[k] = rb.ok[k] && __ldcg(p.store_mask + rb.crow[k]) == 0;
+      }
       if (dbg && EPI == EPI_Q && threadIdx.x == 64) p.debug[34 + (rl0 - warp) / (kWarps * RB) * 2] = globaltimer_ns();
       // (1) combine the partial rows: lane <-> a pair of columns of each piece and its rotary partners
       float2 vlo[RB][BN / CH], vhi[RB][BN / CH];

@@ -129,7 +129,7 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
   base.out_is_cache = 0; base.resid = nullptr; base.ld_resid = 0; base.out_f32 = nullptr; base.b_pair = 0;
   base.rope = reinterpret_cast<const float2*>(B.rope_cs); base.q_prev = B.q_prev;
   base.scores = B.scores; base.has_prev = has_prev ? 1 : 0; base.status = B.status;
-  base.debug = nullptr; base.wait_at_end = 0; base.loop_rows = 0;
+  base.debug = nullptr; base.wait_at_end = 0; base.late_wait = 0; base.loop_rows = 0;
   base.gate_count = nullptr; base.gate_lo = 0; base.gate_hi = 1 << 30; base.store_mask = nullptr;
   // Steps of many row tiles: from these refresh-set sizes on the dense forms of the K/V projection, of attention and of
   // the output projection (results kept for the refreshed rows only) are faster than the listed forms.  Measured on
@@ -196,6 +196,7 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
     // (a selection that refreshes everything reads no scores: behind the two projections it runs beside them)
     select_step(L, g, mode, tau, kv_beside_q && select_all, st, &launches);
   };
+  const bool injected = L->inject != 0;          // (diagnostics: the projection then has to read the list)
   if (!kv_beside_q) select_now();
   // K/V projection with rotary embedding and cache scatter
   {
@@ -209,7 +210,16 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
       p.idx = B.idx; p.count = B.count; p.gather_src = (const bf16*)B.xn;
       const int m_tiles = (T_ + 127) / 128;
       prof_mark(L, SLOT_KV_GEMM, st);
-      if (m_tiles <= 8) {
+      if (T_ <= 128 && !injected) {
+        // One row tile holds every token of the step, refreshed or not: it is projected as it lies, by TMA, while the
+        // selection is still at work, and the rows of the refresh set are stored.  No list, and the main loop is over by
+        // the time the selection is (2 windows of 32 rows, width 4096: step 68.5 -> 61.0 us).
+        p.idx = nullptr; p.count = nullptr; p.gather_src = nullptr;
+        p.n_split = d / 128;
+        p.store_mask = B.delta; p.late_wait = 1;
+        e = launch_gemm_tc(EPI_KV, 128, S.a_xn, S.w_k128, S.w_v128, p, 2 * d / 128, m_tiles_dense, kv_splits(2 * d / 128, kblocks), st);
+        ++launches;
+      } else if (m_tiles <= 8) {
         // Few tokens: the refresh set fits one or two row tiles and the projection is a stream of the weights.
         // Narrower tiles put twice as many CTAs on it; the reduction split is sized for one row tile.
         p.n_split = d / 128;

@@ -58,6 +58,8 @@ struct GemmParams {
   int gate_lo, gate_hi;
   const int* store_mask;
   int loop_rows;         // gathered launch with ONE row of CTAs in the grid: each takes the refresh set's row tiles in turn
+  int late_wait;         // 1: only the finishing pass needs what the predecessor writes (store_mask): the main loop runs
+                         // beside it, its operands come from two or more kernels back
   int wait_at_end;       // 1: the launch reads nothing its predecessor in the stream writes and writes nothing that one
                          // reads, so it runs beside it: its CTAs start as soon as the predecessor's have passed their own
                          // dependency wait (everything further back is then complete), and wait for the predecessor
