@@ -430,6 +430,7 @@ __global__ void __launch_bounds__(kThreads) select_cluster_kernel(const float* _
                                                                   int* __restrict__ idx, int* __restrict__ count_out) {
   __shared__ int warp_sums[32], total, totals[kKthMaxCtas];
   const int ctas = (int)gridDim.x, rank = (int)ptx::cluster_ctarank(), tid = (int)threadIdx.x;
+  ptx::cluster_arrive_relaxed();                      // "this CTA runs": the others may store into its shared memory
   ptx::pdl_wait();
   ptx::pdl_launch_dependents();
   const int iters = (n + ctas * kThreads * 4 - 1) / (ctas * kThreads * 4);   // <= kClusterIters
@@ -451,6 +452,7 @@ __global__ void __launch_bounds__(kThreads) select_cluster_kernel(const float* _
   __syncthreads();
   if ((tid & 31) == 0 && mine != 0) atomicAdd(&total, mine);
   __syncthreads();
+  ptx::cluster_wait();                                // every CTA of the cluster has started
   if (tid < ctas) ptx::st_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&totals[rank]), (uint32_t)tid), (uint32_t)total);
   ptx::cluster_sync_all();
   int out = 0, all = 0;

@@ -326,10 +326,13 @@ __device__ __forceinline__ void bulk_copy_to_cta(uint32_t dst_cluster_addr, uint
                : "memory");
 }
 // Barrier over every thread of the cluster without the release of earlier writes: for points where the threads only
-// tell each other that something they observed complete (an mbarrier phase) is complete.
+// tell each other that something they observed complete (an mbarrier phase) is complete, or that they run at all: a CTA's
+// shared memory may be touched from another one only once it has started.  In two halves where there is work between.
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync_relaxed() {
-  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+  cluster_arrive_relaxed();
+  cluster_wait();
 }
 // Barrier over every thread of the cluster; the release/acquire pair orders the distributed shared-memory stores.
 __device__ __forceinline__ void cluster_sync_all() {
