@@ -139,8 +139,9 @@ dare_status_t dare_layer_step(dare_layer_t* layer, const void* x, int batch, int
  *   tau_t = the reuse_count-th smallest drift score of the step's batch * seq_act tokens,
  * and Eq. 2 is applied with it, so tokens tied with that score are reused as well.  reuse_count = 0 refreshes every
  * token, reuse_count >= batch * seq_act reuses every token; NaN scores sort last and are never reused; negative is
- * rejected.  tau_t is found on the device (an exact four-pass radix selection, one more kernel ahead of the
- * selection) and never travels to the host; dare_layer_last_threshold reads it back afterwards (the threshold of
+ * rejected.  tau_t is found on the device, exactly (inside the selection kernel; with more than 16384 tokens in a kernel
+ * ahead of it, which leaves NaN if its bounded wait ran out: every token is then refreshed and the status word reads
+ * DARE_ERR_TIMEOUT), and never travels to the host; dare_layer_last_threshold reads it back afterwards (the threshold of
  * the last step, whichever call gave it; synchronises the stream if the value is on the device).  A first step and
  * mode = DENSE refresh everything as always.  reuse_count = floor(phi * batch * seq_act) gives the reuse rate phi. */
 dare_status_t dare_layer_step_quantile(dare_layer_t* layer, const void* x, int batch, int seq_act, int pos_begin,
@@ -182,6 +183,9 @@ dare_status_t dare_layer_clear_status(dare_layer_t* layer, void* cuda_stream);
  * dare_layer_debug_inject: the next step overwrites, right after its selection, what = 1: the first entry of the
  *   refresh list with batch * seq_act (one past the step's tokens), what = 2: the list's length with
  *   batch * seq_act + 3; the kernels that consume the selection must flag DARE_ERR_DEVICE_CHECK and skip the access.
+ *   what = 3 (CUDA-core path only, DARE_ERR_UNSUPPORTED otherwise): if the next step is a dare_layer_step_quantile of more
+ *   than 16384 tokens, one of the copies between the thread blocks that work out its threshold is not sent; the wait for it
+ *   gives up after a millisecond, the status word reads DARE_ERR_TIMEOUT and the step refreshes every token.
  *   One step only; what = 0 withdraws it. */
 dare_status_t dare_layer_debug_wait_probe(dare_layer_t* layer, uint64_t limit_ns, uint64_t* waited_ns_host, void* cuda_stream);
 dare_status_t dare_layer_debug_inject(dare_layer_t* layer, int what);
@@ -250,7 +254,7 @@ dare_status_t dare_rmsnorm(const void* x, const float* gain, void* y, int64_t ro
                            void* cuda_stream);
 /* *tau_out (device) = the k-th smallest of n_tokens float32 scores (k clamped to [0, n_tokens]; k = 0: -inf,
  * k = n_tokens or beyond the scores that are numbers: +inf), the threshold that reuses the k least-drifted tokens under
- * Eq. 2 (Sec. 3.1).  Exact; 1 <= n_tokens <= 2^24. */
+ * Eq. 2 (Sec. 3.1).  Exact; 1 <= n_tokens <= 2^24.  NaN if a bounded device-side wait ran out (more than 16384 scores). */
 dare_status_t dare_score_kth(const float* scores, int64_t n_tokens, int64_t k, float* tau_out, void* cuda_stream);
 size_t dare_select_compact_scratch_bytes(int64_t n_tokens);
 dare_status_t dare_select_compact(const float* scores, int64_t n_tokens, float threshold, int32_t* idx, int32_t* count,

@@ -101,7 +101,10 @@ void select_step(dare_layer* L, const StepGeom& g, int mode, float tau, bool bes
   const bool all = !L->has_prev || mode == DARE_MODE_DENSE;
   const bool own = L->reuse_count >= 0 && !all, inside = own && kth_score_in_select(g.tokens());
   L->last_tau_on_device = own;
-  if (own && !inside) { launch_kth_score(B.scores, g.tokens(), L->reuse_count, B.tau_dev, st); ++*launches; }
+  if (own && !inside) {
+    launch_kth_score(B.scores, g.tokens(), L->reuse_count, B.tau_dev, st, B.status, L->inject == 3);
+    ++*launches;
+  }
   launch_select(B.scores, tau, all, g, B.idx, B.count, B.batch_off, B.delta, st, beside_predecessor,
                 own ? B.tau_dev : nullptr, inside ? L->reuse_count : -1);
   ++*launches;
@@ -627,7 +630,8 @@ dare_status_t dare_layer_debug_wait_probe(dare_layer_t* L, uint64_t limit_ns, ui
 dare_status_t dare_layer_debug_inject(dare_layer_t* L, int what) {
   dare_status_t s = check_handle(L);
   if (s != DARE_OK) return s;
-  if (what < 0 || what > 2) return DARE_ERR_INVALID_ARG;
+  if (what < 0 || what > 3) return DARE_ERR_INVALID_ARG;
+  if (what == 3 && L->use_tc) return DARE_ERR_UNSUPPORTED;   // (with a time-out standing that path's waits would give up early)
   L->inject = what;
   return DARE_OK;
 }

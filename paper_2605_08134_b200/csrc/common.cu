@@ -374,8 +374,8 @@ __global__ void __launch_bounds__(1024) kth_score_kernel(const float* __restrict
   if (threadIdx.x == 0) *tau_out = tau;
 }
 bool kth_score_in_select(int n) { return n <= kKthInCta; }
-cudaError_t launch_kth_score(const float* scores, int n, int k, float* tau_out, cudaStream_t st) {
-  if (n > kKthInCta) return launch_kth_score_large(scores, n, k, tau_out, st);
+cudaError_t launch_kth_score(const float* scores, int n, int k, float* tau_out, cudaStream_t st, int* status, bool lose_one) {
+  if (n > kKthInCta) return launch_kth_score_large(scores, n, k, tau_out, st, status, lose_one);
   return launch_pdl(kth_score_kernel, dim3(1), dim3(1024), 0, st, 1, scores, n, k, tau_out);
 }
 

@@ -133,9 +133,12 @@ void launch_select(const float* scores, float tau, bool select_all, const StepGe
 // selection works it out from the scores and leaves it there
 bool kth_score_in_select(int n);
 // *tau_out = the k-th smallest of n scores: one CTA up to kth_score_in_select's limit (common.cu), one cluster beyond
-// (select_large.cu)
-cudaError_t launch_kth_score(const float* scores, int n, int k, float* tau_out, cudaStream_t st);
-cudaError_t launch_kth_score_large(const float* scores, int n, int k, float* tau_out, cudaStream_t st);
+// (select_large.cu), whose CTAs wait for one another: a wait that runs out is recorded in *status (if given) and leaves
+// NaN.  lose_one: diagnostics, lets one run out.
+cudaError_t launch_kth_score(const float* scores, int n, int k, float* tau_out, cudaStream_t st, int* status = nullptr,
+                             bool lose_one = false);
+cudaError_t launch_kth_score_large(const float* scores, int n, int k, float* tau_out, cudaStream_t st, int* status,
+                                   bool lose_one);
 // dst[r, :] = src[idx[r] (or its cache row), :] for the rows of a step's refresh set
 template <typename T>
 void launch_gather_step_rows(const T* src, const int* idx, const int* count, T* dst, const StepGeom& g, bool by_cache_row,

@@ -246,12 +246,19 @@ __global__ void __launch_bounds__(kTileWords) tile_scatter_kernel(const unsigned
 // 256 of them, which most scores lie outside; a bracket that turns out not to hold the rank is given up for all keys.
 // A cluster (rather than a grid) because the call has no scratch memory to meet in: nothing is shared between calls,
 // whatever streams they run on.
+// A CTA that waits in vain for the others' bins records the time-out in the status word (if the caller has one), gives the
+// copies still on their way to it as long again, and says so in place of its total: all CTAs then leave together, and the
+// threshold is NaN, which Eq. 2 reads as "refresh everything".
 constexpr int kKthBins = 2048, kKthMaxCtas = 16, kKthSample = 256;
 constexpr int kKthBracket = 1 << 19;        // the sample costs about 4 us: from this many scores on
 constexpr unsigned kKeyMinusInf = 0x007fffffu, kKeyPlusInf = 0xff800000u;
 
+constexpr int kKthLost = -2;                // s_bin: some CTA's bins never came
+constexpr unsigned long long kKthLoseWaitNs = 1000000ull;
+
+// lose_one (diagnostics): CTA 0 keeps its bins from CTA 1, whose wait for them then runs out, after a millisecond.
 __global__ void __launch_bounds__(kThreads) kth_cluster_kernel(const float* __restrict__ scores, int n, int k,
-                                                               float* __restrict__ tau_out) {
+                                                               float* __restrict__ tau_out, int* status, int lose_one) {
   __shared__ __align__(16) int hist[kKthBins];
   __shared__ __align__(16) int recv[kKthBins];        // [sender][bin of this CTA's slice]
   __shared__ uint64_t recv_bar;
@@ -305,10 +312,10 @@ __global__ void __launch_bounds__(kThreads) kth_cluster_kernel(const float* __re
   __syncthreads();
   unsigned lo = s_lo, hi = s_hi;                      // keys in [lo, hi]
   int rank = k;                                       // of the wanted key: among all of them, then among those in the range
-  bool found = false, numbers = true;                 // numbers: rank k falls among the scores that are numbers
+  bool found = false, numbers = true, lost = false;   // numbers: rank k falls among the scores that are numbers
   ptx::cluster_sync_all();                            // every CTA's barrier is set up
   uint32_t phase = 0;
-  for (bool first = true, whole = lo == kKeyMinusInf && hi == kKeyPlusInf; !found && numbers; ) {
+  for (bool first = true, whole = lo == kKeyMinusInf && hi == kKeyPlusInf; !found && numbers && !lost; ) {
     const unsigned range = hi - lo;
     const int shift = range < (unsigned)kKthBins ? 0 : 21 - __clz((int)range);
     for (int b = tid; b < kKthBins; b += kThreads) hist[b] = 0;
@@ -358,11 +365,13 @@ __global__ void __launch_bounds__(kThreads) kth_cluster_kernel(const float* __re
     if (tid == 0) ptx::mbar_arrive_expect_tx(&recv_bar, (uint32_t)kKthBins * 4u);
     ptx::fence_proxy_async_smem();
     __syncthreads();
-    if (tid < ctas)                                   // slice `tid` of this CTA's bins goes to CTA `tid`
+    if (tid < ctas && !(lose_one && rank_cta == 0 && tid == 1))       // slice `tid` of this CTA's bins goes to CTA `tid`
       ptx::bulk_copy_to_cta(ptx::map_to_cta(ptx::smem_u32(recv + rank_cta * slice), (uint32_t)tid),
                             ptx::smem_u32(hist + tid * slice), (uint32_t)slice * 4u,
                             ptx::map_to_cta(ptx::smem_u32(&recv_bar), (uint32_t)tid));
-    ptx::mbar_wait(&recv_bar, phase, nullptr);
+    const unsigned long long limit = lose_one ? kKthLoseWaitNs : ptx::kWaitLimitNs;
+    const bool came = ptx::mbar_wait(&recv_bar, phase, status, limit);
+    if (!came) ptx::mbar_wait(&recv_bar, phase, nullptr, limit);      // (nobody leaves before what is on its way has landed)
     phase ^= 1;
     if (tid < slice) {
       int mine = 0;
@@ -372,10 +381,10 @@ __global__ void __launch_bounds__(kThreads) kth_cluster_kernel(const float* __re
       mine = __reduce_add_sync(0xffffffffu, mine);
       if (lane == 0) part[tid >> 5] = mine;
     }
-    __syncthreads();
+    const bool all_came = __syncthreads_and(came) != 0;
     if (tid < ctas) {                                 // the slice's total goes to every CTA, and what lies below the range
-      int tot = 0;
-      for (int w = 0; w < slice / 32; ++w) tot += part[w];
+      int tot = all_came ? 0 : -1;
+      for (int w = 0; all_came && w < slice / 32; ++w) tot += part[w];
       ptx::st_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&totals[rank_cta]), (uint32_t)tid), (uint32_t)tot);
       ptx::st_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&below[rank_cta]), (uint32_t)tid), (uint32_t)s_below);
     }
@@ -385,7 +394,9 @@ __global__ void __launch_bounds__(kThreads) kth_cluster_kernel(const float* __re
       if (first) want -= __reduce_add_sync(0xffffffffu, lane < ctas ? below[lane] : 0);
       const int st = lane < ctas ? totals[lane] : 0, inc = scan(st);
       const unsigned hit = __ballot_sync(0xffffffffu, inc - st < want && want <= inc);
-      if (hit != 0u) {
+      if (__any_sync(0xffffffffu, st < 0)) {
+        if (lane == 0) s_bin = kKthLost;
+      } else if (hit != 0u) {
         const int sl = __ffs((int)hit) - 1, per = slice / 32;
         const int before = __shfl_sync(0xffffffffu, inc - st, sl);
         int c[8], tot = 0;
@@ -410,6 +421,8 @@ __global__ void __launch_bounds__(kThreads) kth_cluster_kernel(const float* __re
       rank = s_rank;
       found = shift == 0;
       first = false;
+    } else if (bin == kKthLost) {
+      lost = true;
     } else if (first && !whole) {                     // the bracket does not hold the rank: all keys
       lo = kKeyMinusInf; hi = kKeyPlusInf; whole = true;
     } else {
@@ -417,7 +430,7 @@ __global__ void __launch_bounds__(kThreads) kth_cluster_kernel(const float* __re
     }
     __syncthreads();
   }
-  if (rank_cta == 0 && tid == 0) *tau_out = numbers ? key_score(lo) : __int_as_float(0x7f800000);
+  if (rank_cta == 0 && tid == 0) *tau_out = lost ? __int_as_float(0x7fc00000) : (numbers ? key_score(lo) : __int_as_float(0x7f800000));
   ptx::cluster_sync_all();                            // nobody leaves while its bins are being read
 }
 // ---- compaction of up to kClusterSelect scores by one cluster in one launch: every CTA decides on a contiguous share
@@ -508,12 +521,13 @@ static cudaError_t launch_cluster(void (*kernel)(KArgs...), cudaStream_t st, Arg
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
-cudaError_t launch_kth_score_large(const float* scores, int n, int k, float* tau_out, cudaStream_t st) {
+cudaError_t launch_kth_score_large(const float* scores, int n, int k, float* tau_out, cudaStream_t st, int* status,
+                                   bool lose_one) {
   if (k <= 0 || k >= n) {
     set_float_kernel<<<1, 1, 0, st>>>(tau_out, k <= 0 ? -INFINITY : INFINITY);
     return cudaGetLastError();
   }
-  return launch_cluster(kth_cluster_kernel, st, scores, n, k, tau_out);
+  return launch_cluster(kth_cluster_kernel, st, scores, n, k, tau_out, status, lose_one ? 1 : 0);
 }
 
 int select_large_tiles(long long n) { return (int)((n + kTile - 1) / kTile); }

@@ -92,3 +92,40 @@ def test_selection_values_out_of_range_are_flagged_and_skipped(dare, case, what)
     _two_steps_ok(dare, g, o, hs, shape)
     assert g.status() == dare.OK
     g.close()
+
+
+def test_a_lost_copy_in_the_threshold_exchange_is_flagged_and_refreshes_everything(dare):
+    """More than 16384 tokens: the blocks that work the threshold out wait for one another's bins.  One copy is withheld: the
+    wait gives up, the status word says so, the threshold is NaN and the step is the one that refreshes every token."""
+    shape = wl.scaled(wl.TINY_F32, d_model=64, n_heads=2, head_dim=32, batch=130, seq=127, prompt=60)
+    w = wl.make_weights(shape, 21)
+    hs = wl.HiddenStream(shape, 21)
+    g = dare.Layer(shape, w)
+    o = parity.oracle_layer(shape, w)
+    parity.compare_step(g, o, hs.first(), 3, 0.1, shape, first=True)
+    changed = wl.uniform_positions(hs.rng, shape, 20)
+    k = shape.tokens - int(changed.sum())
+    x = hs.advance(changed)
+    g.inject(3)
+    y = g.step_quantile(parity.to_device(x, shape), 3, k)
+    assert g.status() == dare.ERR_TIMEOUT
+    assert np.isnan(g.last_threshold())
+    sel = g.last_selection(shape.batch, shape.seq)
+    assert sel["count"] == shape.tokens and not sel["delta"].any()
+    yo = o.step(x, 3, -1.0)
+    parity.assert_close("y", y.cpu().numpy(), yo, parity.TOL_F32, rel_rms=parity.TOL_F32)
+    g.clear_status()
+    changed = wl.uniform_positions(hs.rng, shape, 20)             # the handle goes on: the next step is an ordinary one
+    x = hs.advance(changed)
+    y = g.step_quantile(parity.to_device(x, shape), 3, k)
+    yo = o.step(x, 3, 0.1)
+    assert g.status() == dare.OK
+    np.testing.assert_array_equal(g.last_selection(shape.batch, shape.seq)["idx"], o.last_idx)
+    parity.assert_close("y", y.cpu().numpy(), yo, parity.TOL_F32, rel_rms=parity.TOL_F32)
+    with pytest.raises(dare.DareError):
+        g.inject(4)
+    g.close()
+    t = dare.Layer(SMALL_BF16, wl.make_weights(SMALL_BF16, 5), kernel_path=dare.PATH_TENSOR)
+    with pytest.raises(dare.DareError):
+        t.inject(3)
+    t.close()

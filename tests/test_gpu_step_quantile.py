@@ -121,3 +121,47 @@ def test_step_with_its_own_threshold(dare, name, shape, path):
         g.step_quantile(parity.to_device(x1, shape), 3, -1)
     assert g.status() == 0
     g.close()
+
+
+LONG = [("fp32-cuda-core", wl.scaled(wl.TINY_F32, d_model=64, n_heads=2, head_dim=32, batch=130, seq=127, prompt=60), "simt"),
+        ("bf16-tensor", wl.scaled(wl.LLADA_LAYER, d_model=256, n_heads=2, batch=9, seq=1900, prompt=300), "tensor")]
+
+
+@pytest.mark.parametrize("name,shape,path", LONG, ids=[c[0] for c in LONG])
+def test_step_whose_tokens_are_ranked_by_a_cluster(dare, name, shape, path):
+    """More than 16384 tokens: the threshold is a launch of its own.  With as many reused tokens as are unchanged the whole
+    step must be the oracle's at a threshold between the two modes of the scores; at other counts (inside either mode) the
+    threshold is the order statistic of the step's own scores, bit for bit, and the refresh set is Eq. 2 with it."""
+    w = wl.make_weights(shape, 77)
+    hs = wl.HiddenStream(shape, 77)
+    x0 = hs.first()
+    changed = wl.uniform_positions(hs.rng, shape, max(1, shape.seq // 8))
+    x1 = hs.advance(changed)
+    T = shape.tokens
+    k = T - int(changed.sum())
+    assert T > 16384
+    o = parity.oracle_layer(shape, w)
+    o.step(x0, 3, 0.1)
+    yo = o.step(x1, 3, 0.1)
+    g = dare.Layer(shape, w, kernel_path={"simt": dare.PATH_SIMT, "tensor": dare.PATH_TENSOR}[path])
+    g.step(parity.to_device(x0, shape), 3, 0.1)
+    yg = g.step_quantile(parity.to_device(x1, shape), 3, k)
+    sel = g.last_selection(shape.batch, shape.seq)
+    np.testing.assert_array_equal(sel["idx"], o.last_idx)
+    np.testing.assert_array_equal(sel["batch_off"], o.last_batch_off)
+    np.testing.assert_array_equal(sel["delta"], o.delta[:shape.batch, :shape.seq])
+    assert g.last_threshold() == np.sort(sel["scores"])[k - 1]
+    tol = parity.tol_of(shape.dtype)
+    parity.assert_close("y", yg.float().cpu().numpy(), yo, tol, rel_rms=tol)
+    c = g.read_caches(shape.batch, shape.seq)
+    mf = 2.0 if shape.dtype == wl.DTYPE_BF16 else 1.0
+    parity.assert_close("k_cache", c["k"], o.k_cache, tol, max_factor=mf)
+    parity.assert_close("o_cache", c["o"], o.o_cache, tol, max_factor=mf)
+    for i, kk in enumerate((1, k // 2, k + 5, T - 1, 0, T)):
+        g.step_quantile(parity.to_device((x0, x1)[i % 2], shape), (3, 1, 2)[i % 3], kk)
+        sel = g.last_selection(shape.batch, shape.seq)
+        want = np.float32(tor.step_threshold(sel["scores"].tolist(), kk))
+        assert np.float32(g.last_threshold()) == want, (kk, want)
+        np.testing.assert_array_equal(sel["idx"], np.nonzero(orc.refresh_mask(sel["scores"], want))[0])
+    assert g.status() == 0
+    g.close()
