@@ -130,7 +130,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const int ksplit = SPLIT ? (int)gridDim.z : 1;     // = cluster size along z
   const int z = SPLIT ? (int)cluster_ctarank() : 0;
-  const bool dbg = p.debug != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0;
+  const bool dbg = p.debug != nullptr && blockIdx.x == 0 && blockIdx.z == 0;
   if (dbg && threadIdx.x == 0) p.debug[0] = globaltimer_ns();
   const StepGeom& g = p.g;
   // CTA -> (head, sequence, row tile), in launch order:
@@ -141,7 +141,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   //               every row tile again
   int h, b, tile;
   {
-    const int lin = blockIdx.y * gridDim.x + blockIdx.x;
+    const int lin = blockIdx.x;                       // (a flat grid: its other dimensions stop at 65535)
     if (p.idx != nullptr) {
       h = lin % g.n_heads;
       const int rest = lin / g.n_heads;
@@ -639,7 +639,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
   const int tps = (g.seq_act + kPairRows - 1) / kPairRows;
   int h, b, tile;
   {
-    const int lin = blockIdx.y * gridDim.x + blockIdx.x;
+    const int lin = blockIdx.x;                       // (a flat grid: its other dimensions stop at 65535)
     if (idx != nullptr) {
       h = lin % g.n_heads;
       const int rest = lin / g.n_heads;
@@ -658,7 +658,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
   }
   // diagnostics: [0] first CTA's start, [1] its set-up done, [3] its key loop done, [4] its end; over the CTAs with
   // work: [5] latest start, [6] latest end, [7] their number
-  const bool dbg = p.debug != nullptr && blockIdx.x == 0 && blockIdx.y == 0;
+  const bool dbg = p.debug != nullptr && blockIdx.x == 0;
   unsigned long long t_start = 0;
   if (p.debug != nullptr && threadIdx.x == 0) {
     t_start = globaltimer_ns();
@@ -987,12 +987,12 @@ static cudaError_t launch_attention_hd(const KvMaps& maps, const AttnParams& p, 
   int ksplit = 1;
   const bool pair = pick_form(p.g, p.idx != nullptr, &ksplit);
   if (pair) {
-    dim3 grid(p.g.n_heads, p.g.batch * tps2, 1);
-    if (grid.y == 0) return cudaSuccess;
+    dim3 grid(p.g.n_heads * p.g.batch * tps2, 1, 1);
+    if (grid.x == 0) return cudaSuccess;
     return launch_pdl(attn_pair_kernel<HD>, grid, dim3(kThreads), PairSmem<HD>::TOTAL, st, 1, maps.k128, maps.v128, p);
   }
-  dim3 grid(p.g.n_heads, p.g.batch * tps, ksplit);
-  if (grid.y == 0) return cudaSuccess;
+  dim3 grid(p.g.n_heads * p.g.batch * tps, 1, ksplit);
+  if (grid.x == 0) return cudaSuccess;
   return launch_pdl(ksplit > 1 ? attn_tc_kernel<HD, true> : attn_tc_kernel<HD, false>, grid, dim3(kThreads), AttnSmem<HD>::TOTAL, st, ksplit, maps.k64,
                     maps.v64, p);
 }

@@ -391,7 +391,10 @@ __global__ void __launch_bounds__(128 * RG * KG, 1) sattn_kernel(const SattnPara
   const StepGeom& g = p.g;
   const int tid = threadIdx.x, grp = tid / (128 * RG), lt = tid % (128 * RG), tx = tid & 15, ty = lt >> 4;   // key group; row
   const int r0 = (ty >> 3) * 32 + (ty & 7);                             // this thread's rows: r0 + 8 i
-  const int h = blockIdx.x, b = blockIdx.y, tile = blockIdx.z, d = g.d;
+  // one flat grid (the other two dimensions stop at 65535): heads fastest, then sequences, then row tiles, so that the first
+  // row tile of every sequence, the one that has work when a refresh set is small, comes first
+  const int lin = blockIdx.x, rest = lin / g.n_heads, h = lin - rest * g.n_heads;
+  const int tile = rest / g.batch, b = rest - tile * g.batch, d = g.d;
   // The kernel before (the K/V projection) writes the caches only; queries and refresh set come from kernels further back,
   // complete by the time any CTA of this grid runs: they are read, through the L2, ahead of the wait.
   int row0, n_rows;
@@ -596,8 +599,8 @@ cudaError_t launch_sattn_as(const SattnParams& p, cudaStream_t st) {
   static std::atomic<unsigned long long> attr_done{0};
   auto kern = sattn_kernel<T, HD, RG, KG>;
   if (cudaError_t e = ensure_dyn_smem(kern, S::SMEM, attr_done); e != cudaSuccess) return e;
-  return launch_pdl(kern, dim3(p.g.n_heads, p.g.batch, (p.g.seq_act + S::BQ - 1) / S::BQ), dim3(S::THREADS), S::SMEM, st, 1,
-                    p);
+  return launch_pdl(kern, dim3(p.g.n_heads * p.g.batch * ((p.g.seq_act + S::BQ - 1) / S::BQ)), dim3(S::THREADS), S::SMEM, st,
+                    1, p);
 }
 template <typename T, int HD>
 cudaError_t launch_sattn_hd(const SattnParams& p, cudaStream_t st) {
