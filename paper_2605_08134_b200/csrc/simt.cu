@@ -112,7 +112,8 @@ __global__ void __launch_bounds__(kSgThreads, 1) sgemm_kernel(const SgemmParams 
   };
   // the weights do not depend on the kernel before: their first stages are on their way while it drains
   // (row tiles past the first of a gathered launch are usually empty: they look at the count first)
-  const bool likely = p.count == nullptr || blockIdx.y == 0;
+  const int m0 = (int)(blockIdx.z * gridDim.y + blockIdx.y) * BM;
+  const bool likely = p.count == nullptr || m0 == 0;
   auto fetch_w = [&]() {
 #pragma unroll
     for (int kb = 0; kb < kStages - 1; ++kb)
@@ -121,7 +122,6 @@ __global__ void __launch_bounds__(kSgThreads, 1) sgemm_kernel(const SgemmParams 
   if (likely) fetch_w();
   pdl_wait();
   pdl_launch_dependents();
-  const int m0 = (int)blockIdx.y * BM;
   const int m_eff = p.count ? checked_count(*p.count, p.rows, p.status) : p.rows;
   if (m0 >= m_eff) {                             // uniform over the CTA
     cp_async_commit();
@@ -320,7 +320,9 @@ cudaError_t launch_sgemm_as(const SgemmParams& p, int n_tiles, cudaStream_t st) 
   static std::atomic<unsigned long long> attr_done{0};
   auto kern = sgemm_kernel<T, EPI, RM, WM, KG>;
   if (cudaError_t e = ensure_dyn_smem(kern, S::SMEM, attr_done); e != cudaSuccess) return e;
-  return launch_pdl(kern, dim3(n_tiles, (p.rows + S::BM - 1) / S::BM), dim3(S::THREADS), S::SMEM, st, 1, p);
+  // row tiles over y and z: one dimension of a grid stops at 65535 (a CTA past the last tile leaves)
+  const int row_tiles = (p.rows + S::BM - 1) / S::BM, nz = (row_tiles + 65534) / 65535;
+  return launch_pdl(kern, dim3(n_tiles, (row_tiles + nz - 1) / nz, nz), dim3(S::THREADS), S::SMEM, st, 1, p);
 }
 // rows_likely: rows that the launch is sized for (a gathered launch's count is known to the device only).
 template <typename T, int EPI>

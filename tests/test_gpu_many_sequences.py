@@ -52,3 +52,8 @@ def steps_of_many_sequences(dtype, d_model, head_dim, batch, seq, plan):
 @pytest.mark.parametrize("case", range(len(CASES)))
 def test_steps_of_many_short_sequences(case):
     steps_of_many_sequences(*CASES[case], plan=[(3, 0), (1, 0), (3, 1)])
+
+
+def test_steps_of_more_row_tiles_than_one_grid_dimension():
+    """65600 row tiles of 96 in the CUDA-core projections."""
+    steps_of_many_sequences(wl.DTYPE_F32, 32, 32, 65_600, 96, plan=[(3, 0)])
