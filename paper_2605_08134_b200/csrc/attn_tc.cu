@@ -17,7 +17,8 @@
 //                chain S -> softmax -> P V -> S)
 //   warps 4+4s.. four softmax warps, thread <-> query row: reads its row of S from tensor memory, exponentiates, and
 //                writes P as bf16 over the first 32 columns of S (two keys per 32-bit column, the layout of a
-//                tensor-memory A operand), so P never passes through shared memory.  O accumulates in tensor
+//                tensor-memory A operand; heads of 64: a second part over the other 32), so P never passes through
+//                shared memory.  O accumulates in tensor
 //                memory; it is rescaled in place only when the running maximum has grown by more than 2^8 (the
 //                exponentials are taken against the older maximum until then, which changes nothing in exact
 //                arithmetic: numerator and row sum share the factor).
@@ -94,6 +95,13 @@ constexpr uint32_t kTmemCols = 512;
 constexpr int kPairMinDense = 128;      // dense launches with longer windows take the two-tile kernel
 constexpr int kPairMinSparse = 1024;    // row-sparse launches from this window length on
 constexpr float kRescaleStep = 8.f;     // log2 of the growth of the running maximum that triggers a rescale of O
+// Heads of 64: P as two bf16 parts, the rounded weight and what the rounding left (together 16 bits of mantissa), each
+// multiplied with V: the parts of a block of 64 keys take the 64 columns its scores had.  One bf16 part leaves the output
+// 1.37-1.41 times as far from exact as its own bf16 storage does (2.3e-3 against 1.66e-3 relative, 57 to 2048 keys); two
+// parts add nothing to the storage, like the CUDA-core kernels these heads had before.  Heads of 128 have always had one.
+// The second product costs a step of 2 x 512 tokens of width 2048 0.6 of 56.1 us.
+template <int HD>
+constexpr bool kSplitP = HD == 64;
 
 // The HD / 64 chunks of a key (or value) block, 64 columns of KEYS rows each, counted on one barrier.
 template <int HD, int KEYS>
@@ -321,9 +329,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       if (elect_one()) {
         const uint64_t v_desc = v_desc0 + (uint64_t)(rs * (S::V_BYTES >> 4));
 #pragma unroll
-        for (int ks = 0; ks < BK1 / 16; ++ks)       // 16 keys of P = 8 columns
+        for (int ks = 0; ks < BK1 / 16; ++ks) {     // 16 keys of P = 8 columns
           umma_ts(tmem_o, tmem_s + (j & 1) * BK1 + ks * 8, v_desc + ((ks * (16 * 128)) >> 4), idesc_pv,
                   (j | ks) != 0 ? 1u : 0u);
+          if (kSplitP<HD>) umma_ts(tmem_o, tmem_s + (j & 1) * BK1 + 32 + ks * 8, v_desc + ((ks * (16 * 128)) >> 4), idesc_pv, 1u);
+        }
         umma_commit(&o_full[2 * st + (j & 1)]);
         umma_commit(&v_empty[st * kRing1 + rs]);
       }
@@ -403,7 +413,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       // instruction (packed fp32)
       const float2 c2 = make_float2(c, c), nmc2 = make_float2(-m * c, -m * c);
       float2 sum2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-      float pk[BK1 / 2];                            // P as bf16: column i = keys (2i, 2i+1)
+      float pk[BK1 / 2], pl[kSplitP<HD> ? BK1 / 2 : 1];                            // P as bf16: column i = keys (2i, 2i+1)
 #pragma unroll
       for (int i = 0; i < BK1; i += 2) {
         float2 e = __ffma2_rn(make_float2(v[i], v[i + 1]), c2, nmc2);
@@ -412,8 +422,14 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         sum2[(i >> 1) & 1] = __fadd2_rn(sum2[(i >> 1) & 1], e);
         __nv_bfloat162 h2 = __floats2bfloat162_rn(e.x, e.y);
         pk[i >> 1] = __uint_as_float(*reinterpret_cast<uint32_t*>(&h2));
+        if (kSplitP<HD>) {
+          const float2 r = __fadd2_rn(e, make_float2(-__low2float(h2), -__high2float(h2)));
+          __nv_bfloat162 l2 = __floats2bfloat162_rn(r.x, r.y);
+          pl[kSplitP<HD> ? i >> 1 : 0] = __uint_as_float(*reinterpret_cast<uint32_t*>(&l2));
+        }
       }
       tmem_st_32x32_nowait(sbuf, pk);
+      if (kSplitP<HD>) tmem_st_32x32_nowait(sbuf + 32, pl);
       tmem_st_wait();
       l += (sum2[0].x + sum2[0].y) + (sum2[1].x + sum2[1].y);
       tc_fence_before();
@@ -819,9 +835,11 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
         if (elect_one()) {
           const uint64_t v_desc = v_desc0 + (uint64_t)(slot * (S::KV_BYTES >> 4));
 #pragma unroll
-          for (int k4 = 0; k4 < kHalf / 16; ++k4)
-            umma_ts(tmem_o, tmem_s + hb * kHalf + k4 * 8, v_desc + (((hb * (kHalf / 16) + k4) * (16 * 128)) >> 4), idesc_pv,
-                    (hf | k4) != 0 ? 1u : 0u);
+          for (int k4 = 0; k4 < kHalf / 16; ++k4) {
+            const uint64_t v16 = v_desc + (((hb * (kHalf / 16) + k4) * (16 * 128)) >> 4);
+            umma_ts(tmem_o, tmem_s + hb * kHalf + k4 * 8, v16, idesc_pv, (hf | k4) != 0 ? 1u : 0u);
+            if (kSplitP<HD>) umma_ts(tmem_o, tmem_s + hb * kHalf + 32 + k4 * 8, v16, idesc_pv, 1u);
+          }
           umma_commit(&o_full[2 * st + hb]);
           if (hb == 1 || hf == n_half - 1) umma_commit(&v_empty[slot]);
         }
@@ -894,7 +912,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
       }
       const float2 c2 = make_float2(c, c), nmc2 = make_float2(-m * c, -m * c);
       float2 sum2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-      float pk[kHalf / 2];
+      float pk[kHalf / 2], pl[kSplitP<HD> ? kHalf / 2 : 1];
 #pragma unroll
       for (int i = 0; i < kHalf; i += 2) {
         float2 e = __ffma2_rn(make_float2(v[i], v[i + 1]), c2, nmc2);
@@ -903,8 +921,14 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
         sum2[(i >> 1) & 1] = __fadd2_rn(sum2[(i >> 1) & 1], e);
         __nv_bfloat162 h2 = __floats2bfloat162_rn(e.x, e.y);
         pk[i >> 1] = __uint_as_float(*reinterpret_cast<uint32_t*>(&h2));
+        if (kSplitP<HD>) {
+          const float2 r = __fadd2_rn(e, make_float2(-__low2float(h2), -__high2float(h2)));
+          __nv_bfloat162 l2 = __floats2bfloat162_rn(r.x, r.y);
+          pl[kSplitP<HD> ? i >> 1 : 0] = __uint_as_float(*reinterpret_cast<uint32_t*>(&l2));
+        }
       }
       tmem_st_32x32_nowait(sbuf, pk);
+      if (kSplitP<HD>) tmem_st_32x32_nowait(sbuf + 32, pl);
       tmem_st_wait();
       l += (sum2[0].x + sum2[0].y) + (sum2[1].x + sum2[1].y);
       tc_fence_before();
