@@ -640,11 +640,8 @@ const char* dare_kernel_slot_name(int slot) {
   switch (slot) {
     case SLOT_NORM: return "rmsnorm";
     case SLOT_Q_GEMM: return "q_gemm";
-    case SLOT_Q_POST: return "q_post";
     case SLOT_SELECT: return "select_compact";
-    case SLOT_GATHER: return "gather_rows";
     case SLOT_KV_GEMM: return "kv_gemm";
-    case SLOT_KV_POST: return "kv_post";
     case SLOT_ATTN: return "attention";
     case SLOT_OUT_GEMM: return "out_gemm";
   }

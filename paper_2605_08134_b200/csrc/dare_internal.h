@@ -184,8 +184,6 @@ template <typename T>
 cudaError_t launch_out_simt(const SimtStep& s, const T* oc, const T* w_o, T* y, cudaStream_t st);
 
 // ---- tensor-core path (gemm_tc.cu, attn_tc.cu) -----------------------------------------------------------
-struct TcLayerMaps;  // tensor maps and launch state, owned by the handle
 bool tc_supported(const dare_layer_config_t& cfg);
-size_t tc_maps_bytes();
 
 }  // namespace dare

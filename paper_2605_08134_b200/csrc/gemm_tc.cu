@@ -124,7 +124,7 @@ __device__ __forceinline__ void load_row_batch(RowBatch<RB>& rb, const GemmParam
 
 // FLAT: row tiles run on across sequences (p.flat, p.a_piece); a kernel of its own because the row mapping sits on the
 // critical path of every tile (0.5-1 us a launch when all launches carried it).
-// FOUR: the reduction is split in four (for the same reason).
+// FOUR: the reduction is split in four (for the same reason; narrow single-CTA tiles only).
 template <int EPI, int BN, bool PAIR, int HDIM, bool FLAT, bool FOUR>
 __global__ void __launch_bounds__(Warps<BN>::N * 32, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b0,
@@ -687,7 +687,7 @@ static cudaError_t launch_as(const CUtensorMap& a, const CUtensorMap& b0, const 
 template <int EPI, int BN, bool PAIR, int HDIM, bool FLAT>
 static cudaError_t launch_split(const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1, const GemmParams& p,
                                 int n_tiles, int m_tiles, int splits, cudaStream_t st) {
-  if constexpr (BN == 128) {
+  if constexpr (BN == 128 && !PAIR) {
     if (splits == 4) return launch_as<EPI, BN, PAIR, HDIM, FLAT, true>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
   }
   return launch_as<EPI, BN, PAIR, HDIM, FLAT, false>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
@@ -716,7 +716,7 @@ cudaError_t launch_gemm_tc(int epi, int bn, const CUtensorMap& a, const CUtensor
                            const GemmParams& p, int n_tiles, int m_tiles, int splits, cudaStream_t st, int pair) {
   if (m_tiles <= 0 || n_tiles <= 0) return cudaSuccess;
   if (epi == EPI_OUT && p.resid != nullptr) epi = EPI_OUT_RES;
-  if ((splits != 1 && splits != 2 && (splits != 4 || bn != 128)) || p.K / BK % splits != 0) return cudaErrorInvalidValue;
+  if ((splits != 1 && splits != 2 && (splits != 4 || bn != 128 || pair)) || p.K / BK % splits != 0) return cudaErrorInvalidValue;
   if (pair && bn == 128) {
     // narrow pair tiles (256 rows x 128 columns per pair; b0 / b1 with 64-row boxes): twice the CTAs of the wide ones
     // for launches of two row tiles, whose main loops are bound by what one SM can pull from the L2

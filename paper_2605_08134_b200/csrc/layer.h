@@ -30,9 +30,9 @@ struct Buffers {
 
 struct TcState;
 
-// Kernel slots for the optional per-kernel timing.
-enum { SLOT_NORM = 0, SLOT_Q_GEMM, SLOT_Q_POST, SLOT_SELECT, SLOT_GATHER, SLOT_KV_GEMM, SLOT_KV_POST, SLOT_ATTN,
-       SLOT_OUT_GEMM, SLOT_COUNT };
+// Kernel slots for the optional per-kernel timing (the numbers are what callers see: those of kernels that are gone stay
+// unused).
+enum { SLOT_NORM = 0, SLOT_Q_GEMM = 1, SLOT_SELECT = 3, SLOT_KV_GEMM = 5, SLOT_ATTN = 7, SLOT_OUT_GEMM = 8 };
 constexpr int kMaxMarks = 16;
 
 }  // namespace dare

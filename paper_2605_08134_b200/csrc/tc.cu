@@ -70,7 +70,6 @@ bool make_map(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, ui
 bool tc_supported(const dare_layer_config_t& c) {
   return c.dtype == DARE_BF16 && (c.head_dim == 128 || c.head_dim == 64) && c.d_model % 256 == 0;
 }
-size_t tc_maps_bytes() { return sizeof(TcState); }
 
 dare_status_t tc_create(dare_layer* L) {
   TcState* s = new (std::nothrow) TcState();

@@ -6,7 +6,7 @@ import re
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2605_08134_b200", "csrc")
 # what reaches into another CTA of the cluster, and what shows that it has started
-REMOTE = ("st_cluster_u32", "st_cluster_f4", "ld_cluster_u32", "mbar_arrive_cluster", "bulk_copy_to_cta", "tma_load_2d_pair",
+REMOTE = ("st_cluster_u32", "ld_cluster_u32", "mbar_arrive_cluster", "bulk_copy_to_cta", "tma_load_2d_pair",
           "umma2_ss", "umma2_commit")
 BARRIER = ("cluster_sync_all", "cluster_sync_relaxed", "cluster_wait")
 
