@@ -12,7 +12,9 @@ CASES = [
     (512, 4096, 1, 600),      # five: a padding row tile
     (256, 12544, 3, 128),     # three row tiles of 98 column tiles: persistent SwiGLU, single-CTA tiles
     (512, 1024, 1, 129),      # two row tiles, one wave
-    (256, 12544, 2, 77),      # ... more than one wave
+    (256, 12544, 2, 77),      # ... one wave as well: 66 tiles of 192 outputs on 74 SM pairs
+    (256, 19072, 2, 77),      # ... more than one wave: tiles of 256 (the widest), the 75th half full
+    (256, 38016, 3, 40),      # one row tile, more than one wave: the 149th tile of 256 half full
     (4096, 2048, 2, 640),     # ten row tiles: persistent down projection
     (512, 2048, 2, 31),
 ]
