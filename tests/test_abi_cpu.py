@@ -64,7 +64,7 @@ def test_workspace_bytes_validates_config(dare):
     wrong_size = dare.make_config(256, 4, 64, 1, 128, 1e4, 1e-5, dare.F32)
     wrong_size.struct_size = 8
     assert dare.dare_layer_workspace_bytes(wrong_size) == 0
-    # the tensor-core path only exists for bf16 with head_dim 128
+    # the tensor-core path only exists for bf16 (head_dim 64 or 128)
     assert dare.dare_layer_workspace_bytes(
         dare.make_config(256, 4, 64, 1, 128, 1e4, 1e-5, dare.F32, kernel_path=dare.PATH_TENSOR)) == 0
 

@@ -1,5 +1,6 @@
 """CUDA-core kernels at the edges of their tiles against the fp64 oracle: every head width, widths that leave a partial
-column tile or k-block, row counts just past a tile, all three tile heights, key counts around a key block."""
+column tile or k-block, row counts just past a tile, all five tile heights of the projections, all four forms of the
+attention kernel (row groups x key groups) at every head width, key counts around a key block."""
 import numpy as np
 import pytest
 
@@ -20,6 +21,16 @@ CASES = [
     (wl.DTYPE_BF16, 96, 32, 2, 47, 16, 1),
     (wl.DTYPE_BF16, 512, 256, 1, 161, 60, 1),
     (wl.DTYPE_BF16, 320, 64, 2, 97, 33, 4),
+    # forms of the attention kernel's dense steps that the cases above do not reach
+    (wl.DTYPE_F32, 64, 32, 25, 65, 20, 1),       # 2 x 2
+    (wl.DTYPE_F32, 96, 32, 25, 33, 7, 2),        # 3 x 1
+    (wl.DTYPE_F32, 32, 32, 38, 300, 50, 0),      # 4 x 1
+    (wl.DTYPE_F32, 64, 64, 38, 300, 50, 0),
+    (wl.DTYPE_F32, 128, 128, 1, 33, 16, 0),      # 2 x 2
+    (wl.DTYPE_BF16, 256, 128, 32, 193, 60, 1),   # 4 x 1
+    (wl.DTYPE_F32, 768, 256, 25, 33, 8, 2),      # 2 x 2
+    (wl.DTYPE_BF16, 768, 256, 25, 65, 9, 1),     # 3 x 1
+    (wl.DTYPE_F32, 1024, 256, 28, 97, 30, 3),    # 4 x 1
 ]
 
 
