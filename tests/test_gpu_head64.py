@@ -13,7 +13,7 @@ CASES = [
     # d_model, batch, seq, prompt, scoring head
     (256, 1, 57, 20, 1),
     (256, 1, 2300, 252, 0),      # key split
-    (512, 2, 128, 32, 3),        # narrow pair tiles
+    (512, 2, 128, 32, 3),        # narrow tiles split in four, K/V of the dense step in wide pairs
     (512, 5, 1031, 7, 7),        # gathered output projection, 256-wide gathered tiles
     (1024, 8, 1153, 129, 2),     # two query tiles per attention CTA
     (512, 16, 1153, 100, 5),     # persistent projections
