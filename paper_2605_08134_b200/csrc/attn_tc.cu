@@ -991,7 +991,7 @@ bool pick_form(const StepGeom& g, bool row_sparse, int* ksplit_out) {
   // windows are where refresh sets of several tiles are.
   const int tps2 = (g.seq_act + kPairRows - 1) / kPairRows;
   return ksplit == 1 && (row_sparse ? g.seq_act >= kPairMinSparse && g.n_heads * g.batch >= 64
-                                    : g.seq_act > kPairMinDense && g.n_heads * g.batch * tps2 >= 148);
+                                    : g.seq_act > kPairMinDense && g.n_heads * g.batch * tps2 >= kSms);
 }
 }  // namespace
 

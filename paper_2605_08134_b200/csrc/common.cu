@@ -640,7 +640,7 @@ void launch_gather_step_rows(const T* src, const int* idx, const int* count, T* 
                              cudaStream_t st, int* status, int gate_hi) {
   const int T_ = g.tokens();
   if (T_ <= 0) return;
-  const int grid = (T_ + 7) / 8 < 148 * 8 ? (T_ + 7) / 8 : 148 * 8;
+  const int grid = (T_ + 7) / 8 < kSms * 8 ? (T_ + 7) / 8 : kSms * 8;
   launch_pdl(gather_step_rows_kernel<T>, dim3(grid), dim3(256), 0, st, 1, src, idx, count, dst, g, by_cache_row ? 1 : 0,
              status, gate_hi);
 }

@@ -52,6 +52,10 @@ __device__ __forceinline__ float key_score(unsigned key) {
 }
 #endif
 
+// SMs of a B200: what the launch rules count waves with (their constants were measured on it).  A launch that must not be
+// larger than the device, one CTA an SM for good, asks the device instead.
+constexpr int kSms = 148;
+
 // Geometry of one step, passed by value to kernels.
 struct StepGeom {
   int batch;      // B

@@ -538,7 +538,7 @@ cudaError_t launch_drift_scores(const float* a, const float* b, long long rows, 
   if (rows <= 0) return cudaSuccess;
   auto blocks = [&](int rows_per_warp, int per_sm) {
     const long long n = (rows + 8 * rows_per_warp - 1) / (8 * rows_per_warp);
-    return (int)(n < 148 * per_sm ? n : 148 * per_sm);
+    return (int)(n < kSms * per_sm ? n : kSms * per_sm);
   };
   if (hd == 32) drift_score_kernel<8, 1, 4><<<blocks(16, 8), 256, 0, st>>>(a, b, rows, scores);
   else if (hd == 64) drift_score_kernel<16, 1, 4><<<blocks(8, 8), 256, 0, st>>>(a, b, rows, scores);

@@ -329,10 +329,15 @@ template <typename T, int EPI>
 cudaError_t launch_sgemm(const SgemmParams& p, int rows_likely, cudaStream_t st) {
   if (p.rows <= 0) return cudaSuccess;
   const int n_tiles = (p.g.d / 2 + 31) / 32 * (EPI == SG_KV ? 2 : 1);
-  // What a launch takes is its waves of 148 tiles times the tile height over the rate of its inner loop (above), plus what
-  // a tile costs whatever its height (first operands, finishing: measured as about 12 rows).
+  // What a launch takes is its waves of one tile an SM times the tile height over the rate of its inner loop (above), plus
+  // what a tile costs whatever its height (first operands, finishing), about 12 rows: one wave of width 1024 takes 56.0 /
+  // 41.8 / 35.9 / 27.7 / 23.4 us at 96 / 64 / 48 / 32 / 16 rows, 0.51-0.60 us a unit of this cost at every height.
+  // Q projection in us by tile height 96 / 64 / 48 / 32 / 16, fp32, the pick in brackets: width 256, 128 rows 22.8 / 18.4 /
+  // 18.4 / 14.3 / [11.4]; 768, 384 rows 45.9 / 33.9 / 30.6 / [23.6] / 31.9; 512, 768 rows 34.0 / 25.7 / [24.1] / 31.7 / 33.9;
+  // 768, 768 rows 45.9 / [34.8] / 54.0 / 40.4 / 58.9; 1024, 1600 rows [107] / 114 / 125 / 133 / 189.  At all twelve sizes
+  // timed (64 to 1600 rows) the pick was the fastest, for Q and for K/V.
   auto cost = [&](int bm, float f) {
-    return (float)((n_tiles * ((rows_likely + bm - 1) / bm) + 147) / 148) * (12.f + (float)bm * f);
+    return (float)((n_tiles * ((rows_likely + bm - 1) / bm) + kSms - 1) / kSms) * (12.f + (float)bm * f);
   };
   const float c[5] = {cost(96, 1.f), cost(64, 1.1f), cost(48, 1.f), cost(32, 1.1f), cost(16, 1.8f)};
   int best = 0;
@@ -608,10 +613,15 @@ template <typename T, int HD>
 cudaError_t launch_sattn_hd(const SattnParams& p, cudaStream_t st) {
   // rows a sequence is likely to have (a refresh set's size is known to the device only: a quarter of the window)
   const int rows = p.idx ? (p.g.seq_act + 3) / 4 : p.g.seq_act;
-  // waves of 148 CTAs, times the rows of one, times the key blocks its slowest group takes
+  // Waves of one CTA an SM, times the rows of one, times the keys its slowest group takes, times what a row and key cost in
+  // that form beside the 2 x 2 one (heads of 64: 1.2-1.3 / 1 / 1.05-1.1 / 0.97-1.1).  Dense attention in us, row groups x key
+  // groups 1 x 4 / 2 x 2 / 3 x 1 / 4 x 1, fp32, the pick in brackets: 4 heads of 64, 400 rows [24.6] / 36.9 / 51.2 / 63.5; 16
+  // heads of 64, 2 x 384 rows 57.3 / 57.3 / [45.1] / 55.3; 12 heads of 64, 3 x 200 rows 28.7 / [24.6] / 32.8 / 38.9; 8 heads of
+  // 64, 4 x 400 rows [63.5] / 67.6 / 94.2 / 65.5; 4 heads of 256, 4 x 400 rows 143 / [139] / 205 / 262.  Of twelve sizes timed
+  // the pick was the fastest at eleven; 8 heads of 128, 4 x 400 rows: 98.3 / 117 / 176 / [115] (1.15 is too much there).
   auto cost = [&](int bq, int kg, int bkv, float f) {
     const int tiles = p.g.n_heads * p.g.batch * ((rows + bq - 1) / bq), blocks = (p.g.kv_len + bkv - 1) / bkv;
-    return (float)((tiles + 147) / 148) * (float)bq * (float)((blocks + kg - 1) / kg * kg * bkv) * f;
+    return (float)((tiles + kSms - 1) / kSms) * (float)bq * (float)((blocks + kg - 1) / kg * kg * bkv) * f;
   };
   const int b1 = Sa<HD, 1, 4>::BKV, b2 = Sa<HD, 2, 2>::BKV, b3 = Sa<HD, 3, 1>::BKV;
   const float c1 = cost(32, 4, b1, 1.15f), c2 = cost(64, 2, b2, 1.f), c3 = cost(96, 1, b3, 1.05f), c4 = cost(128, 1, b3, 1.f);

@@ -372,7 +372,7 @@ dare_status_t dare_stack_create(const dare_stack_config_t* cfg, const dare_stack
   {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      sms = 148;
+      sms = kSms;
     S->width1 = swiglu_width(cfg->d_ff, sms, false);
     S->width2 = swiglu_width(cfg->d_ff, sms, true);
   }

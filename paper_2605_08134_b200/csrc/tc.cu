@@ -19,7 +19,7 @@ struct TcState {
 namespace {
 
 // units (column tile x pair of row tiles) from which the two-CTA form of a listed launch runs: two rounds of the 74 clusters
-constexpr int kPairUnitGate = 148;
+constexpr int kPairUnitGate = 2 * (kSms / 2);
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
@@ -150,7 +150,7 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
   bool kv_beside_q = !kv_sparse && m_tiles_dense <= 8;
   if (kv_beside_q && persist_pays(2 * d / 256, m_tiles_dense, pick_splits(2 * d / 256 * m_tiles_dense, kblocks))) {
     const int q_ctas = d / 256 * ((m_tiles_dense + 1) / 2 * 2), units = 2 * d / 256 * ((m_tiles_dense + 1) / 2);
-    const float beside = (float)((q_ctas + 2 * d / 256 * m_tiles_dense + 147) / 148) * (9.f + 0.36f * (float)kblocks);
+    const float beside = (float)((q_ctas + 2 * d / 256 * m_tiles_dense + kSms - 1) / kSms) * (9.f + 0.36f * (float)kblocks);
     const float behind = 20.f + 0.33f * (float)(kblocks * (1 + (units + 73) / 74));
     kv_beside_q = beside < behind;
   }

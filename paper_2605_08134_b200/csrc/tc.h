@@ -137,12 +137,24 @@ inline bool pairs_pay(int n_tiles, int m_tiles, int splits) {
 // tiles and more splits (one row tile of 4096 x 4096: 32 CTAs of 32 k-blocks -> 128 of 16), more of them wide ones.
 // Clusters of four CTAs do not cover all 148 SMs, and clusters of eight wait for eight free SMs of one GPC behind the
 // kernel before (a 240-row pass of a 2048-wide stack took 29 % longer with them), so there are none.
+// Q projection in us with an event on either side (the first about 10 us of each figure are those), narrow / narrow split in
+// two / in four / narrow pairs / narrow pairs split in two / wide / wide split in two / wide pairs / wide pairs split in two, the
+// pick in brackets, - where it does not fit one wave:
+//   width 1024,  128 rows: 17.5 / 15.3 / [13.3] / - / - / 19.6 / 17.4 / - / -
+//   width 2048,  512 rows: 22.6 / 17.2 / - / 20.7 / [17.1] / 26.6 / 20.4 / 24.6 / 19.5   (heads of 64; of 128: 17.7 and [17.0])
+//   width 2048, 1024 rows: 23.3 / - / - / 21.5 / - / 26.8 / 20.6 / 25.6 / [20.8]
+//   width 4096,  128 rows: 29.4 / 21.3 / [18.6] / - / - / 38.1 / 25.8 / - / -
+//   width 4096,  256 rows: 30.8 / 22.6 / - / 28.7 / [20.8] / 37.8 / 26.6 / 34.0 / 24.7
+//   width 4096,  512 rows: 31.6 / - / - / 29.0 / - / 38.9 / 27.5 / 34.9 / [26.7]
+//   width 4096, 1024 rows: - / - / - / - / - / 39.6 / - / [37.6] / -
+// At seventeen sizes (widths 512 to 4096, 128 to 1024 rows) the pick is the fastest or within 0.2 us of it, for Q and for the
+// output projection.  (Forms past one wave: two waves of clusters cost 6-8 us more.)
 // `beside`: CTAs of a launch that runs at the same time and should find SMs free; such a form is taken if it takes no
 // longer than `limit_us`, that launch itself.  false: no form.
 struct TileForm { int bn, pair, splits; };
 inline bool pick_one_wave(int d_out, int m_tiles, int kblocks, TileForm* best, int beside = 0,
                           float limit_us = 1e29f) {
-  const float sms = 148.f - (float)beside;
+  const float sms = (float)(kSms - beside);
   float best_us = 1e30f;
   for (int pair = 0; pair < 2; ++pair)
     for (int bn = 128; bn <= 256; bn += 128)
@@ -176,14 +188,14 @@ cudaError_t launch_gemm_persist(int epi, const CUtensorMap& a, const CUtensorMap
                                 const GemmParams& p, int n_tiles, int m_tiles, cudaStream_t st, int pair = 0);
 // ... pays as soon as the tiles are more than one wave: from there on a tile's set-up, pipeline fill and finishing pass
 // hide behind the next tile's main loop.
-inline bool persist_pays(int n_tiles, int m_tiles, int splits) { return splits == 1 && n_tiles * m_tiles > 148; }
+inline bool persist_pays(int n_tiles, int m_tiles, int splits) { return splits == 1 && n_tiles * m_tiles > kSms; }
 // A listed launch comes with a compact copy of its rows and a second form that only looks at the count: from two waves.
-inline bool persist_pays_listed(int n_tiles, int m_tiles) { return n_tiles * m_tiles >= 296; }
+inline bool persist_pays_listed(int n_tiles, int m_tiles) { return n_tiles * m_tiles >= 2 * kSms; }
 // Two-CTA MMAs in it, or single CTAs?  A k-block takes a pair 0.93 of the time it takes a single CTA (644 against 667-690
 // cycles), but pairs walk in waves of 74 units of two row tiles, an odd row tile being padded to a pair.
 inline bool persist_pairs_pay(int n_tiles, int m_tiles) {
   const int units = n_tiles * ((m_tiles + 1) / 2), tiles = n_tiles * m_tiles;
-  return 0.93f * (float)((units + 73) / 74) <= (float)((tiles + 147) / 148);
+  return 0.93f * (float)((units + kSms / 2 - 1) / (kSms / 2)) <= (float)((tiles + kSms - 1) / kSms);
 }
 
 }  // namespace dare
