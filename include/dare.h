@@ -87,9 +87,9 @@ enum {
 
 typedef struct {
   uint32_t struct_size; /* sizeof(dare_layer_config_t), checked */
-  int32_t d_model;      /* = n_heads * head_dim; multiple of 8 */
+  int32_t d_model;      /* = n_heads * head_dim; multiple of 16 */
   int32_t n_heads;
-  int32_t head_dim;     /* even; 32..256 for the SIMT path, 64 or 128 for the tensor-core path */
+  int32_t head_dim;     /* 32, 64, 128 or 256 for the SIMT path, 64 or 128 for the tensor-core path */
   int32_t max_batch;
   int32_t max_seq;
   float rope_theta;     /* rotary base (half-split pairing: element j rotates with j + head_dim/2) */

@@ -70,7 +70,7 @@ size_t carve(const dare_layer_config_t* c, bool use_tc, char* base, Buffers* b) 
   B.debug = (unsigned long long*)take((64 + 3 * 1024) * sizeof(unsigned long long));
   B.x_stage = take(Tm * d * e);
   B.y_stage = take(Tm * d * e);
-  B.tmp = use_tc ? nullptr : (float*)take(Tm * 2 * d * sizeof(float));
+  B.q_raw = use_tc || hd <= 64 ? nullptr : (float*)take(Tm * hd * sizeof(float));
   B.yc = use_tc ? take(Tm * d * e) : nullptr;
   B.tau_dev = (float*)take(sizeof(float));
   return off;
@@ -124,7 +124,7 @@ dare_status_t step_simt(dare_layer_t* L, const T* x, const StepGeom& g, int mode
   const Buffers& B = L->buf;
   const bool kv_sparse = L->has_prev && (mode & DARE_MODE_KV);
   const bool o_sparse = L->has_prev && (mode & DARE_MODE_O);
-  const SimtStep s = {g, B.rope_cs, B.q_prev, B.scores, B.tmp, L->has_prev ? 1 : 0, B.status};
+  const SimtStep s = {g, B.rope_cs, B.q_prev, B.scores, B.q_raw, L->has_prev ? 1 : 0, B.status};
   int launches = 0;
   prof_begin(L);
   // Alg. 1/2 line 1

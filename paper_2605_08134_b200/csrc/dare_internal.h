@@ -166,7 +166,7 @@ struct SimtStep {
   const float* rope_cs;
   float* q_prev;
   float* scores;
-  float* tmp;            // fp32 scratch [T, 2d]
+  float* q_raw;          // heads wider than 64: [T, head_dim] scratch
   int has_prev;
   int* status;
 };

@@ -24,7 +24,7 @@ struct Buffers {
   void* x_stage;    // [T, d] staging for the host-buffer entry point
   void* y_stage;
   void* yc;         // tensor-core path: cache of projected outputs y = W_O O by cache row (gathered output projection)
-  float* tmp;       // SIMT path: fp32 projection results [T, 2d]
+  float* q_raw;     // CUDA-core path, heads wider than 64: [T, head_dim] un-rotated scoring head of every token, fp32
   float* tau_dev;   // [1] threshold of a step that takes it from its own scores (dare_layer_step_quantile)
 };
 

@@ -637,13 +637,13 @@ template <typename T>
 cudaError_t launch_q_simt(const SimtStep& s, const T* xn, const T* w_q, T* q, cudaStream_t st, int* launches) {
   SgemmParams p = {};
   p.a = xn; p.g = s.g; p.rows = s.g.tokens(); p.w0 = w_q; p.out0 = q;
-  p.rope = reinterpret_cast<const float2*>(s.rope_cs); p.q_prev = s.q_prev; p.scores = s.scores; p.q_raw = s.tmp;
+  p.rope = reinterpret_cast<const float2*>(s.rope_cs); p.q_prev = s.q_prev; p.scores = s.scores; p.q_raw = s.q_raw;
   p.has_prev = s.has_prev; p.status = s.status;
   ++*launches;
   if (cudaError_t e = launch_sgemm<T, SG_Q>(p, p.rows, st); e != cudaSuccess) return e;
   if (s.g.head_dim <= 64) return cudaSuccess;
   ++*launches;
-  return launch_pdl(score_kernel, dim3((p.rows + 7) / 8), dim3(256), 0, st, 1, s.tmp, s.q_prev, s.scores, p.has_prev, s.g);
+  return launch_pdl(score_kernel, dim3((p.rows + 7) / 8), dim3(256), 0, st, 1, s.q_raw, s.q_prev, s.scores, p.has_prev, s.g);
 }
 template <typename T>
 cudaError_t launch_kv_simt(const SimtStep& s, const T* xn, const int* idx, const int* count, const T* w_k, const T* w_v,
