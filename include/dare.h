@@ -39,8 +39,8 @@
  *   gives up after two seconds, and the kernel runs on to its normal exit), or a value of the device-side selection
  *   that failed its range check before it was used as an address (a token of the refresh list outside the step, a
  *   list length or a sequence's slice outside the list: the access is skipped and the launch goes on).  A recorded
- *   error stays until `dare_layer_clear_status`; while a time-out stands, every wait gives up at once, so results
- *   are undefined until it is cleared.
+ *   error stays until `dare_layer_clear_status`; while a time-out stands, a wait gives up after half a millisecond: the
+ *   launch it happened in runs out soon, launches that are in order still end in order, and results are not to be relied on.
  *
  * Threading: one host thread per handle at a time.
  */
@@ -183,9 +183,9 @@ dare_status_t dare_layer_clear_status(dare_layer_t* layer, void* cuda_stream);
  * dare_layer_debug_inject: the next step overwrites, right after its selection, what = 1: the first entry of the
  *   refresh list with batch * seq_act (one past the step's tokens), what = 2: the list's length with
  *   batch * seq_act + 3; the kernels that consume the selection must flag DARE_ERR_DEVICE_CHECK and skip the access.
- *   what = 3 (CUDA-core path only, DARE_ERR_UNSUPPORTED otherwise): if the next step is a dare_layer_step_quantile of more
- *   than 16384 tokens, one of the copies between the thread blocks that work out its threshold is not sent; the wait for it
- *   gives up after a millisecond, the status word reads DARE_ERR_TIMEOUT and the step refreshes every token.
+ *   what = 3: if the next step is a dare_layer_step_quantile of more than 16384 tokens, one of the copies between the thread
+ *   blocks that work out its threshold is not sent; the wait for it gives up after a millisecond, the status word reads
+ *   DARE_ERR_TIMEOUT and the step refreshes every token.
  *   One step only; what = 0 withdraws it. */
 dare_status_t dare_layer_debug_wait_probe(dare_layer_t* layer, uint64_t limit_ns, uint64_t* waited_ns_host, void* cuda_stream);
 dare_status_t dare_layer_debug_inject(dare_layer_t* layer, int what);

@@ -631,7 +631,6 @@ dare_status_t dare_layer_debug_inject(dare_layer_t* L, int what) {
   dare_status_t s = check_handle(L);
   if (s != DARE_OK) return s;
   if (what < 0 || what > 3) return DARE_ERR_INVALID_ARG;
-  if (what == 3 && L->use_tc) return DARE_ERR_UNSUPPORTED;   // (with a time-out standing that path's waits would give up early)
   L->inject = what;
   return DARE_OK;
 }

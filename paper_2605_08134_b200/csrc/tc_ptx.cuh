@@ -46,17 +46,19 @@ __device__ __forceinline__ uint64_t globaltimer_ns() {
   return t;
 }
 // Bounded wait for the phase with the given parity.  Returns false (after flagging the status word) on time-out.
-constexpr unsigned long long kWaitLimitNs = 2000000000ull;
+// Once a wait has given up, the others have half a millisecond: the launch it happened in runs out soon, while launches that
+// are in order behind it, whose waits take microseconds, end in order (with no copy still on its way when they leave).
+// (A failed range check is no reason to stop waiting: its access was skipped and the rest of the launch is in order.)
+constexpr unsigned long long kWaitLimitNs = 2000000000ull, kWaitAfterTimeoutNs = 500000ull;
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* status,
                                           unsigned long long limit_ns = kWaitLimitNs) {
   if (mbar_try_wait(bar, parity)) return true;
-  // once a wait has given up, the others do not wait again: the kernel runs out quickly (a failed range check is no
-  // reason to stop waiting: its access was skipped and the rest of the launch is in order)
-  if (status && *reinterpret_cast<volatile int*>(status) == 7 /* DARE_ERR_TIMEOUT */) return false;
+  if (status && *reinterpret_cast<volatile int*>(status) == 7 /* DARE_ERR_TIMEOUT */ && limit_ns > kWaitAfterTimeoutNs)
+    limit_ns = kWaitAfterTimeoutNs;
   const uint64_t t0 = globaltimer_ns();
   uint32_t spins = 0;
-  while (!mbar_try_wait(bar, parity)) {
-    if ((++spins & 0x3ffu) == 0 && globaltimer_ns() - t0 > limit_ns) {
+  while (!mbar_try_wait(bar, parity)) {                 // (a poll suspends the thread for up to about 4 us)
+    if ((++spins & 0x3fu) == 0 && globaltimer_ns() - t0 > limit_ns) {
       if (status) atomicExch(status, 7 /* DARE_ERR_TIMEOUT */);      // (takes the place of a recorded range-check failure)
       return false;
     }

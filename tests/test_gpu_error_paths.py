@@ -94,10 +94,15 @@ def test_selection_values_out_of_range_are_flagged_and_skipped(dare, case, what)
     g.close()
 
 
-def test_a_lost_copy_in_the_threshold_exchange_is_flagged_and_refreshes_everything(dare):
+@pytest.mark.parametrize("path", ["simt", "tensor"])
+def test_a_lost_copy_in_the_threshold_exchange_is_flagged_and_refreshes_everything(dare, path):
     """More than 16384 tokens: the blocks that work the threshold out wait for one another's bins.  One copy is withheld: the
-    wait gives up, the status word says so, the threshold is NaN and the step is the one that refreshes every token."""
+    wait gives up, the status word says so, the threshold is NaN and the step is the one that refreshes every token; its
+    other launches, which run with the time-out standing, are in order and end in order."""
     shape = wl.scaled(wl.TINY_F32, d_model=64, n_heads=2, head_dim=32, batch=130, seq=127, prompt=60)
+    if path == "tensor":
+        shape = wl.scaled(wl.LLADA_LAYER, d_model=256, n_heads=4, head_dim=64, batch=130, seq=127, prompt=60)
+    tol = parity.tol_of(shape.dtype)
     w = wl.make_weights(shape, 21)
     hs = wl.HiddenStream(shape, 21)
     g = dare.Layer(shape, w)
@@ -113,7 +118,7 @@ def test_a_lost_copy_in_the_threshold_exchange_is_flagged_and_refreshes_everythi
     sel = g.last_selection(shape.batch, shape.seq)
     assert sel["count"] == shape.tokens and not sel["delta"].any()
     yo = o.step(x, 3, -1.0)
-    parity.assert_close("y", y.cpu().numpy(), yo, parity.TOL_F32, rel_rms=parity.TOL_F32)
+    parity.assert_close("y", y.float().cpu().numpy(), yo, tol, rel_rms=tol)
     g.clear_status()
     changed = wl.uniform_positions(hs.rng, shape, 20)             # the handle goes on: the next step is an ordinary one
     x = hs.advance(changed)
@@ -121,11 +126,7 @@ def test_a_lost_copy_in_the_threshold_exchange_is_flagged_and_refreshes_everythi
     yo = o.step(x, 3, 0.1)
     assert g.status() == dare.OK
     np.testing.assert_array_equal(g.last_selection(shape.batch, shape.seq)["idx"], o.last_idx)
-    parity.assert_close("y", y.cpu().numpy(), yo, parity.TOL_F32, rel_rms=parity.TOL_F32)
+    parity.assert_close("y", y.float().cpu().numpy(), yo, tol, rel_rms=tol)
     with pytest.raises(dare.DareError):
         g.inject(4)
     g.close()
-    t = dare.Layer(SMALL_BF16, wl.make_weights(SMALL_BF16, 5), kernel_path=dare.PATH_TENSOR)
-    with pytest.raises(dare.DareError):
-        t.inject(3)
-    t.close()
