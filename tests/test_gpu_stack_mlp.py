@@ -15,6 +15,7 @@ CASES = [
     (256, 12544, 2, 77),      # ... one wave as well: 66 tiles of 192 outputs on 74 SM pairs
     (256, 19072, 2, 77),      # ... more than one wave: tiles of 256 (the widest), the 75th half full
     (256, 38016, 3, 40),      # one row tile, more than one wave: the 149th tile of 256 half full
+    (4096, 12544, 3, 256),    # groups of column tiles of unequal width: 98 over nine groups of 11
     (4096, 2048, 2, 640),     # ten row tiles: persistent down projection
     (512, 2048, 2, 31),
 ]
