@@ -27,7 +27,7 @@
 // traffic (ncu: tensor pipe 87 % active).  Both CTAs' TMA loads complete on the even CTA's barriers, stages and
 // accumulators are released to both by one commit each, and the finishing warps of both CTAs hand an accumulator
 // back by arriving on the even CTA's barrier.
-// No reduction split, epilogues Q, K/V, OUT, OUT_RES, F32 (logits of listed rows), SWIGLU (a tile then holds the gate and the up projection of the same
+// No reduction split, epilogues Q, K/V, QKV, OUT, OUT_RES, F32 (logits of listed rows), SWIGLU (a tile then holds the gate and the up projection of the same
 // 128 outputs, and a finishing chunk 32 columns of each: eight row tiles of 4096 x 2 x 12288 took 251 us in the
 // one-tile-per-CTA kernel, 6 waves of CTAs that each fill and drain on their own, and 175 us here).
 #include "layer.h"
@@ -65,17 +65,19 @@ constexpr int kWarps = 2 + kFinish;
 constexpr int kGroupBytes = 24 << 20;
 
 struct TileGeom {
-  int nt, mt, n0, is_b1;
+  int nt, mt, n0, mat;               // mat: which of the matrices W0 / W1 / W2
   int t0, rows_valid, a_row, pos0;
   size_t crow0;
 };
 // n_rows: rows of a gathered launch (the device-side count), unused otherwise
+template <bool kThree>
 __device__ __forceinline__ TileGeom tile_geom(const GemmParams& p, int nt, int mt, bool gather, int n_rows) {
   TileGeom t;
   t.nt = nt;
   t.mt = mt;
-  t.is_b1 = t.nt >= p.n_split;
-  t.n0 = p.b_pair ? t.nt * (BN / 2) : (t.is_b1 ? t.nt - p.n_split : t.nt) * BN;
+  t.mat = t.nt >= p.n_split ? 1 : 0;
+  if (kThree && t.nt - p.n_split >= p.n_split) t.mat = 2;
+  t.n0 = p.b_pair ? t.nt * (BN / 2) : (t.nt - t.mat * p.n_split) * BN;
   if (gather) {                      // rows t0 .. of the index list; position and cache row come from the tokens
     t.t0 = t.mt * BM;
     t.rows_valid = min(BM, n_rows - t.t0);
@@ -98,8 +100,10 @@ __device__ __forceinline__ TileGeom tile_geom(const GemmParams& p, int nt, int m
 template <int EPI, bool GATHER, bool PAIR, int HDIM>
 __global__ void __launch_bounds__(kWarps * 32, 1)
 gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b0,
-                    const __grid_constant__ CUtensorMap tm_b1, const GemmParams p, const int n_tiles,
+                    const __grid_constant__ CUtensorMap tm_b1, const __grid_constant__ CUtensorMap tm_b2,
+                    const GemmParams p, const int n_tiles,
                     const int total_tiles_dense, const int n_group) {
+  constexpr bool kThree = EPI == EPI_QKV, kKv = EPI == EPI_KV || EPI == EPI_QKV;
   constexpr int STAGES = Ring<PAIR>::STAGES, STAGE_BYTES = Ring<PAIR>::STAGE_BYTES, B_BYTES = Ring<PAIR>::B_BYTES;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -124,6 +128,7 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
     prefetch_tmap(&tm_a);
     prefetch_tmap(&tm_b0);
     prefetch_tmap(&tm_b1);
+    if (kThree) prefetch_tmap(&tm_b2);
   }
   if (warp == 1) {
     if (PAIR) { tmem_alloc2(tmem_slot, 512); tmem_relinquish2(); }
@@ -162,16 +167,22 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
   const int m_units = PAIR ? (m_tiles_live + 1) / 2 : m_tiles_live;
   auto tile_of = [&](int u) {
     // column tiles in groups of n_group, a group over all row tiles (or pairs of them) before the next, columns fastest
-    const int in_group = n_group * m_units, grp = u / in_group, r = u - grp * in_group;
-    const int width = min(n_group, n_tiles - grp * n_group), mu = r / width, nt = grp * n_group + r - mu * width;
-    if (!PAIR) return tile_geom(p, nt, mu, GATHER, n_rows);
+    int width = n_tiles, nt0 = 0, r = u;
+    if (n_group < n_tiles) {
+      const int in_group = n_group * m_units, grp = u / in_group;
+      r = u - grp * in_group;
+      nt0 = grp * n_group;
+      width = min(n_group, n_tiles - nt0);
+    }
+    const int mu = r / width, nt = nt0 + r - mu * width;
+    if (!PAIR) return tile_geom<kThree>(p, nt, mu, GATHER, n_rows);
     const int mt = 2 * mu + pr;
     if (GATHER) {                      // (the tile past an odd count has no rows: nothing stored)
-      TileGeom t = tile_geom(p, nt, mt, true, n_rows);
+      TileGeom t = tile_geom<kThree>(p, nt, mt, true, n_rows);
       t.rows_valid = max(t.rows_valid, 0);
       return t;
     }
-    TileGeom t = tile_geom(p, nt, mt < p.m_tiles ? mt : mt - 1, false, 0);
+    TileGeom t = tile_geom<kThree>(p, nt, mt < p.m_tiles ? mt : mt - 1, false, 0);
     if (mt >= p.m_tiles) t.rows_valid = 0;
     return t;
   };
@@ -181,7 +192,7 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
     uint32_t it = 0;
     for (int tile = walker; tile < total_tiles; tile += n_walkers) {
       const TileGeom t = tile_of(tile);
-      const CUtensorMap* tm_b = t.is_b1 ? &tm_b1 : &tm_b0;
+      const CUtensorMap* tm_b = kThree && t.mat == 2 ? &tm_b2 : (t.mat == 1 ? &tm_b1 : &tm_b0);
       for (int kb = 0; kb < KB; ++kb, ++it) {
         const int s = it % STAGES;
         mbar_wait(&empty_bar[s], ((it / STAGES) & 1) ^ 1, p.status);
@@ -277,9 +288,10 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
         if ((unsigned)tok_first >= (unsigned)p.g.tokens()) tok_first = 0;
       }
       const FlatRows fr(p.g, t.t0, p.flat != 0);
-      const bool rotate = (EPI == EPI_Q) || (EPI == EPI_KV && !t.is_b1);
+      const bool rotate = (EPI == EPI_Q) || (kKv && t.mat != 1);
       const int score_col = (EPI == EPI_Q) ? p.g.score_head * HDIM - t.n0 : -1;   // first column of the scoring head in this tile
-      __nv_bfloat16* out = t.is_b1 ? p.out1 : p.out0;
+      const bool by_token = kThree && t.mat == 2;
+      __nv_bfloat16* out = by_token ? p.out2 : (t.mat == 1 ? p.out1 : p.out0);
 #pragma unroll 1
       for (int chunk = 0; chunk < 4; ++chunk) {
         // tile columns [c_lo, c_lo + 16) and their partners + PART: of the rotary embedding (h_col: the columns' place in
@@ -336,7 +348,7 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
               fr.at(rc, &pos, &crowr);
             }
             tok_k[k] = tokr; crow_k[k] = crowr;
-            if (!GATHER && EPI == EPI_KV && p.store_mask != nullptr && ok[k] && p.store_mask[crowr] != 0) ok[k] = false;
+            if (!GATHER && kKv && p.store_mask != nullptr && ok[k] && p.store_mask[crowr] != 0) ok[k] = false;
             const uint8_t* row = stg + rr * STG_ROW_BYTES + (l8 & 1) * 8;
             lo[k] = *reinterpret_cast<const float2*>(row + unit_at(rr, l8 >> 1));
             hi[k] = *reinterpret_cast<const float2*>(row + unit_at(rr, 4 + (l8 >> 1)));
@@ -403,7 +415,7 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
               const float2 fa = __bfloat1622float2(ra[k]), fb = __bfloat1622float2(rb[k]);
               vlo.x += fa.x; vlo.y += fa.y; vhi.x += fb.x; vhi.y += fb.y;
             }
-            const size_t orow = p.out_is_cache == 1 ? crow : (p.out_is_cache == 2 ? (size_t)(t.t0 + r) : (size_t)tok);
+            const size_t orow = p.out_is_cache == 1 && !by_token ? crow : (p.out_is_cache == 2 ? (size_t)(t.t0 + r) : (size_t)tok);
             if (EPI == EPI_F32) {
               float* d32 = p.out_f32 + orow * p.ld_out + t.n0 + c_lo + 2 * l8;
               *reinterpret_cast<float2*>(d32) = vlo;
@@ -442,8 +454,8 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
 }
 
 template <int EPI, bool GATHER, bool PAIR, int HDIM>
-static cudaError_t launch_persist_hd(const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1, const GemmParams& p,
-                                  int n_tiles, int m_tiles, cudaStream_t st) {
+static cudaError_t launch_persist_hd(const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1, const CUtensorMap& b2,
+                                     const GemmParams& p, int n_tiles, int m_tiles, cudaStream_t st) {
   static std::atomic<unsigned long long> attr_done{0};
   auto kern = gemm_persist_kernel<EPI, GATHER, PAIR, HDIM>;
   if (cudaError_t e = ensure_dyn_smem(kern, SMEM_TOTAL, attr_done); e != cudaSuccess) return e;
@@ -458,25 +470,25 @@ static cudaError_t launch_persist_hd(const CUtensorMap& a, const CUtensorMap& b0
   const int n_group = (n_tiles + groups - 1) / groups;
   if (PAIR) {
     const int units = n_tiles * ((m_tiles + 1) / 2), clusters = units < sms / 2 ? units : sms / 2;
-    return launch_pdl_xz(kern, dim3(2 * clusters), dim3(kWarps * 32), SMEM_TOTAL, st, 2, 1, a, b0, b1, q, n_tiles, total, n_group);
+    return launch_pdl_xz(kern, dim3(2 * clusters), dim3(kWarps * 32), SMEM_TOTAL, st, 2, 1, a, b0, b1, b2, q, n_tiles, total, n_group);
   }
   return launch_pdl(kern, dim3(total < sms ? total : sms), dim3(kWarps * 32), SMEM_TOTAL, st,
-                    1, a, b0, b1, q, n_tiles, total, n_group);
+                    1, a, b0, b1, b2, q, n_tiles, total, n_group);
 }
 
 template <int EPI, bool GATHER, bool PAIR = false>
-static cudaError_t launch_persist(const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1, const GemmParams& p,
-                                  int n_tiles, int m_tiles, cudaStream_t st) {
-  if constexpr (EPI == EPI_Q || EPI == EPI_KV) {
-    if (p.g.head_dim == 64) return launch_persist_hd<EPI, GATHER, PAIR, 64>(a, b0, b1, p, n_tiles, m_tiles, st);
+static cudaError_t launch_persist(const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1, const CUtensorMap& b2,
+                                  const GemmParams& p, int n_tiles, int m_tiles, cudaStream_t st) {
+  if constexpr (EPI == EPI_Q || EPI == EPI_KV || EPI == EPI_QKV) {
+    if (p.g.head_dim == 64) return launch_persist_hd<EPI, GATHER, PAIR, 64>(a, b0, b1, b2, p, n_tiles, m_tiles, st);
   }
-  return launch_persist_hd<EPI, GATHER, PAIR, 128>(a, b0, b1, p, n_tiles, m_tiles, st);
+  return launch_persist_hd<EPI, GATHER, PAIR, 128>(a, b0, b1, b2, p, n_tiles, m_tiles, st);
 }
 
 // 256-wide tiles, no reduction split; b0 / b1 are maps with 256-row boxes (128-row boxes with pair != 0, and for SWIGLU).  Listed
 // launches (idx and count set, gather_src not; m_tiles = capacity of the row list in tiles): `a` maps a compact copy of
 // the listed rows (row r of the list = row r of the copy).
-cudaError_t launch_gemm_persist(int epi, const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1,
+cudaError_t launch_gemm_persist(int epi, const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1, const CUtensorMap& b2,
                                 const GemmParams& p, int n_tiles, int m_tiles, cudaStream_t st, int pair) {
   if (m_tiles <= 0 || n_tiles <= 0) return cudaSuccess;
   if ((p.b_pair != 0) != (epi == EPI_SWIGLU) || p.K % BK != 0) return cudaErrorInvalidValue;
@@ -486,28 +498,31 @@ cudaError_t launch_gemm_persist(int epi, const CUtensorMap& a, const CUtensorMap
   if (gather) return cudaErrorInvalidValue;       // (rows fetched by index inside the kernel: gemm_tc.cu)
   if (listed) {          // A = compact copy of the listed rows
     if (pair) {
-      if (epi == EPI_KV) return launch_persist<EPI_KV, true, true>(a, b0, b1, p, n_tiles, m_tiles, st);
-      if (epi == EPI_OUT) return launch_persist<EPI_OUT, true, true>(a, b0, b1, p, n_tiles, m_tiles, st);
+      if (epi == EPI_QKV) return launch_persist<EPI_QKV, true, true>(a, b0, b1, b2, p, n_tiles, m_tiles, st);
+      if (epi == EPI_KV) return launch_persist<EPI_KV, true, true>(a, b0, b1, b2, p, n_tiles, m_tiles, st);
+      if (epi == EPI_OUT) return launch_persist<EPI_OUT, true, true>(a, b0, b1, b2, p, n_tiles, m_tiles, st);
     } else {
-      if (epi == EPI_KV) return launch_persist<EPI_KV, true, false>(a, b0, b1, p, n_tiles, m_tiles, st);
-      if (epi == EPI_OUT) return launch_persist<EPI_OUT, true, false>(a, b0, b1, p, n_tiles, m_tiles, st);
-      if (epi == EPI_F32) return launch_persist<EPI_F32, true, false>(a, b0, b1, p, n_tiles, m_tiles, st);
+      if (epi == EPI_QKV) return launch_persist<EPI_QKV, true, false>(a, b0, b1, b2, p, n_tiles, m_tiles, st);
+      if (epi == EPI_KV) return launch_persist<EPI_KV, true, false>(a, b0, b1, b2, p, n_tiles, m_tiles, st);
+      if (epi == EPI_OUT) return launch_persist<EPI_OUT, true, false>(a, b0, b1, b2, p, n_tiles, m_tiles, st);
+      if (epi == EPI_F32) return launch_persist<EPI_F32, true, false>(a, b0, b1, b2, p, n_tiles, m_tiles, st);
     }
     return cudaErrorInvalidValue;
   }
   if (pair) {            // two-CTA MMAs: b0 / b1 are maps with 128-row boxes
-    if (epi == EPI_Q) return launch_persist<EPI_Q, false, true>(a, b0, b1, p, n_tiles, m_tiles, st);
-    if (epi == EPI_KV) return launch_persist<EPI_KV, false, true>(a, b0, b1, p, n_tiles, m_tiles, st);
-    if (epi == EPI_OUT) return launch_persist<EPI_OUT, false, true>(a, b0, b1, p, n_tiles, m_tiles, st);
-    if (epi == EPI_OUT_RES) return launch_persist<EPI_OUT_RES, false, true>(a, b0, b1, p, n_tiles, m_tiles, st);
-    if (epi == EPI_SWIGLU) return launch_persist<EPI_SWIGLU, false, true>(a, b0, b1, p, n_tiles, m_tiles, st);
+    if (epi == EPI_Q) return launch_persist<EPI_Q, false, true>(a, b0, b1, b2, p, n_tiles, m_tiles, st);
+    if (epi == EPI_QKV) return launch_persist<EPI_QKV, false, true>(a, b0, b1, b2, p, n_tiles, m_tiles, st);
+    if (epi == EPI_KV) return launch_persist<EPI_KV, false, true>(a, b0, b1, b2, p, n_tiles, m_tiles, st);
+    if (epi == EPI_OUT) return launch_persist<EPI_OUT, false, true>(a, b0, b1, b2, p, n_tiles, m_tiles, st);
+    if (epi == EPI_OUT_RES) return launch_persist<EPI_OUT_RES, false, true>(a, b0, b1, b2, p, n_tiles, m_tiles, st);
+    if (epi == EPI_SWIGLU) return launch_persist<EPI_SWIGLU, false, true>(a, b0, b1, b2, p, n_tiles, m_tiles, st);
     return cudaErrorInvalidValue;
   }
-  if (epi == EPI_Q) return launch_persist<EPI_Q, false>(a, b0, b1, p, n_tiles, m_tiles, st);
-  if (epi == EPI_KV) return launch_persist<EPI_KV, false>(a, b0, b1, p, n_tiles, m_tiles, st);
-  if (epi == EPI_OUT) return launch_persist<EPI_OUT, false>(a, b0, b1, p, n_tiles, m_tiles, st);
-  if (epi == EPI_OUT_RES) return launch_persist<EPI_OUT_RES, false>(a, b0, b1, p, n_tiles, m_tiles, st);
-  if (epi == EPI_SWIGLU) return launch_persist<EPI_SWIGLU, false>(a, b0, b1, p, n_tiles, m_tiles, st);
+  if (epi == EPI_Q) return launch_persist<EPI_Q, false>(a, b0, b1, b2, p, n_tiles, m_tiles, st);
+  if (epi == EPI_KV) return launch_persist<EPI_KV, false>(a, b0, b1, b2, p, n_tiles, m_tiles, st);
+  if (epi == EPI_OUT) return launch_persist<EPI_OUT, false>(a, b0, b1, b2, p, n_tiles, m_tiles, st);
+  if (epi == EPI_OUT_RES) return launch_persist<EPI_OUT_RES, false>(a, b0, b1, b2, p, n_tiles, m_tiles, st);
+  if (epi == EPI_SWIGLU) return launch_persist<EPI_SWIGLU, false>(a, b0, b1, b2, p, n_tiles, m_tiles, st);
   return cudaErrorInvalidValue;
 }
 

@@ -17,6 +17,7 @@
 // of its warps: one warp per row, lane <-> column pairs, so that table reads and output stores are contiguous.
 // The fused epilogue work is thereby spread over both CTAs as well.
 // Fused epilogues:
+//   SCORE  the scoring head's columns alone: score and store of the new query (steps of many tokens, tc.cu)
 //   Q    drift score of the scoring head against the stored query (Sec. 3.1), store of the new query, rotary
 //        embedding, bf16 store
 //   K/V  rotary embedding of K, scatter of both rows into the caches at the refresh-set rows (Eq. 3)
@@ -107,7 +108,7 @@ __device__ __forceinline__ void load_row_batch(RowBatch<RB>& rb, const GemmParam
     }
     // no instruction consumes these loads before the finishing pass, so they stay in flight across the exchange
     if (rotate) rb.cs[k] = *reinterpret_cast<const float4*>(p.rope + (size_t)pos * L::HALF + L::in_head(lane));
-    if (EPI == EPI_Q && score_tile && p.has_prev) {
+    if ((EPI == EPI_Q || EPI == EPI_SCORE) && score_tile && p.has_prev) {
       rb.qa[k] = *reinterpret_cast<const float2*>(p.q_prev + rb.crow[k] * HDIM + L::in_head(lane));
       rb.qb[k] = *reinterpret_cast<const float2*>(p.q_prev + rb.crow[k] * HDIM + L::HALF + L::in_head(lane));
     }
@@ -146,7 +147,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
   // it to be uniform over the warp
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   // (a pair launch has the row tiles along x: the two CTAs of an MMA pair are neighbours in x)
-  const int nt = PAIR ? blockIdx.y : blockIdx.x, mt_first = PAIR ? blockIdx.x : blockIdx.y;
+  const int nt = EPI == EPI_SCORE ? p.g.score_head * HDIM / BN : (int)(PAIR ? blockIdx.y : blockIdx.x), mt_first = PAIR ? blockIdx.x : blockIdx.y;
   const int cl_splits = gridDim.z;              // = cluster size along z: slices of the reduction
   // cluster = (PAIR ? 2 : 1, 1, splits): rank = place in the MMA pair + 2 * reduction slice
   const int crank = (int)cluster_ctarank();
@@ -309,7 +310,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
   const int nkb = KB / splits;                    // k-blocks this CTA walks for the tile
   const int quarter = warp & 3;                   // TMEM lanes a warp may touch: 32*quarter .. +31
   const bool rotate = (EPI == EPI_Q) || (EPI == EPI_KV && !is_b1);
-  const int score_col = (EPI == EPI_Q) ? p.g.score_head * HDIM - n0 : -1;       // first column of the scoring head in this tile
+  const int score_col = (EPI == EPI_Q || EPI == EPI_SCORE) ? p.g.score_head * HDIM - n0 : -1;       // first column of the scoring head in this tile
   const bool score_tile = score_col >= 0 && score_col < BN;
   RowBatch<RB> rb;
 
@@ -551,7 +552,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       }
       // (2) Sec. 3.1 on the un-rotated query of the scoring head: 1 - cos(current, stored), all rows of the batch
       //     reduced across the lanes together; lane k finishes row k.  Then the current query is stored.
-      if (EPI == EPI_Q && score_tile) {
+      if ((EPI == EPI_Q || EPI == EPI_SCORE) && score_tile) {
         float dot[RB], n1[RB], n2[RB];
         const bool mine = HDIM == CH || (lane >> 4) == ((score_col / HDIM) & 1);   // this lane holds columns of the scoring head
 #pragma unroll
@@ -597,7 +598,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       // (3) the projection's own tail and the store
 #pragma unroll
       for (int k = 0; k < RB; ++k) {
-        if (!rb.ok[k]) continue;
+        if (!rb.ok[k] || EPI == EPI_SCORE) continue;
         const size_t orow = p.out_is_cache == 1 ? rb.crow[k] : (p.out_is_cache == 2 ? (size_t)rb.row[k] : (size_t)rb.tok[k]);
         if (EPI == EPI_SWIGLU) {
           // columns [0, 128) of a 256-wide tile are the gate, [128, 256) the up projection of the same 128 outputs
@@ -704,7 +705,7 @@ static cudaError_t launch_hd(const CUtensorMap& a, const CUtensorMap& b0, const 
 template <int EPI, int BN, bool PAIR>
 static cudaError_t launch_one(const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1, const GemmParams& p,
                               int n_tiles, int m_tiles, int splits, cudaStream_t st) {
-  if constexpr (EPI == EPI_Q || EPI == EPI_KV) {
+  if constexpr (EPI == EPI_Q || EPI == EPI_SCORE || EPI == EPI_KV) {
     if (p.g.head_dim == 64) return launch_hd<EPI, BN, PAIR, 64>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
   }
   return launch_hd<EPI, BN, PAIR, 128>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
@@ -721,6 +722,7 @@ cudaError_t launch_gemm_tc(int epi, int bn, const CUtensorMap& a, const CUtensor
     // narrow pair tiles (256 rows x 128 columns per pair; b0 / b1 with 64-row boxes): twice the CTAs of the wide ones
     // for launches of two row tiles, whose main loops are bound by what one SM can pull from the L2
     if (p.gather_src != nullptr || p.count != nullptr || p.b_pair) return cudaErrorInvalidValue;
+    if (epi == EPI_SCORE) return launch_one<EPI_SCORE, 128, true>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
     if (epi == EPI_Q) return launch_one<EPI_Q, 128, true>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
     if (epi == EPI_OUT) return launch_one<EPI_OUT, 128, true>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
     if (epi == EPI_OUT_RES) return launch_one<EPI_OUT_RES, 128, true>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
@@ -745,6 +747,7 @@ cudaError_t launch_gemm_tc(int epi, int bn, const CUtensorMap& a, const CUtensor
   }
   if (bn == 128 && !p.b_pair) {
     if (epi == EPI_KV) return launch_one<EPI_KV, 128, false>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
+    if (epi == EPI_SCORE) return launch_one<EPI_SCORE, 128, false>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
     if (epi == EPI_Q) return launch_one<EPI_Q, 128, false>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
     if (epi == EPI_OUT) return launch_one<EPI_OUT, 128, false>(a, b0, b1, p, n_tiles, m_tiles, splits, st);
     if (epi == EPI_OUT_RES) return launch_one<EPI_OUT_RES, 128, false>(a, b0, b1, p, n_tiles, m_tiles, splits, st);

@@ -154,13 +154,59 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
     const float behind = 20.f + 0.33f * (float)(kblocks * (1 + (units + 73) / 74));
     kv_beside_q = beside < behind;
   }
+  // A projection of the refresh set's rows of x_norm (p.idx, p.count): a compact copy of them, then the launch in three forms,
+  // each of which looks at the count: listed in two-CTA and in one-CTA tiles; from gate_kv refreshed tokens on dense, every row
+  // of the step projected and the refresh set's stored.
+  auto listed_projection = [&](int epi, GemmParams p, const CUtensorMap& b0, const CUtensorMap& b1, const CUtensorMap& b2, const CUtensorMap& b0h,
+                               const CUtensorMap& b1h, const CUtensorMap& b2h, int n_tiles) {
+    const int m_tiles = (T_ + 127) / 128;
+    const bool dense_form = persist_pays_listed(n_tiles, m_tiles_dense);
+    const int hi = dense_form ? gate_kv : 1 << 30;
+    launch_gather_step_rows((const bf16*)B.xn, B.idx, B.count, (bf16*)B.x_stage, g, false, st, B.status, hi); ++launches;
+    p.gather_src = nullptr;
+    p.unit_gate = kPairUnitGate;
+    p.gate_count = B.count; p.gate_hi = hi;
+    cudaError_t err = launch_gemm_persist(epi, S.a_xg, b0h, b1h, b2h, p, n_tiles, m_tiles, st, 1); ++launches;
+    if (err == cudaSuccess) { err = launch_gemm_persist(epi, S.a_xg, b0, b1, b2, p, n_tiles, m_tiles, st, 0); ++launches; }
+    if (dense_form && err == cudaSuccess) {
+      p.idx = nullptr; p.count = nullptr; p.unit_gate = 0;
+      p.gate_lo = gate_kv; p.gate_hi = 1 << 30; p.store_mask = B.delta;
+      err = launch_gemm_persist(epi, S.a_xn, b0h, b1h, b2h, p, n_tiles, m_tiles_dense, st, 1); ++launches;
+    }
+    return err;
+  };
   prof_begin(L);
   // Alg. 1/2 line 1
   prof_mark(L, SLOT_NORM, st);
   launch_rmsnorm<bf16>((const bf16*)x, L->w.rms_gain, (bf16*)B.xn, T_, d, L->cfg.rms_eps, st, dbg ? dbg + 40 : nullptr);
   ++launches;
-  // line 2 + line 3 + stored-query update + rotary embedding, one kernel
-  {
+  // A step of many tokens that reuses attention outputs needs the scoring head of every token (the score, the stored query),
+  // and of the other heads only the queries that attend, the refresh set's (Alg. 2 line 8): the scoring head's 128 columns are
+  // projected first, and the refresh set's queries behind the selection, beside its K and V where those are listed as well.
+  // 4 x 4096 tokens of width 4096, both rules, 15 % refreshed: 1019 -> 692 us; 8 x 1024, output reuse, 13 %: 783 -> 634 us.
+  // With (nearly) all tokens refreshed the scoring head is projected twice, one launch for nothing: 1-2 % of a step, which is
+  // why the rule asks for a query projection of some size (us before / with it, every token refreshed, and at 13 to 30 %):
+  //   both:   1 x 1152 of 4096 (39 GFLOP) 238 / 238, 148 / 139    8 x 1700 of 1536 (64) 490 / 494, 237 / 188
+  //   output: 2 x 1250 of 4096 (84 GFLOP) 419 / 417, 327 / 284    4 x 2300 of 2048 (77) 496 / 507, 349 / 315
+  // A step given its reuse rate knows when more than three quarters will be refreshed.  (Up to eight row tiles the projections
+  // are streams of the weights whatever the rows: 90 us this way against 78 at 512 tokens of width 4096.)
+  const int n_listed = (kv_sparse ? 3 : 1) * (d / 256);
+  const double q_flop = 2.0 * T_ * (double)d * d;
+  const bool many_known = L->reuse_count >= 0 && 4ll * (T_ - L->reuse_count) > 3ll * T_;
+  const bool q_pays = !many_known && q_flop >= (kv_sparse ? 34e9 : 80e9);
+  const bool q_listed = o_sparse && m_tiles_dense > 8 && compact_ok && q_pays && persist_pays_listed(n_listed, (T_ + 127) / 128);
+  if (q_listed) {
+    GemmParams p = base;
+    p.debug = dbg;
+    prof_mark(L, SLOT_Q_GEMM, st);
+    TileForm f;
+    if (!pick_one_wave(128, m_tiles_dense, kblocks, &f)) f = TileForm{128, 0, 1};
+    const CUtensorMap& wq = f.pair ? S.w_q64 : S.w_q128;
+    e = launch_gemm_tc(EPI_SCORE, 128, S.a_xn, wq, wq, p, 1, m_tiles_dense, f.splits, st, f.pair);
+    ++launches;
+    if (e != cudaSuccess) return DARE_ERR_CUDA;
+  } else {
+    // line 2 + line 3 + stored-query update + rotary embedding, one kernel
     GemmParams p = base;
     p.out0 = (bf16*)B.q;
     p.debug = dbg;
@@ -228,31 +274,27 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
         ++launches;
       } else {
         // Many tokens: even a small refreshed fraction fills the GPU with 256-wide tiles, which re-read the least.
-        if (persist_pays_listed(n_tiles, m_tiles) && compact_ok) {
+        const int n_listed_tiles = q_listed ? n_listed : n_tiles;
+        if (persist_pays_listed(n_listed_tiles, m_tiles) && compact_ok) {
           // a compact copy of the refresh set's rows first (a stream of n x d elements), then the projection with
           // every operand through TMA and two-CTA MMAs; beyond gate_kv refreshed tokens the dense form instead: every
           // row of the step projected, the rows of the refresh set stored (the others keep their cached K and V)
-          const bool dense_form = persist_pays_listed(n_tiles, m_tiles_dense);
-          const int hi = dense_form ? gate_kv : 1 << 30;
-          launch_gather_step_rows((const bf16*)B.xn, B.idx, B.count, (bf16*)B.x_stage, g, false, st, B.status, hi); ++launches;
-          p.gather_src = nullptr;
-          p.unit_gate = kPairUnitGate;
-          p.gate_count = B.count; p.gate_hi = hi;
-          e = launch_gemm_persist(EPI_KV, S.a_xg, S.w_k128, S.w_v128, p, n_tiles, m_tiles, st, 1); ++launches;
-          if (e == cudaSuccess) e = launch_gemm_persist(EPI_KV, S.a_xg, S.w_k, S.w_v, p, n_tiles, m_tiles, st, 0);
-          if (dense_form && e == cudaSuccess) {
-            GemmParams pd = p;
-            pd.idx = nullptr; pd.count = nullptr; pd.unit_gate = 0;
-            pd.gate_lo = gate_kv; pd.gate_hi = 1 << 30; pd.store_mask = B.delta;
-            ++launches;
-            e = launch_gemm_persist(EPI_KV, S.a_xn, S.w_k128, S.w_v128, pd, n_tiles, m_tiles_dense, st, 1);
-          }
+          if (q_listed) p.out2 = (bf16*)B.q;
+          e = listed_projection(q_listed ? EPI_QKV : EPI_KV, p, S.w_k, S.w_v, S.w_q, S.w_k128, S.w_v128, S.w_q128, n_listed_tiles);
+          --launches;                                    // (counted below)
         } else
           e = launch_gemm_tc(EPI_KV, 256, S.a_xn, S.w_k, S.w_v, p, n_tiles, m_tiles, 1, st);
         ++launches;
       }
     } else {
       prof_mark(L, SLOT_KV_GEMM, st);
+      if (q_listed) {
+        GemmParams pq = base;
+        pq.out0 = (bf16*)B.q;
+        pq.idx = B.idx; pq.count = B.count;
+        e = listed_projection(EPI_KV, pq, S.w_q, S.w_q, S.w_q, S.w_q128, S.w_q128, S.w_q128, n_listed);
+        if (e != cudaSuccess) return DARE_ERR_CUDA;
+      }
       p.wait_at_end = kv_beside_q ? 1 : 0;
       const int sp = pick_splits(n_tiles * m_tiles_dense, kblocks);
       if (!kv_beside_q && persist_pays(n_tiles, m_tiles_dense, sp)) {
@@ -282,7 +324,8 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
     p.debug = dbg ? dbg + 16 : nullptr;
     // the refresh set then comes from the kernel right before; or the two kernels before ran beside the Q projection
     // without waiting for it, so the queries are not known to be complete before this kernel's own wait
-    p.wait_first = kv_beside_q ? 1 : 0;
+    // (or the kernel before wrote the queries themselves)
+    p.wait_first = kv_beside_q || (q_listed && kv_sparse) ? 1 : 0;
     p.gate_count = nullptr; p.gate_lo = 0; p.gate_hi = 1 << 30; p.store_mask = nullptr;
     // a long row-sparse step is issued in both forms: over the refresh set's rows, and dense with only the refreshed
     // rows stored (tiles without one skipped); the size of the set decides on the device which of them runs

@@ -8,7 +8,9 @@
 namespace dare {
 
 enum { EPI_Q = 0, EPI_KV = 1, EPI_OUT = 2, EPI_SWIGLU = 3, EPI_F32 = 4,
-       EPI_OUT_RES = 5 };   // EPI_OUT plus a residual row (chosen by the launcher when GemmParams::resid is set)
+       EPI_OUT_RES = 5,     // EPI_OUT plus a residual row (chosen by the launcher when GemmParams::resid is set)
+       EPI_SCORE = 6,       // the one column tile of the scoring head: scored and kept (as in EPI_Q), no query stored
+       EPI_QKV = 7 };       // EPI_KV and a third matrix: the queries of the same rows (persistent kernel)
 
 struct GemmParams {
   int K;                 // reduction length (multiple of 64)
@@ -30,7 +32,8 @@ struct GemmParams {
                          // gives it at least this many (column tile, row-tile pair) units, the one-CTA form otherwise;
                          // 0: no gate
   StepGeom g;
-  int n_split;           // n-tiles [0, n_split) use W0/out0, the rest W1/out1
+  int n_split;           // n-tiles [0, n_split) use W0/out0, the next n_split W1/out1 and (EPI_QKV) the last n_split
+                         // W2/out2: rotated, stored by token
   __nv_bfloat16* out0;
   __nv_bfloat16* out1;
   int ld_out;
@@ -38,7 +41,10 @@ struct GemmParams {
                          // in the gathered list (2)
   const __nv_bfloat16* resid;  // EPI_OUT: rows added to the result (indexed like a token-addressed output), or nullptr
   int ld_resid;
-  float* out_f32;        // EPI_F32: fp32 output instead of out0
+  union {                // (no larger: every launch carries the struct, and 8 bytes more cost short steps 0.5 %)
+    float* out_f32;        // EPI_F32: fp32 output instead of out0
+    __nv_bfloat16* out2;   // EPI_QKV: see n_split
+  };
   int b_pair;            // the W tile is BN/2 rows of W0 followed by BN/2 rows of W1, both at row nt*BN/2 (EPI_SWIGLU:
                          // gate and up projections of the same BN/2 outputs)
   const float2* rope;    // rotary table [max_seq][head_dim/2]
@@ -183,9 +189,13 @@ cudaError_t launch_swiglu(const CUtensorMap& x, const CUtensorMap& gate, const C
 
 // Persistent form for launches of many row tiles (dense rows, 256-wide tiles, no reduction split, epilogues Q, K/V,
 // OUT): one CTA per SM walks the tiles, finishing pass overlapped with the next tile's main loop.
-// pair != 0 (dense launches only): two-CTA MMAs over pairs of row tiles, b0 / b1 with 128-row boxes.
-cudaError_t launch_gemm_persist(int epi, const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1,
+// pair != 0: two-CTA MMAs over pairs of row tiles, b0 / b1 / b2 with 128-row boxes.
+cudaError_t launch_gemm_persist(int epi, const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1, const CUtensorMap& b2,
                                 const GemmParams& p, int n_tiles, int m_tiles, cudaStream_t st, int pair = 0);
+inline cudaError_t launch_gemm_persist(int epi, const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1,
+                                       const GemmParams& p, int n_tiles, int m_tiles, cudaStream_t st, int pair = 0) {
+  return launch_gemm_persist(epi, a, b0, b1, b1, p, n_tiles, m_tiles, st, pair);
+}
 // ... pays as soon as the tiles are more than one wave: from there on a tile's set-up, pipeline fill and finishing pass
 // hide behind the next tile's main loop.
 inline bool persist_pays(int n_tiles, int m_tiles, int splits) { return splits == 1 && n_tiles * m_tiles > kSms; }
