@@ -51,7 +51,10 @@ template <int BN, bool PAIR = false>
 struct Cfg {
   static constexpr int B_BYTES = (PAIR ? BN / 2 : BN) * BK * 2;     // this CTA's part of the W tile
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr int STAGES = (PAIR || BN != 256) ? 6 : 4;
+  // (narrow pairs are streams of the weights from the HBM, and of a stage's 24 KB only 8 are weights: nine stages keep as much of
+  // them in flight as fits.  Decoding step of an eight-layer stack, 256 rows of width 4096: 1406 -> 1375 us against six stages;
+  // a seventh stage for the others made no difference.)
+  static constexpr int STAGES = PAIR && BN == 128 ? 9 : ((PAIR || BN != 256) ? 6 : 4);
   static constexpr int BAR_OFFSET = STAGES * STAGE_BYTES;
   static constexpr int SMEM_TOTAL = BAR_OFFSET + 256 + 1024;  // barriers + slack for 1024-byte alignment
   static constexpr int PROW_BYTES = BN * 4;
@@ -241,7 +244,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
   }
   // The weights do not depend on the previous kernel in the stream: the producer starts their first tiles now, so
   // that they stream in while that kernel drains.  Everything it produced is needed only after pdl_wait().
-  const int n_early = likely && iter == 0 ? (KB / cl_splits < STAGES ? KB / cl_splits : STAGES) : 0;
+  // (Four stages of them: more only take bandwidth from that kernel's tail.  Six / four / three / two early stages, step in us:
+  // 2 x 32 rows of width 4096 60.8 / 59.9 / 60.0 / 60.9, 2 x 512 of 2048, heads of 64, 56.9 / 56.1 / 56.0 / 55.8, 2 x 128 of 2048
+  // 44.8 / 44.0 / 44.1 / 44.3, 512 of 4096 73.4 / 73.0 / 73.0 / 73.2.)
+  constexpr int EARLY = 4;
+  const int n_early = likely && iter == 0 ? (KB / cl_splits < EARLY ? KB / cl_splits : EARLY) : 0;
   if (warp == 0 && lane == 0) {
     for (int i = 0; i < n_early; ++i) {
       uint8_t* b_dst = smem + i * STAGE_BYTES + A_BYTES;
