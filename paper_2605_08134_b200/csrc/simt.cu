@@ -1,9 +1,11 @@
 // CUDA-core (SIMT) kernel path: fp32 accumulate everywhere, any supported geometry.  This is the path of the
-// fp32 configuration (tensor-core tf32 would not hold a 1e-4 bound) and the cross-check for the tensor-core path.
+// fp32 configuration (whose larger projections go to the tensor cores in split operands, gemm_f32.cu) and the cross-check for
+// the tensor-core path.
 // Six launches a step (seven with heads wider than 64), chained with programmatic dependent launch:
 //   RMSNorm -> Q projection (+ score, stored query, rotary embedding) -> selection -> K/V projection of the refresh set
 //   (+ rotary embedding, cache scatter) -> attention -> output projection.
-#include "dare_internal.h"
+#include <type_traits>
+#include "sgemm.h"
 #include "tc_ptx.cuh"
 
 namespace dare {
@@ -41,25 +43,6 @@ __device__ __forceinline__ void fetch4(float* dst, const __nv_bfloat16* src, boo
 // Bound by the FMA pipe and the registers that feed it: the inner loop alone reaches 53 TFLOP/s at RM = 6, 48 at RM = 4,
 // 30 at RM = 2.  (Two CTAs of 256 threads an SM were slower: a launch of one wave filled SMs two by two and left the
 // others idle.)
-enum { SG_Q = 0, SG_KV = 1, SG_OUT = 2 };
-struct SgemmParams {
-  const void* a;
-  const int* idx;        // gathered rows of A (tokens), or nullptr
-  const int* count;      // device count of them
-  int a_cache_rows;      // A is addressed by cache row
-  StepGeom g;
-  int rows;              // rows of the launch (capacity of the list if gathered)
-  const void* w0;
-  const void* w1;        // SG_KV: W_V
-  void* out0;
-  void* out1;
-  const float2* rope;
-  float* q_prev;
-  float* scores;
-  float* q_raw;          // heads wider than 64: un-rotated scoring head of every token, for score_kernel
-  int has_prev;
-  int* status;
-};
 constexpr int kStages = 3, kSgThreads = 512;
 
 template <int RM, int WM, int KG>
@@ -343,6 +326,15 @@ cudaError_t launch_sgemm(const SgemmParams& p, int rows_likely, cudaStream_t st)
   int best = 0;
   for (int i = 1; i < 5; ++i)
     if (c[i] < c[best]) best = i;
+  // fp32 on the tensor cores (gemm_f32.cu) instead?  A unit of the cost above is 0.42 us at width 1024; a tile of 128 rows takes
+  // 4.5 us and 1 us a block of 64 k-elements there.  Steps in us, here / there with every projection (heads of 64, every row): 64
+  // rows of width 384 30.4 / 38.8, 2 x 384 of 384 58.1 / 57.1, 4 x 400 of 384 131 / 97.7, 2 x 128 of 512 42.8 / 51.1, 2 x 384 of
+  // 512 89.7 / 70.9, 128 of 1024 66.7 / 72.6, 256 of 1024 96.8 / 83.0, 4 x 400 of 1024 498 / 269.
+  if constexpr (std::is_same<T, float>::value) {
+    const int tiles = p.g.d / 64 * (EPI == SG_KV ? 2 : 1) * ((rows_likely + 127) / 128);
+    const float there = (float)((tiles + kSms - 1) / kSms) * (4.5f + (float)(p.g.d / 64));
+    if (p.g.d % 64 == 0 && there < 0.42f * (float)p.g.d / 1024.f * c[best]) return launch_gemm_f32(EPI, p, st);
+  }
   switch (best) {
     case 0: return launch_sgemm_as<T, EPI, 6, 4, 2>(p, n_tiles, st);
     case 1: return launch_sgemm_as<T, EPI, 4, 4, 2>(p, n_tiles, st);
