@@ -5,8 +5,9 @@
 //     (1) per-tile count of refreshed tokens and the decisions themselves, a plain bit array -> scratch
 //     (2) exclusive scan of the tile counts (one CTA) -> scratch, total -> *count
 //     (3) per-tile compaction from the decision bits, written at the tile's offset: ascending index list
-// No CTA waits for another; the order of the list does not depend on scheduling.  Passes 2 and 3 are launched
-// programmatically dependent: their launch latency hides behind the pass before.
+// No CTA waits for another; the order of the list does not depend on scheduling.  Every kernel here is launched programmatically
+// dependent, its launch latency hidden behind the kernel before: with the drift scores and pass 1 among them, scores, quantile
+// and compaction of 20000 rows of 64 take 19.9 us, 22.5 before.
 // A single pass (tiles handed out by ticket, every CTA publishing its tile's count and adding up the counts published
 // before it back to the nearest known running total, entries staged in shared memory and written as whole lines) was
 // built as well, list and count identical, and measured on the same 2^24 scores against 22.6 us for the three passes:
@@ -35,6 +36,8 @@ template <int LPR, int VPL, int U>
 __global__ void __launch_bounds__(256) drift_score_kernel(const float* __restrict__ a, const float* __restrict__ b,
                                                           long long rows, float* __restrict__ scores) {
   constexpr int RPW = 32 / LPR * U, HD = 4 * LPR * VPL;      // rows a warp takes at once
+  ptx::pdl_wait();
+  ptx::pdl_launch_dependents();
   const int lane = threadIdx.x & 31, sub = lane & (LPR - 1), grp = lane / LPR;
   const long long warp0 = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
@@ -76,6 +79,8 @@ __global__ void __launch_bounds__(256) drift_score_kernel(const float* __restric
 // any other row length
 __global__ void __launch_bounds__(256) drift_score_any_kernel(const float* __restrict__ a, const float* __restrict__ b,
                                                               long long rows, int hd, float* __restrict__ scores) {
+  ptx::pdl_wait();
+  ptx::pdl_launch_dependents();
   const int lane = threadIdx.x & 31;
   const long long warp0 = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
@@ -171,6 +176,7 @@ __global__ void __launch_bounds__(kThreads) tile_flag_kernel(const float* __rest
                                                              int* __restrict__ tile_counts,
                                                              unsigned* __restrict__ flags) {
   __shared__ int total;
+  ptx::pdl_wait();
   ptx::pdl_launch_dependents();            // the scan's CTA may take its place now; it waits for this grid to complete
   if (threadIdx.x == 0) total = 0;
   __syncthreads();
@@ -244,6 +250,8 @@ __global__ void __launch_bounds__(kTileWords) tile_scatter_kernel(const unsigned
 // shared-memory atomic takes a cycle a lane whatever it meets, so the first pass costs a cycle a score of the CTA's share
 // (copies of the histogram changed nothing): with many scores the range starts as a bracket around rank k from a sample of
 // 256 of them, which most scores lie outside; a bracket that turns out not to hold the rank is given up for all keys.
+// The bracket's keys (about a seventh of the scores) are kept in shared memory as they are found, so the narrowing passes read
+// them and not the scores again: a call of 2^20 scores 2-4 us shorter; a kernel of its own, for the code cost 20000 scores 0.6 us.
 // A cluster (rather than a grid) because the call has no scratch memory to meet in: nothing is shared between calls,
 // whatever streams they run on.
 // A CTA that waits in vain for the others' bins records the time-out in the status word (if the caller has one), gives the
@@ -251,6 +259,7 @@ __global__ void __launch_bounds__(kTileWords) tile_scatter_kernel(const unsigned
 // threshold is NaN, which Eq. 2 reads as "refresh everything".
 constexpr int kKthBins = 2048, kKthMaxCtas = 16, kKthSample = 256;
 constexpr int kKthBracket = 1 << 19;        // the sample costs about 4 us: from this many scores on
+constexpr int kKthList = 48 * 1024;         // keys of the bracket that a CTA keeps in shared memory (one CTA an SM)
 constexpr unsigned kKeyMinusInf = 0x007fffffu, kKeyPlusInf = 0xff800000u;
 
 constexpr int kKthLost = -2;                // s_bin: some CTA's bins never came
@@ -265,6 +274,7 @@ __device__ __noinline__ bool kth_wait(uint64_t* bar, uint32_t phase, int* status
   return false;
 }
 // lose_one (diagnostics): CTA 0 keeps its bins from CTA 1, whose wait for them then runs out, after a millisecond.
+template <bool kBracket>       // n >= kKthBracket
 __global__ void __launch_bounds__(kThreads) kth_cluster_kernel(const float* __restrict__ scores, int n, int k,
                                                                float* __restrict__ tau_out, int* status, int lose_one) {
   __shared__ __align__(16) int hist[kKthBins];
@@ -274,6 +284,8 @@ __global__ void __launch_bounds__(kThreads) kth_cluster_kernel(const float* __re
   __shared__ __align__(16) unsigned sample[kKthSample];
   __shared__ int part[kKthBins / 8 / 32], totals[kKthMaxCtas], below[kKthMaxCtas], s_below, s_bin, s_rank;
   __shared__ unsigned s_lo, s_hi;
+  __shared__ int s_list, s_under;
+  extern __shared__ unsigned list[];                  // (bracket only: kKthList keys)
   const int ctas = (int)gridDim.x, rank_cta = (int)ptx::cluster_ctarank(), lane = threadIdx.x & 31, tid = (int)threadIdx.x;
   const int slice = kKthBins / ctas;                  // 128 or 256: whole warps, four or eight bins to a lane
   ptx::pdl_wait();
@@ -291,15 +303,15 @@ __global__ void __launch_bounds__(kThreads) kth_cluster_kernel(const float* __re
     return v;
   };
   // ---- the bracket, the same in every CTA: the sample's keys four standard deviations of its rank either side of k
-  const bool bracket = n >= kKthBracket;
-  if (bracket && tid < kKthSample) sample[tid] = score_key(scores[(int)(((long long)tid * n) / kKthSample)]);
+  if (kBracket && tid < kKthSample) sample[tid] = score_key(scores[(int)(((long long)tid * n) / kKthSample)]);
   if (tid == 0) {
     s_lo = kKeyMinusInf; s_hi = kKeyPlusInf;
+    s_list = 0; s_under = 0;
     ptx::mbar_init(&recv_bar, 1);
     ptx::fence_mbar_init();
   }
   __syncthreads();
-  if (bracket) {
+  if (kBracket) {
     const float p = (float)k / (float)n;
     const int c = (int)(p * kKthSample), w = (int)(4.f * sqrtf(p * (1.f - p) * kKthSample)) + 2;
     const int me = tid >> 2;                          // four threads to a sample key
@@ -321,13 +333,73 @@ __global__ void __launch_bounds__(kThreads) kth_cluster_kernel(const float* __re
   unsigned lo = s_lo, hi = s_hi;                      // keys in [lo, hi]
   int rank = k;                                       // of the wanted key: among all of them, then among those in the range
   bool found = false, numbers = true, lost = false;   // numbers: rank k falls among the scores that are numbers
+  // ---- the bracket's keys into shared memory: the passes below then read the scores no more (a CTA whose list overflows reads
+  // them again, whatever the others do)
+  auto raw_key = [](float f) {                        // score_key of a number; NaN goes below -inf or above +inf
+    const unsigned u = __float_as_uint(f);
+    return u ^ ((unsigned)((int)u >> 31) | 0x80000000u);
+  };
+  bool listed = false;
+  if (kBracket) {
+    const unsigned range = hi - lo;
+    int under = 0;
+    auto inside = [&](unsigned key) { return key - lo <= range; };
+    auto lower = [&](unsigned key) { return key - kKeyMinusInf < lo - kKeyMinusInf ? 1 : 0; };
+    auto one = [&](float f) {
+      const unsigned key = raw_key(f);
+      under += lower(key);
+      if (!inside(key)) return;
+      const int at = atomicAdd(&s_list, 1);
+      if (at < kKthList) list[at] = key;
+    };
+    constexpr int U = 4;                              // vectors a thread has in flight; a warp's share of the list in one piece
+    const int step = ctas * kThreads;
+    for (int base = rank_cta * kThreads + (tid & ~31); base < n4; base += U * step) {
+      unsigned key[U][4];
+      int mine = 0;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int i = base + lane + u * step;
+        const float4 v = i < n4 ? body[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+        key[u][0] = raw_key(v.x); key[u][1] = raw_key(v.y); key[u][2] = raw_key(v.z); key[u][3] = raw_key(v.w);
+        if (i >= n4) key[u][0] = key[u][1] = key[u][2] = key[u][3] = kKeyNaN;        // (neither inside nor below)
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          under += lower(key[u][e]);
+          mine += inside(key[u][e]) ? 1 : 0;
+        }
+      const int inc = scan(mine);
+      int at = 0;
+      if (lane == 31) at = atomicAdd(&s_list, inc);
+      at = __shfl_sync(0xffffffffu, at, 31) + inc - mine;
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (inside(key[u][e])) {
+            if (at < kKthList) list[at] = key[u][e];
+            ++at;
+          }
+    }
+    if (rank_cta == 0) {
+      if (tid < head) one(scores[tid]);
+      if (tid < n - tail0) one(scores[tail0 + tid]);
+    }
+    under = __reduce_add_sync(0xffffffffu, under);
+    if (lane == 0 && under != 0) atomicAdd(&s_under, under);
+    __syncthreads();
+    listed = s_list <= kKthList;
+  }
   ptx::cluster_sync_all();                            // every CTA's barrier is set up
   uint32_t phase = 0;
   for (bool first = true, whole = lo == kKeyMinusInf && hi == kKeyPlusInf; !found && numbers && !lost; ) {
     const unsigned range = hi - lo;
     const int shift = range < (unsigned)kKthBins ? 0 : 21 - __clz((int)range);
     for (int b = tid; b < kKthBins; b += kThreads) hist[b] = 0;
-    if (tid == 0) { s_bin = -1; s_below = 0; }
+    if (tid == 0) { s_bin = -1; s_below = first && !whole ? s_under : 0; }
     __syncthreads();
     int under = 0;
     auto walk = [&](auto count) {
@@ -350,15 +422,13 @@ __global__ void __launch_bounds__(kThreads) kth_cluster_kernel(const float* __re
         if (tid < n - tail0) count(scores[tail0 + tid]);
       }
     };
-    auto raw_key = [](float f) {                      // score_key of a number; NaN goes below -inf or above +inf
-      const unsigned u = __float_as_uint(f);
-      return u ^ ((unsigned)((int)u >> 31) | 0x80000000u);
-    };
     auto bin_of = [&](unsigned key) {
       const unsigned d = key - lo;
       if (d <= range) atomicAdd(&hist[d >> shift], 1);
     };
-    if (first)
+    if (kBracket && listed)
+      for (int i = tid; i < s_list; i += kThreads) bin_of(list[i]);
+    else if (first && whole)
       walk([&](float f) {
         const unsigned key = raw_key(f);
         under += key - kKeyMinusInf < lo - kKeyMinusInf ? 1 : 0;
@@ -366,7 +436,7 @@ __global__ void __launch_bounds__(kThreads) kth_cluster_kernel(const float* __re
       });
     else
       walk([&](float f) { bin_of(raw_key(f)); });
-    if (first) {
+    if (first && whole) {
       under = __reduce_add_sync(0xffffffffu, under);
       if (lane == 0 && under != 0) atomicAdd(&s_below, under);
     }
@@ -430,7 +500,7 @@ __global__ void __launch_bounds__(kThreads) kth_cluster_kernel(const float* __re
     } else if (bin == kKthLost) {
       lost = true;
     } else if (first && !whole) {                     // the bracket does not hold the rank: all keys
-      lo = kKeyMinusInf; hi = kKeyPlusInf; whole = true;
+      lo = kKeyMinusInf; hi = kKeyPlusInf; whole = true; listed = false;
     } else {
       numbers = false;
     }
@@ -493,15 +563,16 @@ __global__ void set_float_kernel(float* dst, float value) { *dst = value; }
 
 // One cluster of 16 CTAs where the device takes one of that size (asked once per device and kernel), of the portable 8
 // otherwise.
-template <typename... KArgs, typename... Args>
-static cudaError_t launch_cluster(void (*kernel)(KArgs...), cudaStream_t st, Args... args) {
-  static std::atomic<unsigned long long> asked{0}, wide{0};      // (per kernel signature: the two kernels' differ)
+template <bool kTag, typename... KArgs, typename... Args>
+static cudaError_t launch_cluster(void (*kernel)(KArgs...), int smem, cudaStream_t st, Args... args) {
+  static std::atomic<unsigned long long> asked{0}, wide{0};      // (per kernel: signature and tag tell them apart)
   int dev = 0;
   if (cudaError_t e = cudaGetDevice(&dev); e != cudaSuccess) return e;
   const unsigned long long bit = 1ull << (dev & 63);
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[2];
   cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cfg.attrs = attr;
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -513,6 +584,7 @@ static cudaError_t launch_cluster(void (*kernel)(KArgs...), cudaStream_t st, Arg
     cfg.gridDim = dim3(kKthMaxCtas);
     attr[0].val.clusterDim.x = kKthMaxCtas;
     cfg.numAttrs = 1;
+    if (cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); e != cudaSuccess) return e;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
         cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) == cudaSuccess && clusters > 0)
       wide.fetch_or(bit);
@@ -533,7 +605,9 @@ cudaError_t launch_kth_score_large(const float* scores, int n, int k, float* tau
     set_float_kernel<<<1, 1, 0, st>>>(tau_out, k <= 0 ? -INFINITY : INFINITY);
     return cudaGetLastError();
   }
-  return launch_cluster(kth_cluster_kernel, st, scores, n, k, tau_out, status, lose_one ? 1 : 0);
+  if (n >= kKthBracket)
+    return launch_cluster<true>(kth_cluster_kernel<true>, kKthList * 4, st, scores, n, k, tau_out, status, lose_one ? 1 : 0);
+  return launch_cluster<false>(kth_cluster_kernel<false>, 0, st, scores, n, k, tau_out, status, lose_one ? 1 : 0);
 }
 
 int select_large_tiles(long long n) { return (int)((n + kTile - 1) / kTile); }
@@ -546,12 +620,12 @@ cudaError_t launch_drift_scores(const float* a, const float* b, long long rows, 
     const long long n = (rows + 8 * rows_per_warp - 1) / (8 * rows_per_warp);
     return (int)(n < kSms * per_sm ? n : kSms * per_sm);
   };
-  if (hd == 32) drift_score_kernel<8, 1, 4><<<blocks(16, 8), 256, 0, st>>>(a, b, rows, scores);
-  else if (hd == 64) drift_score_kernel<16, 1, 4><<<blocks(8, 8), 256, 0, st>>>(a, b, rows, scores);
-  else if (hd == 128) drift_score_kernel<32, 1, 4><<<blocks(4, 8), 256, 0, st>>>(a, b, rows, scores);
-  else if (hd == 256) drift_score_kernel<32, 2, 2><<<blocks(2, 8), 256, 0, st>>>(a, b, rows, scores);
-  else drift_score_any_kernel<<<blocks(1, 16), 256, 0, st>>>(a, b, rows, hd, scores);
-  return cudaGetLastError();
+  auto launch = [&](auto kernel, int grid, auto... args) { return launch_pdl(kernel, dim3(grid), dim3(256), 0, st, 1, args...); };
+  if (hd == 32) return launch(drift_score_kernel<8, 1, 4>, blocks(16, 8), a, b, rows, scores);
+  if (hd == 64) return launch(drift_score_kernel<16, 1, 4>, blocks(8, 8), a, b, rows, scores);
+  if (hd == 128) return launch(drift_score_kernel<32, 1, 4>, blocks(4, 8), a, b, rows, scores);
+  if (hd == 256) return launch(drift_score_kernel<32, 2, 2>, blocks(2, 8), a, b, rows, scores);
+  return launch(drift_score_any_kernel, blocks(1, 16), a, b, rows, hd, scores);
 }
 
 // tile_counts and tile_offsets: device arrays of select_large_tiles(n) ints each; flags: 512 32-bit words per tile
@@ -559,9 +633,10 @@ cudaError_t launch_select_large(const float* scores, long long n, float tau, int
                                 int* tile_offsets, unsigned* flags, cudaStream_t st) {
   const int tiles = select_large_tiles(n);
   if (tiles == 0) return cudaMemsetAsync(count, 0, sizeof(int), st);
-  if (n <= kClusterSelect) return launch_cluster(select_cluster_kernel, st, scores, (int)n, tau, idx, count);
-  tile_flag_kernel<<<tiles, kThreads, 0, st>>>(scores, n, tau, tile_counts, flags);
-  cudaError_t e = launch_pdl(tile_scan_kernel, dim3(1), dim3(kThreads), 0, st, 1, (const int*)tile_counts, tiles,
+  if (n <= kClusterSelect) return launch_cluster<false>(select_cluster_kernel, 0, st, scores, (int)n, tau, idx, count);
+  cudaError_t e = launch_pdl(tile_flag_kernel, dim3(tiles), dim3(kThreads), 0, st, 1, scores, n, tau, tile_counts, flags);
+  if (e != cudaSuccess) return e;
+  e = launch_pdl(tile_scan_kernel, dim3(1), dim3(kThreads), 0, st, 1, (const int*)tile_counts, tiles,
                              tile_offsets, count);
   if (e != cudaSuccess) return e;
   e = launch_pdl(tile_scatter_kernel, dim3(tiles), dim3(kTileWords), 0, st, 1, (const unsigned*)flags,

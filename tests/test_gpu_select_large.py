@@ -164,6 +164,28 @@ def test_kth_of_many_scores(n, kind):
             assert got == (np.inf if np.isnan(want) else want), (kind, k, got, want)
 
 
+@pytest.mark.parametrize("kind", ["two values", "ascending", "spread"])
+def test_kth_with_more_keys_in_the_bracket_than_are_kept(kind):
+    """Two million scores: a bracket of tied keys overflows what a cluster's CTAs keep of it in shared memory, in all of them
+    or (sorted scores with one long tie) in some; against sort-and-index."""
+    import torch
+    from paper_2605_08134_b200 import dare
+    n = 2_100_003
+    rng = np.random.default_rng(5)
+    s = rng.standard_normal(n).astype(np.float32)
+    if kind == "two values":
+        s = np.where(rng.random(n) < 0.4, np.float32(0.25), np.float32(-3.0)).astype(np.float32)
+    elif kind == "ascending":
+        s.sort()
+        s[n // 3: n // 3 + 900_000] = s[n // 3]
+    sd = torch.from_numpy(s).cuda()
+    out = torch.zeros(1, device="cuda")
+    srt = np.sort(s)
+    for k in (1, n // 10, n // 2, int(0.93 * n), n - 1):
+        assert dare.dare_score_kth(sd.data_ptr(), n, k, out.data_ptr(), torch.cuda.current_stream().cuda_stream) == 0
+        assert out.cpu().numpy()[0] == srt[k - 1], (kind, k)
+
+
 @pytest.mark.parametrize("n", [1, 3, 4096, 65_536, 65_537, 262_143, 262_144, 262_145])
 def test_compaction_in_one_launch_and_in_three(n):
     """Around the size up to which one cluster compacts in a single launch: list, count, nothing past the list touched."""
