@@ -89,7 +89,10 @@ swiglu_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ 
     if (PAIR) tma_load_2d_pair(dst, &tm_x, i * BK, pr * BM, map_to_cta(smem_u32(&full_bar[s]), 0));
     else tma_load_2d(dst, &tm_x, i * BK, 0, &full_bar[s]);
   };
-  const int n_early = min(stages, KB);
+  // Weights asked for while the kernel before (a short norm) finishes: four stages; all of them took bandwidth from it.  Decoding
+  // step with every stage / four / three / two early, us: six layers of width 2048, 256 rows 500.2 / 496.9 / 497.0 / 498.1, 2 x 32
+  // rows 491.6 / 485.5 / 485.5 / 483.7; eight of 4096, 256 rows 1388.7 / 1384.5 / 1385.8 / 1386.6.
+  const int n_early = min(min(stages, 4), KB);
   if (warp == 0 && lane == 0)
     for (int i = 0; i < n_early; ++i) load_w(i, i);
   pdl_wait();
