@@ -14,6 +14,7 @@ CASES = [
     (1024, 128, 3, 300, 299),    # scores from the stored head; windows
     (512, 32, 5, 230, 0),        # two heads a tile
     (768, 256, 3, 257, 0),       # a head over four tiles
+    (992, 32, 3, 257, 0),        # width no multiple of 64: stays on the CUDA cores, tiles of 96 and 48 rows
     (448, 64, 7, 200, 190),      # seven blocks (an odd number), seven column tiles
 ]
 
