@@ -59,8 +59,8 @@ constexpr int kWarps = 2 + kFinish;
 // Column tiles are walked in groups, a group over all row tiles before the next.  What an SM pulls for a tile is the same in any
 // order, but not what has to come from the HBM: with all columns of a wide matrix innermost, each pair of row tiles streamed the
 // whole matrix through the L2 again (gate and up projections of width 12288: 200 MB, four times for 1024 rows), with a group of
-// 24 MB the matrix is read once and the rows, fewer bytes, once a group.  Four blocks of 2 x 512 rows a pass of a width 4096 stack
-// 3.70 -> 3.46 ms, output reuse over 8 x 1024 tokens 672 -> 635 us, dense step of 4 x 4096 2.88 -> 2.81 ms (at the power cap:
+// 24 MB the matrix is read once and the rows, fewer bytes, once a group.  First pass of eight layers of width 4096 over
+// 2 x 512 rows 3.70 -> 3.46 ms, output reuse over 8 x 1024 tokens 672 -> 635 us, dense step of 4 x 4096 2.88 -> 2.81 ms (at the power cap:
 // bytes not moved are clock); groups of 16, 20, 32 and 40 MB were all within 1 % of this.
 constexpr int kGroupBytes = 24 << 20;
 

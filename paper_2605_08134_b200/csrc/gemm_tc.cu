@@ -1,7 +1,7 @@
 // bf16 projection GEMMs on the 5th-generation tensor cores: C[m, n] = sum_k A[m, k] * W[n, k]  (W = [out, in],
 // Alg. 1 lines 2, 7, 11).  One CTA = one 128 x 256 output tile over one slice of the reduction dimension:
 //   warp 0    TMA producer: a 128-row A tile and a 256-row W tile per 64 k-elements (128 bytes per row, 128-byte
-//             swizzle) into a ring of 4 stages
+//             swizzle) into a ring of 4 stages (narrower tiles: more)
 //   warp 1    allocates tensor memory; one elected lane issues tcgen05.mma (M = 128, N = 256, K = 16) into a
 //             128 x 256 fp32 accumulator and commits each stage back to the producer.  The tensor pipe runs at full
 //             rate down to N = 128, but what an SM can pull from the L2 bounds the main loop of these projections,

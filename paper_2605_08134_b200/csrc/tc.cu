@@ -183,7 +183,7 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
   // A step of many tokens that reuses attention outputs needs the scoring head of every token (the score, the stored query),
   // and of the other heads only the queries that attend, the refresh set's (Alg. 2 line 8): the scoring head's 128 columns are
   // projected first, and the refresh set's queries behind the selection, beside its K and V where those are listed as well.
-  // 4 x 4096 tokens of width 4096, both rules, 15 % refreshed: 1019 -> 692 us; 8 x 1024, output reuse, 13 %: 783 -> 634 us.
+  // 4 x 4096 tokens of width 4096, both rules, 15 % refreshed: 1019 -> 684 us; 8 x 1024, output reuse, 13 %: 783 -> 627 us.
   // With (nearly) all tokens refreshed the scoring head is projected twice, one launch for nothing: 1-2 % of a step, which is
   // why the rule asks for a query projection of some size (us before / with it, every token refreshed, and at 13 to 30 %):
   //   both:   1 x 1152 of 4096 (39 GFLOP) 238 / 238, 148 / 139    8 x 1700 of 1536 (64) 490 / 494, 237 / 188
