@@ -1,19 +1,27 @@
 // fp32 projections on the tensor cores: C[m, n] = sum_k A[m, k] * W[n, k] with fp32 operands and fp32 accuracy.
-// An fp32 number is the sum of three bf16 numbers, exactly (8 + 8 + 8 bits of mantissa): x = h + m + l.  Of the nine products
-// of two such sums six are taken, hh, hm, mh, mm, hl, lh; the others are below 2^-25 of the product.  Products of bf16 are
-// exact on the tensor core, so what is left to lose is the accumulation: the tensor core's adds truncate, each by up to an ulp
-// of the running sum.  The reduction is therefore cut into blocks of 64: a block's products go into an accumulator of its
-// own, the small ones first (the four hh steps are the only ones that add to a sum of full size), and the blocks are added up
-// in fp32 registers, rounded to nearest.  Error against fp64, in units of 2^-24 (relative, widths 256 / 512 / 768 / 1024): 1.5 /
-// 1.6 / 1.7 / 1.85, where the chains of the CUDA-core kernel leave 1.9 / 2.6 / 4.2 / 4.9.
-// Bound by the MMAs: 24 of them take about 1450 cycles (their operands are 144 KB of shared-memory reads a block), the splitting
-// about 1050 beside them.  768 rows of width 1024: 46 us on the CUDA cores, 21 here; a step of 2 x 384 tokens 171.5 -> 118 us, of
-// 4 x 400 498 -> 266 us.  (With the issuing thread adding up blocks as well the tensor core idled 40 % of the time: 126 us.)
+// An fp32 number is the sum of three bf16 numbers (8 + 8 + 8 bits of mantissa): x = h + m + l, the split of Henry, Tang and
+// Heinecke, "Leveraging the bfloat16 Artificial Intelligence Datatype for Higher-Precision Computations" (ARITH 2019).  Of the
+// nine products of two such sums six are taken, hh, hm, mh, mm, hl, lh; the others are below 2^-25 of the product.  Products of
+// bf16 are exact on the tensor core, so what is left to lose is the accumulation: the tensor core's adds truncate, each by up to
+// an ulp of the running sum, and where the sum does not cancel these errors share a sign.  So no sum of full size is added to
+// there: every 16 k-elements of hh have an accumulator of their own (16 products of 8 x 8 bits fit its 24 bits nearly always), only
+// the small products, 2^-8 of the sum and less, add up over the whole reduction.  The rest is added in fp32 registers, rounded to
+// nearest: the four accumulators of a block of 64 as a tree, the blocks in chains of two to eight, the chains.
+// Error of V against fp64 in units of 2^-24 (2-norms), split / CUDA-core tiles that the launch rule takes otherwise, and (four hh
+// steps into one accumulator, as it was first):
+//   width               128                384                512                1024               4096
+//   zero-mean normal    0.96 / 1.49 (1.39) 1.13 / 2.26 (1.55) 1.18 / 3.47 (1.61) 1.30 / 4.86 (1.83) 1.83 / 6.85 (2.79)
+//   their magnitudes    0.72 / 0.75 (1.45) 0.87 / 0.95 (1.54) 0.77 / 1.46 (1.54) 0.81 / 2.01 (1.67) 0.94 / 2.06 (2.37)
+//   exp(2 normal)       2.23 / 1.32 (8.14) 2.04 / 1.77 (5.99) 2.07 / 2.83 (6.11) 2.14 / 4.29 (5.72) 1.94 / 5.68 (5.59)
+// (the last line: 16 products of one sign that span far more than 2^8, whose small ones are cut where they are lined up)
+// Bound by the splitting, about 1050 cycles a block of which the adding up slows each, beside 24 MMAs of 1450 in all (their operands
+// are 144 KB of shared-memory reads a block).  768 rows of width 1024: 46 us on the CUDA cores, 22 here; a step of 2 x 384 tokens,
+// key and value reuse, 171.5 -> 122 us (one accumulator a block, less accurate: 117), of 4 x 400 498 -> 272 us (264).
 // A CTA takes 128 rows x 64 columns: 32 rotary pairs, columns (j, j + head_dim / 2) of the heads they belong to, as in simt.cu.
-//   warps 0-3   add up the blocks: thread <-> row, tensor memory -> registers, into the finished tile
+//   warps 0-3   add up: thread <-> row, tensor memory -> registers, into the finished tile
 //   warps 4-11  fetch the operands (16 bytes a lane, whole lines), a block ahead of the one they split, and write the parts
 //               into a ring of two stages (72 KB each: 192 rows x 64 k x 3 parts) in the 128-byte-swizzled layout
-//   warp 12     issues the 24 MMAs (M 128, N 64, K 16) of a block into one of four accumulators
+//   warp 12     issues the 24 MMAs (M 128, N 64, K 16) of a block
 #include "sgemm.h"
 #include "tc_ptx.cuh"
 
@@ -22,7 +30,11 @@ namespace dare {
 using namespace ptx;
 
 namespace {
-constexpr int BM = 128, BN = 64, BK = 64, STAGES = 2, ACCS = 4, kSplitters = 256, kThreads = 128 + kSplitters + 32;
+constexpr int BM = 128, BN = 64, BK = 64, STAGES = 2, kSplitters = 256, kThreads = 128 + kSplitters + 32;
+// Tensor memory, 64 columns each: an accumulator for the hh products of every 16 k-elements of a block, one for the small products
+// of the whole reduction, and the sums put aside.
+constexpr int HH = BK / 16, ACC_SMALL = HH * BN, ACC_ASIDE = ACC_SMALL + BN, TMEM_COLS = 512;
+static_assert(HH == 4 && ACC_ASIDE + BN <= TMEM_COLS, "tensor memory of one CTA");
 constexpr int A_PART = BM * BK * 2, W_PART = BN * BK * 2, STAGE_BYTES = 3 * (A_PART + W_PART), W_OFFSET = 3 * A_PART;
 constexpr int CHUNKS = (BM + BN) * (BK / 4) / kSplitters;              // 16-byte chunks of a stage per splitting thread
 constexpr int ROWS = kSplitters / (BK / 4), W_CHUNKS = BN / ROWS;      // 16 rows a chunk index
@@ -61,8 +73,9 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f32_kernel(const SgemmParams
   uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem + BAR_OFFSET);
   uint64_t* empty_bar = full_bar + STAGES;
   uint64_t* acc_full = empty_bar + STAGES;
-  uint64_t* acc_empty = acc_full + ACCS;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + ACCS);
+  uint64_t* acc_empty = acc_full + 1;
+  uint64_t* all_done = acc_empty + 1;          // every MMA of the tile complete
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(all_done + 1);
   float* tile = reinterpret_cast<float*>(smem);
   // of a row: its token (-1: no such row), its row of A (then the first one's, dropped at the end), cache row and position
   __shared__ int s_tok[BM], s_pos[BM];
@@ -82,11 +95,11 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f32_kernel(const SgemmParams
   }
   if (tid == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(&full_bar[s], kSplitters / 32); mbar_init(&empty_bar[s], 1); }
-    for (int b = 0; b < ACCS; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], 4); }
+    mbar_init(acc_full, 1); mbar_init(acc_empty, 4); mbar_init(all_done, 1);
     fence_mbar_init();
   }
   if (warp == 1) {
-    tmem_alloc(tmem_slot, ACCS * BN);
+    tmem_alloc(tmem_slot, TMEM_COLS);
     tmem_relinquish();
   }
   // a splitting thread's chunks: rows row_of + 16 i of W's 64 and A's 128, elements kc .. kc + 3 of a block.  The weights do not
@@ -188,25 +201,30 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f32_kernel(const SgemmParams
   } else if (active && warp == 12) {
     constexpr uint32_t idesc = idesc_bf16(BM, BN);
     for (int kb = 0; kb < KB; ++kb) {
-      const int s = kb % STAGES, b = kb % ACCS;
+      const int s = kb % STAGES;
       mbar_wait(&full_bar[s], (kb / STAGES) & 1, p.status);
-      mbar_wait(&acc_empty[b], ((kb / ACCS) & 1) ^ 1, p.status);
+      mbar_wait(acc_empty, (kb & 1) ^ 1, p.status);
       tc_fence_after();
       if (elect_one()) {
-        const uint32_t stage = smem_u32(smem) + (uint32_t)(s * STAGE_BYTES), d = tmem_base + b * BN;
+        const uint32_t stage = smem_u32(smem) + (uint32_t)(s * STAGE_BYTES);
         uint64_t ad[3], wd[3];
 #pragma unroll
         for (int part = 0; part < 3; ++part) {
           ad[part] = smem_desc_k_sw128(stage + part * A_PART);
           wd[part] = smem_desc_k_sw128(stage + W_OFFSET + part * W_PART);
         }
-        constexpr int pa[6] = {2, 0, 1, 1, 0, 0}, pw[6] = {0, 2, 1, 0, 1, 0};    // the small products first
+        // hh first: while the small products run, the other warps read these four
 #pragma unroll
-        for (int j = 0; j < 6; ++j)
+        for (int k = 0; k < HH; ++k) umma_ss(tmem_base + k * BN, ad[0] + 2 * k, wd[0] + 2 * k, idesc, 0u);
+        umma_commit(acc_full);
+        constexpr int pa[5] = {2, 0, 1, 1, 0}, pw[5] = {0, 2, 1, 0, 1};
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k) umma_ss(d, ad[pa[j]] + 2 * k, wd[pw[j]] + 2 * k, idesc, (j | k) != 0 ? 1u : 0u);
+        for (int j = 0; j < 5; ++j)
+#pragma unroll
+          for (int k = 0; k < HH; ++k)
+            umma_ss(tmem_base + ACC_SMALL, ad[pa[j]] + 2 * k, wd[pw[j]] + 2 * k, idesc, (kb | j | k) != 0 ? 1u : 0u);
         umma_commit(&empty_bar[s]);
-        umma_commit(&acc_full[b]);
+        if (kb == KB - 1) umma_commit(all_done);
       }
       __syncwarp();
     }
@@ -215,20 +233,58 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f32_kernel(const SgemmParams
     float2 acc[BN / 2];
 #pragma unroll
     for (int c = 0; c < BN / 2; ++c) acc[c] = make_float2(0.f, 0.f);
-    for (int kb = 0; kb < KB; ++kb) {
-      const int b = kb % ACCS;
-      mbar_wait(&acc_full[b], (kb / ACCS) & 1, p.status);
-      tc_fence_after();
-      float v[BN / 2];
-      tmem_ld_32x32(t_lane + b * BN, v);
+    auto pair = [](const float* v, int e) { return make_float2(v[e], v[e + 1]); };
+    const float none[8] = {};
 #pragma unroll
-      for (int c = 0; c < 16; ++c) acc[c] = __fadd2_rn(acc[c], make_float2(v[2 * c], v[2 * c + 1]));
-      tmem_ld_32x32(t_lane + b * BN + 32, v);
+    for (int c = 0; c < BN; c += 8) tmem_st_32x8(t_lane + ACC_ASIDE + c, none);
+    const int chain = KB <= 6 ? 2 : max(4, KB / 8);                          // then its sum is put aside
+    int left = chain;
+#pragma unroll 1
+    for (int kb = 0; kb < KB; ++kb) {
+      mbar_wait(acc_full, kb & 1, p.status);
+      tc_fence_after();
+#pragma unroll
+      for (int c = 0; c < BN; c += 8) {
+        float v[HH][8];
+#pragma unroll
+        for (int k = 0; k < HH; ++k) tmem_ld_32x8_nowait(t_lane + k * BN + c, v[k]);
+        tmem_ld_wait();
+#pragma unroll
+        for (int e = 0; e < 8; e += 2)
+          acc[(c + e) / 2] = __fadd2_rn(acc[(c + e) / 2], __fadd2_rn(__fadd2_rn(pair(v[0], e), pair(v[1], e)),
+                                                                     __fadd2_rn(pair(v[2], e), pair(v[3], e))));
+      }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&acc_empty[b]);
+      if (lane == 0) mbar_arrive(acc_empty);
+      if (--left == 0) {
+        left = chain;
 #pragma unroll
-      for (int c = 0; c < 16; ++c) acc[16 + c] = __fadd2_rn(acc[16 + c], make_float2(v[2 * c], v[2 * c + 1]));
+        for (int c = 0; c < BN; c += 8) {
+          float sum[8];
+          tmem_ld_32x8_nowait(t_lane + ACC_ASIDE + c, sum);
+          tmem_ld_wait();
+#pragma unroll
+          for (int e = 0; e < 8; e += 2) {
+            const float2 x = __fadd2_rn(pair(sum, e), acc[(c + e) / 2]);
+            sum[e] = x.x; sum[e + 1] = x.y;
+            acc[(c + e) / 2] = make_float2(0.f, 0.f);
+          }
+          tmem_st_32x8(t_lane + ACC_ASIDE + c, sum);
+        }
+      }
+    }
+    mbar_wait(all_done, 0, p.status);
+    tc_fence_after();
+#pragma unroll
+    for (int c = 0; c < BN; c += 8) {
+      float small[8], sum[8];
+      tmem_ld_32x8_nowait(t_lane + ACC_SMALL + c, small);
+      tmem_ld_32x8_nowait(t_lane + ACC_ASIDE + c, sum);
+      tmem_ld_wait();
+#pragma unroll
+      for (int e = 0; e < 8; e += 2)
+        acc[(c + e) / 2] = __fadd2_rn(__fadd2_rn(acc[(c + e) / 2], pair(small, e)), pair(sum, e));
     }
     // the tile through the ring, idle by now (every MMA that read it is complete)
 #pragma unroll
@@ -306,7 +362,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f32_kernel(const SgemmParams
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 1) tmem_dealloc(tmem_base, ACCS * BN);
+  if (warp == 1) tmem_dealloc(tmem_base, TMEM_COLS);
 }
 
 template <int EPI>

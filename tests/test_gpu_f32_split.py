@@ -46,8 +46,9 @@ def test_steps_against_the_oracle(case):
     g.close()
 
 
-def _values(d, seq, spoil=None):
-    """The V cache of a dense step over 3 x `seq` rows and its operands, fp64 (x_norm from the fp32 kernel that makes it)."""
+def _values(d, seq, spoil=None, batch=3, rows=0):
+    """The V cache of a dense step over `batch` x `seq` rows (of which `rows` > 0: only the first of the first sequence are given to
+    the layer) and its operands, fp64 (x_norm from the fp32 kernel that makes it)."""
     import torch
     from paper_2605_08134_b200 import build
     build.build()
@@ -55,30 +56,52 @@ def _values(d, seq, spoil=None):
     gen = torch.Generator(device="cuda")
     gen.manual_seed(d + seq)
     draw = lambda *s: torch.empty(s, device="cuda").normal_(0, 1, generator=gen)
-    shape = _shape(d, 64, 3, seq)
+    shape = _shape(d, 64, 1, rows) if rows else _shape(d, 64, batch, seq)
     w = {k: draw(d, d) * 0.02 for k in ("w_q", "w_k", "w_v", "w_o")}
     w["rms_gain"] = torch.ones(d, device="cuda")
-    x = draw(3, seq, d)
+    x = draw(batch, seq, d)
     if spoil:
         spoil(w, x)
+    if rows:
+        x, batch, seq = x[:1, :rows].contiguous(), 1, rows
     layer = dare.Layer(shape, w)
     layer.step(x, 0, 0.1)
     xn = torch.empty_like(x)
-    assert dare.dare_rmsnorm(x.data_ptr(), w["rms_gain"].data_ptr(), xn.data_ptr(), 3 * seq, d, shape.rms_eps, wl.DTYPE_F32, 0) == 0
+    assert dare.dare_rmsnorm(x.data_ptr(), w["rms_gain"].data_ptr(), xn.data_ptr(), batch * seq, d, shape.rms_eps, wl.DTYPE_F32, 0) == 0
     torch.cuda.synchronize()
-    v = np.asarray(layer.read_caches(3, seq)["v"], np.float64)
+    v = np.asarray(layer.read_caches(batch, seq)["v"], np.float64)
     layer.close()
     return v, xn.double().cpu().numpy(), w["w_v"].double().cpu().numpy()
 
 
 @pytest.mark.parametrize("d,seq", [(512, 300), (1024, 257)])
 def test_accuracy(d, seq):
-    """A block of 64 ends in four truncated adds of up to 2^-23 of its sum each, the d / 64 <= 16 blocks are added with 2^-24
-    each: 4 x 2/3 + sqrt(16 / 6) units of 2^-24 at most on average, where the CUDA-core kernel's chains of d / 4 lose sqrt(d / 24)
-    (6.5 at 1024).  Measured 1.6 and 1.85; 3 is asked for, below what the chains leave at these widths."""
+    """16 products of an accumulator are cut by less than an ulp (2 units of 2^-24 of their sum, half of it on average), the
+    adds in registers leave 0.3 ulp each at a chain's, a tree's or the whole sum's size: below 2 units in all, where the CUDA-core
+    kernel's chains of d / 4 products lose sqrt(d / 24) (6.5 at 1024).  Measured 1.2 and 1.3; 3 is asked for."""
     v, xn, wv = _values(d, seq)
     want = xn @ wv.T
     assert np.linalg.norm(v - want) / np.linalg.norm(want) < 3 * 2.0 ** -24
+
+
+def _magnitudes(w, x):
+    for t in (*w.values(), x):
+        t.abs_()
+
+
+@pytest.mark.parametrize("d", [384, 512, 1024])
+@pytest.mark.parametrize("kind", ["normal", "one sign"])
+def test_no_less_accurate_than_the_cuda_core_kernel(d, kind):
+    """The same operands through both kernels (60 rows stay on the CUDA cores, 1200 do not), sums that cancel and sums that do not:
+    the split form's error against fp64 is at most the other's, up to 5 %, the spread of a norm over 60 x d rounding errors being
+    below one."""
+    spoil = _magnitudes if kind == "one sign" else None
+    err = []
+    for rows in (60, 0):
+        v, xn, wv = _values(d, 400, spoil, rows=rows)
+        want = xn @ wv.T
+        err.append(np.linalg.norm(v - want) / np.linalg.norm(want) * 2.0 ** 24)
+    assert err[1] <= 1.05 * err[0], err
 
 
 def test_infinities_and_nan():
