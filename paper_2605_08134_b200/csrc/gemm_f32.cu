@@ -1,27 +1,31 @@
 // fp32 projections on the tensor cores: C[m, n] = sum_k A[m, k] * W[n, k] with fp32 operands and fp32 accuracy.
-// An fp32 number is the sum of three bf16 numbers (8 + 8 + 8 bits of mantissa): x = h + m + l, the split of Henry, Tang and
-// Heinecke, "Leveraging the bfloat16 Artificial Intelligence Datatype for Higher-Precision Computations" (ARITH 2019).  Of the
-// nine products of two such sums six are taken, hh, hm, mh, mm, hl, lh; the others are below 2^-25 of the product.  Products of
-// bf16 are exact on the tensor core, so what is left to lose is the accumulation: the tensor core's adds truncate, each by up to
-// an ulp of the running sum, and where the sum does not cancel these errors share a sign.  So no sum of full size is added to
-// there: every 16 k-elements of hh have an accumulator of their own (16 products of 8 x 8 bits fit its 24 bits nearly always), only
-// the small products, 2^-8 of the sum and less, add up over the whole reduction.  The rest is added in fp32 registers, rounded to
-// nearest: the four accumulators of a block of 64 as a tree, the blocks in chains of two to eight, the chains.
+// An fp32 number is the sum of three bf16 numbers (8 + 8 + 8 bits of mantissa), here scaled: x = h + m / 2^8 + l / 2^16, the split
+// of Henry, Tang and Heinecke, "Leveraging the bfloat16 Artificial Intelligence Datatype for Higher-Precision Computations" (ARITH
+// 2019).  With the scales it holds exactly for every finite x that does not round up to infinity: h, m and l are multiples of 2^-133,
+// bf16's smallest number, however small x is (without them the last part is lost below about 2^-110, and weights of size 1e-35 left
+// 44 units of the error below).  Of the nine products of two such sums six are taken, hh, hm, mh, mm, hl, lh; the others are below
+// 2^-25 of the product.  Products of bf16 are exact on the tensor core, so what is left to lose is the accumulation: the tensor
+// core's adds truncate, each by up to an ulp of the running sum, and where the sum does not cancel these errors share a sign.  So
+// no sum of full size is added to there: every 16 k-elements of hh have an accumulator of their own (16 products of 8 x 8 bits fit
+// its 24 bits nearly always), only the small products, 2^-8 of the sum and less, add up over the whole reduction, those of scale
+// 2^8 and of 2^16 apart.  The rest is added in fp32 registers, rounded to nearest: the four accumulators of a block of 64 as a
+// tree, the blocks in chains of two to eight, the chains.
 // Error of V against fp64 in units of 2^-24 (2-norms), split / CUDA-core tiles that the launch rule takes otherwise, and (four hh
 // steps into one accumulator, as it was first):
 //   width               128                384                512                1024               4096
-//   zero-mean normal    0.96 / 1.49 (1.39) 1.13 / 2.26 (1.55) 1.18 / 3.47 (1.61) 1.30 / 4.86 (1.83) 1.83 / 6.85 (2.79)
+//   zero-mean normal    0.96 / 1.49 (1.39) 1.12 / 2.26 (1.55) 1.18 / 3.47 (1.61) 1.28 / 4.86 (1.83) 1.62 / 6.85 (2.79)
 //   their magnitudes    0.72 / 0.75 (1.45) 0.87 / 0.95 (1.54) 0.77 / 1.46 (1.54) 0.81 / 2.01 (1.67) 0.94 / 2.06 (2.37)
-//   exp(2 normal)       2.23 / 1.32 (8.14) 2.04 / 1.77 (5.99) 2.07 / 2.83 (6.11) 2.14 / 4.29 (5.72) 1.94 / 5.68 (5.59)
+//   exp(2 normal)       2.24 / 1.32 (8.14) 2.04 / 1.77 (5.99) 2.07 / 2.83 (6.11) 2.13 / 4.29 (5.72) 1.91 / 5.68 (5.59)
 // (the last line: 16 products of one sign that span far more than 2^8, whose small ones are cut where they are lined up)
-// Bound by the splitting, about 1050 cycles a block of which the adding up slows each, beside 24 MMAs of 1450 in all (their operands
-// are 144 KB of shared-memory reads a block).  768 rows of width 1024: 46 us on the CUDA cores, 22 here; a step of 2 x 384 tokens,
-// key and value reuse, 171.5 -> 122 us (one accumulator a block, less accurate: 117), of 4 x 400 498 -> 272 us (264).
+// Bound by the splitting, which the adding up beside it slows.  The products of one part of A with two parts of W that lie side by
+// side are one MMA, with the accumulators of both scales side by side as well: 16 MMAs a block that read 112 KB of shared memory,
+// not 24 that read 144.  A step of 2 x 384 tokens of width 1024, key and value reuse, 171.5 us on the CUDA cores, 122 here (24 MMAs:
+// 124; unscaled, one accumulator a block, less accurate: 117), dense of 4 x 400 498 -> 275 us (277; 264).
 // A CTA takes 128 rows x 64 columns: 32 rotary pairs, columns (j, j + head_dim / 2) of the heads they belong to, as in simt.cu.
 //   warps 0-3   add up: thread <-> row, tensor memory -> registers, into the finished tile
 //   warps 4-11  fetch the operands (16 bytes a lane, whole lines), a block ahead of the one they split, and write the parts
 //               into a ring of two stages (72 KB each: 192 rows x 64 k x 3 parts) in the 128-byte-swizzled layout
-//   warp 12     issues the 24 MMAs (M 128, N 64, K 16) of a block
+//   warp 12     issues the 16 MMAs (M 128, N 64 or 128, K 16) of a block
 #include "sgemm.h"
 #include "tc_ptx.cuh"
 
@@ -31,9 +35,9 @@ using namespace ptx;
 
 namespace {
 constexpr int BM = 128, BN = 64, BK = 64, STAGES = 2, kSplitters = 256, kThreads = 128 + kSplitters + 32;
-// Tensor memory, 64 columns each: an accumulator for the hh products of every 16 k-elements of a block, one for the small products
-// of the whole reduction, and the sums put aside.
-constexpr int HH = BK / 16, ACC_SMALL = HH * BN, ACC_ASIDE = ACC_SMALL + BN, TMEM_COLS = 512;
+// Tensor memory, 64 columns each: an accumulator for the hh products of every 16 k-elements of a block, the small products of the
+// whole reduction by their scale (2^8: hm, mh; 2^16: hl, mm, lh), and the sums put aside.
+constexpr int HH = BK / 16, ACC_MID = HH * BN, ACC_LOW = ACC_MID + BN, ACC_ASIDE = ACC_LOW + BN, TMEM_COLS = 512;
 static_assert(HH == 4 && ACC_ASIDE + BN <= TMEM_COLS, "tensor memory of one CTA");
 constexpr int A_PART = BM * BK * 2, W_PART = BN * BK * 2, STAGE_BYTES = 3 * (A_PART + W_PART), W_OFFSET = 3 * A_PART;
 constexpr int CHUNKS = (BM + BN) * (BK / 4) / kSplitters;              // 16-byte chunks of a stage per splitting thread
@@ -160,8 +164,9 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f32_kernel(const SgemmParams
       for (int part = 0; part < 3; ++part) {
         const __nv_bfloat162 b = __floats2bfloat162_rn(v.x, v.y);
         o[part] = *reinterpret_cast<const uint32_t*>(&b);
-        // (minus the rounded pair: the sign bits flipped on the way)
-        if (part < 2) v = __fadd2_rn(v, make_float2(-__uint_as_float(o[part] << 16), -__uint_as_float(o[part] & 0xffff0000u)));
+        if (part < 2)
+          v = __fmul2_rn(__ffma2_rn(make_float2(__uint_as_float(o[part] << 16), __uint_as_float(o[part] & 0xffff0000u)),
+                                    make_float2(-1.f, -1.f), v), make_float2(256.f, 256.f));
       }
     };
     const uint32_t thread_at = smem_u32(smem) + (uint32_t)(row_of * 128 + (((kc >> 3) ^ (row_of & 7)) << 4) + (kc & 4) * 2);
@@ -199,7 +204,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f32_kernel(const SgemmParams
       }
     }
   } else if (active && warp == 12) {
-    constexpr uint32_t idesc = idesc_bf16(BM, BN);
+    constexpr uint32_t idesc = idesc_bf16(BM, BN), idesc2 = idesc_bf16(BM, 2 * BN);
     for (int kb = 0; kb < KB; ++kb) {
       const int s = kb % STAGES;
       mbar_wait(&full_bar[s], (kb / STAGES) & 1, p.status);
@@ -217,12 +222,12 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f32_kernel(const SgemmParams
 #pragma unroll
         for (int k = 0; k < HH; ++k) umma_ss(tmem_base + k * BN, ad[0] + 2 * k, wd[0] + 2 * k, idesc, 0u);
         umma_commit(acc_full);
-        constexpr int pa[5] = {2, 0, 1, 1, 0}, pw[5] = {0, 2, 1, 0, 1};
 #pragma unroll
-        for (int j = 0; j < 5; ++j)
+        for (int k = 0; k < HH; ++k) umma_ss(tmem_base + ACC_MID, ad[0] + 2 * k, wd[1] + 2 * k, idesc2, (kb | k) != 0 ? 1u : 0u);   // hm, hl
 #pragma unroll
-          for (int k = 0; k < HH; ++k)
-            umma_ss(tmem_base + ACC_SMALL, ad[pa[j]] + 2 * k, wd[pw[j]] + 2 * k, idesc, (kb | j | k) != 0 ? 1u : 0u);
+        for (int k = 0; k < HH; ++k) umma_ss(tmem_base + ACC_MID, ad[1] + 2 * k, wd[0] + 2 * k, idesc2, 1u);                        // mh, mm
+#pragma unroll
+        for (int k = 0; k < HH; ++k) umma_ss(tmem_base + ACC_LOW, ad[2] + 2 * k, wd[0] + 2 * k, idesc, 1u);                         // lh
         umma_commit(&empty_bar[s]);
         if (kb == KB - 1) umma_commit(all_done);
       }
@@ -276,15 +281,17 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f32_kernel(const SgemmParams
     }
     mbar_wait(all_done, 0, p.status);
     tc_fence_after();
+    const float2 down = make_float2(1.f / 256.f, 1.f / 256.f);
 #pragma unroll
     for (int c = 0; c < BN; c += 8) {
-      float small[8], sum[8];
-      tmem_ld_32x8_nowait(t_lane + ACC_SMALL + c, small);
+      float mid[8], low[8], sum[8];
+      tmem_ld_32x8_nowait(t_lane + ACC_MID + c, mid);
+      tmem_ld_32x8_nowait(t_lane + ACC_LOW + c, low);
       tmem_ld_32x8_nowait(t_lane + ACC_ASIDE + c, sum);
       tmem_ld_wait();
 #pragma unroll
       for (int e = 0; e < 8; e += 2)
-        acc[(c + e) / 2] = __fadd2_rn(__fadd2_rn(acc[(c + e) / 2], pair(small, e)), pair(sum, e));
+        acc[(c + e) / 2] = __fadd2_rn(__ffma2_rn(__ffma2_rn(pair(low, e), down, pair(mid, e)), down, acc[(c + e) / 2]), pair(sum, e));
     }
     // the tile through the ring, idle by now (every MMA that read it is complete)
 #pragma unroll

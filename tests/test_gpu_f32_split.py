@@ -104,6 +104,16 @@ def test_no_less_accurate_than_the_cuda_core_kernel(d, kind):
     assert err[1] <= 1.05 * err[0], err
 
 
+@pytest.mark.parametrize("size", [1e-35, 1e-37, 1e34])
+def test_weights_of_any_size(size):
+    """Weights of any size split exactly (here products and sums stay normal numbers): the bound of test_accuracy."""
+    def spoil(w, x):
+        w["w_v"].mul_(size / 0.02)
+    v, xn, wv = _values(512, 300, spoil)
+    want = xn @ wv.T
+    assert np.linalg.norm(v / size - want / size) / np.linalg.norm(want / size) < 3 * 2.0 ** -24
+
+
 def test_infinities_and_nan():
     def spoil(w, x):
         w["w_v"][7, 11] = float("inf")        # a column of V: +-inf by the sign of the row's element 11
