@@ -16,6 +16,9 @@ CASES = [
     (768, 256, 3, 257, 0),       # a head over four tiles
     (992, 32, 3, 257, 0),        # width no multiple of 64: stays on the CUDA cores, tiles of 96 and 48 rows
     (448, 64, 7, 200, 190),      # seven blocks (an odd number), seven column tiles
+    (128, 32, 4, 2100, 0),       # the narrowest that it takes: two blocks, one chain
+    (192, 64, 4, 600, 0),        # three blocks, the last in a chain of its own
+    (2048, 128, 1, 130, 0),      # wider than the launch rule's other sizes: 32 blocks, chains of four
 ]
 
 
