@@ -17,6 +17,7 @@
 // whole wave back, and a CTA's loads do not overlap its walk: the chain per tile (scores -> scan -> publish -> walk
 // -> write) is several microseconds long, and what a CTA has in flight during it does not cover it.
 #include <math.h>
+#include <algorithm>
 #include <mutex>
 
 #include "dare_internal.h"
@@ -250,8 +251,8 @@ __global__ void __launch_bounds__(kTileWords) tile_scatter_kernel(const unsigned
 // shared-memory atomic takes a cycle a lane whatever it meets, so the first pass costs a cycle a score of the CTA's share
 // (copies of the histogram changed nothing): with many scores the range starts as a bracket around rank k from a sample of
 // 256 of them, which most scores lie outside; a bracket that turns out not to hold the rank is given up for all keys.
-// The bracket's keys (about a seventh of the scores) are kept in shared memory as they are found, so the narrowing passes read
-// them and not the scores again: a call of 2^20 scores 2-4 us shorter; a kernel of its own, for the code cost 20000 scores 0.6 us.
+// Where the bracket's keys fit (kth_list_keys), they are kept in shared memory as they are found, and the narrowing passes read
+// them, not the scores again: a call of 2^19 to 2^21 scores 1-10 % shorter; a kernel of its own, for the code cost 20000 scores 0.6 us.
 // A cluster (rather than a grid) because the call has no scratch memory to meet in: nothing is shared between calls,
 // whatever streams they run on.
 // A CTA that waits in vain for the others' bins records the time-out in the status word (if the caller has one), gives the
@@ -259,8 +260,25 @@ __global__ void __launch_bounds__(kTileWords) tile_scatter_kernel(const unsigned
 // threshold is NaN, which Eq. 2 reads as "refresh everything".
 constexpr int kKthBins = 2048, kKthMaxCtas = 16, kKthSample = 256;
 constexpr int kKthBracket = 1 << 19;        // the sample costs about 4 us: from this many scores on
-constexpr int kKthList = 48 * 1024;         // keys of the bracket that a CTA keeps in shared memory (one CTA an SM)
+constexpr int kKthList = 48 * 1024;         // keys of the bracket that a CTA keeps in shared memory, at most (one CTA an SM)
 constexpr unsigned kKeyMinusInf = 0x007fffffu, kKeyPlusInf = 0xff800000u;
+
+// The bracket around rank k: the sample's keys four standard deviations of its rank either side.
+__host__ __device__ __forceinline__ void kth_bracket(int n, int k, int* lo, int* hi) {
+  const float p = (float)k / (float)n;
+  const int c = (int)(p * kKthSample), w = (int)(4.f * sqrtf(p * (1.f - p) * kKthSample)) + 2;
+  *lo = c - w; *hi = c + w;
+}
+// Keys that a CTA keeps of it: its share of the scores between those two keys (27 % at the median, 18 % for k = 0.87 n, 14 % for
+// 0.93 n) and four standard deviations of that share, as far as they fit; none where not even two would, from 2.4, 3.4 and 4.1
+// million scores on (collected and then of no use, they made calls of 4 to 16 million 50-65 % longer).
+int kth_list_keys(int n, int k, int ctas) {
+  int lo, hi;
+  kth_bracket(n, k, &lo, &hi);
+  const float share = (float)(std::min(hi + 1, kKthSample) - std::max(lo, 0)) / (float)kKthSample;
+  const float sd = sqrtf(share * (1.f - share) / (float)kKthSample), scores = (float)n / (float)ctas;
+  return (share + 2.f * sd) * scores <= (float)kKthList ? std::min(kKthList, (int)((share + 4.f * sd) * scores)) : 0;
+}
 
 constexpr int kKthLost = -2;                // s_bin: some CTA's bins never came
 constexpr unsigned long long kKthLoseWaitNs = 1000000ull;
@@ -285,7 +303,8 @@ __global__ void __launch_bounds__(kThreads) kth_cluster_kernel(const float* __re
   __shared__ int part[kKthBins / 8 / 32], totals[kKthMaxCtas], below[kKthMaxCtas], s_below, s_bin, s_rank;
   __shared__ unsigned s_lo, s_hi;
   __shared__ int s_list, s_under;
-  extern __shared__ unsigned list[];                  // (bracket only: kKthList keys)
+  extern __shared__ unsigned list[];                  // (bracket only, and only where the launch gave it room)
+  int list_keys = kBracket ? (int)(ptx::dynamic_smem_bytes() / 4u) : 0;
   const int ctas = (int)gridDim.x, rank_cta = (int)ptx::cluster_ctarank(), lane = threadIdx.x & 31, tid = (int)threadIdx.x;
   const int slice = kKthBins / ctas;                  // 128 or 256: whole warps, four or eight bins to a lane
   ptx::pdl_wait();
@@ -302,7 +321,7 @@ __global__ void __launch_bounds__(kThreads) kth_cluster_kernel(const float* __re
     }
     return v;
   };
-  // ---- the bracket, the same in every CTA: the sample's keys four standard deviations of its rank either side of k
+  // ---- the bracket, the same in every CTA
   if (kBracket && tid < kKthSample) sample[tid] = score_key(scores[(int)(((long long)tid * n) / kKthSample)]);
   if (tid == 0) {
     s_lo = kKeyMinusInf; s_hi = kKeyPlusInf;
@@ -312,8 +331,8 @@ __global__ void __launch_bounds__(kThreads) kth_cluster_kernel(const float* __re
   }
   __syncthreads();
   if (kBracket) {
-    const float p = (float)k / (float)n;
-    const int c = (int)(p * kKthSample), w = (int)(4.f * sqrtf(p * (1.f - p) * kKthSample)) + 2;
+    int at_lo, at_hi;
+    kth_bracket(n, k, &at_lo, &at_hi);
     const int me = tid >> 2;                          // four threads to a sample key
     const unsigned mine = sample[me];
     int r = 0;
@@ -325,121 +344,131 @@ __global__ void __launch_bounds__(kThreads) kth_cluster_kernel(const float* __re
     r += __shfl_xor_sync(0xffffffffu, r, 1);
     r += __shfl_xor_sync(0xffffffffu, r, 2);
     if ((tid & 3) == 0) {
-      if (r == c - w && mine != kKeyNaN) s_lo = mine;
-      if (r == c + w && mine != kKeyNaN) s_hi = mine;
+      if (r == at_lo && mine != kKeyNaN) s_lo = mine;
+      if (r == at_hi && mine != kKeyNaN) s_hi = mine;
     }
   }
   __syncthreads();
   unsigned lo = s_lo, hi = s_hi;                      // keys in [lo, hi]
   int rank = k;                                       // of the wanted key: among all of them, then among those in the range
   bool found = false, numbers = true, lost = false;   // numbers: rank k falls among the scores that are numbers
-  // ---- the bracket's keys into shared memory: the passes below then read the scores no more (a CTA whose list overflows reads
-  // them again, whatever the others do)
   auto raw_key = [](float f) {                        // score_key of a number; NaN goes below -inf or above +inf
     const unsigned u = __float_as_uint(f);
     return u ^ ((unsigned)((int)u >> 31) | 0x80000000u);
   };
-  bool listed = false;
-  if (kBracket) {
-    const unsigned range = hi - lo;
-    int under = 0;
-    auto inside = [&](unsigned key) { return key - lo <= range; };
-    auto lower = [&](unsigned key) { return key - kKeyMinusInf < lo - kKeyMinusInf ? 1 : 0; };
-    auto one = [&](float f) {
-      const unsigned key = raw_key(f);
-      under += lower(key);
-      if (!inside(key)) return;
-      const int at = atomicAdd(&s_list, 1);
-      if (at < kKthList) list[at] = key;
-    };
-    constexpr int U = 4;                              // vectors a thread has in flight; a warp's share of the list in one piece
+  // width of a bin of [lo, hi], as a shift
+  auto shift_now = [&]() { return hi - lo < (unsigned)kKthBins ? 0 : 21 - __clz((int)(hi - lo)); };
+  auto lower = [&](unsigned key) { return key - kKeyMinusInf < lo - kKeyMinusInf ? 1 : 0; };
+  auto walk = [&](auto count) {
+    constexpr int U = 8;                            // vectors a thread has in flight
     const int step = ctas * kThreads;
-    for (int base = rank_cta * kThreads + (tid & ~31); base < n4; base += U * step) {
-      unsigned key[U][4];
-      int mine = 0;
+    int i = rank_cta * kThreads + tid;
+    for (; i + (U - 1) * step < n4; i += U * step) {
+      float4 v[U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int i = base + lane + u * step;
-        const float4 v = i < n4 ? body[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-        key[u][0] = raw_key(v.x); key[u][1] = raw_key(v.y); key[u][2] = raw_key(v.z); key[u][3] = raw_key(v.w);
-        if (i >= n4) key[u][0] = key[u][1] = key[u][2] = key[u][3] = kKeyNaN;        // (neither inside nor below)
-      }
+      for (int u = 0; u < U; ++u) v[u] = body[i + u * step];
 #pragma unroll
-      for (int u = 0; u < U; ++u)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          under += lower(key[u][e]);
-          mine += inside(key[u][e]) ? 1 : 0;
-        }
-      const int inc = scan(mine);
-      int at = 0;
-      if (lane == 31) at = atomicAdd(&s_list, inc);
-      at = __shfl_sync(0xffffffffu, at, 31) + inc - mine;
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-          if (inside(key[u][e])) {
-            if (at < kKthList) list[at] = key[u][e];
-            ++at;
-          }
+      for (int u = 0; u < U; ++u) { count(v[u].x); count(v[u].y); count(v[u].z); count(v[u].w); }
+    }
+    for (; i < n4; i += step) {
+      const float4 v = body[i];
+      count(v.x); count(v.y); count(v.z); count(v.w);
     }
     if (rank_cta == 0) {
-      if (tid < head) one(scores[tid]);
-      if (tid < n - tail0) one(scores[tail0 + tid]);
+      if (tid < head) count(scores[tid]);
+      if (tid < n - tail0) count(scores[tail0 + tid]);
+    }
+  };
+  // ---- the first pass over a bracket: what lies below it, and its keys, kept for all passes that follow (a CTA whose keys turn out to
+  // be more than it has room for reads the scores for them, whatever the others do), or the first pass's bins
+  bool listed = false, binned = false;                // binned: the bins of [lo, hi] are there
+  if (kBracket) {
+    const unsigned range = hi - lo;
+    const int shift = shift_now();
+    int under = 0;
+    for (int b = tid; b < kKthBins; b += kThreads) hist[b] = 0;
+    // No keys kept where one pass is all (a bracket of one tied score, say), or where the sample says that they will not fit (a
+    // tie with one of the bracket's ends)
+    const int in_sample = __syncthreads_count(tid < kKthSample && sample[tid & (kKthSample - 1)] - lo <= range);
+    if (shift == 0 || (float)in_sample * (float)n > (float)list_keys * (float)(kKthSample * ctas)) list_keys = 0;
+    auto bin = [&](float f) {
+      const unsigned key = raw_key(f);
+      under += lower(key);
+      if (key - lo <= range) atomicAdd(&hist[(key - lo) >> shift], 1);
+    };
+    auto keep = [&](float f) {
+      const unsigned key = raw_key(f);
+      under += lower(key);
+      if (key - lo > range) return;
+      const int at = atomicAdd(&s_list, 1);
+      if (at < list_keys) list[at] = key;
+    };
+    if (list_keys > 0) {
+      constexpr int U = 4;                            // vectors a thread has in flight; a warp's share of the list in one piece
+      const int step = ctas * kThreads;
+      for (int base = rank_cta * kThreads + (tid & ~31); base < n4; base += U * step) {
+        unsigned key[U][4];
+        int mine = 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int i = base + lane + u * step;
+          const float4 v = i < n4 ? body[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+          key[u][0] = raw_key(v.x); key[u][1] = raw_key(v.y); key[u][2] = raw_key(v.z); key[u][3] = raw_key(v.w);
+          if (i >= n4) key[u][0] = key[u][1] = key[u][2] = key[u][3] = kKeyNaN;      // (neither inside nor below)
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            under += lower(key[u][e]);
+            mine += key[u][e] - lo <= range ? 1 : 0;
+          }
+        const int inc = scan(mine);
+        int at = 0;
+        if (lane == 31) at = atomicAdd(&s_list, inc);
+        at = __shfl_sync(0xffffffffu, at, 31) + inc - mine;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            if (key[u][e] - lo <= range) {
+              if (at < list_keys) list[at] = key[u][e];
+              ++at;
+            }
+      }
+      if (rank_cta == 0) {
+        if (tid < head) keep(scores[tid]);
+        if (tid < n - tail0) keep(scores[tail0 + tid]);
+      }
+    } else {
+      walk(bin);
+      binned = true;
     }
     under = __reduce_add_sync(0xffffffffu, under);
     if (lane == 0 && under != 0) atomicAdd(&s_under, under);
     __syncthreads();
-    listed = s_list <= kKthList;
+    listed = list_keys > 0 && s_list <= list_keys;
   }
   ptx::cluster_sync_all();                            // every CTA's barrier is set up
   uint32_t phase = 0;
   for (bool first = true, whole = lo == kKeyMinusInf && hi == kKeyPlusInf; !found && numbers && !lost; ) {
-    const unsigned range = hi - lo;
-    const int shift = range < (unsigned)kKthBins ? 0 : 21 - __clz((int)range);
-    for (int b = tid; b < kKthBins; b += kThreads) hist[b] = 0;
-    if (tid == 0) { s_bin = -1; s_below = first && !whole ? s_under : 0; }
+    const int shift = shift_now();
+    if (!binned)
+      for (int b = tid; b < kKthBins; b += kThreads) hist[b] = 0;
+    if (tid == 0) { s_bin = -1; s_below = kBracket && first && !whole ? s_under : 0; }
     __syncthreads();
-    int under = 0;
-    auto walk = [&](auto count) {
-      constexpr int U = 8;                            // vectors a thread has in flight
-      const int step = ctas * kThreads;
-      int i = rank_cta * kThreads + tid;
-      for (; i + (U - 1) * step < n4; i += U * step) {
-        float4 v[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) v[u] = body[i + u * step];
-#pragma unroll
-        for (int u = 0; u < U; ++u) { count(v[u].x); count(v[u].y); count(v[u].z); count(v[u].w); }
-      }
-      for (; i < n4; i += step) {
-        const float4 v = body[i];
-        count(v.x); count(v.y); count(v.z); count(v.w);
-      }
-      if (rank_cta == 0) {
-        if (tid < head) count(scores[tid]);
-        if (tid < n - tail0) count(scores[tail0 + tid]);
-      }
-    };
-    auto bin_of = [&](unsigned key) {
-      const unsigned d = key - lo;
-      if (d <= range) atomicAdd(&hist[d >> shift], 1);
-    };
-    if (kBracket && listed)
-      for (int i = tid; i < s_list; i += kThreads) bin_of(list[i]);
-    else if (first && whole)
-      walk([&](float f) {
-        const unsigned key = raw_key(f);
-        under += key - kKeyMinusInf < lo - kKeyMinusInf ? 1 : 0;
-        bin_of(key);
-      });
-    else
-      walk([&](float f) { bin_of(raw_key(f)); });
-    if (first && whole) {
-      under = __reduce_add_sync(0xffffffffu, under);
-      if (lane == 0 && under != 0) atomicAdd(&s_below, under);
+    if (!binned) {
+      const unsigned range = hi - lo;
+      auto bin_of = [&](unsigned key) {
+        const unsigned d = key - lo;
+        if (d <= range) atomicAdd(&hist[d >> shift], 1);
+      };
+      if (kBracket && listed)
+        for (int i = tid; i < s_list; i += kThreads) bin_of(list[i]);
+      else
+        walk([&](float f) { bin_of(raw_key(f)); });
     }
+    binned = false;
     if (tid == 0) ptx::mbar_arrive_expect_tx(&recv_bar, (uint32_t)kKthBins * 4u);
     ptx::fence_proxy_async_smem();
     __syncthreads();
@@ -563,8 +592,9 @@ __global__ void set_float_kernel(float* dst, float value) { *dst = value; }
 
 // One cluster of 16 CTAs where the device takes one of that size (asked once per device and kernel), of the portable 8
 // otherwise.
-template <bool kTag, typename... KArgs, typename... Args>
-static cudaError_t launch_cluster(void (*kernel)(KArgs...), int smem, cudaStream_t st, Args... args) {
+// smem(number of CTAs): dynamic shared memory of a CTA, at most max_smem.
+template <bool kTag, typename Smem, typename... KArgs, typename... Args>
+static cudaError_t launch_cluster(void (*kernel)(KArgs...), int max_smem, Smem smem, cudaStream_t st, Args... args) {
   static std::atomic<unsigned long long> asked{0}, wide{0};      // (per kernel: signature and tag tell them apart)
   int dev = 0;
   if (cudaError_t e = cudaGetDevice(&dev); e != cudaSuccess) return e;
@@ -572,7 +602,6 @@ static cudaError_t launch_cluster(void (*kernel)(KArgs...), int smem, cudaStream
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[2];
   cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cfg.attrs = attr;
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -584,7 +613,8 @@ static cudaError_t launch_cluster(void (*kernel)(KArgs...), int smem, cudaStream
     cfg.gridDim = dim3(kKthMaxCtas);
     attr[0].val.clusterDim.x = kKthMaxCtas;
     cfg.numAttrs = 1;
-    if (cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); e != cudaSuccess) return e;
+    cfg.dynamicSmemBytes = max_smem;
+    if (cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem); e != cudaSuccess) return e;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
         cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) == cudaSuccess && clusters > 0)
       wide.fetch_or(bit);
@@ -596,6 +626,7 @@ static cudaError_t launch_cluster(void (*kernel)(KArgs...), int smem, cudaStream
   cfg.gridDim = dim3(ctas);
   attr[0].val.clusterDim.x = ctas;
   cfg.numAttrs = 2;
+  cfg.dynamicSmemBytes = smem((int)ctas);
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
@@ -606,8 +637,10 @@ cudaError_t launch_kth_score_large(const float* scores, int n, int k, float* tau
     return cudaGetLastError();
   }
   if (n >= kKthBracket)
-    return launch_cluster<true>(kth_cluster_kernel<true>, kKthList * 4, st, scores, n, k, tau_out, status, lose_one ? 1 : 0);
-  return launch_cluster<false>(kth_cluster_kernel<false>, 0, st, scores, n, k, tau_out, status, lose_one ? 1 : 0);
+    return launch_cluster<true>(kth_cluster_kernel<true>, kKthList * 4, [&](int ctas) { return kth_list_keys(n, k, ctas) * 4; }, st,
+                                scores, n, k, tau_out, status, lose_one ? 1 : 0);
+  return launch_cluster<false>(kth_cluster_kernel<false>, 0, [](int) { return 0; }, st, scores, n, k, tau_out, status,
+                               lose_one ? 1 : 0);
 }
 
 int select_large_tiles(long long n) { return (int)((n + kTile - 1) / kTile); }
@@ -633,7 +666,7 @@ cudaError_t launch_select_large(const float* scores, long long n, float tau, int
                                 int* tile_offsets, unsigned* flags, cudaStream_t st) {
   const int tiles = select_large_tiles(n);
   if (tiles == 0) return cudaMemsetAsync(count, 0, sizeof(int), st);
-  if (n <= kClusterSelect) return launch_cluster<false>(select_cluster_kernel, 0, st, scores, (int)n, tau, idx, count);
+  if (n <= kClusterSelect) return launch_cluster<false>(select_cluster_kernel, 0, [](int) { return 0; }, st, scores, (int)n, tau, idx, count);
   cudaError_t e = launch_pdl(tile_flag_kernel, dim3(tiles), dim3(kThreads), 0, st, 1, scores, n, tau, tile_counts, flags);
   if (e != cudaSuccess) return e;
   e = launch_pdl(tile_scan_kernel, dim3(1), dim3(kThreads), 0, st, 1, (const int*)tile_counts, tiles,

@@ -186,6 +186,31 @@ def test_kth_with_more_keys_in_the_bracket_than_are_kept(kind):
         assert out.cpu().numpy()[0] == srt[k - 1], (kind, k)
 
 
+@pytest.mark.parametrize("n", [2_000_001, 2_900_002, 3_600_003, (1 << 24) - 1])
+@pytest.mark.parametrize("kind", ["spread", "bimodal", "two values", "far"])
+def test_kth_of_millions_of_scores(n, kind):
+    """Around the sizes from which a bracket's keys are not kept (at the median, at k = 0.87 n and 0.93 n), and the largest:
+    the first pass bins the bracket whether or not it keeps the keys; "far": the sample sees none of the scores around rank k, so
+    the bracket is given up.  Against torch's sort."""
+    import torch
+    from paper_2605_08134_b200 import dare
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(n)
+    s = torch.empty(n, device="cuda").normal_(0, 1, generator=gen)
+    if kind == "bimodal":
+        hot = torch.rand(n, device="cuda", generator=gen) < 0.13
+        s = torch.where(hot, s.abs() + 0.3, s * 1e-5)
+    elif kind == "two values":
+        s = torch.where(s < 0.25, -3.0, 0.25)
+    elif kind == "far":
+        s[torch.arange(256, device="cuda") * n // 256] = 50.0
+    out = torch.zeros(1, device="cuda")
+    srt = torch.sort(s).values
+    for k in (1, n // 8, n // 2, int(0.87 * n), int(0.93 * n), n - 1):
+        assert dare.dare_score_kth(s.data_ptr(), n, k, out.data_ptr(), torch.cuda.current_stream().cuda_stream) == 0
+        assert out.item() == srt[k - 1].item(), (kind, k)
+
+
 @pytest.mark.parametrize("n", [1, 3, 4096, 65_536, 65_537, 262_143, 262_144, 262_145])
 def test_compaction_in_one_launch_and_in_three(n):
     """Around the size up to which one cluster compacts in a single launch: list, count, nothing past the list touched."""
