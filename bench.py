@@ -399,11 +399,12 @@ def run_ours(args):
     #   in and out, index list out.
     many = shape.batch * ((shape.seq + 127) // 128) > 8
     n_out = n if ((mode & 2) and many) else T
-    # ... and of Q, from a size on, every token's scoring head (a stream of x_norm) and the refresh set's rows, in the K/V slot
-    score_first = bool(mode & 2) and many and 2.0 * T * d * d >= (34e9 if mode & 1 else 80e9)
+    # ... and of Q, where the step says that it took that schedule, every token's scoring head (a stream of x_norm, the stored
+    # query in and out) and the refresh set's rows, in the K/V slot
+    score_first = bool(layers[0].forms() & dare.FORM_SCORE_FIRST)
     n_q = n if score_first else 0
     work = {
-        "q_gemm": ("hbm", 2.0 * T * d) if score_first else ("tensor", 2.0 * T * d * d),
+        "q_gemm": ("hbm", 2.0 * T * d + 8.0 * T * shape.head_dim) if score_first else ("tensor", 2.0 * T * d * d),
         "out_gemm": ("tensor", 2.0 * n_out * d * d),
         "kv_gemm": ("hbm", 2.0 * d * d * 2 + 3.0 * n_kv * d * 2) if n_kv <= 215 else ("tensor", 4.0 * n_kv * d * d + 2.0 * n_q * d * d),
         "attention": ("tensor", 4.0 * n_o * shape.seq * d),   # n_o counts rows of all sequences

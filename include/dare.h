@@ -281,6 +281,17 @@ dare_status_t dare_select_compact_static(const float* scores, int64_t n_tokens, 
 /* Number of kernels the last dare_layer_step enqueued (for launch accounting in benchmarks). */
 int dare_layer_last_launch_count(const dare_layer_t* layer);
 
+/* Which of its forms the last dare_layer_step took where its launch rules have a choice that the shapes of its inputs do not
+ * show (an OR of DARE_FORM_*): for tests that are about one of them, and for accounting of the work a step really did. */
+enum {
+  DARE_FORM_SCORE_FIRST = 1,   /* many tokens, attention outputs reused: the scoring head of every token projected first, the other
+                                * queries of the refresh set only, behind the selection */
+  DARE_FORM_SPLIT_Q = 2,       /* fp32: the Q projection, the K/V projection, the output projection ran on the tensor cores, operands */
+  DARE_FORM_SPLIT_KV = 4,      /* split into three bf16 parts */
+  DARE_FORM_SPLIT_OUT = 8
+};
+int dare_layer_last_forms(const dare_layer_t* layer);
+
 const char* dare_status_string(dare_status_t s);
 
 /* Version of this ABI (bumped when a signature changes). */

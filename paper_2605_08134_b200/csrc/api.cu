@@ -124,8 +124,8 @@ dare_status_t step_simt(dare_layer_t* L, const T* x, const StepGeom& g, int mode
   const Buffers& B = L->buf;
   const bool kv_sparse = L->has_prev && (mode & DARE_MODE_KV);
   const bool o_sparse = L->has_prev && (mode & DARE_MODE_O);
-  const SimtStep s = {g, B.rope_cs, B.q_prev, B.scores, B.q_raw, L->has_prev ? 1 : 0, B.status};
-  int launches = 0;
+  int launches = 0, forms = 0;
+  const SimtStep s = {g, B.rope_cs, B.q_prev, B.scores, B.q_raw, L->has_prev ? 1 : 0, B.status, &forms};
   prof_begin(L);
   // Alg. 1/2 line 1
   prof_mark(L, SLOT_NORM, st);
@@ -149,6 +149,7 @@ dare_status_t step_simt(dare_layer_t* L, const T* x, const StepGeom& g, int mode
   CUDA_TRY(launch_out_simt<T>(s, (const T*)B.oc, (const T*)L->w.w_o, y, st)); ++launches;
   prof_end(L, st);
   L->last_launches = launches;
+  L->last_forms = forms;
   CUDA_TRY(cudaGetLastError());
   return DARE_OK;
 }
@@ -261,6 +262,7 @@ dare_status_t dare_layer_create(const dare_layer_config_t* cfg, const dare_layer
   L->batch = 0;
   L->kv_len = 0;
   L->last_launches = 0;
+  L->last_forms = 0;
   L->tc = nullptr;
   L->prof_on = false;
   L->prof_n = 0;
@@ -696,6 +698,10 @@ dare_status_t dare_select_compact(const float* scores, int64_t n_tokens, float t
 int dare_layer_last_launch_count(const dare_layer_t* L) {
   if (check_handle(L) != DARE_OK) return 0;
   return L->last_launches;
+}
+int dare_layer_last_forms(const dare_layer_t* L) {
+  if (check_handle(L) != DARE_OK) return 0;
+  return L->last_forms;
 }
 
 }  // extern "C"

@@ -169,6 +169,7 @@ struct SimtStep {
   float* q_raw;          // heads wider than 64: [T, head_dim] scratch
   int has_prev;
   int* status;
+  int* forms;            // DARE_FORM_* of what was launched are added
 };
 // Q projection with its tail: score of the scoring head against q_prev (fp32, cache rows), q_prev update, rotary
 // embedding, store in the layer dtype (heads wider than 64: the score is a launch of its own).

@@ -50,6 +50,7 @@ struct dare_layer {
   int batch;
   int kv_len;
   int last_launches;
+  int last_forms;   // DARE_FORM_* of the last step
   dare::StepGeom last_geom;
   dare::TcState* tc;
   // optional per-kernel timing (events recorded between the kernels of a step)

@@ -309,7 +309,7 @@ cudaError_t launch_sgemm_as(const SgemmParams& p, int n_tiles, cudaStream_t st) 
 }
 // rows_likely: rows that the launch is sized for (a gathered launch's count is known to the device only).
 template <typename T, int EPI>
-cudaError_t launch_sgemm(const SgemmParams& p, int rows_likely, cudaStream_t st) {
+cudaError_t launch_sgemm(const SgemmParams& p, int rows_likely, int* forms, cudaStream_t st) {
   if (p.rows <= 0) return cudaSuccess;
   const int n_tiles = (p.g.d / 2 + 31) / 32 * (EPI == SG_KV ? 2 : 1);
   // What a launch takes is its waves of one tile an SM times the tile height over the rate of its inner loop (above), plus
@@ -340,7 +340,10 @@ cudaError_t launch_sgemm(const SgemmParams& p, int rows_likely, cudaStream_t st)
   if constexpr (std::is_same<T, float>::value) {
     const int tiles = p.g.d / 64 * (EPI == SG_KV ? 2 : 1) * ((rows_likely + 127) / 128);
     const float there = (float)((tiles + kSms - 1) / kSms) * (4.5f + (p.g.d <= 1024 ? 1.f : 1.2f) * (float)(p.g.d / 64));
-    if (p.g.d % 64 == 0 && there < 0.42f * (float)p.g.d / 1024.f * c[best]) return launch_gemm_f32(EPI, p, st);
+    if (p.g.d % 64 == 0 && there < 0.42f * (float)p.g.d / 1024.f * c[best]) {
+      *forms |= EPI == SG_Q ? DARE_FORM_SPLIT_Q : (EPI == SG_KV ? DARE_FORM_SPLIT_KV : DARE_FORM_SPLIT_OUT);
+      return launch_gemm_f32(EPI, p, st);
+    }
   }
   switch (best) {
     case 0: return launch_sgemm_as<T, EPI, 6, 4, 2>(p, n_tiles, st);
@@ -639,7 +642,7 @@ cudaError_t launch_q_simt(const SimtStep& s, const T* xn, const T* w_q, T* q, cu
   p.rope = reinterpret_cast<const float2*>(s.rope_cs); p.q_prev = s.q_prev; p.scores = s.scores; p.q_raw = s.q_raw;
   p.has_prev = s.has_prev; p.status = s.status;
   ++*launches;
-  if (cudaError_t e = launch_sgemm<T, SG_Q>(p, p.rows, st); e != cudaSuccess) return e;
+  if (cudaError_t e = launch_sgemm<T, SG_Q>(p, p.rows, s.forms, st); e != cudaSuccess) return e;
   if (s.g.head_dim <= 64) return cudaSuccess;
   ++*launches;
   return launch_pdl(score_kernel, dim3((p.rows + 7) / 8), dim3(256), 0, st, 1, s.q_raw, s.q_prev, s.scores, p.has_prev, s.g);
@@ -651,7 +654,7 @@ cudaError_t launch_kv_simt(const SimtStep& s, const T* xn, const int* idx, const
   p.a = xn; p.idx = idx; p.count = count; p.g = s.g; p.rows = s.g.tokens(); p.w0 = w_k; p.w1 = w_v; p.out0 = kc; p.out1 = vc;
   p.rope = reinterpret_cast<const float2*>(s.rope_cs); p.status = s.status;
   // (a refresh set is sized for a quarter of the tokens)
-  return launch_sgemm<T, SG_KV>(p, idx ? (p.rows + 3) / 4 : p.rows, st);
+  return launch_sgemm<T, SG_KV>(p, idx ? (p.rows + 3) / 4 : p.rows, s.forms, st);
 }
 template <typename T>
 cudaError_t launch_attention_simt(const SimtStep& s, const T* q, const T* kc, const T* vc, const int* idx,
@@ -669,7 +672,7 @@ template <typename T>
 cudaError_t launch_out_simt(const SimtStep& s, const T* oc, const T* w_o, T* y, cudaStream_t st) {
   SgemmParams p = {};
   p.a = oc; p.a_cache_rows = 1; p.g = s.g; p.rows = s.g.tokens(); p.w0 = w_o; p.out0 = y; p.status = s.status;
-  return launch_sgemm<T, SG_OUT>(p, p.rows, st);
+  return launch_sgemm<T, SG_OUT>(p, p.rows, s.forms, st);
 }
 #define SIMT_LAUNCHES(T)                                                                                                   \
   template cudaError_t launch_q_simt<T>(const SimtStep&, const T*, const T*, T*, cudaStream_t, int*);                     \

@@ -155,7 +155,7 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
     kv_beside_q = beside < behind;
   }
   // A projection of the refresh set's rows of x_norm (p.idx, p.count): a compact copy of them, then the launch in three forms,
-  // each of which looks at the count: listed in two-CTA and in one-CTA tiles; from gate_kv refreshed tokens on dense, every row
+  // each of which looks at the count (launches counted here): listed in two-CTA and in one-CTA tiles; from gate_kv refreshed tokens on dense, every row
   // of the step projected and the refresh set's stored.
   auto listed_projection = [&](int epi, GemmParams p, const CUtensorMap& b0, const CUtensorMap& b1, const CUtensorMap& b2, const CUtensorMap& b0h,
                                const CUtensorMap& b1h, const CUtensorMap& b2h, int n_tiles) {
@@ -281,10 +281,10 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
           // row of the step projected, the rows of the refresh set stored (the others keep their cached K and V)
           if (q_listed) p.out2 = (bf16*)B.q;
           e = listed_projection(q_listed ? EPI_QKV : EPI_KV, p, S.w_k, S.w_v, S.w_q, S.w_k128, S.w_v128, S.w_q128, n_listed_tiles);
-          --launches;                                    // (counted below)
-        } else
+        } else {
           e = launch_gemm_tc(EPI_KV, 256, S.a_xn, S.w_k, S.w_v, p, n_tiles, m_tiles, 1, st);
-        ++launches;
+          ++launches;
+        }
       }
     } else {
       prof_mark(L, SLOT_KV_GEMM, st);
@@ -419,6 +419,7 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
   }
   prof_end(L, st);
   L->last_launches = launches;
+  L->last_forms = q_listed ? DARE_FORM_SCORE_FIRST : 0;
   if (cudaGetLastError() != cudaSuccess) return DARE_ERR_CUDA;
   return DARE_OK;
 }

@@ -15,6 +15,7 @@ OK = 0
 ERR_INVALID_ARG, ERR_SHAPE, ERR_STATE, ERR_ALIGN, ERR_WORKSPACE, ERR_CUDA, ERR_TIMEOUT, ERR_UNSUPPORTED, \
     ERR_DEVICE_CHECK = range(1, 10)
 MODE_DENSE, MODE_KV, MODE_O, MODE_BOTH = 0, 1, 2, 3
+FORM_SCORE_FIRST, FORM_SPLIT_Q, FORM_SPLIT_KV, FORM_SPLIT_OUT = 1, 2, 4, 8
 F32, BF16 = 0, 1
 PATH_AUTO, PATH_SIMT, PATH_TENSOR = 0, 1, 2
 
@@ -82,6 +83,7 @@ def _load():
         "dare_layer_export_state": (C.c_int, [vp, vp, sz, vp]),
         "dare_layer_import_state": (C.c_int, [vp, vp, sz, vp]),
         "dare_layer_last_launch_count": (C.c_int, [vp]),
+        "dare_layer_last_forms": (C.c_int, [vp]),
         "dare_layer_set_profiling": (C.c_int, [vp, i32]),
         "dare_layer_last_kernel_times": (C.c_int, [vp, vp, vp, i32, C.POINTER(C.c_int)]),
         "dare_kernel_slot_name": (C.c_char_p, [C.c_int]),
@@ -222,6 +224,11 @@ def dare_layer_import_state(handle, src_ptr, nbytes, stream=0) -> int:
 
 def dare_layer_last_launch_count(handle) -> int:
     return _lib.dare_layer_last_launch_count(handle)
+
+
+def dare_layer_last_forms(handle) -> int:
+    """FORM_* flags of the last step."""
+    return _lib.dare_layer_last_forms(handle)
 
 
 def dare_layer_set_profiling(handle, enable: int) -> int:
@@ -488,6 +495,9 @@ class Layer:
 
     def launch_count(self) -> int:
         return dare_layer_last_launch_count(self.handle)
+
+    def forms(self) -> int:
+        return dare_layer_last_forms(self.handle)
 
     def close(self):
         if getattr(self, "handle", None):

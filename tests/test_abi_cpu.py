@@ -98,3 +98,4 @@ def test_calls_on_a_null_handle(dare):
     assert dare.dare_layer_status(None) == dare.ERR_INVALID_ARG
     assert dare.dare_layer_state_bytes(None) == 0
     assert dare.dare_layer_last_launch_count(None) == 0
+    assert dare.dare_layer_last_forms(None) == 0

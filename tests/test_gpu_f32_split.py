@@ -9,16 +9,16 @@ from tests import parity
 pytestmark = pytest.mark.gpu
 
 CASES = [
-    # d_model, head_dim, batch, seq, window
-    (1024, 64, 2, 385, 0),       # the last row tile has two rows
-    (1024, 128, 3, 300, 299),    # scores from the stored head; windows
-    (512, 32, 5, 230, 0),        # two heads a tile
-    (768, 256, 3, 257, 0),       # a head over four tiles
-    (992, 32, 3, 257, 0),        # width no multiple of 64: stays on the CUDA cores, tiles of 96 and 48 rows
-    (448, 64, 7, 200, 190),      # seven blocks (an odd number), seven column tiles
-    (128, 32, 4, 2100, 0),       # the narrowest that it takes: two blocks, one chain
-    (192, 64, 4, 600, 0),        # three blocks, the last in a chain of its own
-    (2048, 128, 1, 130, 0),      # wider than the launch rule's other sizes: 32 blocks, chains of four
+    # d_model, head_dim, batch, seq, window, projections that run on the tensor cores: of a dense step, with listed K/V rows
+    (1024, 64, 2, 385, 0, "QKO", "QKO"),      # the last row tile has two rows
+    (1024, 128, 3, 300, 299, "QKO", "QKO"),   # scores from the stored head; windows
+    (512, 32, 5, 230, 0, "QKO", "QO"),        # two heads a tile
+    (768, 256, 3, 257, 0, "QKO", "QKO"),      # a head over four tiles
+    (992, 32, 3, 257, 0, "", ""),             # width no multiple of 64: stays on the CUDA cores, tiles of 96 and 48 rows
+    (448, 64, 7, 200, 190, "QKO", "QO"),      # seven blocks (an odd number), seven column tiles
+    (128, 32, 4, 2100, 0, "QKO", "QO"),       # the narrowest that it takes: two blocks, one chain
+    (192, 64, 4, 600, 0, "K", ""),            # three blocks, the last in a chain of its own
+    (2048, 128, 1, 130, 0, "QKO", "QO"),      # wider than the launch rule's other sizes: 32 blocks, chains of four
 ]
 
 
@@ -29,13 +29,19 @@ def _layer(shape, w):
     return dare.Layer(shape, w)
 
 
+def _split(layer):
+    """Which projections of its last step ran on the tensor cores: of Q, K (and V), O."""
+    from paper_2605_08134_b200 import dare
+    return "".join(n for n, f in (("Q", dare.FORM_SPLIT_Q), ("K", dare.FORM_SPLIT_KV), ("O", dare.FORM_SPLIT_OUT)) if layer.forms() & f)
+
+
 def _shape(d, hd, batch, seq):
     return wl.LayerShape("split", d, d // hd, hd, batch, seq, seq // 2, 1e4, wl.DTYPE_F32)
 
 
 @pytest.mark.parametrize("case", range(len(CASES)))
 def test_steps_against_the_oracle(case):
-    d, hd, batch, seq, window = CASES[case]
+    d, hd, batch, seq, window, dense, listed = CASES[case]
     shape = _shape(d, hd, batch, seq)
     w = wl.make_weights(shape, 1700 + case)
     hs = wl.HiddenStream(shape, 1700 + case)
@@ -46,6 +52,7 @@ def test_steps_against_the_oracle(case):
     for mode, frac in [(0, 0.1), (3, 0.2), (1, 0.9), (2, 0.6)]:
         x = hs.advance(wl.uniform_positions(hs.rng, shape, max(1, int(round(frac * seq)))))
         parity.compare_step(g, o, np.ascontiguousarray(x[:, at:]), mode, 0.1, shape, pos_begin=at)
+        assert _split(g) == (listed if mode & 1 else dense)
     g.close()
 
 
@@ -69,6 +76,7 @@ def _values(d, seq, spoil=None, batch=3, rows=0):
         x, batch, seq = x[:1, :rows].contiguous(), 1, rows
     layer = dare.Layer(shape, w)
     layer.step(x, 0, 0.1)
+    assert ("K" in _split(layer)) == (not rows)                  # V by the kernel that the caller is about
     xn = torch.empty_like(x)
     assert dare.dare_rmsnorm(x.data_ptr(), w["rms_gain"].data_ptr(), xn.data_ptr(), batch * seq, d, shape.rms_eps, wl.DTYPE_F32, 0) == 0
     torch.cuda.synchronize()
@@ -81,10 +89,10 @@ def _values(d, seq, spoil=None, batch=3, rows=0):
 def test_accuracy(d, seq):
     """16 products of an accumulator are cut by less than an ulp (2 units of 2^-24 of their sum, half of it on average), the
     adds in registers leave 0.3 ulp each at a chain's, a tree's or the whole sum's size: below 2 units in all, where the CUDA-core
-    kernel's chains of d / 4 products lose sqrt(d / 24) (6.5 at 1024).  Measured 1.2 and 1.3; 3 is asked for."""
+    kernel's chains leave 3.5 and 4.9 at these widths.  Measured 1.2 and 1.3; 2 is asked for."""
     v, xn, wv = _values(d, seq)
     want = xn @ wv.T
-    assert np.linalg.norm(v - want) / np.linalg.norm(want) < 3 * 2.0 ** -24
+    assert np.linalg.norm(v - want) / np.linalg.norm(want) < 2 * 2.0 ** -24
 
 
 def _magnitudes(w, x):
@@ -114,7 +122,7 @@ def test_weights_of_any_size(size):
         w["w_v"].mul_(size / 0.02)
     v, xn, wv = _values(512, 300, spoil)
     want = xn @ wv.T
-    assert np.linalg.norm(v / size - want / size) / np.linalg.norm(want / size) < 3 * 2.0 ** -24
+    assert np.linalg.norm(v / size - want / size) / np.linalg.norm(want / size) < 2 * 2.0 ** -24
 
 
 def test_infinities_and_nan():
