@@ -184,16 +184,23 @@ dare_status_t step_tc(dare_layer* L, const void* x, const StepGeom& g, int mode,
   // and of the other heads only the queries that attend, the refresh set's (Alg. 2 line 8): the scoring head's 128 columns are
   // projected first, and the refresh set's queries behind the selection, beside its K and V where those are listed as well.
   // 4 x 4096 tokens of width 4096, both rules, 15 % refreshed: 1019 -> 684 us; 8 x 1024, output reuse, 13 %: 783 -> 627 us.
-  // With (nearly) all tokens refreshed the scoring head is projected twice, one launch for nothing: 1-2 % of a step, which is
-  // why the rule asks for a query projection of some size (us before / with it, every token refreshed, and at 13 to 30 %):
-  //   both:   1 x 1152 of 4096 (39 GFLOP) 238 / 238, 148 / 139    8 x 1700 of 1536 (64) 490 / 494, 237 / 188
-  //   output: 2 x 1250 of 4096 (84 GFLOP) 419 / 417, 327 / 284    4 x 2300 of 2048 (77) 496 / 507, 349 / 315
-  // A step given its reuse rate knows when more than three quarters will be refreshed.  (Up to eight row tiles the projections
-  // are streams of the weights whatever the rows: 90 us this way against 78 at 512 tokens of width 4096.)
+  // With (nearly) all tokens refreshed the scoring head is projected twice and launches are added that only look at the count, which
+  // costs up to 4 % of a step; hence a query projection of some size, and of some width: the scoring head's launch streams x_norm,
+  // 360 / d of the time of the whole query projection.  In us, one projection of all queries / scoring head first, at 15 %, 50 %
+  // and all tokens refreshed:
+  //   both:   4 x 4096 of 4096  954 / 656, 1737 / 1543, 2808 / 2770    16 x 288 of 2048 (34 GFLOP) 144 / 122, 207 / 193, 243 / 251
+  //           8 x 1700 of 1536  220 / 171, 339 / 294, 489 / 496        32 x 1024 of 1024 300 / 246, 432 / 389, 579 / 595
+  //   output: 4 x 4096 of 4096  1574 / 1186, 2250 / 1905, 2799 / 2764  2 x 1250 of 4096 (84 GFLOP) 324 / 282, 388 / 373, 417 / 416
+  //           4 x 4096 of 2048  593 / 542, 980 / 905, 1046 / 1035      4 x 2300 of 2048 (77 GFLOP) 349 / 315, -, 496 / 507
+  //   widths below the rule's, both: 32 x 1024 of 768 247 / 211, -, 432 / 450    64 x 1100 of 512 396 / 352, -, 826 / 875
+  //           128 x 2100 of 256 964 / 934, -, 2128 / 2247
+  // A step that is given its reuse rate knows when more than three quarters will be refreshed, one with a threshold below every
+  // score that all will.  (Up to eight row tiles the projections are streams of the weights whatever the rows: 90 us this way
+  // against 78 at 512 tokens of width 4096.)
   const int n_listed = (kv_sparse ? 3 : 1) * (d / 256);
   const double q_flop = 2.0 * T_ * (double)d * d;
-  const bool many_known = L->reuse_count >= 0 && 4ll * (T_ - L->reuse_count) > 3ll * T_;
-  const bool q_pays = !many_known && q_flop >= (kv_sparse ? 34e9 : 80e9);
+  const bool many_known = L->reuse_count >= 0 ? 4ll * (T_ - L->reuse_count) > 3ll * T_ : tau < 0.f;
+  const bool q_pays = !many_known && d >= 1024 && q_flop >= (kv_sparse ? 34e9 : 80e9);
   const bool q_listed = o_sparse && m_tiles_dense > 8 && compact_ok && q_pays && persist_pays_listed(n_listed, (T_ + 127) / 128);
   if (q_listed) {
     GemmParams p = base;
