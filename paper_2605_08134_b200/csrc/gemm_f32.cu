@@ -81,7 +81,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f32_kernel(const SgemmParams
   uint64_t* all_done = acc_empty + 1;          // every MMA of the tile complete
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(all_done + 1);
   float* tile = reinterpret_cast<float*>(smem);
-  // of a row: its token (-1: no such row), its row of A (then the first one's, dropped at the end), cache row and position
+  // of a row: its token (-1: no such row, or one whose token failed its check), its row of A (then that of token 0: read, and the
+  // result not written), cache row and position
   __shared__ int s_tok[BM], s_pos[BM];
   __shared__ size_t s_row[BM], s_crow[BM];
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31, tid = (int)threadIdx.x;
@@ -126,7 +127,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f32_kernel(const SgemmParams
   const bool active = m0 < m_eff;                // uniform over the CTA
   if (tid < BM) {
     int t = m0 + tid < m_eff ? (p.idx ? p.idx[m0 + tid] : m0 + tid) : -1;
-    if (p.idx && t != -1 && !token_ok(t, p.g.tokens(), p.status)) t = -1;   // read as zeros, not written
+    if (p.idx && t != -1 && !token_ok(t, p.g.tokens(), p.status)) t = -1;   // (not written)
     const int tc = max(t, 0);
     s_tok[tid] = t;
     s_pos[tid] = p.g.position(tc);

@@ -152,7 +152,7 @@ gemm_persist_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
 
   const int KB = p.K / BK;
   const int n_rows = GATHER ? checked_count(*p.count, p.m_total, p.status) : 0;
-  // (PAIR: units = column tiles x pairs of row tiles; this CTA's row tile of unit u is 2 * (u / n_tiles) + pr, and
+  // (PAIR: units = column tiles x pairs of row tiles, in the order of tile_of; this CTA has row tile pr of a unit's pair, and
   // a row tile past the end of an odd count runs the main loop for its partner's sake and finishes no rows)
   const int m_tiles_live = GATHER ? (n_rows + BM - 1) / BM : p.m_tiles;
   int total_tiles = PAIR ? n_tiles * ((m_tiles_live + 1) / 2) : (GATHER ? m_tiles_live * n_tiles : total_tiles_dense);

@@ -246,7 +246,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
   // that they stream in while that kernel drains.  Everything it produced is needed only after pdl_wait().
   // (Four stages of them: more only take bandwidth from that kernel's tail.  Six / four / three / two early stages, step in us:
   // 2 x 32 rows of width 4096 60.8 / 59.9 / 60.0 / 60.9, 2 x 512 of 2048, heads of 64, 56.9 / 56.1 / 56.0 / 55.8, 2 x 128 of 2048
-  // 44.8 / 44.0 / 44.1 / 44.3, 512 of 4096 73.4 / 73.0 / 73.0 / 73.2.)
+  // 44.8 / 44.0 / 44.1 / 44.3, 512 of 4096 73.4 / 73.0 / 73.0 / 73.2.  Against six, at widths 256 to 2048, 32 to 1024 rows, every
+  // mode: within 1 %, but for dense steps of 32 to 100 rows of 1536, 1.5-2.2 % longer, and of 256 rows of 2048, 1.5 %; asking for all
+  // of a share of up to six blocks lost 1-4 % nearly everywhere.)
   constexpr int EARLY = 4;
   const int n_early = likely && iter == 0 ? (KB / cl_splits < EARLY ? KB / cl_splits : EARLY) : 0;
   if (warp == 0 && lane == 0) {
