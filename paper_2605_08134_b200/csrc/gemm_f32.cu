@@ -10,13 +10,17 @@
 // its 24 bits nearly always), only the small products, 2^-8 of the sum and less, add up over the whole reduction, those of scale
 // 2^8 and of 2^16 apart.  The rest is added in fp32 registers, rounded to nearest: the four accumulators of a block of 64 as a
 // tree, the blocks in chains of two to eight, the chains.
-// Error of V against fp64 in units of 2^-24 (2-norms), split / CUDA-core tiles that the launch rule takes otherwise, and (four hh
-// steps into one accumulator, as it was first):
-//   width               128                384                512                1024               4096
-//   zero-mean normal    0.96 / 1.49 (1.39) 1.12 / 2.26 (1.55) 1.18 / 3.47 (1.61) 1.28 / 4.86 (1.83) 1.62 / 6.85 (2.79)
-//   their magnitudes    0.72 / 0.75 (1.45) 0.87 / 0.95 (1.54) 0.77 / 1.46 (1.54) 0.81 / 2.01 (1.67) 0.94 / 2.06 (2.37)
-//   exp(2 normal)       2.24 / 1.32 (8.14) 2.04 / 1.77 (5.99) 2.07 / 2.83 (6.11) 2.13 / 4.29 (5.72) 1.91 / 5.68 (5.59)
-// (the last line: 16 products of one sign that span far more than 2^8, whose small ones are cut where they are lined up)
+// Error of V against fp64 in units of 2^-24 (2-norms), CUDA-core tiles that the launch rule takes otherwise / split, by operands:
+//   width                        128          192          256          384          448          512          1024
+//   zero-mean normal             1.49 / 0.95  2.20 / 0.96  2.51 / 1.06  2.26 / 1.12  3.25 / 1.11  3.47 / 1.18  4.86 / 1.28
+//   their magnitudes             0.75 / 0.72  1.11 / 0.72  1.10 / 0.72  0.95 / 0.87  1.46 / 0.77  1.46 / 0.76  2.01 / 0.82
+//   normal + 1                   0.78 / 0.79  1.07 / 0.71  1.14 / 0.76  0.95 / 0.81  1.40 / 0.71  1.46 / 0.73  1.94 / 0.75
+//   normal, every 61st x 60      1.37 / 1.24  2.32 / 1.24  2.59 / 1.32  2.27 / 1.37  3.37 / 1.36  3.58 / 1.41  4.99 / 1.51
+//   +- exp(2 normal)             1.49 / 1.26  2.42 / 1.20  2.31 / 1.34  2.16 / 1.32  3.02 / 1.37  3.22 / 1.38  4.17 / 1.39
+//   exp(normal)                  0.81 / 0.80  1.10 / 0.73  1.20 / 0.81  0.95 / 0.84  1.50 / 0.79  1.57 / 0.86  2.13 / 0.89
+//   exp(2 normal), one sign      1.28 / 2.25  2.00 / 2.11  2.02 / 1.99  1.68 / 2.09  4.65 / 2.25  3.19 / 2.31  4.41 / 2.51
+// (the last line: 16 products of one sign that span far more than 2^8, whose small ones are cut where they are lined up.  Four hh steps
+// into one accumulator, as it was first: 1.39 to 1.83 on the first line, 1.45 to 1.67 on the second, 5.7 to 8.1 on the last.)
 // Bound by the splitting, which the adding up beside it slows.  The products of one part of A with two parts of W that lie side by
 // side are one MMA, with the accumulators of both scales side by side as well: 16 MMAs a block that read 112 KB of shared memory,
 // not 24 that read 144.  A step of 2 x 384 tokens of width 1024, key and value reuse, 171.5 us on the CUDA cores, 122 here (24 MMAs:

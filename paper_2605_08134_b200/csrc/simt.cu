@@ -329,18 +329,19 @@ cudaError_t launch_sgemm(const SgemmParams& p, int rows_likely, int* forms, cuda
   // fp32 on the tensor cores (gemm_f32.cu) instead?  A unit of the cost above is 0.42 us at width 1024; a tile of 128 rows takes
   // 4.5 us and 1 us a block of 64 k-elements there, 1.2 beyond width 1024, where most of the step's weights come from the HBM.
   // Dense steps in us, here / there with every projection / as the rule below picks for each:
-  //   64 rows of width 384 30.4 / 41.7 / 30.4    2 x 200 of 256 33.9 / 45.5 / 33.9      4 x 1000 of 128 106 / 101 / 99
-  //   2 x 384 of 384 58.1 / 59.1 / 53.8          4 x 400 of 256 73.8 / 68.1 / 68.0      4 x 2200 of 128 360 / 327 / 327
-  //   4 x 400 of 384 131 / 98.7 / 98.8           2 x 128 of 512 42.8 / 53.5 / 42.8      4 x 1000 of 192 162 / 148 / 148
+  //   64 rows of width 384 30.4 / 41.7 / 30.4    2 x 200 of 256 33.9 / 45.5 / 33.9      4 x 1000 of 128 106 / 101 / 106
+  //   2 x 384 of 384 58.1 / 59.1 / 53.8          4 x 400 of 256 73.8 / 68.1 / 68.0      4 x 2200 of 128 360 / 327 / 360
+  //   4 x 400 of 384 131 / 98.7 / 98.8           2 x 128 of 512 42.8 / 53.5 / 42.8      4 x 1000 of 192 162 / 148 / 162
   //   2 x 384 of 512 89.6 / 73.7 / 73.7          300 of 640 67.4 / 68.4 / 64.0          300 of 768 81.9 / 76.4 / 73.5
   //   128 of 1024 66.6 / 77.8 / 66.6             256 of 1024 96.5 / 85.3 / 82.7         4 x 400 of 1024 498 / 275 / 275
   //   64 of 1536 95.5 / 116 / 95.6               100 of 1536 117 / 114 / 109            200 of 1536 174 / 125 / 125
   //   64 of 2048 119 / 147 / 119                 100 of 2048 165 / 140 / 136            200 of 2048 299 / 156 / 156
   //   32 of 4096 211 / 304 / 211                 64 of 4096 305 / 282 / 266             200 of 4096 1052 / 381 / 379
+  // Widths below 256 stay here: little to gain, and short sums are the ones that this kernel rounds least (gemm_f32.cu).
   if constexpr (std::is_same<T, float>::value) {
     const int tiles = p.g.d / 64 * (EPI == SG_KV ? 2 : 1) * ((rows_likely + 127) / 128);
     const float there = (float)((tiles + kSms - 1) / kSms) * (4.5f + (p.g.d <= 1024 ? 1.f : 1.2f) * (float)(p.g.d / 64));
-    if (p.g.d % 64 == 0 && there < 0.42f * (float)p.g.d / 1024.f * c[best]) {
+    if (p.g.d % 64 == 0 && p.g.d >= 256 && there < 0.42f * (float)p.g.d / 1024.f * c[best]) {
       *forms |= EPI == SG_Q ? DARE_FORM_SPLIT_Q : (EPI == SG_KV ? DARE_FORM_SPLIT_KV : DARE_FORM_SPLIT_OUT);
       return launch_gemm_f32(EPI, p, st);
     }

@@ -16,8 +16,9 @@ CASES = [
     (768, 256, 3, 257, 0, "QKO", "QKO"),      # a head over four tiles
     (992, 32, 3, 257, 0, "", ""),             # width no multiple of 64: stays on the CUDA cores, tiles of 96 and 48 rows
     (448, 64, 7, 200, 190, "QKO", "QO"),      # seven blocks (an odd number), seven column tiles
-    (128, 32, 4, 2100, 0, "QKO", "QO"),       # the narrowest that it takes: two blocks, one chain
-    (192, 64, 4, 600, 0, "K", ""),            # three blocks, the last in a chain of its own
+    (256, 32, 4, 500, 0, "QKO", "QO"),        # the narrowest that it takes: four blocks, two chains
+    (320, 64, 4, 600, 0, "QKO", "QO"),        # five blocks, the last in a chain of its own
+    (192, 64, 4, 600, 0, "", ""),             # narrower: stays on the CUDA cores
     (2048, 128, 1, 130, 0, "QKO", "QO"),      # wider than the launch rule's other sizes: 32 blocks, chains of four
 ]
 
